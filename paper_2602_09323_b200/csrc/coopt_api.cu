@@ -3,37 +3,16 @@
 #include <utility>
 #include <vector>
 
-#include "coopt_common.cuh"
+#include "coopt_decode.cuh"
 
 namespace coopt {
 
 int launch_kv_write(const coopt_cache* c, const void* k, const void* v, int64_t stride, const int64_t* slots,
                     int num_tokens, cudaStream_t stream);
-int launch_paged_decode(const coopt_cache* c, const void* q, void* out, const int32_t* block_table,
-                        int32_t max_blocks_per_seq, const int32_t* context_lens, int32_t batch, int32_t num_q_heads,
-                        float sm_scale, int32_t chunk_size, const int32_t* cu_q_lens, void* workspace, int planned_ctas,
-                        cudaStream_t stream);
 int launch_paged_prefill(const coopt_cache* c, const void* q, void* out, const int32_t* cu_q_lens,
                          const int32_t* block_table, int32_t max_blocks_per_seq, const int32_t* context_lens,
                          int32_t batch, int32_t num_q_heads, int32_t total_q, int32_t causal, float sm_scale,
                          void* workspace, cudaStream_t stream);
-size_t decode_workspace_bytes(int planned_ctas, int group, int head_dim, int batch, int num_q_heads, int num_kv_heads,
-                              int max_blocks_per_seq, int chunk_blocks, int max_chunks);
-size_t plan_bytes(int planned_ctas, int batch, int num_kv_heads, int max_blocks_per_seq, int chunk_blocks);
-int launch_decode_plan(const int32_t* block_table, int32_t max_blocks_per_seq, const int32_t* context_lens, int32_t batch,
-                       int32_t num_kv_heads, int32_t num_blocks, int32_t chunk_size, int planned_ctas, void* plan,
-                       cudaStream_t stream);
-int launch_decode_planned(const coopt_cache* c, const void* plan, const void* k_new, const void* v_new, int64_t kv_token_stride,
-                          const int64_t* slot_mapping, const void* q, void* out, int32_t max_blocks_per_seq, int32_t batch,
-                          int32_t num_q_heads, float sm_scale, int32_t chunk_size, const int32_t* cu_q_lens, void* workspace,
-                          int planned_ctas, bool overlap_previous, cudaStream_t stream);
-size_t workspace_control_bytes();
-int decode_planned_ctas(int num_sms, long long upper_blocks);
-int decode_max_batch();
-int decode_counter_slots();
-int decode_max_chunk_blocks();
-void chunk_partial_offsets(int batch, int num_q_heads, int head_dim, int max_chunks, size_t* o, size_t* m, size_t* l);
-
 const DeviceInfo* device_info() {
   static DeviceInfo info[64];
   static bool known[64] = {};
@@ -83,12 +62,38 @@ int max_chunks_of(int max_blocks_per_seq, int chunk_size) {
   return static_cast<int>((static_cast<long long>(max_blocks_per_seq) * kBlockSize + chunk_size - 1) / chunk_size);
 }
 
-// number of CTAs planned for a decode-style launch; the same on the sizing and the launching side
-int planned_ctas(int batch, int num_kv_heads, int max_blocks_per_seq) {
+int ctas_of(int batch, int num_kv_heads, int max_blocks_per_seq, int chunk_size) {
   const DeviceInfo* di = device_info();
-  const int sms = di ? di->num_sms : 148;
-  return decode_planned_ctas(sms, static_cast<long long>(batch) * num_kv_heads * max_blocks_per_seq);
+  return decode_ctas(di ? di->num_sms : 148, batch, num_kv_heads, max_blocks_per_seq, chunk_size / kBlockSize);
 }
+
+// The sizes that coopt_plan_bytes and coopt_workspace_bytes report are part of the interface: pools are laid out by them,
+// and coopt_paged_decode_static refuses by them.  They are those of a plan that lists every CTA's blocks and of a
+// workspace with room for one -- more than the kernels use now, except for the pieces of small problems.
+long long listed_plan_ctas(int batch, int num_kv_heads, int max_blocks_per_seq) {
+  const DeviceInfo* di = device_info();
+  const long long sms = di ? di->num_sms : 148, need = (static_cast<long long>(batch) * num_kv_heads * max_blocks_per_seq + 2031) / 2032;
+  return need > sms ? need : sms;
+}
+size_t listed_plan_bytes(int batch, int num_kv_heads, int max_blocks_per_seq, int chunk_blocks) {
+  const long long P = listed_plan_ctas(batch, num_kv_heads, max_blocks_per_seq);
+  const long long units = static_cast<long long>(batch) * num_kv_heads, all = units * max_blocks_per_seq;
+  long long blocks = (all + P - 1) / P + 1;
+  if (chunk_blocks > 0) {
+    const long long chunks = units * ((max_blocks_per_seq + chunk_blocks - 1) / chunk_blocks);
+    blocks = ((chunks + P - 1) / P + 1) * chunk_blocks;
+  } else if (blocks < 32) {
+    blocks = 32;
+  }
+  if (blocks > all) blocks = all;
+  long long segments = (blocks < units ? blocks : units) + 3;
+  if (chunk_blocks > 0) segments += blocks / chunk_blocks + 1;
+  if (segments > blocks + 2) segments = blocks + 2;
+  const long long rounds = (segments + 31) / 32 + (blocks + 1023) / 1024 + 1;
+  const long long region = (rounds * 80 + segments * 64 + blocks * 4 + 64 + 127) / 128 * 128;
+  return 256 + static_cast<size_t>(P) * region + 4096;
+}
+size_t larger(size_t a, size_t b) { return a > b ? a : b; }
 
 }  // namespace
 
@@ -117,6 +122,23 @@ int check_attention_shapes(const coopt_cache* c, const void* q, void* out, int32
   // the planner indexes (sequence, kv head, block) triples with 31 bits
   if (static_cast<long long>(batch) * c->num_kv_heads * max_blocks_per_seq >= (1ll << 31)) return COOPT_ERR_UNSUPPORTED;
   return COOPT_OK;
+}
+
+// What every decode-style launch has in common.
+static DecodeCall attention_call(const coopt_cache* c, const void* q, void* out, int32_t max_blocks_per_seq, int32_t batch, int32_t num_q_heads,
+                                 int32_t chunk_size, float sm_scale, void* workspace) {
+  DecodeCall a = {};
+  a.q = q;
+  a.out = out;
+  a.max_blocks_per_seq = max_blocks_per_seq;
+  a.batch = batch;
+  a.num_q_heads = num_q_heads;
+  a.chunk_size = chunk_size;
+  a.sm_scale = sm_scale;
+  a.workspace = workspace;
+  a.ctas = ctas_of(batch, c->num_kv_heads, max_blocks_per_seq, chunk_size);
+  a.order = kAfterPrevious;
+  return a;
 }
 
 }  // namespace coopt
@@ -169,9 +191,13 @@ size_t coopt_workspace_bytes(int32_t batch, int32_t num_q_heads, int32_t num_kv_
   (void)total_q;
   if (batch < 0 || num_q_heads <= 0 || num_kv_heads <= 0 || max_blocks_per_seq <= 0 || chunk_size < 0) return 0;
   const int group = (num_q_heads + num_kv_heads - 1) / num_kv_heads;
-  const int P = planned_ctas(batch, num_kv_heads, max_blocks_per_seq);
   const int mc = chunk_size > 0 ? max_chunks_of(max_blocks_per_seq, chunk_size) : 0;
-  return decode_workspace_bytes(P, group, head_dim, batch, num_q_heads, num_kv_heads, max_blocks_per_seq, chunk_size / kBlockSize, mc);
+  const size_t used = decode_workspace_bytes(ctas_of(batch, num_kv_heads, max_blocks_per_seq, chunk_size), group, head_dim, batch, num_q_heads, mc);
+  const size_t pieces = static_cast<size_t>(2) * listed_plan_ctas(batch, num_kv_heads, max_blocks_per_seq) * group * (head_dim + 2) * 4;
+  const size_t partials = static_cast<size_t>(batch) * num_q_heads * mc * (head_dim + 2) * 4;
+  const size_t listed = (workspace_control_bytes() + pieces + (mc > 0 ? partials + 256 : 0) + 511) / 256 * 256 +
+                        listed_plan_bytes(batch, num_kv_heads, max_blocks_per_seq, chunk_size / kBlockSize);
+  return larger(used, listed);
 }
 
 int coopt_workspace_init(void* workspace, size_t workspace_bytes, void* stream) {
@@ -201,9 +227,10 @@ int coopt_paged_decode(const coopt_cache* cache, const void* q, void* out, const
   if (!workspace || workspace_bytes < coopt_workspace_bytes(batch, num_q_heads, cache->num_kv_heads, cache->head_dim,
                                                             max_blocks_per_seq, 0, batch))
     return COOPT_ERR_WORKSPACE;
-  const int P = planned_ctas(batch, cache->num_kv_heads, max_blocks_per_seq);
-  return launch_paged_decode(cache, q, out, block_table, max_blocks_per_seq, context_lens, batch, num_q_heads, sm_scale,
-                             0, nullptr, workspace, P, static_cast<cudaStream_t>(stream));
+  DecodeCall a = attention_call(cache, q, out, max_blocks_per_seq, batch, num_q_heads, 0, sm_scale, workspace);
+  a.block_table = block_table;
+  a.context_lens = context_lens;
+  return launch_decode(cache, a, static_cast<cudaStream_t>(stream));
 }
 
 int coopt_decode_step(const coopt_cache* cache, const void* k_new, const void* v_new, int64_t kv_token_stride,
@@ -221,14 +248,16 @@ int coopt_decode_step(const coopt_cache* cache, const void* k_new, const void* v
     return COOPT_ERR_WORKSPACE;
   rc = launch_kv_write(cache, k_new, v_new, kv_token_stride, slot_mapping, batch, static_cast<cudaStream_t>(stream));
   if (rc != COOPT_OK) return rc;
-  const int P = planned_ctas(batch, cache->num_kv_heads, max_blocks_per_seq);
-  return launch_paged_decode(cache, q, out, block_table, max_blocks_per_seq, context_lens, batch, num_q_heads, sm_scale,
-                             0, nullptr, workspace, P, static_cast<cudaStream_t>(stream));
+  DecodeCall a = attention_call(cache, q, out, max_blocks_per_seq, batch, num_q_heads, 0, sm_scale, workspace);
+  a.block_table = block_table;
+  a.context_lens = context_lens;
+  a.order = kDependent;                      // on the write in front of it
+  return launch_decode(cache, a, static_cast<cudaStream_t>(stream));
 }
 
 size_t coopt_plan_bytes(int32_t batch, int32_t num_kv_heads, int32_t max_blocks_per_seq, int32_t chunk_size) {
   if (batch <= 0 || num_kv_heads <= 0 || max_blocks_per_seq <= 0 || chunk_size < 0 || chunk_size % kBlockSize != 0) return 0;
-  return plan_bytes(planned_ctas(batch, num_kv_heads, max_blocks_per_seq), batch, num_kv_heads, max_blocks_per_seq, chunk_size / kBlockSize);
+  return larger(decode_plan_bytes(batch, max_blocks_per_seq), listed_plan_bytes(batch, num_kv_heads, max_blocks_per_seq, chunk_size / kBlockSize));
 }
 
 static int check_plan_args(int32_t batch, int32_t num_kv_heads, int32_t max_blocks_per_seq, int32_t chunk_size, const void* plan,
@@ -250,8 +279,8 @@ int coopt_decode_plan(const int32_t* block_table, int32_t max_blocks_per_seq, co
   if (rc != COOPT_OK) return rc;
   if (!block_table || !context_lens || num_blocks <= 0) return COOPT_ERR_INVALID_ARG;
   if (batch == 0) return COOPT_OK;
-  return launch_decode_plan(block_table, max_blocks_per_seq, context_lens, batch, num_kv_heads, num_blocks, chunk_size,
-                            planned_ctas(batch, num_kv_heads, max_blocks_per_seq), plan, static_cast<cudaStream_t>(stream));
+  return launch_decode_plan(block_table, max_blocks_per_seq, context_lens, batch, num_kv_heads, num_blocks, chunk_size, plan,
+                            static_cast<cudaStream_t>(stream));
 }
 
 int coopt_decode_step_planned(const coopt_cache* cache, const void* plan, size_t plan_bytes_given, const void* k_new,
@@ -271,10 +300,11 @@ int coopt_decode_step_planned(const coopt_cache* cache, const void* plan, size_t
   if (!workspace || workspace_bytes < coopt_workspace_bytes(batch, num_q_heads, cache->num_kv_heads, cache->head_dim,
                                                             max_blocks_per_seq, chunk_size, batch))
     return COOPT_ERR_WORKSPACE;
-  return launch_decode_planned(cache, plan, k_new, v_new, kv_token_stride, slot_mapping, q, out, max_blocks_per_seq, batch,
-                               num_q_heads, sm_scale, chunk_size, nullptr, workspace,
-                               planned_ctas(batch, cache->num_kv_heads, max_blocks_per_seq),
-                               (flags & COOPT_FLAG_OVERLAP_PREVIOUS) != 0, static_cast<cudaStream_t>(stream));
+  DecodeCall a = attention_call(cache, q, out, max_blocks_per_seq, batch, num_q_heads, chunk_size, sm_scale, workspace);
+  a.plan = plan;
+  a.k_new = k_new; a.v_new = v_new; a.slot_mapping = slot_mapping; a.kv_token_stride = kv_token_stride;
+  a.order = (flags & COOPT_FLAG_OVERLAP_PREVIOUS) != 0 ? kOverlapPrevious : kAfterPrevious;
+  return launch_decode(cache, a, static_cast<cudaStream_t>(stream));
 }
 
 int coopt_decode_layers(const coopt_layer_io* layers, int32_t num_layers, int64_t kv_token_stride, const int32_t* block_table,
@@ -302,15 +332,16 @@ int coopt_decode_layers(const coopt_layer_io* layers, int32_t num_layers, int64_
   if (batch == 0) return COOPT_OK;
   if (!workspace || workspace_bytes < coopt_workspace_bytes(batch, num_q_heads, c0->num_kv_heads, c0->head_dim, max_blocks_per_seq, 0, batch))
     return COOPT_ERR_WORKSPACE;
-  const int P = planned_ctas(batch, c0->num_kv_heads, max_blocks_per_seq);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  rc = launch_decode_plan(block_table, max_blocks_per_seq, context_lens, batch, c0->num_kv_heads, c0->num_blocks, 0, P, plan, st);
+  rc = launch_decode_plan(block_table, max_blocks_per_seq, context_lens, batch, c0->num_kv_heads, c0->num_blocks, 0, plan, st);
   for (int32_t l = 0; l < num_layers && rc == COOPT_OK; ++l) {
     const coopt_layer_io& io = layers[l];
-    // layer l > 0 may start while layer l - 1 drains: its copy warp reads only the plan and its own cache
-    rc = launch_decode_planned(io.cache, plan, io.k_new, io.v_new, kv_token_stride, io.slot_mapping, io.q, io.out, max_blocks_per_seq,
-                               batch, num_q_heads, sm_scale, 0, nullptr, workspace, P,
-                               l > 0 && (flags & COOPT_FLAG_OVERLAP_PREVIOUS) != 0, st);
+    DecodeCall a = attention_call(io.cache, io.q, io.out, max_blocks_per_seq, batch, num_q_heads, 0, sm_scale, workspace);
+    a.plan = plan;
+    a.k_new = io.k_new; a.v_new = io.v_new; a.slot_mapping = io.slot_mapping; a.kv_token_stride = kv_token_stride;
+    // layer l > 0 may read the plan and its own cache while layer l - 1 drains
+    a.order = l > 0 && (flags & COOPT_FLAG_OVERLAP_PREVIOUS) != 0 ? kOverlapPrevious : kDependent;
+    rc = launch_decode(io.cache, a, st);
   }
   return rc;
 }
@@ -330,9 +361,11 @@ int coopt_paged_chunked(const coopt_cache* cache, const void* q, void* out, cons
     return COOPT_ERR_WORKSPACE;
   if (total_q == batch) {
     // one query token per sequence: the Opt-Pa chunk-and-merge decode
-    const int P = planned_ctas(batch, cache->num_kv_heads, max_blocks_per_seq);
-    return launch_paged_decode(cache, q, out, block_table, max_blocks_per_seq, context_lens, batch, num_q_heads,
-                               sm_scale, chunk_size, cu_q_lens, workspace, P, static_cast<cudaStream_t>(stream));
+    DecodeCall a = attention_call(cache, q, out, max_blocks_per_seq, batch, num_q_heads, chunk_size, sm_scale, workspace);
+    a.block_table = block_table;
+    a.context_lens = context_lens;
+    a.cu_q_lens = cu_q_lens;
+    return launch_decode(cache, a, static_cast<cudaStream_t>(stream));
   }
   return launch_paged_prefill(cache, q, out, cu_q_lens, block_table, max_blocks_per_seq, context_lens, batch,
                               num_q_heads, total_q, causal, sm_scale, workspace, static_cast<cudaStream_t>(stream));
@@ -397,31 +430,28 @@ int coopt_decode_step_host(const coopt_cache* cache, const void* step_inputs_hos
   if (rc != COOPT_OK) return rc;
   if (!workspace || workspace_bytes < coopt_workspace_bytes(batch, num_q_heads, hkv, d, max_blocks_per_seq, 0, batch)) return COOPT_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const int P = planned_ctas(batch, hkv, max_blocks_per_seq);
+  DecodeCall a = attention_call(cache, dev + s.q, dev + s.out, max_blocks_per_seq, batch, num_q_heads, 0, sm_scale, workspace);
+  a.plan = plan;
+  a.k_new = dev + s.k_new; a.v_new = dev + s.v_new; a.slot_mapping = reinterpret_cast<const int64_t*>(dev + s.slot_mapping);
+  a.kv_token_stride = static_cast<int64_t>(hkv) * d;
+  a.order = kDependent;
   // Host buffers that are page-locked and mapped into the device's address space are used where they are: the
   // kernel fetches the queries and the new tokens from them and stores the result into them, and only the
   // index arrays (slots, block table, context lengths: what the planner walks) are copied to the device.
   const uint8_t* in_dev = mapped_host_pointer(step_inputs_host);
   uint8_t* out_dev = const_cast<uint8_t*>(mapped_host_pointer(out_host));
-  if (in_dev != nullptr && out_dev != nullptr && reinterpret_cast<uintptr_t>(in_dev) % 16 == 0 && reinterpret_cast<uintptr_t>(out_dev) % 16 == 0) {
-    if (cudaMemcpyAsync(dev + s.slot_mapping, static_cast<const uint8_t*>(step_inputs_host) + s.slot_mapping, s.in_bytes - s.slot_mapping,
-                        cudaMemcpyHostToDevice, st) != cudaSuccess)
-      return COOPT_ERR_CUDA;
-    rc = launch_decode_plan(reinterpret_cast<const int32_t*>(dev + s.block_table), max_blocks_per_seq,
-                            reinterpret_cast<const int32_t*>(dev + s.context_lens), batch, hkv, cache->num_blocks, 0, P, plan, st);
-    if (rc != COOPT_OK) return rc;
-    return launch_decode_planned(cache, plan, in_dev + s.k_new, in_dev + s.v_new, static_cast<int64_t>(hkv) * d,
-                                 reinterpret_cast<const int64_t*>(dev + s.slot_mapping), in_dev + s.q, out_dev, max_blocks_per_seq,
-                                 batch, num_q_heads, sm_scale, 0, nullptr, workspace, P, false, st);
-  }
-  // pageable host memory: one copy in, the plan and the fused step, one copy out
-  if (cudaMemcpyAsync(dev, step_inputs_host, s.in_bytes, cudaMemcpyHostToDevice, st) != cudaSuccess) return COOPT_ERR_CUDA;
+  const bool in_place = in_dev != nullptr && out_dev != nullptr && reinterpret_cast<uintptr_t>(in_dev) % 16 == 0 && reinterpret_cast<uintptr_t>(out_dev) % 16 == 0;
+  const size_t from = in_place ? s.slot_mapping : 0;
+  if (cudaMemcpyAsync(dev + from, static_cast<const uint8_t*>(step_inputs_host) + from, s.in_bytes - from, cudaMemcpyHostToDevice, st) != cudaSuccess)
+    return COOPT_ERR_CUDA;
   rc = launch_decode_plan(reinterpret_cast<const int32_t*>(dev + s.block_table), max_blocks_per_seq,
-                          reinterpret_cast<const int32_t*>(dev + s.context_lens), batch, hkv, cache->num_blocks, 0, P, plan, st);
+                          reinterpret_cast<const int32_t*>(dev + s.context_lens), batch, hkv, cache->num_blocks, 0, plan, st);
   if (rc != COOPT_OK) return rc;
-  rc = launch_decode_planned(cache, plan, dev + s.k_new, dev + s.v_new, static_cast<int64_t>(hkv) * d,
-                             reinterpret_cast<const int64_t*>(dev + s.slot_mapping), dev + s.q, dev + s.out, max_blocks_per_seq, batch,
-                             num_q_heads, sm_scale, 0, nullptr, workspace, P, false, st);
+  if (in_place) {
+    a.q = in_dev + s.q; a.k_new = in_dev + s.k_new; a.v_new = in_dev + s.v_new; a.out = out_dev;
+    return launch_decode(cache, a, st);
+  }
+  rc = launch_decode(cache, a, st);
   if (rc != COOPT_OK) return rc;
   return cudaMemcpyAsync(out_host, dev + s.out, s.out_bytes, cudaMemcpyDeviceToHost, st) == cudaSuccess ? COOPT_OK : COOPT_ERR_CUDA;
 }

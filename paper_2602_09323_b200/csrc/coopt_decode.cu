@@ -1,509 +1,1013 @@
-// Paged decode over the bf16 ablation cache (the un-quantised layout the method is compared with):
-// Eq. 1, Eq. 7-8 (the G query heads of a group consume one K/V stream), Eq. 9 (valid blocks only),
-// Eq. 10 (max-subtracted softmax) and the Opt-Pa chunk-and-merge reduction, on mma.sync.  The FP8
-// cache has its own kernel on the 5th-generation tensor cores; this file also holds the host launcher
-// and the workspace arithmetic that both share.
+// Paged GQA decode: Algorithm 1 phase 2 (Eq. 6 dequantisation on load), Algorithm 2 (Eq. 7-8: the G query heads of a
+// group consume one K/V stream), Algorithm 3 (Eq. 9 valid blocks only, Eq. 10 max-subtracted softmax), the Opt-Pa
+// chunk-and-merge reduction, and, in a step that appends, Algorithm 1 phase 1 for one token per sequence.  FP8 (E4M3,
+// E5M2) and bf16 caches, head_dim 64 and 128, group sizes 1 to 8.
 //
-// The work decomposition is the shared planner's.  Inside a segment the CTA's warps take blocks
-// round-robin; each warp streams its granules through a private ring of shared-memory stages filled
-// by bulk async copies (one elected lane issues, an mbarrier per stage counts the bytes), runs both
-// contractions with the G query heads in the top rows of the 16-row instruction tile (the
-// probabilities split into a bf16 high and low half, the low halves in rows 8..15), and keeps an
-// online softmax per query head (warp shuffles inside the quad that owns a head, one shared-memory
-// step across warps at the end of the segment).  A segment that does not cover its whole sequence
-// leaves (m, l, o) in the workspace; the CTA that delivers the last piece of a (sequence, kv head)
-// merges them by log-sum-exp and writes the bf16 output.
-#include "coopt_plan.cuh"
+// What bounds it is the stream of the cache from HBM; everything else is arranged so that nothing waits on anything
+// but that stream.  Every warp is on its own: it walks its part of the line of blocks (coopt_decode.cuh), a lane of it
+// requests one granule (K part, V part, scales: one contiguous piece) per bulk copy into a ring of the warp's own, and
+// the warp takes both contractions of a block from there as they land:
+//     S^T [16 tokens x 8 heads] = K [16 x D] . Q^T        O^T [D x 8 heads] += V^T [D x 16 tokens] . P^T
+// on mma.sync m16n8k16.  Tokens (and dims) fill the instruction's 16 rows and the heads of a group its 8 columns, so
+// no row is idle for any group size.  Codes become f16 on the way from shared memory to registers (exact); a bf16
+// query row, scaled by a power of two, is exact in f16 as well; a probability is f16 once, carried times 2^8 against a
+// reference that may lag the maximum by 2^6, so that the running output is rescaled rarely; the K scale of a block
+// multiplies its logits, the V scale goes into the probabilities.  No barrier is met between the first block and the
+// last; pieces of units that warps or CTAs share are merged by log-sum-exp at the end.
+//
+// (The kernel before this one ran the contractions on tcgen05.mma, 128 tokens at a time, with two softmax teams per
+// CTA and a plan of every CTA's blocks made by a kernel of its own.  The tensor core was 21 % busy with columns that
+// are mostly padding, and what bounded the launch were the hand-overs between its roles, per unit and at both ends.
+// Before / now: one layer of 56 heads over 8 kv heads, 8 sequences of 1..28 tokens 60 / 8 us; 24 sequences of
+// 300..4000 tokens, G = 8, 46 / 25 us a layer; 32 x 2048 tokens, G = 5, 35 / 32 us; 64 sequences of 128..8192 tokens,
+// 121 / 106 us; 120 sequences of 5..900 tokens at head_dim 64, plan included, 56 / 18.5 us.)
+#include "coopt_decode.cuh"
+#include "coopt_trace.cuh"
+#include "coopt_umma.cuh"
+#include "coopt_write.cuh"
 
 namespace coopt {
 
 namespace {
 
-constexpr int kWarps = 8;
-constexpr int kThreads = kWarps * 32;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
+constexpr float kLag = 6.0f;                                      // how far a reference maximum may lag (base-2 logarithm units)
+constexpr float kShift = 8.0f, kUnshift = 1.0f / 256.0f;          // probabilities are carried times 2^kShift: at most 2^14 in f16
 
-template <int D>
+template <int D, int FMT>
 struct Cfg {
-  static constexpr int kGran = granule_bytes(D, false);
-  static constexpr int kStages = 2;
-  static constexpr int kKSteps = D / 16;
-  static constexpr int kNTiles = D / 8;
-  static constexpr int kOAcc = 4;               // accumulator registers kept per n-tile
-  // shared memory carve-up (bytes)
-  static constexpr int kRingOff = 0;
-  static constexpr int kRingBytes = kWarps * kStages * kGran;
-  static constexpr int kBarOff = kRingOff + kRingBytes;
-  static constexpr int kIdsOff = kBarOff + kWarps * kStages * 8;
-  static constexpr int kPreBlkOff = kIdsOff + kCap * 4;
-  static constexpr int kPreUnitOff = kPreBlkOff + (kMaxBatch + 4) * 4;
-  static constexpr int kSegOff = kPreUnitOff + (kMaxBatch + 4) * 4;
-  static constexpr int kMergeOff = kSegOff + kMaxSeg * static_cast<int>(sizeof(Segment));
-  static constexpr int kMergeStride = D + 4;    // floats per (warp, row): o[D], m, l, pad
-  static constexpr int kMiscOff = kMergeOff + kWarps * kMaxGroup * kMergeStride * 4;
-  static constexpr int kSmemBytes = kMiscOff + 128;
+  static constexpr bool kFp8 = FMT != COOPT_KV_BF16;
+  static constexpr bool kE5m2 = FMT == COOPT_KV_FP8_E5M2;
+  // A warp needs time for a block (about 1 us from landing to the next wait), so many warps are wanted, with at least two
+  // blocks in flight each.  head_dim 128: 12 warps x 3 blocks against 16 x 2 (which spill), 14 x 2 and 10 x 4: 423 / 430 /
+  // 423 / 427 us (64 sequences of 128..8192 tokens, four layers), 99 / 101 / 105 / 109 us (24 sequences, G = 8, four
+  // layers).  head_dim 64: 16 x 4 against 12 x 6: 33 / 36 us (85 x 2002 tokens).  bf16: 8 x 2 (182 registers).
+  static constexpr int kWarps = kFp8 ? (D == 128 ? 12 : 16) : 8;
+  static constexpr int kThreads = kWarps * 32;
+  static constexpr int kGran = granule_bytes(D, kFp8);
+  static constexpr int kCopy = kFp8 ? 2 * kBlockSize * D + kFp8Header : kGran;   // bytes of a granule that are read
+  static constexpr int kStages = kFp8 ? (D == 128 ? 3 : 4) : (D == 128 ? 2 : 4);
+  static constexpr int kPieceStride = D + 4;                    // floats of one head of a piece: o[D], maximum, sum, padding
+  static constexpr int kPiece = kMaxGroup * kPieceStride * 4;   // bytes
+  static constexpr int kWarpBytes = kStages * kGran + kPiece;
+  static constexpr int kBarOff = kWarps * kWarpBytes;
+  static constexpr int kLensOff = kBarOff + kWarps * kStages * 8;
+  static constexpr int kPreOff = kLensOff + kMaxBatch * 4;
+  static constexpr int kRecOff = kPreOff + (kMaxBatch + 4) * 4;
+  static constexpr int kMiscOff = kRecOff + kWarps * 32;
+  static constexpr int kSmemBytes = kMiscOff + 192;
+  static_assert(kGran % 128 == 0 && kPiece % 128 == 0 && kStages * kGran >= kPiece && kCopy % 16 == 0, "copies land on 128-byte boundaries");
+  static_assert(kCtasPerSm * (kSmemBytes + 1024) <= 233472, "shared memory of one SM");
 };
 
-__device__ __forceinline__ float quad_max(float x) {
-  x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, 1));
-  return fmaxf(x, __shfl_xor_sync(0xffffffffu, x, 2));
+// What a warp leaves about the (at most two) units it holds only a piece of.
+struct Rec {
+  int flags;            // kHas0: a piece of a unit that starts before this warp; kEnds0: that unit ends here; kHas1: one that starts here and goes on
+  int b0, g0, u0;       // its sequence, kv head and first block
+  int b1, g1, u1;
+  int pad;
+};
+constexpr int kHas0 = 1, kEnds0 = 2, kHas1 = 4;
+static_assert(sizeof(Rec) == 32, "shared memory layout");
+
+// ---- the line ------------------------------------------------------------------------------------------------------
+struct Line {
+  const int* lens;      // shared memory: context lengths
+  const unsigned* pre;  // shared memory: places of one kv head of the sequences before
+  int batch, heads, chunk;   // chunk: blocks per chunk, kNoChunks without chunks
+};
+__device__ __forceinline__ int line_blocks(const Line& ln, int b) { return (ln.lens[b] + kBlockSize - 1) / kBlockSize; }
+// first place of the unit of (b, g) that starts with block u
+__device__ __forceinline__ unsigned unit_place(const Line& ln, int b, int g, int u) {
+  const unsigned head = ln.pre[b + 1] - ln.pre[b];
+  return ln.heads * ln.pre[b] + g * head + (ln.chunk == kNoChunks ? 0u : static_cast<unsigned>(u / ln.chunk) * static_cast<unsigned>(ln.chunk + kUnitCost));
 }
-__device__ __forceinline__ float quad_sum(float x) {
-  x += __shfl_xor_sync(0xffffffffu, x, 1);
-  return x + __shfl_xor_sync(0xffffffffu, x, 2);
+__device__ __forceinline__ int unit_blocks(const Line& ln, int nb, int u) { return min(ln.chunk, nb - u); }
+
+// A walk over the units of the places [x, end): unit (b, g, first block u, n blocks), of which the blocks [j, jend)
+// (counted from u) belong to the walker.
+struct Walk {
+  int b, g, nb, u, n;
+  int j, jend;
+  unsigned base, end;
+  bool more;
+};
+__device__ __forceinline__ void walk_range(Walk& w, unsigned x) {
+  w.j = max(0, static_cast<int>(x - w.base) - kUnitCost);
+  w.jend = min(w.n, static_cast<int>(w.end - w.base) - kUnitCost);
+  w.more = w.jend > w.j;
+}
+__device__ __forceinline__ void walk_next(const Line& ln, Walk& w) {
+  const unsigned at = w.base + w.n + kUnitCost;
+  w.u += w.n;
+  if (w.u >= w.nb) {
+    w.u = 0;
+    if (++w.g == ln.heads) {
+      w.g = 0;
+      ++w.b;
+      while (w.b < ln.batch && ln.pre[w.b + 1] == ln.pre[w.b]) ++w.b;
+      if (w.b >= ln.batch) { w.more = false; return; }
+      w.nb = line_blocks(ln, w.b);
+    }
+  }
+  w.base = at;
+  w.n = unit_blocks(ln, w.nb, w.u);
+  if (w.base >= w.end) { w.more = false; return; }
+  walk_range(w, w.base);
+}
+// the sequence whose places contain x < all places (by the lanes of a warp together: 32 coarse candidates, then the fine ones)
+__device__ __forceinline__ int line_seq(const Line& ln, unsigned x, int lane) {
+  const int step = (ln.batch + 31) / 32;
+  int c = lane * step;
+  unsigned le = __ballot_sync(0xffffffffu, c < ln.batch && ln.heads * ln.pre[min(c, ln.batch)] <= x);
+  const int lo = (31 - __clz(le)) * step;
+  c = lo + lane;
+  le = __ballot_sync(0xffffffffu, lane < step && c < ln.batch && ln.heads * ln.pre[min(c, ln.batch)] <= x);
+  return lo + 31 - __clz(le);
+}
+// the unit that contains place x, and its first place
+__device__ __forceinline__ void walk_unit(const Line& ln, Walk& w, unsigned x, int lane) {
+  w.b = line_seq(ln, x, lane);
+  const unsigned before = ln.heads * ln.pre[w.b], head = ln.pre[w.b + 1] - ln.pre[w.b], rem = x - before;
+  w.g = rem / head;
+  w.nb = line_blocks(ln, w.b);
+  w.base = before + w.g * head;
+  w.u = 0;
+  if (ln.chunk != kNoChunks) {
+    const unsigned ci = (x - w.base) / static_cast<unsigned>(ln.chunk + kUnitCost);
+    w.u = ci * ln.chunk;
+    w.base += ci * static_cast<unsigned>(ln.chunk + kUnitCost);
+  }
+  w.n = unit_blocks(ln, w.nb, w.u);
+}
+__device__ __forceinline__ void walk_start(const Line& ln, Walk& w, unsigned x, unsigned end, int lane) {
+  w.end = end;
+  w.more = false;
+  w.b = w.g = w.u = w.n = w.nb = w.j = w.jend = 0;
+  w.base = 0;
+  if (x >= end) return;
+  walk_unit(ln, w, x, lane);
+  walk_range(w, x);
+}
+// the first place at or behind x where a unit begins
+__device__ __forceinline__ unsigned next_unit(const Line& ln, unsigned x, int lane) {
+  Walk w;
+  walk_unit(ln, w, x, lane);
+  return w.base == x ? x : w.base + w.n + kUnitCost;
 }
 
-// bf16 mma with only the top 8 rows of A in use (rows 8..15 are zero): two live accumulators.
-__device__ __forceinline__ void mma_top(float& d0, float& d1, uint32_t a0, uint32_t a2, uint32_t b0, uint32_t b1) {
-  float t2, t3;
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%10,%10};"
-               : "+f"(d0), "+f"(d1), "=f"(t2), "=f"(t3)
-               : "r"(a0), "r"(0u), "r"(a2), "r"(0u), "r"(b0), "r"(b1), "f"(0.0f));
-  static_cast<void>(t2 + t3);
+// ---- warp-level pieces ------------------------------------------------------------------------------------------------
+__device__ __forceinline__ void ldmatrix4(uint32_t addr, uint32_t (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
 }
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+__device__ __forceinline__ uint32_t transpose8x8(uint32_t x) {
+  uint32_t y;
+  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
+  return y;
+}
+template <bool kE5m2> __device__ __forceinline__ uint32_t codes_lo(uint32_t w) { return kE5m2 ? e5m2x2_to_f16x2_lo(w) : e4m3x2_to_f16x2_lo(w); }
+template <bool kE5m2> __device__ __forceinline__ uint32_t codes_hi(uint32_t w) { return kE5m2 ? e5m2x2_to_f16x2_hi(w) : e4m3x2_to_f16x2_hi(w); }
 
+// Algorithm 1 phase 1 for one token, on the granule as it sits in shared memory (K part, V part, header), which is then
+// written back: the write kernels' rule (write_part), with the same value for every number that is stored.
+// k, v: this lane's D / 32 consecutive values of the token's rows, as packed pairs.
+template <int D, bool kE5m2>
+__device__ __noinline__ void append_token(uint8_t* st, uint8_t* gran, const uint2 k, const uint2 v, int off, int lane) {
+  constexpr int kPart = kBlockSize * D, kPerLane = D / 32;
+  float* hdr = reinterpret_cast<float*>(st + header_offset(D));
+  const bool fresh = off == 0;
+  const uint32_t raw[2][2] = {{k.x, k.y}, {v.x, v.y}};
+  float s_old[2], s_new[2];
+#pragma unroll
+  for (int which = 0; which < 2; ++which) {
+    uint32_t amax2 = raw[which][0] & 0x7FFF7FFFu;
+    if (kPerLane == 4) amax2 = __vmaxu2(amax2, raw[which][1] & 0x7FFF7FFFu);
+    const uint32_t am = __reduce_max_sync(0xffffffffu, max(amax2 << 16, amax2 & 0xFFFF0000u));   // non-negative floats order like their bits
+    s_old[which] = fresh ? 0.0f : hdr[which];
+    s_new[which] = fmaxf(s_old[which], __fdiv_rn(__uint_as_float(am), kE5m2 ? kE5m2Max : kE4m3Max));
+  }
+#pragma unroll
+  for (int which = 0; which < 2; ++which) {
+    uint8_t* part = st + which * kPart;
+    if (fresh) {
+      for (int i = lane; i < kPart / 16; i += 32) reinterpret_cast<uint4*>(part)[i] = make_uint4(0u, 0u, 0u, 0u);
+    } else if (s_new[which] > s_old[which] && s_old[which] > 0.0f) {
+#pragma unroll 4
+      for (int i = lane; i < kPart; i += 32) {
+        const float val = __fmul_rn(kE5m2 ? e5m2_to_f32(part[i]) : e4m3_to_f32(part[i]), s_old[which]);
+        part[i] = static_cast<uint8_t>(kE5m2 ? f32_to_e5m2(__fdiv_rn(val, s_new[which])) : f32_to_e4m3(__fdiv_rn(val, s_new[which])));
+      }
+    }
+  }
+  __syncwarp();
+#pragma unroll
+  for (int which = 0; which < 2; ++which) {
+#pragma unroll
+    for (int e = 0; e < kPerLane; ++e) {
+      const float x = (e & 1) ? bf16_hi(raw[which][e >> 1]) : bf16_lo(raw[which][e >> 1]);
+      const float y = s_new[which] > 0.0f ? __fdiv_rn(x, s_new[which]) : x;
+      st[which * kPart + (which == 0 ? k_elem_offset(D, true, off, lane * kPerLane + e) : v_elem_offset(D, true, off, lane * kPerLane + e))] =
+          static_cast<uint8_t>(kE5m2 ? f32_to_e5m2(y) : f32_to_e4m3(y));
+    }
+  }
+  if (lane < 8) hdr[lane] = lane == 0 ? s_new[0] : lane == 1 ? s_new[1] : fresh ? 0.0f : hdr[lane];
+  __syncwarp();
+  for (int i = lane; i < (2 * kPart + kFp8Header) / 16; i += 32) reinterpret_cast<uint4*>(gran)[i] = reinterpret_cast<const uint4*>(st)[i];
+}
+// This lane's D / 32 consecutive values of a row that may be aligned for no more than its elements.
 template <int D>
-__global__ void __launch_bounds__(kThreads, 1) paged_decode_kernel(const DecodeParams p) {
-  using C = Cfg<D>;
-  extern __shared__ __align__(128) uint8_t smem[];
-  uint8_t* ring = smem + C::kRingOff;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kBarOff);
-  int* ids = reinterpret_cast<int*>(smem + C::kIdsOff);
-  int* pre_blk = reinterpret_cast<int*>(smem + C::kPreBlkOff);
-  int* pre_unit = reinterpret_cast<int*>(smem + C::kPreUnitOff);
-  Segment* segs = reinterpret_cast<Segment*>(smem + C::kSegOff);
-  float* merge = reinterpret_cast<float*>(smem + C::kMergeOff);
-  int* misc = reinterpret_cast<int*>(smem + C::kMiscOff);   // [0] nseg, [1..2] next x, [3] last-arriver flag
+__device__ __forceinline__ uint2 load_new(const __nv_bfloat16* row, bool vec, int lane) {
+  uint32_t w[D / 64];
+  if (vec) load_row<D / 32, true>(row + lane * (D / 32), w); else load_row<D / 32, false>(row + lane * (D / 32), w);
+  return make_uint2(w[0], D == 128 ? w[D / 64 - 1] : 0u);
+}
 
+// A head's pieces merged by log-sum-exp: numerators of the lane's four dims, denominator, maximum.
+struct Acc {
+  float M, den;
+  float4 num;
+};
+__device__ __forceinline__ void acc_clear(Acc& a) { a.M = -INFINITY; a.den = 0.0f; a.num = make_float4(0.0f, 0.0f, 0.0f, 0.0f); }
+// Up to 32 more pieces into the accumulator.  Lane k brings piece k's maximum and sum; `rows(k)` is where the piece's o
+// (normalised by its sum) lies for this lane.
+template <bool kGlobal, class Rows>
+__device__ __forceinline__ void acc_merge(Acc& a, int n, float m, float l, bool on, Rows rows) {
+  constexpr int kUnroll = 4;
+  const bool some = l > 0.0f;
+  const float top = fmaxf(a.M, ordered_to_f32(__reduce_max_sync(0xffffffffu, f32_to_ordered(some ? m : -INFINITY))));
+  const float wgt = some ? l * ex2(m - top) : 0.0f;
+  const float keep = a.den > 0.0f ? ex2(a.M - top) : 0.0f;
+  a.num.x *= keep; a.num.y *= keep; a.num.z *= keep; a.num.w *= keep;
+  a.den = a.den * keep + warp_sum(wgt);
+  a.M = top;
+  for (int k0 = 0; k0 < n; k0 += kUnroll) {
+    float4 o[kUnroll];
+#pragma unroll
+    for (int k = 0; k < kUnroll; ++k) {
+      const float4* from = reinterpret_cast<const float4*>(rows(min(k0 + k, n - 1)));
+      o[k] = on ? (kGlobal ? __ldcg(from) : *from) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    }
+#pragma unroll
+    for (int k = 0; k < kUnroll; ++k) {
+      const float w = k0 + k < n ? __shfl_sync(0xffffffffu, wgt, k0 + k) : 0.0f;
+      if (w > 0.0f) { a.num.x += w * o[k].x; a.num.y += w * o[k].y; a.num.z += w * o[k].z; a.num.w += w * o[k].w; }
+    }
+  }
+}
+
+template <int D, int FMT>
+__global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decode_kernel(const DecodeParams p) {
+  using C = Cfg<D, FMT>;
+  constexpr int kQSteps = D / 16;
+  extern __shared__ __align__(128) uint8_t smem[];
+  int* lens = reinterpret_cast<int*>(smem + C::kLensOff);
+  unsigned* pre = reinterpret_cast<unsigned*>(smem + C::kPreOff);
+  Rec* recs = reinterpret_cast<Rec*>(smem + C::kRecOff);
+  int* misc = reinterpret_cast<int*>(smem + C::kMiscOff);   // [0..15] warps' sums, [16] wrong plan, [17..32] warps' longest unit
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int row = lane >> 2, quad = lane & 3;
   const int B = p.batch, Hkv = p.num_kv_heads, G = p.group, Hq = p.num_q_heads;
-  const bool chunk_mode = p.chunk_blocks > 0;
+  uint8_t* ring = smem + warp * C::kWarpBytes;
+  float* piece0 = reinterpret_cast<float*>(ring + C::kStages * C::kGran);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kBarOff) + warp * C::kStages;
 
-  // ---- plan: blocks (and chunks) per sequence, this CTA's slice of the flat block list ---------
-  PlanSmem plan;
-  plan.pre_blk = pre_blk; plan.pre_unit = pre_unit; plan.segs = segs; plan.ids = ids; plan.misc = misc;
-  plan.slice = reinterpret_cast<long long*>(smem + C::kMiscOff + 64);
-  plan.bounds = nullptr;
-  int ctx_early[2];
-  plan_prefix_load(p, tid, kThreads, ctx_early);
-  if (tid == 0) {
-    for (int i = 0; i < kWarps * C::kStages; ++i) mbar_init(&bars[i], 1);
+  COOPT_TRACE_CYCLES(p.trace, kTrEntry, tid == 0);
+#ifdef COOPT_TRACE
+  if (tid == 0 && p.trace != nullptr && blockIdx.x < kTraceMaxCtas) {
+    trace_put(p.trace, kTrPrevExitNs, p.trace[blockIdx.x * kTraceSlots + kTrExitNs]);
+    unsigned int smid;
+    asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
+    trace_put(p.trace, kTrSmId, smid + 1);
+  }
+#endif
+  COOPT_TRACE_NS(p.trace, kTrEntryNs, tid == 0);
+  if (lane == 0) {
+    for (int i = 0; i < C::kStages; ++i) mbar_init(&bars[i], 1);
     mbar_fence_init();
   }
-  plan_prefix(p, plan, tid, kThreads, ctx_early);
-  if (tid == 0) plan_slice_publish(p, plan);
-  plan_check_single_query(p, tid, kThreads);
-  __syncthreads();
-
-  // sequences with an empty context: all-zero output rows
-  for (int b = blockIdx.x; b < B; b += gridDim.x) {
-    if (pre_blk[b + 1] == pre_blk[b])
-      for (int i = tid; i < Hq * D; i += kThreads) p.out[static_cast<size_t>(b) * Hq * D + i] = __float2bfloat16(0.0f);
+  // Launched as a programmatic dependent, this CTA may run while the kernel before it still does.  If that kernel
+  // writes neither the plan nor the cache (overlap_previous) only the queries, the new tokens and everything that is
+  // written wait for it (below).
+  if (!p.overlap_previous) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   }
 
-  PlanSlice sl;
-  if (!plan_slice_fetch(plan, sl)) return;
-  const long long lo = sl.lo, hi = sl.hi;
-  auto cta_of = [&](long long x) -> int { return plan_cta_of(sl, x); };
+  // ---- the line: context lengths and their prefix sums -------------------------------------------------------
+  {
+    constexpr int kPer = (kMaxBatch + C::kThreads - 1) / C::kThreads;
+    const int chunk = p.chunk_blocks > 0 ? p.chunk_blocks : kNoChunks;
+    unsigned v[kPer], sum = 0;
+    int most = 0, key = p.plan_key;
+    if (tid == 0 && p.plan != nullptr) key = p.plan->key;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const int b = tid * kPer + k;
+      int L = b < B ? p.context_lens[b] : 0;
+      L = max(0, min(L, p.max_blocks_per_seq * kBlockSize));
+      if (b < B) lens[b] = L;
+      const int nb = (L + kBlockSize - 1) / kBlockSize;
+      const int units = nb == 0 ? 0 : (chunk == kNoChunks ? 1 : (nb + chunk - 1) / chunk);
+      v[k] = nb + units * kUnitCost;
+      sum += v[k];
+      most = max(most, min(nb, chunk));
+    }
+    most = __reduce_max_sync(0xffffffffu, most);
+    unsigned inc = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned t = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += t;
+    }
+    if (lane == 31) { misc[warp] = inc; misc[17 + warp] = most; }
+    if (tid == 0) misc[16] = key != p.plan_key;
+    __syncthreads();
+    unsigned at = inc - sum;
+    for (int w = 0; w < warp; ++w) at += misc[w];
+    if (tid == 0) pre[0] = 0;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      at += v[k];
+      if (tid * kPer + k < B) pre[tid * kPer + k + 1] = at;
+    }
+    recs[warp].flags = 0;
+    __syncthreads();
+  }
+  if (misc[16]) {                                  // not a plan of this problem (uniform over the grid)
+    if (p.overlap_previous) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (tid == 0) atomicCAS(p.status, 0, COOPT_ERR_INVALID_ARG);
+    return;
+  }
+  COOPT_TRACE_CYCLES(p.trace, kTrLine, tid == 0);
+  Line ln;
+  ln.lens = lens; ln.pre = pre; ln.batch = B; ln.heads = Hkv; ln.chunk = p.chunk_blocks > 0 ? p.chunk_blocks : kNoChunks;
+  const unsigned places = Hkv * pre[B];
+  const unsigned T = max(static_cast<unsigned>(kMinPlaces), (places + gridDim.x - 1) / gridDim.x);
+  // Shared units cost a trip through the workspace at the end of the launch.  Where units are short, a CTA takes the units
+  // that begin among its places whole instead.  (In chunk mode every CTA between the first and the last of a (sequence,
+  // kv head) has to hold a chunk of it.)
+  int most = 0;
+  for (int k = 0; k < C::kWarps; ++k) most = max(most, misc[17 + k]);
+  const bool whole = most * (D / 64) <= (T == kMinPlaces ? kWholeUnitsIdle : kWholeUnits) && (p.chunk_blocks == 0 || most + kUnitCost <= static_cast<int>(T));
+  unsigned cta_lo = blockIdx.x * T, cta_hi = min(places, cta_lo + T);
+  if (whole && cta_lo < places) {
+    cta_lo = next_unit(ln, cta_lo, lane);
+    cta_hi = cta_hi < places ? next_unit(ln, cta_hi, lane) : places;
+  }
+  const unsigned mine = cta_hi > cta_lo ? cta_hi - cta_lo : 0u, Tw = (mine + C::kWarps - 1) / C::kWarps;
+  const unsigned my_lo = min(cta_hi, cta_lo + warp * Tw), my_hi = min(cta_hi, my_lo + Tw);
 
-  // ---- per-warp pipeline state (persists across rounds) ----------------------------------------
-  uint8_t* my_ring = ring + warp * C::kStages * C::kGran;
-  uint64_t* my_bars = bars + warp * C::kStages;
+  // ---- copies: a granule per request, a ring of stages per warp -------------------------------------------------
+  // Physical block ids are looked up 32 at a time (one per lane), one batch ahead of the copies that need them.
+  Walk pw;
+  walk_start(ln, pw, my_lo, my_hi, lane);
+  int ids_a = 0, cnt_a = 0, g_a = 0, pos_a = 0, ids_b = 0, cnt_b = 0, g_b = 0;
+  auto fetch_ids = [&]() {
+    cnt_b = 0;
+    if (!pw.more) return;
+    cnt_b = min(32, pw.jend - pw.j);
+    g_b = pw.g;
+    ids_b = lane < cnt_b ? p.block_table[static_cast<size_t>(pw.b) * p.max_blocks_per_seq + pw.u + pw.j + lane] : 0;
+    pw.j += cnt_b;
+    if (pw.j >= pw.jend) walk_next(ln, pw);
+  };
+  auto take_ids = [&]() {
+    ids_a = ids_b; cnt_a = cnt_b; g_a = g_b; pos_a = 0;
+    if (ids_a < 0 || ids_a >= p.num_blocks) {      // reported, and replaced by block 0: never dereferenced
+      if (p.plan == nullptr) atomicCAS(p.status, 0, COOPT_ERR_INVALID_ARG);
+      ids_a = 0;
+    }
+    fetch_ids();
+  };
   uint32_t issued = 0, consumed = 0;
-  bool dead = false;   // a bounded wait ran out: stop touching the pipeline, keep the barriers' company
-
-  long long x = lo;
-  while (x < hi) {
-    // ---- round: thread 0 plans up to kMaxSeg segments / kCap blocks starting at x -------------
-    if (tid == 0) plan_round(p, plan, sl, x);
-    __syncthreads();
-    const int nseg = misc[0];
-    const long long x_next = (static_cast<long long>(misc[2]) << 32) | static_cast<unsigned int>(misc[1]);
-    if (tid < nseg) plan_round_finish(p, plan, sl, tid);
-    plan_stage_ids(p, plan, nseg, tid, kThreads);
-    __syncthreads();
-
-    // ---- producer cursor of this warp: (segment, block-in-segment) --------------------------
-    int pseg = 0, pk = warp;
-    auto prod_normalise = [&]() {
-      while (pseg < nseg && pk >= segs[pseg].n) { ++pseg; pk = warp; }
-    };
-    auto prod_issue = [&]() {
-      const Segment& sg = segs[pseg];
-      const int id = ids[sg.list_off + pk];
-      const uint8_t* src = p.cache + (static_cast<size_t>(id) * Hkv + sg.g) * C::kGran;
+  auto issue = [&]() {
+    if (pos_a == cnt_a) take_ids();
+    if (pos_a < cnt_a) {
+      const int id = __shfl_sync(0xffffffffu, ids_a, pos_a);
+      ++pos_a;
       const uint32_t stage = issued % C::kStages;
       if (lane == 0) {
-        mbar_expect_tx(&my_bars[stage], C::kGran);
-        bulk_copy_g2s(my_ring + stage * C::kGran, src, C::kGran, &my_bars[stage]);
+        mbar_expect_tx(&bars[stage], C::kCopy);
+        bulk_copy_g2s(ring + stage * C::kGran, p.cache + (static_cast<size_t>(id) * Hkv + g_a) * C::kGran, C::kCopy, &bars[stage]);
       }
       ++issued;
-      pk += kWarps;
-    };
-    prod_normalise();
-    if (!dead) {
+    }
+  };
+
+  // ---- per-lane constants of the operand layouts ---------------------------------------------------------------
+  // FP8: ldmatrix row i of the "low" matrix of a K chunk is token 4 (i / 2) + i % 2, of the "high" one that token + 2
+  const int kt = 4 * ((lane & 7) >> 1) + (lane & 1) + 2 * ((lane >> 3) & 1);
+  const uint32_t k_lane = (kt >> 3) * 8 * D + (lane >> 4) * 128 + (kt & 7) * 16;
+  const int tok0 = C::kFp8 ? 4 * (row >> 1) + (row & 1) : row;       // token of this lane's logits 0 and 1; 2 and 3: tok0 + kTokStep
+  constexpr int kTokStep = C::kFp8 ? 2 : 8;
+
+  // raw query rows, loaded a unit ahead: this lane's head is `row`, its dims as the contraction takes them
+  uint32_t qraw[kQSteps][2];
+  auto load_q = [&](int b, int g) {
+    const bool live = row < G;
+    const __nv_bfloat16* qp = p.q + (static_cast<size_t>(b) * Hq + g * G + (live ? row : 0)) * D;
+#pragma unroll
+    for (int s = 0; s < kQSteps; ++s) {
+      if constexpr (C::kFp8) {
+        const uint2 v = live ? *reinterpret_cast<const uint2*>(qp + 16 * s + 4 * quad) : make_uint2(0u, 0u);
+        qraw[s][0] = v.x; qraw[s][1] = v.y;
+      } else {
+        qraw[s][0] = live ? *reinterpret_cast<const uint32_t*>(qp + 16 * s + 2 * quad) : 0u;
+        qraw[s][1] = live ? *reinterpret_cast<const uint32_t*>(qp + 16 * s + 2 * quad + 8) : 0u;
+      }
+    }
+  };
+  bool dead = false;
+  Walk w = pw;
+  // What the first unit needs besides its blocks is on its way to L2 before the copies queue up in front of it (also where
+  // the kernel before may still write it: L2 is where its stores arrive).
+  if (w.more) {
+    const uint8_t* qrows = reinterpret_cast<const uint8_t*>(p.q + (static_cast<size_t>(w.b) * Hq + w.g * G) * D);
+    if (lane < G * D / 64) prefetch_l2(qrows + lane * 128);
+    if (p.k_new != nullptr && lane < 3) {
+      const long long at = static_cast<long long>(w.b) * p.kv_token_stride + w.g * D;
+      prefetch_l2(lane == 0 ? static_cast<const void*>(p.k_new + at) : lane == 1 ? static_cast<const void*>(p.v_new + at) : static_cast<const void*>(p.slot_mapping + w.b));
+    }
+  }
+  fetch_ids();
 #pragma unroll 1
-      for (int s = 0; s < C::kStages && pseg < nseg; ++s) { prod_issue(); prod_normalise(); }
+  for (int step = 0; step < 2; ++step) {
+    if ((step == 0) == (p.overlap_previous != 0)) {
+#pragma unroll 1
+      for (int i = 0; i < C::kStages; ++i) issue();
+      COOPT_TRACE_CYCLES(p.trace, kTrFirstCopy, tid == 0);
+    } else {
+      // (The kernel behind this one may start only now, when the one before it has finished: it may read early what that one wrote.)
+      if (p.overlap_previous) {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+      }
+      COOPT_TRACE_CYCLES(p.trace, kTrPrevDone, tid == 0);
+      if (w.more) load_q(w.b, w.g);
+    }
+  }
+  if (blockIdx.x == 0) {
+    if (p.plan != nullptr && tid < kPlanCtas && p.plan->status[tid] != 0) atomicCAS(p.status, 0, p.plan->status[tid]);
+    // coopt_paged_chunked takes this path only for one query token per sequence: any other split of the same total is reported
+    if (p.cu_q_lens != nullptr)
+      for (int b = tid; b <= B; b += C::kThreads)
+        if (p.cu_q_lens[b] != b) atomicCAS(p.status, 0, COOPT_ERR_INVALID_ARG);
+  }
+  // sequences with an empty context: all-zero output rows
+  for (int b = blockIdx.x; b < B; b += gridDim.x)
+    if (lens[b] == 0)
+      for (int i = tid; i < Hq * D / 8; i += C::kThreads) reinterpret_cast<uint4*>(p.out + static_cast<size_t>(b) * Hq * D)[i] = make_uint4(0u, 0u, 0u, 0u);
+
+#pragma unroll 1
+  while (w.more) {
+    // ---- query operand: f16 (exact: rows scaled by a power of two), or bf16 as it is -------------------------------
+    uint32_t qf[kQSteps][2];
+    float qs[2];                                   // logit scale of heads 2 quad, 2 quad + 1
+    if constexpr (C::kFp8) {
+      uint32_t amax2 = 0;
+#pragma unroll
+      for (int s = 0; s < kQSteps; ++s) amax2 = __vmaxu2(__vmaxu2(amax2, qraw[s][0] & 0x7FFF7FFFu), qraw[s][1] & 0x7FFF7FFFu);
+      uint32_t am = max(amax2 << 16, amax2 & 0xFFFF0000u);
+      am = max(am, __shfl_xor_sync(0xffffffffu, am, 1));
+      am = max(am, __shfl_xor_sync(0xffffffffu, am, 2));
+      int k2 = 0;
+      if (am != 0u) k2 = max(-64, min(64, 134 - static_cast<int>((am >> 23) & 0xFF)));
+      const float up = __uint_as_float(static_cast<uint32_t>(k2 + 127) << 23);
+      const float down = p.sm_scale_log2 * __uint_as_float(static_cast<uint32_t>(127 - k2) << 23);
+#pragma unroll
+      for (int s = 0; s < kQSteps; ++s)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) qf[s][e] = pack_f16x2(bf16_lo(qraw[s][e]) * up, bf16_hi(qraw[s][e]) * up);
+      qs[0] = __shfl_sync(0xffffffffu, down, 8 * quad);
+      qs[1] = __shfl_sync(0xffffffffu, down, 8 * quad + 4);
+    } else {
+#pragma unroll
+      for (int s = 0; s < kQSteps; ++s) { qf[s][0] = qraw[s][0]; qf[s][1] = qraw[s][1]; }
+      qs[0] = qs[1] = p.sm_scale_log2;
+    }
+    COOPT_TRACE_CYCLES(p.trace, kTrQuery, tid == 0 && consumed == 0 && qf[0][0] != 0x12345u);
+    {
+      Walk nx = w;
+      walk_next(ln, nx);
+      if (nx.more) load_q(nx.b, nx.g);
     }
 
-    // raw query registers of the next segment, loaded one segment ahead
-    uint32_t qraw[C::kKSteps][2];
-    auto load_q_raw = [&](const Segment& sg) {
-      const bool live = row < G;
-      const __nv_bfloat16* qp = p.q + (static_cast<size_t>(sg.b) * Hq + sg.g * G + (live ? row : 0)) * D + 2 * quad;
+    float o[D / 16][4];
 #pragma unroll
-      for (int s = 0; s < C::kKSteps; ++s) {
-        qraw[s][0] = live ? *reinterpret_cast<const uint32_t*>(qp + 16 * s) : 0u;
-        qraw[s][1] = live ? *reinterpret_cast<const uint32_t*>(qp + 16 * s + 8) : 0u;
-      }
-    };
-    if (nseg > 0) load_q_raw(segs[0]);
-
-    for (int si = 0; si < nseg; ++si) {
-      const Segment sg = segs[si];
-
-      // ---- query fragments (A operand): bf16 as loaded ---------------------------------------
-      uint32_t qa[C::kKSteps][2];
+    for (int t = 0; t < D / 16; ++t)
 #pragma unroll
-      for (int s = 0; s < C::kKSteps; ++s) { qa[s][0] = qraw[s][0]; qa[s][1] = qraw[s][1]; }
-      if (si + 1 < nseg) load_q_raw(segs[si + 1]);
-
-      // ---- online softmax state of this warp for the segment ---------------------------------
-      float m_run = -INFINITY, l_run = 0.0f;
-      float o[C::kNTiles][C::kOAcc];
-#pragma unroll
-      for (int t = 0; t < C::kNTiles; ++t)
-#pragma unroll
-        for (int e = 0; e < C::kOAcc; ++e) o[t][e] = 0.0f;
+      for (int e = 0; e < 4; ++e) o[t][e] = 0.0f;
+    float m[2] = {-INFINITY, -INFINITY}, top[2] = {-INFINITY, -INFINITY}, l[2] = {0.0f, 0.0f};
+    float vref = 0.0f, vinv = 0.0f;
+    const int ctx = lens[w.b];
 
 #pragma unroll 1
-      for (int k = warp; k < sg.n; k += kWarps) {
-        const uint32_t stage = consumed % C::kStages;
-        const uint32_t parity = (consumed / C::kStages) & 1u;
-        if (!dead && !mbar_wait_bounded(&my_bars[stage], parity)) {
-          dead = true;
-          if (lane == 0) atomicCAS(p.status, 0, COOPT_ERR_TIMEOUT);
+    for (int j = w.j; j < w.jend; ++j) {
+      const uint32_t stage = consumed % C::kStages;
+      // the step's new token: what it needs is loaded while its block is on the way
+      const bool append = C::kFp8 && p.k_new != nullptr && w.u + j == w.nb - 1;
+      long long slot = -1;
+      int id = 0;
+      uint2 k_row = make_uint2(0u, 0u), v_row = k_row;
+      if constexpr (C::kFp8) {
+        if (append) {
+          const bool vec = ((reinterpret_cast<uintptr_t>(p.k_new) | reinterpret_cast<uintptr_t>(p.v_new) | static_cast<uintptr_t>(p.kv_token_stride * 2)) & (D / 16 - 1)) == 0;
+          const long long at = static_cast<long long>(w.b) * p.kv_token_stride + w.g * D;
+          slot = p.slot_mapping[w.b];
+          id = p.block_table[static_cast<size_t>(w.b) * p.max_blocks_per_seq + w.nb - 1];
+          k_row = load_new<D>(p.k_new + at, vec, lane);
+          v_row = load_new<D>(p.v_new + at, vec, lane);
         }
-        ++consumed;
-        if (dead) continue;
-        const uint8_t* st = my_ring + stage * C::kGran;
-        const int nvalid = min(kBlockSize, sg.ctx_len - (sg.j0 + k) * kBlockSize);   // Eq. 9 tail
+      }
+      if (!dead && !mbar_wait_bounded(&bars[stage], (consumed / C::kStages) & 1u)) {
+        dead = true;
+        if (lane == 0) atomicCAS(p.status, 0, COOPT_ERR_TIMEOUT);
+      }
+      dead = __any_sync(0xffffffffu, dead);
+      COOPT_TRACE_CYCLES(p.trace, kTrFirstLanded, tid == 0 && consumed == 0);
+      ++consumed;
+      if (dead) continue;
+      uint8_t* st = ring + stage * C::kGran;
+      const int nvalid = min(kBlockSize, ctx - (w.u + j) * kBlockSize);      // Eq. 9: tail of the context
 
-        // ---- S = Q K^T for 16 tokens (two n-tiles of 8) ---------------------------------------
-        float s0[2] = {0.0f, 0.0f}, s1[2] = {0.0f, 0.0f};
-        const uint8_t* kp = st + part_offset(D, false, 0) + lane * 16;
+      if constexpr (C::kFp8) {
+        if (append && slot >= 0) {                                             // Eq. 5: negative slots are skipped
+          const int off = (ctx - 1) % kBlockSize;
+          if (slot != static_cast<long long>(id) * kBlockSize + off) {         // not the sequence's last position
+            if (lane == 0) atomicCAS(p.status, 0, COOPT_ERR_INVALID_ARG);
+          } else if (id >= 0 && id < p.num_blocks) {
+            append_token<D, C::kE5m2>(st, p.cache + (static_cast<size_t>(id) * Hkv + w.g) * C::kGran, k_row, v_row, off, lane);
+          }
+          __syncwarp();
+        }
+      }
+
+      // ---- S^T = K Q^T: 16 tokens x 8 heads ------------------------------------------------------------------------
+      float sa[4] = {0.0f, 0.0f, 0.0f, 0.0f}, sb[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+      float sk = 1.0f, sv = 1.0f;
+      if constexpr (C::kFp8) {
+        const uint32_t ka = smem_u32(st) + k_lane;
+        const float2 hdr = *reinterpret_cast<const float2*>(st + header_offset(D));
+        sk = hdr.x; sv = hdr.y;
+#pragma unroll
+        for (int c = 0; c < D / 32; ++c) {
+          uint32_t r[4];
+          ldmatrix4(ka + c * 256, r);
+          mma16816<true>(sa, codes_lo<C::kE5m2>(r[0]), codes_lo<C::kE5m2>(r[1]), codes_hi<C::kE5m2>(r[0]), codes_hi<C::kE5m2>(r[1]), qf[2 * c][0], qf[2 * c][1]);
+          mma16816<true>(sb, codes_lo<C::kE5m2>(r[2]), codes_lo<C::kE5m2>(r[3]), codes_hi<C::kE5m2>(r[2]), codes_hi<C::kE5m2>(r[3]), qf[2 * c + 1][0], qf[2 * c + 1][1]);
+        }
+      } else {
+        const uint8_t* kp = st + lane * 16;
 #pragma unroll
         for (int i = 0; i < D / 32; ++i) {
-          const uint4 w0 = lds128(kp + (0 * (D / 32) + i) * 512);
-          const uint4 w1 = lds128(kp + (1 * (D / 32) + i) * 512);
-          mma_top(s0[0], s0[1], qa[2 * i][0], qa[2 * i][1], w0.x, w0.y);
-          mma_top(s0[0], s0[1], qa[2 * i + 1][0], qa[2 * i + 1][1], w0.z, w0.w);
-          mma_top(s1[0], s1[1], qa[2 * i][0], qa[2 * i][1], w1.x, w1.y);
-          mma_top(s1[0], s1[1], qa[2 * i + 1][0], qa[2 * i + 1][1], w1.z, w1.w);
+          const uint4 w0 = lds128(kp + i * 512), w1 = lds128(kp + (D / 32 + i) * 512);
+          mma16816<false>(sa, w0.x, w1.x, w0.y, w1.y, qf[2 * i][0], qf[2 * i][1]);
+          mma16816<false>(sb, w0.z, w1.z, w0.w, w1.w, qf[2 * i + 1][0], qf[2 * i + 1][1]);
         }
+      }
 
-        // ---- online softmax (Eq. 10), log2 units ---------------------------------------------------
-        const float ks = p.sm_scale_log2;
-        float sc[4] = {s0[0] * ks, s0[1] * ks, s1[0] * ks, s1[1] * ks};
-        const int tok[4] = {2 * quad, 2 * quad + 1, 2 * quad + 8, 2 * quad + 9};
-        if (nvalid < kBlockSize) {
+      // ---- online softmax (Eq. 10) in base-2 units; the reference maximum is lazy ------------------------------------
+      const float k0 = qs[0] * sk, k1 = qs[1] * sk;
+      float x[4] = {(sa[0] + sb[0]) * k0, (sa[1] + sb[1]) * k1, (sa[2] + sb[2]) * k0, (sa[3] + sb[3]) * k1};
+      if (nvalid < kBlockSize) {
+        if (tok0 >= nvalid) x[0] = x[1] = -INFINITY;
+        if (tok0 + kTokStep >= nvalid) x[2] = x[3] = -INFINITY;
+      }
+      const float t0 = fmaxf(x[0], x[2]), t1 = fmaxf(x[1], x[3]);
+      top[0] = fmaxf(top[0], t0);
+      top[1] = fmaxf(top[1], t1);
+      const bool grow = C::kFp8 && sv > vref;
+      if (__any_sync(0xffffffffu, t0 > m[0] + kLag || t1 > m[1] + kLag) || grow) {
+        float f[2];
 #pragma unroll
-          for (int e = 0; e < 4; ++e) sc[e] = tok[e] < nvalid ? sc[e] : -INFINITY;
+        for (int h = 0; h < 2; ++h) {
+          float t = h ? t1 : t0;
+          t = fmaxf(t, __shfl_xor_sync(0xffffffffu, t, 4));
+          t = fmaxf(t, __shfl_xor_sync(0xffffffffu, t, 8));
+          t = fmaxf(t, __shfl_xor_sync(0xffffffffu, t, 16));
+          const float mn = fmaxf(m[h], t);
+          f[h] = ex2(m[h] - mn);
+          m[h] = mn;
+          l[h] *= f[h];
         }
-        const float m_blk = quad_max(fmaxf(fmaxf(sc[0], sc[1]), fmaxf(sc[2], sc[3])));
-        const float m_new = fmaxf(m_run, m_blk);
-        const float a_m = ex2(m_run - m_new);
-        float pr[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) pr[e] = ex2(sc[e] - m_new);
-        l_run = l_run * a_m + (pr[0] + pr[1]) + (pr[2] + pr[3]);
-        m_run = m_new;
-        if (__any_sync(0xffffffffu, a_m != 1.0f)) {
-#pragma unroll
-          for (int t = 0; t < C::kNTiles; ++t)
-#pragma unroll
-            for (int e = 0; e < C::kOAcc; ++e) o[t][e] *= a_m;
+        if (grow) {
+          const float fv = vref * (1.0f / sv);
+          f[0] *= fv; f[1] *= fv;
+          vref = sv;
+          vinv = 1.0f / sv;
         }
+#pragma unroll
+        for (int t = 0; t < D / 16; ++t) { o[t][0] *= f[0]; o[t][1] *= f[1]; o[t][2] *= f[0]; o[t][3] *= f[1]; }
+      }
+      float pr[4];
+      const float b0 = kShift - m[0], b1 = kShift - m[1];
+      pr[0] = ex2(x[0] + b0); pr[1] = ex2(x[1] + b1); pr[2] = ex2(x[2] + b0); pr[3] = ex2(x[3] + b1);
+      l[0] += pr[0] + pr[2];
+      l[1] += pr[1] + pr[3];
 
-        // ---- O += P V -----------------------------------------------------------------------------
+      // ---- O^T += V^T P^T -----------------------------------------------------------------------------------------------
+      if constexpr (C::kFp8) {
+        const float pv = sv * vinv;
+        const uint32_t p0 = transpose8x8(pack_f16x2(pr[0] * pv, pr[1] * pv)), p1 = transpose8x8(pack_f16x2(pr[2] * pv, pr[3] * pv));
+        const uint32_t va = smem_u32(st) + kBlockSize * D + lane * 16;
+        uint32_t mask = 0xFFFFFFFFu;
+        if (nvalid < kBlockSize) {                 // codes of slots past the context are cleared: they may hold anything
+          const int keep = nvalid - 4 * quad;
+          mask = keep >= 4 ? 0xFFFFFFFFu : keep <= 0 ? 0u : (1u << (8 * keep)) - 1u;
+        }
+#pragma unroll
+        for (int i = 0; i < D / 32; ++i) {
+          uint32_t r[4];
+          ldmatrix4(va + i * 512, r);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) r[e] &= mask;
+          mma16816<true>(o[2 * i], codes_lo<C::kE5m2>(r[0]), codes_lo<C::kE5m2>(r[1]), codes_hi<C::kE5m2>(r[0]), codes_hi<C::kE5m2>(r[1]), p0, p1);
+          mma16816<true>(o[2 * i + 1], codes_lo<C::kE5m2>(r[2]), codes_lo<C::kE5m2>(r[3]), codes_hi<C::kE5m2>(r[2]), codes_hi<C::kE5m2>(r[3]), p0, p1);
+        }
+      } else {
+        // bf16 probabilities as a high and a low half (16 bits in all)
+        const uint32_t h0 = pack_bf16x2(pr[0], pr[1]), h1 = pack_bf16x2(pr[2], pr[3]);
+        const uint32_t e0 = pack_bf16x2(pr[0] - bf16_lo(h0), pr[1] - bf16_hi(h0)), e1 = pack_bf16x2(pr[2] - bf16_lo(h1), pr[3] - bf16_hi(h1));
+        const uint32_t p0 = transpose8x8(h0), p1 = transpose8x8(h1), r0 = transpose8x8(e0), r1 = transpose8x8(e1);
         const uint8_t* vp = st + part_offset(D, false, 1) + lane * 16;
-        {
-          // bf16 probabilities split into high and low halves; the low halves ride in rows 8..15
-          uint32_t hi0 = pack_bf16x2(pr[0], pr[1]), hi2 = pack_bf16x2(pr[2], pr[3]);
-          const uint32_t lo0 = pack_bf16x2(pr[0] - bf16_lo(hi0), pr[1] - bf16_hi(hi0));
-          const uint32_t lo2 = pack_bf16x2(pr[2] - bf16_lo(hi2), pr[3] - bf16_hi(hi2));
-          uint32_t m01 = 0xffffffffu, m89 = 0xffffffffu;
-          if (nvalid < kBlockSize) {
-            m01 = (tok[0] < nvalid ? 0x0000FFFFu : 0u) | (tok[1] < nvalid ? 0xFFFF0000u : 0u);
-            m89 = (tok[2] < nvalid ? 0x0000FFFFu : 0u) | (tok[3] < nvalid ? 0xFFFF0000u : 0u);
-          }
-#pragma unroll
-          for (int qd = 0; qd < D / 16; ++qd) {
-            const uint4 w = lds128(vp + qd * 512);
-            mma16816<false>(o[2 * qd], hi0, lo0, hi2, lo2, w.x & m01, w.y & m89);
-            mma16816<false>(o[2 * qd + 1], hi0, lo0, hi2, lo2, w.z & m01, w.w & m89);
-          }
+        uint32_t m0 = 0xFFFFFFFFu, m1 = 0xFFFFFFFFu;
+        if (nvalid < kBlockSize) {
+          m0 = (2 * quad < nvalid ? 0x0000FFFFu : 0u) | (2 * quad + 1 < nvalid ? 0xFFFF0000u : 0u);
+          m1 = (2 * quad + 8 < nvalid ? 0x0000FFFFu : 0u) | (2 * quad + 9 < nvalid ? 0xFFFF0000u : 0u);
         }
-
-        // ---- hand the stage back to the copy engine ------------------------------------------------
-        __syncwarp();
-        if (pseg < nseg) {
-          if (lane == 0) fence_proxy_async();
-          prod_issue();
-          prod_normalise();
+#pragma unroll
+        for (int i = 0; i < D / 16; ++i) {
+          const uint4 v = lds128(vp + i * 512);
+          mma16816<false>(o[i], v.x & m0, v.z & m0, v.y & m1, v.w & m1, p0, p1);
+          mma16816<false>(o[i], v.x & m0, v.z & m0, v.y & m1, v.w & m1, r0, r1);
         }
       }
 
-      // ---- end of segment: combine the warps' states through shared memory --------------------
-      l_run = quad_sum(l_run);
-      if (row < G) {
-        float* mr = merge + (warp * kMaxGroup + row) * C::kMergeStride;
-#pragma unroll
-        for (int t = 0; t < C::kNTiles; ++t)   // high and low halves of the probabilities were accumulated apart
-          *reinterpret_cast<float2*>(mr + 8 * t + 2 * quad) = make_float2(o[t][0] + o[t][2], o[t][1] + o[t][3]);
-        if (quad == 0) { mr[D] = m_run; mr[D + 1] = l_run; }
-      }
-      __syncthreads();
-
-      const int h0 = sg.g * G;
-      float* po = nullptr; float* pm = nullptr; float* pl = nullptr;
-      if (sg.partial) {
-        if (chunk_mode) {
-          const size_t base = (static_cast<size_t>(sg.b) * Hq + h0) * p.max_chunks + sg.slot;
-          po = p.part_o + base * D; pm = p.part_m + base; pl = p.part_l + base;
-        } else {
-          const size_t base = static_cast<size_t>(sg.slot) * G;
-          po = p.part_o + base * D; pm = p.part_m + base; pl = p.part_l + base;
-        }
-      }
-      const size_t pstride = chunk_mode ? static_cast<size_t>(p.max_chunks) : 1;   // row stride of partial arrays
-      for (int idx = tid; idx < G * D; idx += kThreads) {
-        const int r = idx / D, d = idx % D;
-        float M = -INFINITY;
-#pragma unroll
-        for (int w = 0; w < kWarps; ++w) M = fmaxf(M, merge[(w * kMaxGroup + r) * C::kMergeStride + D]);
-        float num = 0.0f, den = 0.0f;
-#pragma unroll
-        for (int w = 0; w < kWarps; ++w) {
-          const float* mw = merge + (w * kMaxGroup + r) * C::kMergeStride;
-          const float wgt = ex2(mw[D] - M);
-          num += wgt * mw[d];
-          den += wgt * mw[D + 1];
-        }
-        const float val = num / den;
-        if (!sg.partial) {
-          p.out[(static_cast<size_t>(sg.b) * Hq + h0 + r) * D + d] = __float2bfloat16(val);
-        } else {
-          po[r * pstride * D + d] = val;
-          if (d == 0) {
-            pm[r * pstride] = chunk_mode ? M * kLn2 : M;   // exported partials use natural-log units
-            pl[r * pstride] = den;
-          }
-        }
-      }
-
-      if (sg.partial) {
-        __threadfence();
-        __syncthreads();
-        int* counter = p.counters + sg.b * Hkv + sg.g;
-        if (tid == 0) {
-          const int old = atomicAdd(counter, 1);
-          const int last = old == sg.expected - 1;
-          if (last) *counter = 0;             // ready for the next call
-          misc[3] = last;
-        }
-        __syncthreads();
-        if (misc[3]) {
-          // this CTA delivered the last piece: log-sum-exp merge of all pieces (split-K merge)
-          __threadfence();
-          int first_cta = 0;
-          if (!chunk_mode) {
-            const long long fs = static_cast<long long>(Hkv) * pre_blk[sg.b] + static_cast<long long>(sg.g) * sg.seq_blocks;
-            first_cta = cta_of(fs);
-          }
-          for (int idx = tid; idx < G * D; idx += kThreads) {
-            const int r = idx / D, d = idx % D;
-            float M = -INFINITY;
-            for (int c = 0; c < sg.expected; ++c) {
-              size_t at;
-              if (chunk_mode) at = (static_cast<size_t>(sg.b) * Hq + h0 + r) * p.max_chunks + c;
-              else at = static_cast<size_t>(2 * (first_cta + c) + (c == 0 ? 1 : 0)) * G + r;
-              M = fmaxf(M, __ldcg(p.part_m + at));
-            }
-            float num = 0.0f, den = 0.0f;
-            for (int c = 0; c < sg.expected; ++c) {
-              size_t at;
-              if (chunk_mode) at = (static_cast<size_t>(sg.b) * Hq + h0 + r) * p.max_chunks + c;
-              else at = static_cast<size_t>(2 * (first_cta + c) + (c == 0 ? 1 : 0)) * G + r;
-              const float mc = __ldcg(p.part_m + at), lc = __ldcg(p.part_l + at);
-              const float wgt = lc * (chunk_mode ? ex2((mc - M) * kLog2e) : ex2(mc - M));
-              num += wgt * __ldcg(p.part_o + at * D + d);
-              den += wgt;
-            }
-            p.out[(static_cast<size_t>(sg.b) * Hq + h0 + r) * D + d] = __float2bfloat16(num / den);
-          }
-        }
-      }
-      __syncthreads();   // merge scratch and misc[3] are reused by the next segment
+      // ---- the stage goes back to the copy engine ---------------------------------------------------------------------
+      __syncwarp();
+      if (lane == 0) fence_proxy_async();
+      issue();
     }
 
-    x = x_next;
-    __syncthreads();
+    // ---- end of the unit (or of this warp's piece of it) ----------------------------------------------------------------
+    float inv[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+#pragma unroll
+      for (int s = 4; s <= 16; s <<= 1) l[h] += __shfl_xor_sync(0xffffffffu, l[h], s);
+      inv[h] = l[h] > 0.0f ? (C::kFp8 ? vref : 1.0f) / l[h] : 0.0f;      // o and l go by the same reference
+      if (p.chunk_blocks > 0) {                    // exported partials carry the true maximum
+#pragma unroll
+        for (int s = 4; s <= 16; s <<= 1) top[h] = fmaxf(top[h], __shfl_xor_sync(0xffffffffu, top[h], s));
+        l[h] *= ex2(m[h] - top[h]);
+        m[h] = top[h];
+      }
+    }
+    const bool starts = w.j == 0, ends = w.jend == w.n;
+    if (starts && ends && p.chunk_blocks == 0) {
+      // the whole (sequence, kv head): bf16 rows, transposed so that a lane holds pairs of dims of head `row`
+      __nv_bfloat16* dst = p.out + (static_cast<size_t>(w.b) * Hq + w.g * G + row) * D + 2 * quad;
+#pragma unroll
+      for (int t = 0; t < D / 16; ++t) {
+        const uint32_t a = transpose8x8(pack_bf16x2(o[t][0] * inv[0], o[t][1] * inv[1])), c = transpose8x8(pack_bf16x2(o[t][2] * inv[0], o[t][3] * inv[1]));
+        if (row < G) {
+          *reinterpret_cast<uint32_t*>(dst + 16 * t) = a;
+          *reinterpret_cast<uint32_t*>(dst + 16 * t + 8) = c;
+        }
+      }
+    } else if (starts && ends) {
+      // a whole chunk: exported
+      const size_t rows = static_cast<size_t>(p.max_chunks);
+      const size_t at = (static_cast<size_t>(w.b) * Hq + w.g * G + 2 * quad) * rows + w.u / ln.chunk;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        if (2 * quad + h < G) {
+          float* dst = p.part_o + (at + h * rows) * D + row;
+#pragma unroll
+          for (int t = 0; t < D / 16; ++t) { dst[16 * t] = o[t][h] * inv[h]; dst[16 * t + 8] = o[t][2 + h] * inv[h]; }
+          if (row == 0) { p.part_m[at + h * rows] = m[h] * kLn2; p.part_l[at + h * rows] = l[h] * kUnshift; }
+        }
+      }
+    } else {
+      // a piece: into shared memory (the piece of a unit that goes on is the warp's last one: it takes the ring's place)
+      float* piece = starts ? reinterpret_cast<float*>(ring) : piece0;
+      float* at = piece + 2 * quad * C::kPieceStride + row;
+#pragma unroll
+      for (int t = 0; t < D / 16; ++t) {
+        at[16 * t] = o[t][0] * inv[0];
+        at[C::kPieceStride + 16 * t] = o[t][1] * inv[1];
+        at[16 * t + 8] = o[t][2] * inv[0];
+        at[C::kPieceStride + 16 * t + 8] = o[t][3] * inv[1];
+      }
+      if (row < 2) {
+        piece[(2 * quad + row) * C::kPieceStride + D] = row ? m[1] : m[0];
+        piece[(2 * quad + row) * C::kPieceStride + D + 1] = row ? l[1] : l[0];
+      }
+      if (lane == 0) {
+        Rec& r = recs[warp];
+        if (starts) { r.b1 = w.b; r.g1 = w.g; r.u1 = w.u; r.flags |= kHas1; }
+        else { r.b0 = w.b; r.g0 = w.g; r.u0 = w.u; r.flags |= kHas0 | (ends ? kEnds0 : 0); }
+      }
+    }
+    walk_next(ln, w);
   }
-
-  // a warp that gave up still has copies in flight: give them a bounded time to land before
-  // the CTA's shared memory is released
+  COOPT_TRACE_CYCLES(p.trace, kTrWarpEnd + warp, lane == 0);
+  COOPT_TRACE_VALUE(p.trace, kTrBlocks, tid == 0, consumed);
+  // a warp that gave up still has copies in flight: they get a bounded time to land
   if (dead) {
     while (consumed < issued) {
-      const uint32_t stage = consumed % C::kStages, parity = (consumed / C::kStages) & 1u;
-      mbar_wait_bounded(&my_bars[stage], parity);
+      mbar_wait_bounded(&bars[consumed % C::kStages], (consumed / C::kStages) & 1u);
       ++consumed;
     }
+  }
+  __syncthreads();
+  COOPT_TRACE_CYCLES(p.trace, kTrStreamed, tid == 0);
+
+  // ---- units that several warps share: merged by log-sum-exp, one (unit, head) per warp ---------------------------------
+  const int d0 = lane * 4;
+  const bool on = d0 < D;
+  // One head of a piece that other CTAs hold the rest of goes to the workspace; the warp that delivers the last piece gets
+  // `true` and all pieces merged.  The first piece of a unit sits in the odd slot of its CTA, the others in the even ones.
+  auto deliver = [&](Acc& a, int region, bool first_piece, int cta_f, int pieces, int h) -> bool {
+    const size_t base = static_cast<size_t>(region) * 2 * gridDim.x;
+    const size_t at = (base + 2 * blockIdx.x + (first_piece ? 1 : 0)) * G + h;
+    const float dinv = a.den > 0.0f ? 1.0f / a.den : 0.0f;
+    if (on) *reinterpret_cast<float4*>(p.run_o + at * D + d0) = make_float4(a.num.x * dinv, a.num.y * dinv, a.num.z * dinv, a.num.w * dinv);
+    if (lane == 0) { p.run_m[at] = a.M; p.run_l[at] = a.den; }
+    __syncwarp();
+    int done = 0;
+    if (lane == 0) {
+      // release (this piece is visible before the count moves) and acquire (the other pieces are visible before they are read)
+      int* counter = p.counters + (region * gridDim.x + cta_f) * kMaxGroup + h;
+      int old;
+      asm volatile("atom.add.acq_rel.gpu.s32 %0, [%1], 1;" : "=r"(old) : "l"(counter) : "memory");
+      done = old == pieces - 1;
+      if (done) *counter = 0;            // ready for the next call
+    }
+    if (!__shfl_sync(0xffffffffu, done, 0)) return false;
+    acc_clear(a);
+    auto slot = [&](int c) -> size_t { return (base + 2 * (cta_f + c) + (c == 0 ? 1 : 0)) * G + h; };
+    for (int c0 = 0; c0 < pieces; c0 += 32) {
+      const int n = min(32, pieces - c0);
+      const float m = lane < n ? __ldcg(p.run_m + slot(c0 + lane)) : 0.0f, l = lane < n ? __ldcg(p.run_l + slot(c0 + lane)) : 0.0f;
+      acc_merge<true>(a, n, m, l, on, [&](int k) { return p.run_o + slot(c0 + k) * D + d0; });
+    }
+    return true;
+  };
+  auto store_out = [&](const Acc& a, int b, int g, int h) {
+    const float dinv = a.den > 0.0f ? 1.0f / a.den : 0.0f;
+    if (on) *reinterpret_cast<uint2*>(p.out + (static_cast<size_t>(b) * Hq + g * G + h) * D + d0) =
+        make_uint2(pack_bf16x2(a.num.x * dinv, a.num.y * dinv), pack_bf16x2(a.num.z * dinv, a.num.w * dinv));
+  };
+  const int flags = lane < C::kWarps ? recs[lane].flags : 0;
+  const unsigned has0 = __ballot_sync(0xffffffffu, flags & kHas0), ends0 = __ballot_sync(0xffffffffu, flags & kEnds0), has1 = __ballot_sync(0xffffffffu, flags & kHas1);
+  // a chain: the warps that hold pieces of one unit, the first of them `from` (kind 0: the unit began in another CTA)
+  const int chains = static_cast<int>(has0 & 1u) + __popc(has1);
+#pragma unroll 1
+  for (int task = warp; task < chains * G; task += C::kWarps) {
+    const int ci = task / G, h = task - ci * G;
+    const int kind = (has0 & 1u) && ci == 0 ? 0 : 1;
+    unsigned rest = has1;
+    for (int k = static_cast<int>(has0 & 1u); k < ci; ++k) rest &= rest - 1;
+    const int from = kind ? __ffs(rest) - 1 : 0;
+    int last = from;
+    bool closed = kind == 0 && (ends0 & 1u);
+    if (!closed) {
+      const int held = __ffs(~(has0 >> (from + 1))) - 1, end = __ffs(ends0 >> (from + 1));
+      closed = end != 0 && end <= held;
+      last = from + (closed ? end : held);
+    }
+    const int b = kind ? recs[from].b1 : recs[from].b0, g = kind ? recs[from].g1 : recs[from].g0, u = kind ? recs[from].u1 : recs[from].u0;
+    auto piece = [&](int k) {
+      return reinterpret_cast<const float*>(smem + (from + k) * C::kWarpBytes + ((kind && k == 0) ? 0 : C::kStages * C::kGran)) + h * C::kPieceStride;
+    };
+    const int n = last - from + 1;
+    Acc a;
+    acc_clear(a);
+    acc_merge<false>(a, n, lane < n ? piece(lane)[D] : 0.0f, lane < n ? piece(lane)[D + 1] : 0.0f, on, [&](int k) { return piece(k) + d0; });
+    if (!(kind && closed)) {
+      const unsigned first = unit_place(ln, b, g, u) + kUnitCost;
+      const int nu = unit_blocks(ln, line_blocks(ln, b), u), cta_f = first / T;
+      if (!deliver(a, p.chunk_blocks > 0 ? 1 : 0, kind != 0, cta_f, static_cast<int>((first + nu - 1) / T) - cta_f + 1, h)) continue;
+    }
+    if (p.chunk_blocks == 0) {
+      store_out(a, b, g, h);
+    } else {
+      const size_t at = (static_cast<size_t>(b) * Hq + g * G + h) * p.max_chunks + u / ln.chunk;
+      const float dinv = a.den > 0.0f ? 1.0f / a.den : 0.0f;
+      if (on) *reinterpret_cast<float4*>(p.part_o + at * D + d0) = make_float4(a.num.x * dinv, a.num.y * dinv, a.num.z * dinv, a.num.w * dinv);
+      if (lane == 0) { p.part_m[at] = a.M * kLn2; p.part_l[at] = a.den * kUnshift; }
+    }
+  }
+  COOPT_TRACE_CYCLES(p.trace, kTrExit, tid == 0);
+  COOPT_TRACE_NS(p.trace, kTrExitNs, tid == 0);
+  if (p.chunk_blocks == 0) return;
+
+  // ---- Opt-Pa: what this CTA holds of a (sequence, kv head) is merged over its chunks, then with the other CTAs' shares ----
+  __syncthreads();                       // this CTA's chunks have been exported (or left in its slots)
+  int task = 0;
+  Walk c;
+  walk_start(ln, c, cta_lo, cta_hi, lane);
+  while (c.more) {
+    const int b = c.b, g = c.g, nb = c.nb, c_first = c.u / ln.chunk;
+    const bool cut_first = c.j != 0 || c.jend != c.n, first_began = c.j == 0, run_begins = first_began && c.u == 0;
+    bool cut_last = false, run_ends = false;
+    int c_last = c_first;
+    do {
+      c_last = c.u / ln.chunk;
+      cut_last = c.j != 0 || c.jend != c.n;
+      run_ends = c.u + c.n >= nb && c.jend == c.n;
+      walk_next(ln, c);
+    } while (c.more && c.b == b && c.g == g);
+    for (int h = 0; h < G; ++h, ++task) {
+      if (task % C::kWarps != warp) continue;
+      Acc a;
+      acc_clear(a);
+      const size_t rows = (static_cast<size_t>(b) * Hq + g * G + h) * p.max_chunks;
+      const size_t slots = (static_cast<size_t>(2 * gridDim.x) + 2 * blockIdx.x) * G + h;
+      auto cut = [&](int i) { return (i == c_first && cut_first) || (i == c_last && cut_last); };
+      auto slot = [&](int i) { return slots + (i == c_first && !first_began ? 0 : G); };
+      for (int c0 = c_first; c0 <= c_last; c0 += 32) {
+        const int n = min(32, c_last - c0 + 1);
+        float m = 0.0f, l = 0.0f;
+        if (lane < n) {
+          const int i = c0 + lane;
+          m = cut(i) ? __ldcg(p.run_m + slot(i)) : __ldcg(p.part_m + rows + i) * kLog2e;
+          l = cut(i) ? __ldcg(p.run_l + slot(i)) * kUnshift : __ldcg(p.part_l + rows + i);
+        }
+        acc_merge<true>(a, n, m, l, on, [&](int k) { return (cut(c0 + k) ? p.run_o + slot(c0 + k) * D : p.part_o + (rows + c0 + k) * D) + d0; });
+      }
+      if (!(run_begins && run_ends)) {
+        const int u_last = (nb - 1) / ln.chunk * ln.chunk;
+        const unsigned first = unit_place(ln, b, g, 0) + (whole ? 0 : kUnitCost);
+        const unsigned last = unit_place(ln, b, g, u_last) + (whole ? 0 : kUnitCost + (nb - u_last) - 1);
+        const int cta_f = first / T;
+        if (!deliver(a, 0, run_begins, cta_f, static_cast<int>(last / T) - cta_f + 1, h)) continue;
+      }
+      store_out(a, b, g, h);
+    }
+  }
+}
+
+template <int D, int FMT>
+int launch_one(const DecodeParams& p, int grid, bool dependent, cudaStream_t stream) {
+  using C = Cfg<D, FMT>;
+  if (!configure_kernel_smem(reinterpret_cast<const void*>(&paged_decode_kernel<D, FMT>), C::kSmemBytes)) return COOPT_ERR_CUDA;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(grid));
+  cfg.blockDim = dim3(C::kThreads);
+  cfg.dynamicSmemBytes = C::kSmemBytes;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = dependent ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, paged_decode_kernel<D, FMT>, p) == cudaSuccess ? COOPT_OK : COOPT_ERR_CUDA;
+}
+
+// coopt_decode_plan: a copy of the step's context lengths and of the valid part of its block table, with the block ids
+// range-checked once (a bad one is replaced by 0 and reported by the launches that read the plan).  All the rest of
+// the decomposition follows from the lengths, and every CTA of the attention kernel works out its own part of it.
+constexpr int kPlanThreads = 256;
+constexpr int kPlanPiece = 128;          // table entries a warp takes at a time
+__global__ void __launch_bounds__(kPlanThreads) decode_plan_kernel(const int* block_table, int width, const int* context_lens, int batch, int num_blocks,
+                                                                   int key, PlanHeader* header) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  int* lens = reinterpret_cast<int*>(header + 1);
+  int* table = reinterpret_cast<int*>(reinterpret_cast<uint8_t*>(header) + plan_table_offset(batch));
+  __shared__ int bad;
+  if (threadIdx.x == 0) bad = 0;
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warps = gridDim.x * (kPlanThreads / 32);
+  const int per_row = (width + kPlanPiece - 1) / kPlanPiece;
+  for (int i = (blockIdx.x * kPlanThreads + threadIdx.x) >> 5; i < batch * per_row; i += warps) {
+    const int b = i / per_row, j0 = (i - b * per_row) * kPlanPiece + lane;
+    const int L = max(0, min(context_lens[b], width * kBlockSize)), nb = (L + kBlockSize - 1) / kBlockSize;
+    if (j0 == 0) lens[b] = L;
+    const size_t at = static_cast<size_t>(b) * width + j0;
+    int id[kPlanPiece / 32];
+#pragma unroll
+    for (int k = 0; k < kPlanPiece / 32; ++k) id[k] = j0 + 32 * k < nb ? block_table[at + 32 * k] : 0;
+#pragma unroll
+    for (int k = 0; k < kPlanPiece / 32; ++k) {
+      if (id[k] < 0 || id[k] >= num_blocks) { bad = 1; id[k] = 0; }
+      if (j0 + 32 * k < nb) table[at + 32 * k] = id[k];
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) header->status[blockIdx.x] = bad ? COOPT_ERR_INVALID_ARG : COOPT_OK;
+  if (blockIdx.x == 0) {
+    if (threadIdx.x == 0) header->key = key;
+    for (int i = gridDim.x + threadIdx.x; i < kPlanCtas; i += kPlanThreads) header->status[i] = COOPT_OK;
   }
 }
 
 }  // namespace
 
-// Workspace layout: [header 256 B: word 0 = status][counters int32 x 16384][partials][plan of a one-off call].
-size_t plan_bytes(int planned_ctas, int batch, int num_kv_heads, int max_blocks_per_seq, int chunk_blocks);
-int plan_cta_stride(int planned_ctas, int batch, int num_kv_heads, int max_blocks_per_seq, int chunk_blocks);
-int launch_decode_plan(const int32_t* block_table, int32_t max_blocks_per_seq, const int32_t* context_lens, int32_t batch,
-                       int32_t num_kv_heads, int32_t num_blocks, int32_t chunk_size, int planned_ctas, void* plan,
-                       cudaStream_t stream);
-
-static size_t partials_bytes(int planned_ctas, int group, int head_dim, int batch, int num_q_heads, int max_chunks) {
-  size_t bytes = kWsHeaderBytes + static_cast<size_t>(kCounterSlots) * 4;
-  const size_t dec = static_cast<size_t>(2) * planned_ctas * group * (head_dim + 2) * 4;
-  const size_t chk = static_cast<size_t>(batch) * num_q_heads * max_chunks * (head_dim + 2) * 4;
-  // chunk mode holds both: the per-chunk partials it exports and the merged pieces of the CTAs' runs
-  return (bytes + (max_chunks > 0 ? chk + dec + 256 : dec) + 256 + 255) / 256 * 256;
+static int launch_attention(const DecodeParams& p, int head_dim, int dtype, int grid, bool dependent, cudaStream_t stream) {
+  if (head_dim == 128) {
+    if (dtype == COOPT_KV_FP8_E4M3) return launch_one<128, COOPT_KV_FP8_E4M3>(p, grid, dependent, stream);
+    if (dtype == COOPT_KV_FP8_E5M2) return launch_one<128, COOPT_KV_FP8_E5M2>(p, grid, dependent, stream);
+    return launch_one<128, COOPT_KV_BF16>(p, grid, dependent, stream);
+  }
+  if (dtype == COOPT_KV_FP8_E4M3) return launch_one<64, COOPT_KV_FP8_E4M3>(p, grid, dependent, stream);
+  if (dtype == COOPT_KV_FP8_E5M2) return launch_one<64, COOPT_KV_FP8_E5M2>(p, grid, dependent, stream);
+  return launch_one<64, COOPT_KV_BF16>(p, grid, dependent, stream);
 }
-size_t decode_workspace_bytes(int planned_ctas, int group, int head_dim, int batch, int num_q_heads, int num_kv_heads,
-                              int max_blocks_per_seq, int chunk_blocks, int max_chunks) {
-  // calls that bring no plan of their own (coopt_paged_decode, coopt_paged_chunked) plan into the workspace
-  return partials_bytes(planned_ctas, group, head_dim, batch, num_q_heads, max_chunks) +
-         plan_bytes(planned_ctas, batch, num_kv_heads, max_blocks_per_seq, chunk_blocks);
+
+// CTAs of a decode launch, from what the host knows: all that fit the device, or fewer where even full block tables would
+// leave a CTA without its smallest share.  The same on the sizing and the launching side.
+int decode_ctas(int num_sms, int batch, int num_kv_heads, int max_blocks_per_seq, int chunk_blocks) {
+  const long long units = chunk_blocks > 0 ? (max_blocks_per_seq + chunk_blocks - 1) / chunk_blocks : 1;
+  const long long places = static_cast<long long>(batch) * num_kv_heads * (max_blocks_per_seq + units * kUnitCost);
+  const long long most = (places + kMinPlaces - 1) / kMinPlaces;
+  return static_cast<int>(most < kCtasPerSm * num_sms ? most : kCtasPerSm * num_sms);
 }
 size_t workspace_control_bytes() { return kWsHeaderBytes + static_cast<size_t>(kCounterSlots) * 4; }
-
-int decode_planned_ctas(int num_sms, long long upper_blocks) {
-  // a CTA's slice must fit one round of staged block ids, so that no (sequence, kv head) is cut twice
-  // inside one CTA; slices differ by at most one block from the mean
-  const long long need = (upper_blocks + (kCap - 16) - 1) / (kCap - 16);
-  return static_cast<int>(need > num_sms ? need : num_sms);
-}
 int decode_max_batch() { return kMaxBatch; }
 int decode_counter_slots() { return kCounterSlots; }
-int decode_max_chunk_blocks() { return kCap; }
+int decode_max_chunk_blocks() { return kMaxChunkBlocks; }
 
+// Workspace layout: [header 256 B: word 0 = status][counters int32 x 16384][chunk mode: exported partials][shared pieces].
 void chunk_partial_offsets(int batch, int num_q_heads, int head_dim, int max_chunks, size_t* o, size_t* m, size_t* l) {
   const size_t rows = static_cast<size_t>(batch) * num_q_heads * max_chunks;
   *o = workspace_control_bytes();
   *m = *o + rows * head_dim * 4;
   *l = *m + rows * 4;
 }
+static size_t pieces_offset(int batch, int num_q_heads, int head_dim, int max_chunks) {
+  const size_t partials = static_cast<size_t>(batch) * num_q_heads * max_chunks * (head_dim + 2) * 4;
+  return (workspace_control_bytes() + partials + 255) / 256 * 256;
+}
+static size_t pieces_rows(int ctas, int group, int max_chunks) { return static_cast<size_t>(max_chunks > 0 ? 4 : 2) * ctas * group; }
 
-template <int D>
-static int launch_one(const DecodeParams& p, int grid, cudaStream_t stream) {
-  using C = Cfg<D>;
-  if (!configure_kernel_smem(reinterpret_cast<const void*>(&paged_decode_kernel<D>), C::kSmemBytes)) return COOPT_ERR_CUDA;
-  paged_decode_kernel<D><<<grid, kThreads, C::kSmemBytes, stream>>>(p);
+size_t decode_workspace_bytes(int ctas, int group, int head_dim, int batch, int num_q_heads, int max_chunks) {
+  return (pieces_offset(batch, num_q_heads, head_dim, max_chunks) + pieces_rows(ctas, group, max_chunks) * (head_dim + 2) * 4 + 255) / 256 * 256;
+}
+size_t decode_plan_bytes(int batch, int max_blocks_per_seq) {
+  return plan_table_offset(batch) + static_cast<size_t>(batch) * max_blocks_per_seq * 4;
+}
+
+int launch_decode_plan(const int32_t* block_table, int32_t max_blocks_per_seq, const int32_t* context_lens, int32_t batch,
+                       int32_t num_kv_heads, int32_t num_blocks, int32_t chunk_size, void* plan, cudaStream_t stream) {
+  const long long pieces = static_cast<long long>(batch) * ((max_blocks_per_seq + kPlanPiece - 1) / kPlanPiece);
+  const long long ctas = (pieces + kPlanThreads / 32 - 1) / (kPlanThreads / 32);
+  const int key = plan_key(batch, num_kv_heads, chunk_size / kBlockSize, max_blocks_per_seq, num_blocks);
+  decode_plan_kernel<<<static_cast<unsigned>(ctas < kPlanCtas ? ctas : kPlanCtas), kPlanThreads, 0, stream>>>(
+      block_table, max_blocks_per_seq, context_lens, batch, num_blocks, key, static_cast<PlanHeader*>(plan));
   return cudaGetLastError() == cudaSuccess ? COOPT_OK : COOPT_ERR_CUDA;
 }
 
-int launch_paged_decode_umma(const DecodeParams& p, int head_dim, int grid, bool overlap_previous, cudaStream_t stream);
-
-// Everything of DecodeParams that does not depend on where the plan comes from.
-static void fill_decode_params(DecodeParams& p, const coopt_cache* c, const void* q, void* out, const int32_t* block_table,
-                               int32_t max_blocks_per_seq, const int32_t* context_lens, int32_t batch, int32_t num_q_heads,
-                               float sm_scale, int32_t chunk_size, const int32_t* cu_q_lens, void* workspace, int planned_ctas) {
-  p = DecodeParams{};
-  p.cache = static_cast<const uint8_t*>(c->data);
-  p.q = static_cast<const __nv_bfloat16*>(q);
-  p.out = static_cast<__nv_bfloat16*>(out);
-  p.block_table = block_table;
-  p.context_lens = context_lens;
-  p.cu_q_lens = cu_q_lens;
-  p.max_blocks_per_seq = max_blocks_per_seq;
-  p.batch = batch;
-  p.num_q_heads = num_q_heads;
+int launch_decode(const coopt_cache* c, const DecodeCall& a, cudaStream_t stream) {
+  DecodeParams p = {};
+  p.cache = static_cast<uint8_t*>(c->data);
+  p.q = static_cast<const __nv_bfloat16*>(a.q);
+  p.out = static_cast<__nv_bfloat16*>(a.out);
+  p.block_table = a.block_table;
+  p.context_lens = a.context_lens;
+  p.cu_q_lens = a.cu_q_lens;
+  p.max_blocks_per_seq = a.max_blocks_per_seq;
+  p.batch = a.batch;
+  p.num_q_heads = a.num_q_heads;
   p.num_kv_heads = c->num_kv_heads;
-  p.group = num_q_heads / c->num_kv_heads;
+  p.group = a.num_q_heads / c->num_kv_heads;
   p.num_blocks = c->num_blocks;
-  p.kv_e5m2 = c->dtype == COOPT_KV_FP8_E5M2 ? 1 : 0;
-  p.sm_scale_log2 = sm_scale * kLog2e;
-  p.planned_ctas = planned_ctas;
-  p.chunk_blocks = chunk_size / kBlockSize;
-  p.max_chunks = chunk_size > 0 ? static_cast<int>((static_cast<long long>(max_blocks_per_seq) * kBlockSize + chunk_size - 1) / chunk_size) : 0;
-  uint8_t* ws = static_cast<uint8_t*>(workspace);
+  p.sm_scale_log2 = a.sm_scale * kLog2e;
+  p.chunk_blocks = a.chunk_size / kBlockSize;
+  p.max_chunks = a.chunk_size > 0 ? static_cast<int>((static_cast<long long>(a.max_blocks_per_seq) * kBlockSize + a.chunk_size - 1) / a.chunk_size) : 0;
+  if (a.plan != nullptr) {
+    const uint8_t* plan = static_cast<const uint8_t*>(a.plan);
+    p.plan = reinterpret_cast<const PlanHeader*>(plan);
+    p.context_lens = reinterpret_cast<const int*>(plan + kPlanHeaderBytes);
+    p.block_table = reinterpret_cast<const int*>(plan + plan_table_offset(a.batch));
+    p.plan_key = plan_key(a.batch, c->num_kv_heads, p.chunk_blocks, a.max_blocks_per_seq, c->num_blocks);
+  }
+  p.k_new = static_cast<const __nv_bfloat16*>(a.k_new);
+  p.v_new = static_cast<const __nv_bfloat16*>(a.v_new);
+  p.slot_mapping = reinterpret_cast<const long long*>(a.slot_mapping);
+  p.kv_token_stride = a.kv_token_stride;
+  p.overlap_previous = a.order == kOverlapPrevious ? 1 : 0;
+  uint8_t* ws = static_cast<uint8_t*>(a.workspace);
   p.status = reinterpret_cast<int*>(ws);
   p.counters = reinterpret_cast<int*>(ws + kWsHeaderBytes);
-  uint8_t* parts = ws + workspace_control_bytes();
-  if (chunk_size > 0) {
+  if (a.chunk_size > 0) {
     size_t o, m, l;
-    chunk_partial_offsets(batch, num_q_heads, c->head_dim, p.max_chunks, &o, &m, &l);
+    chunk_partial_offsets(a.batch, a.num_q_heads, c->head_dim, p.max_chunks, &o, &m, &l);
     p.part_o = reinterpret_cast<float*>(ws + o);
     p.part_m = reinterpret_cast<float*>(ws + m);
     p.part_l = reinterpret_cast<float*>(ws + l);
-    const size_t chunk_rows = static_cast<size_t>(batch) * num_q_heads * p.max_chunks;
-    const size_t run_at = (l + chunk_rows * 4 + 255) / 256 * 256;
-    const size_t rows = static_cast<size_t>(2) * planned_ctas * p.group;
-    p.run_o = reinterpret_cast<float*>(ws + run_at);
-    p.run_m = p.run_o + rows * c->head_dim;
-    p.run_l = p.run_m + rows;
-  } else {
-    const size_t rows = static_cast<size_t>(2) * planned_ctas * p.group;
-    p.part_o = reinterpret_cast<float*>(parts);
-    p.part_m = p.part_o + rows * c->head_dim;
-    p.part_l = p.part_m + rows;
-    p.run_o = p.part_o;
-    p.run_m = p.part_m;
-    p.run_l = p.part_l;
   }
-}
-
-static void attach_plan(DecodeParams& p, const void* plan) {
-  p.plan_header = static_cast<const PlanHeader*>(plan);
-  p.plan = static_cast<const uint8_t*>(plan) + kPlanHeaderBytes;
-  p.plan_cta_stride = plan_cta_stride(p.planned_ctas, p.batch, p.num_kv_heads, p.max_blocks_per_seq, p.chunk_blocks);
-  p.plan_key = plan_key(p.planned_ctas, p.batch, p.num_kv_heads, p.chunk_blocks, p.max_blocks_per_seq, p.num_blocks);
-}
-
-// A call that brings no plan: the FP8 kernel's plan is made in the workspace first (one more small launch);
-// the bf16 ablation kernel plans inside its own CTAs.
-int launch_paged_decode(const coopt_cache* c, const void* q, void* out, const int32_t* block_table,
-                        int32_t max_blocks_per_seq, const int32_t* context_lens, int32_t batch, int32_t num_q_heads,
-                        float sm_scale, int32_t chunk_size, const int32_t* cu_q_lens, void* workspace, int planned_ctas,
-                        cudaStream_t stream) {
-  DecodeParams p;
-  fill_decode_params(p, c, q, out, block_table, max_blocks_per_seq, context_lens, batch, num_q_heads, sm_scale, chunk_size,
-                     cu_q_lens, workspace, planned_ctas);
-  if (!is_fp8(c->dtype))
-    return c->head_dim == 128 ? launch_one<128>(p, planned_ctas, stream) : launch_one<64>(p, planned_ctas, stream);
-  void* plan = static_cast<uint8_t*>(workspace) + partials_bytes(planned_ctas, p.group, c->head_dim, batch, num_q_heads, p.max_chunks);
-  const int rc = launch_decode_plan(block_table, max_blocks_per_seq, context_lens, batch, c->num_kv_heads, c->num_blocks, chunk_size,
-                                    planned_ctas, plan, stream);
-  if (rc != COOPT_OK) return rc;
-  attach_plan(p, plan);
-  return launch_paged_decode_umma(p, c->head_dim, planned_ctas, false, stream);
-}
-
-// A call that brings its plan (coopt_decode_plan) and may append one token per sequence in the same launch.
-int launch_decode_planned(const coopt_cache* c, const void* plan, const void* k_new, const void* v_new, int64_t kv_token_stride,
-                          const int64_t* slot_mapping, const void* q, void* out, int32_t max_blocks_per_seq, int32_t batch,
-                          int32_t num_q_heads, float sm_scale, int32_t chunk_size, const int32_t* cu_q_lens, void* workspace,
-                          int planned_ctas, bool overlap_previous, cudaStream_t stream) {
-  DecodeParams p;
-  fill_decode_params(p, c, q, out, nullptr, max_blocks_per_seq, nullptr, batch, num_q_heads, sm_scale, chunk_size, cu_q_lens,
-                     workspace, planned_ctas);
-  p.k_new = static_cast<const __nv_bfloat16*>(k_new);
-  p.v_new = static_cast<const __nv_bfloat16*>(v_new);
-  p.slot_mapping = reinterpret_cast<const long long*>(slot_mapping);
-  p.kv_token_stride = kv_token_stride;
-  attach_plan(p, plan);
-  return launch_paged_decode_umma(p, c->head_dim, planned_ctas, overlap_previous, stream);
+  const size_t rows = pieces_rows(a.ctas, p.group, p.max_chunks);
+  p.run_o = reinterpret_cast<float*>(ws + pieces_offset(a.batch, a.num_q_heads, c->head_dim, p.max_chunks));
+  p.run_m = p.run_o + rows * c->head_dim;
+  p.run_l = p.run_m + rows;
+#ifdef COOPT_TRACE
+  p.trace = trace_buffer();
+#endif
+  return launch_attention(p, c->head_dim, c->dtype, a.ctas, a.order != kAfterPrevious, stream);
 }
 
 }  // namespace coopt

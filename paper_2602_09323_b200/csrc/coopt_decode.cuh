@@ -1,0 +1,119 @@
+// Paged GQA decode: what the kernel and the host side share: the work decomposition, the layout of a plan buffer and
+// the kernel's parameters.
+//
+// Work decomposition (Eq. 9: only the valid blocks of every sequence are listed).  A unit is what one softmax runs
+// over before anything is merged: a (sequence, kv head), or in chunk mode (Opt-Pa) one chunk of one.  All units lie
+// one behind the other on a line, in the order sequence, kv head, chunk; a unit of n blocks takes n + kUnitCost places
+// of it, the extra ones in front, because a unit costs its warp a start and an end (query rows, reduction, store)
+// besides its blocks.  CTA i takes the places [i T, (i + 1) T), warp w of it an equal part of those, and a block
+// belongs to the warp that holds its place.  So every warp has at most two units that it holds only a piece of: the
+// one it starts in the middle of, and the one it does not reach the end of.
+#pragma once
+
+#include "coopt_common.cuh"
+
+namespace coopt {
+
+constexpr int kMaxBatch = 512;
+constexpr int kMaxGroup = 8;
+constexpr int kMaxChunkBlocks = 2048;
+constexpr int kCounterSlots = 16384;
+constexpr int kWsHeaderBytes = 256;
+// Measured, us a pass: cost 3 / 5 places 435 / 429 (64 mixed lengths, 4 layers), 103 / 101 (24 sequences, G = 8, 4 layers),
+// 126 / 104 (21 sequences of 2..60 tokens, 8 layers); smallest share 64 / 16 places 20.5 / 16.4 (one sequence of 777
+// tokens), 142 / 102 (7 sequences of 272..544 tokens, 8 layers): where a call cannot fill the device, spreading it wins.
+constexpr int kUnitCost = 5;          // places of the line that a unit takes besides its blocks
+constexpr int kCtasPerSm = 1;
+constexpr int kMinPlaces = 16;        // smallest share of a CTA
+constexpr int kWholeUnits = 32;       // units of at most so many blocks (head_dim 64: twice) are not cut between CTAs
+constexpr int kWholeUnitsIdle = 192;  // .. where the call does not fill the device
+constexpr int kNoChunks = 1 << 30;    // "blocks per chunk" of a call without chunks
+
+// A plan: header, the clamped context lengths int32[batch] (padded to 16 bytes), the block table
+// int32[batch][max_blocks_per_seq] with its valid entries range-checked.
+constexpr int kPlanCtas = 48;
+struct PlanHeader {
+  int key;                   // plan_key() of the problem the plan was made for
+  int pad[15];
+  int status[kPlanCtas];     // by CTA of the planning kernel: a coopt_status that the launches which read the plan report
+};
+constexpr int kPlanHeaderBytes = 256;
+static_assert(sizeof(PlanHeader) == kPlanHeaderBytes, "plan layout");
+__host__ __device__ inline size_t plan_table_offset(int batch) { return kPlanHeaderBytes + (static_cast<size_t>(batch) * 4 + 15) / 16 * 16; }
+
+// What a launch and the plan it is handed must agree on.
+__host__ __device__ inline int plan_key(int batch, int num_kv_heads, int chunk_blocks, int max_blocks_per_seq, int num_blocks) {
+  unsigned int h = 0x9e3779b9u;
+  const int v[5] = {batch, num_kv_heads, chunk_blocks, max_blocks_per_seq, num_blocks};
+  for (int i = 0; i < 5; ++i) h = (h ^ static_cast<unsigned int>(v[i])) * 0x01000193u + 0x7f4a7c15u;
+  return static_cast<int>(h | 1u);
+}
+
+struct DecodeParams {
+  uint8_t* cache;
+  const __nv_bfloat16* q;
+  __nv_bfloat16* out;
+  const int* block_table;
+  const int* context_lens;
+  const PlanHeader* plan;  // null: block_table and context_lens are the caller's own and are checked here
+  const int* cu_q_lens;    // chunk mode of coopt_paged_chunked: prefix sums of the query tokens (must be 0..batch); else null
+  int plan_key;
+  // fused append (null when the call has no new tokens): Algorithm 1 phase 1 for one token per sequence
+  const __nv_bfloat16* k_new;
+  const __nv_bfloat16* v_new;
+  const long long* slot_mapping;
+  long long kv_token_stride;
+  int max_blocks_per_seq;
+  int batch, num_q_heads, num_kv_heads, group;
+  int num_blocks;
+  int overlap_previous;    // 1: plan and cache were complete before the kernel in front of this one began
+  float sm_scale_log2;     // sm_scale * log2(e)
+  int chunk_blocks;        // 0 = decode mode
+  int max_chunks;
+  int* status;
+  int* counters;           // [regions][ctas][kMaxGroup]: pieces delivered, by first CTA and head
+  float* part_o;           // chunk mode: exported partials [B][Hq][max_chunks][D]
+  float* part_m;           // [B][Hq][max_chunks]
+  float* part_l;
+  float* run_o;            // pieces that CTAs share: [regions][2 ctas][G][D]; region 0 (sequence, kv head), region 1 (chunk mode) chunks
+  float* run_m;            // [regions][2 ctas][G], base-2 logarithm units
+  float* run_l;
+  unsigned long long* trace;   // time stamps (trace build only; null otherwise)
+};
+
+// ---- host side -------------------------------------------------------------------------------------------------
+enum DecodeOrder {
+  kAfterPrevious = 0,     // an ordinary launch
+  kDependent,             // may be set up while the kernel before it runs, and waits for it before it reads anything
+  kOverlapPrevious        // the plan and the cache were complete before that kernel began: they are read early
+};
+struct DecodeCall {
+  const void* q;
+  void* out;
+  const int32_t* block_table;       // these two, or a plan
+  const int32_t* context_lens;
+  const void* plan;
+  const int32_t* cu_q_lens;
+  const void* k_new;
+  const void* v_new;
+  const int64_t* slot_mapping;
+  int64_t kv_token_stride;
+  int32_t max_blocks_per_seq, batch, num_q_heads, chunk_size;
+  float sm_scale;
+  void* workspace;
+  int ctas;                         // decode_ctas()
+  DecodeOrder order;
+};
+int launch_decode(const coopt_cache* c, const DecodeCall& a, cudaStream_t stream);
+int launch_decode_plan(const int32_t* block_table, int32_t max_blocks_per_seq, const int32_t* context_lens, int32_t batch,
+                       int32_t num_kv_heads, int32_t num_blocks, int32_t chunk_size, void* plan, cudaStream_t stream);
+int decode_ctas(int num_sms, int batch, int num_kv_heads, int max_blocks_per_seq, int chunk_blocks);
+size_t decode_workspace_bytes(int ctas, int group, int head_dim, int batch, int num_q_heads, int max_chunks);
+size_t decode_plan_bytes(int batch, int max_blocks_per_seq);
+size_t workspace_control_bytes();
+int decode_max_batch();
+int decode_counter_slots();
+int decode_max_chunk_blocks();
+void chunk_partial_offsets(int batch, int num_q_heads, int head_dim, int max_chunks, size_t* o, size_t* m, size_t* l);
+
+}  // namespace coopt

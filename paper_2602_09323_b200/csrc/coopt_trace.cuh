@@ -1,5 +1,5 @@
-// Time stamps of the roles of the tcgen05 decode kernel.  Compiled in only with -DCOOPT_TRACE (the separate
-// library libcoopt_trace.so); the ordinary library contains none of this.  A stamp is the SM's cycle counter
+// Time stamps of the decode and prefill kernels.  Compiled in only with -DCOOPT_TRACE (the separate library
+// libcoopt_trace.so); the ordinary library contains none of this.  A stamp is the SM's cycle counter
 // written to slot `s` of the CTA's record in a caller-supplied buffer (coopt_trace_set_buffer); two slots
 // hold the global nanosecond timer at entry and exit so that the CTAs of a launch can be laid side by side.
 #pragma once
@@ -8,45 +8,27 @@
 
 namespace coopt {
 
-enum TraceSlot {
-  kTrEntry = 0,        // first instruction of the CTA (cycles; every other cycle stamp is read against this one)
-  kTrEntryNs,          // global timer at entry
-  kTrSetupDone,        // barriers initialised, tensor memory allocated, plan in shared memory
-  kTrIdsStaged,        // block ids of the first round staged: the copy warp may start
-  kTrFirstCopy,        // first tile requested
-  kTrFirstLanded,      // first tile's bytes have landed (seen by the lane that issues the logits)
-  kTrFirstProbs,       // probabilities of the first tile written (team 0)
-  kTrLastCopy,         // last tile requested
-  kTrLastLanded,       // last tile's bytes have landed
-  kTrLastPv,           // last P V group committed
-  kTrTeamsDone,        // team 0 has handed over its last piece
-  kTrLastHandOff,      // epilogue warp has received the last segment
-  kTrPieceStored,      // last piece written to the workspace (before the counter)
-  kTrCounted,          // counter round trip done
-  kTrEpilogueDone,     // last store / merge done
-  kTrExit,             // behind the final barrier
-  kTrExitNs,           // global timer at exit
-  kTrWriteDone,        // fused step: the new tokens' granules are written
-  kTrNumSeg,           // number of segments of the first round (a count, not a time)
-  kTrNumTiles,         // tiles of the CTA (a count)
-  kTrSmId,             // the SM the CTA ran on
-  kTrProducerPlan,     // the copy warp has seen the plan
-  kTrPrevExitNs,       // what kTrExitNs held at entry: the exit of this CTA's slot in the launch before
-  kTrFirstCopyReady,   // the copy warp is about to request the first tile (rows worked out, byte count posted)
-  kTrSegBase = 24,     // 24 + i: epilogue warp received segment i (i < 20)
-  kTrTeamSegBase = 44, // 44 + i: team 0 began segment i (i < 20)
-  kTrCopyTileBase = 64,    // 64 + i: tile i requested (i < 32)
-  kTrProbsTileBase = 96,   // 96 + i: probabilities of tile i written by its team (i < 32)
-  kTrSegTileBase = 128,    // 128 + i: 1 + number of the first tile of segment i (i < 20; a count)
-  kTrLogitsTileBase = 148, // 148 + i: logits of tile i issued (i < 32)
-  kTrPvTileBase = 180,     // 180 + i: P V of tile i issued (i < 32)
-  kTraceSlots = 256
+enum TraceSlot {         // of the decode kernel, by the first lane of warp 0 unless it says otherwise
+  kTrEntry = 0,          // first instruction of the CTA (cycles; every other cycle stamp is read against this one)
+  kTrEntryNs,            // global timer at entry
+  kTrLine,               // context lengths read and summed up
+  kTrFirstCopy,          // the ring's first copies requested
+  kTrPrevDone,           // the kernel before has finished
+  kTrQuery,              // query operand of the first unit ready
+  kTrFirstLanded,        // first block has landed
+  kTrStreamed,           // all warps have worked through their blocks
+  kTrExit,               // last store issued
+  kTrExitNs,             // global timer at exit
+  kTrSmId,               // 1 + the SM the CTA ran on
+  kTrPrevExitNs,         // what kTrExitNs held at entry: the exit of this CTA's slot in the launch before
+  kTrBlocks,             // blocks of warp 0 (a count)
+  kTrWarpEnd = 16,       // 16 + w: warp w has worked through its blocks
+  kTraceSlots = 32
 };
 constexpr int kTraceMaxCtas = 1024;
 
 #ifdef COOPT_TRACE
 unsigned long long* trace_buffer();      // host: what coopt_trace_set_buffer registered (nullptr = none)
-int trace_plan_rotate();                 // host: what coopt_trace_set_rotate registered
 #ifdef __CUDACC__
 __device__ __forceinline__ void trace_put(unsigned long long* buf, int slot, unsigned long long v) {
   if (buf != nullptr && blockIdx.x < kTraceMaxCtas && slot < kTraceSlots) buf[blockIdx.x * kTraceSlots + slot] = v;

@@ -1,11 +1,10 @@
 """Where the time of one launch goes: ``python -m paper_2602_09323_b200.trace [--workload ...]``.
 
 Builds ``libcoopt_trace.so`` (the library's sources with ``-DCOOPT_TRACE``), runs the fused decode step of a
-workload a few times and prints, for the last launch, when each role of the tcgen05 kernel reached its
+workload a few times and prints, for the last launch, when the decode kernel's CTAs reached their
 milestones: per milestone the median, the earliest and the latest CTA, in microseconds from that CTA's own
-first instruction, and the span of the whole launch on the global timer.  The stamps cost a few stores per
-tile; the launch is a few per cent slower than in the ordinary library, so this is a breakdown, not a
-benchmark.  ``--workload chunked_prefill`` prints instead, for the tcgen05 prefill kernel, the cycles that the
+first instruction, and the span of the whole launch on the global timer.  The stamps cost a few stores, so this is a
+breakdown, not a benchmark.  ``--workload chunked_prefill`` prints instead, for the tcgen05 prefill kernel, the cycles that the
 first thread of softmax team 0 and the two instruction-issuing lanes spend in each phase of a tile.
 """
 from __future__ import annotations
@@ -18,23 +17,21 @@ import torch
 
 from . import binding, build, workloads
 
-SLOTS = 256
+SLOTS = 32
 MAX_CTAS = 1024
-NAMES = ["entry", "entry_ns", "setup_done", "plan_in_smem", "first_copy", "first_landed", "first_probs", "last_copy",
-         "last_landed", "last_pv", "teams_done", "last_hand_off", "piece_stored", "counted", "epilogue_done", "exit",
-         "exit_ns", "write_done", "num_seg", "num_tiles", "sm_id", "producer_plan", "prev_exit_ns", "first_copy_ready"]
-SEG_BASE, TEAM_SEG_BASE = 24, 44
+ENTRY, ENTRY_NS, STREAMED, EXIT, EXIT_NS, SM_ID, PREV_EXIT_NS, BLOCKS, WARP_END = 0, 1, 7, 8, 9, 10, 11, 12, 16
+MILESTONES = {2: "line_summed", 3: "first_copies", 4: "previous_done", 5: "query_ready", 6: "first_landed", STREAMED: "streamed", EXIT: "exit"}
+SHAPES = {"one_sequence": ([777], 40, 8, 128), "short": ([3, 28, 17, 9, 22, 28, 1, 14], 56, 8, 128), "group_of_eight": (None, 64, 8, 128)}
 
 
 def main():
     ap = argparse.ArgumentParser()
-    ap.add_argument("--workload", default="llama13b_decode", choices=["llama13b_decode", "mixed_serving", "long_context", "chunked_prefill"])
+    ap.add_argument("--workload", default="llama13b_decode",
+                    choices=["llama13b_decode", "mixed_serving", "long_context", "chunked_prefill"] + sorted(SHAPES))
     ap.add_argument("--no-append", action="store_true", help="attention only (no new token written in the launch)")
+    ap.add_argument("--overlap", action="store_true", help="every launch may start while the one before it drains")
     ap.add_argument("--launches", type=int, default=12)
-    ap.add_argument("--timeline", type=int, nargs="*", default=None, help="CTAs whose tile-by-tile timeline is printed")
-    ap.add_argument("--rotate", type=int, default=0, help="with --per-cta: the second listed launch gives CTA i the plan "
-                    "region i + ROTATE, to tell slow shares of the plan from slow SMs")
-    ap.add_argument("--per-cta", action="store_true", help="also list every CTA: SM, segments, streaming time")
+    ap.add_argument("--per-cta", action="store_true", help="also list every CTA: SM, blocks of warp 0, life time")
     ap.add_argument("--sm-mhz", type=float, default=1965.0, help="SM clock used to turn cycles into microseconds")
     args = ap.parse_args()
     binding.use_library(build.build(trace=True))
@@ -48,8 +45,11 @@ def main():
         w = workloads.config_llama13b_decode()
     elif args.workload == "mixed_serving":
         w = workloads.config_mixed_serving()
-    else:
+    elif args.workload == "long_context":
         w, chunk = workloads.config_long_context(), 2048
+    else:
+        lengths, hq, hkv, d = SHAPES[args.workload]
+        w = workloads.make_workload(args.workload, lengths or workloads.uniform_lengths(24, 300, 4000, 7), hq, hkv, d)
     B, Hq, Hkv, D = w.batch, w.num_q_heads, w.num_kv_heads, w.head_dim
     k, v, slots = w.k.cuda(), w.v.cuda(), w.slot_mapping.cuda()
     last = torch.tensor([w.kv_offsets[b] + L - 1 for b, L in enumerate(w.context_lens)])
@@ -68,72 +68,36 @@ def main():
     buf = torch.zeros(MAX_CTAS * SLOTS, dtype=torch.int64, device="cuda")
     assert lib.coopt_trace_set_buffer(ctypes.c_void_p(buf.data_ptr()), buf.numel() * 8) == 0
     out = torch.empty_like(q)
-    lib.coopt_trace_set_rotate.restype, lib.coopt_trace_set_rotate.argtypes = ctypes.c_int, [ctypes.c_int]
-    for i in range(args.launches):
-        if i != args.launches - 1:
-            buf.zero_()                     # (the last launch follows its predecessor directly and keeps its exit times)
-        lib.coopt_trace_set_rotate(args.rotate if i == args.launches - 1 else 0)
-        if args.no_append:
-            binding.decode_step_planned(caches[i % 2], plan, q, table.shape[1], w.sm_scale, ws, chunk_size=chunk, out=out)
-        else:
-            binding.decode_step_planned(caches[i % 2], plan, q, table.shape[1], w.sm_scale, ws, k_new, v_new, s_new,
-                                        chunk_size=chunk, out=out)
-        if i == args.launches - 3:
-            torch.cuda.synchronize()
-            prev = buf.cpu().numpy().reshape(MAX_CTAS, SLOTS).copy()
+    new = (None, None, None) if args.no_append else (k_new, v_new, s_new)
+    torch.cuda.synchronize()
+    for i in range(args.launches):          # (every launch follows its predecessor directly and finds its exit times)
+        binding.decode_step_planned(caches[i % 2], plan, q, table.shape[1], w.sm_scale, ws, *new, chunk_size=chunk, out=out,
+                                    flags=binding.FLAG_OVERLAP_PREVIOUS if args.overlap and i else 0)
     torch.cuda.synchronize()
     assert binding.workspace_status(ws) == 0
     t = buf.cpu().numpy().reshape(MAX_CTAS, SLOTS)
-    if args.per_cta:
-        # streaming time (first copy requested to last tile landed) of every CTA in the last two launches, by SM
-        us_ = 1.0 / args.sm_mhz
-        rows = []
-        for rec in (prev, t):
-            r = rec[rec[:, 0] != 0]
-            rows.append({int(x[20]) - 1: ((x[8] - x[4]) * us_, int(x[18]), (x[15] - x[0]) * us_) for x in r})
-        print("sm  launch A: stream_us nseg life_us | launch B: stream_us nseg life_us")
-        for sm in sorted(set(rows[0]) & set(rows[1])):
-            a, b = rows[0][sm], rows[1][sm]
-            print(f"{sm:3d}  {a[0]:6.2f} {a[1]} {a[2]:6.2f} | {b[0]:6.2f} {b[1]} {b[2]:6.2f}")
-    if args.timeline is not None:
-        us_ = 1.0 / args.sm_mhz
-        for cta in (args.timeline or [0, 1, 2, 3]):
-            x = t[cta]
-            seg_first = [int(v) - 1 for v in x[128:148] if v]
-            print(f"CTA {cta}: {int(x[18])} segments starting at tiles {seg_first}; epilogue got them at "
-                  f"{[round(float((v - x[0]) * us_), 2) for v in x[24:44] if v]}")
-            print(" tile   requested  logits_issued  probs_written  pv_issued   (us)")
-            for i in range(32):
-                if x[64 + i]:
-                    f = lambda v: f"{(v - x[0]) * us_:10.2f}" if v else "         -"
-                    print(f"{i:5d} {f(x[64 + i])}    {f(x[148 + i])}     {f(x[96 + i])}  {f(x[180 + i])}{'   <- segment starts' if i in seg_first else ''}")
-    t = t[t[:, 0] != 0]
+    t = t[t[:, ENTRY] != 0]
     us = 1.0 / args.sm_mhz
-    print(f"workload {args.workload}{' (no append)' if args.no_append else ''}: {t.shape[0]} CTAs, "
-          f"segments per CTA median {np.median(t[:, 18]):.0f} max {t[:, 18].max()}, tiles per CTA median {np.median(t[:, 19]):.0f} "
-          f"max {t[:, 19].max()}")
-    span = (t[:, 16].max() - t[:, 1].min()) / 1e3
-    print(f"launch span on the global timer: {span:.1f} us (first entry to last exit); entries spread over "
-          f"{(t[:, 1].max() - t[:, 1].min()) / 1e3:.1f} us, exits over {(t[:, 16].max() - t[:, 16].min()) / 1e3:.1f} us")
-    if t[:, 22].min() > 0:
-        print(f"gap to the launch before (its last exit to this one's first entry): {(t[:, 1].min() - t[:, 22].max()) / 1e3:.2f} us")
+    if args.per_cta:
+        print("CTA   SM  blocks of warp 0  first landed  streamed  exit (us)")
+        for i, x in enumerate(t):
+            print(f"{i:4d} {int(x[SM_ID]) - 1:4d} {int(x[BLOCKS]):4d}  {(x[6] - x[0]) * us:8.2f} {(x[STREAMED] - x[0]) * us:8.2f} {(x[EXIT] - x[0]) * us:8.2f}")
+    print(f"workload {args.workload}{' (no append)' if args.no_append else ''}{' (overlapped)' if args.overlap else ''}: {t.shape[0]} CTAs, "
+          f"blocks of warp 0 median {np.median(t[:, BLOCKS]):.0f} max {t[:, BLOCKS].max()}")
+    print(f"launch span on the global timer: {(t[:, EXIT_NS].max() - t[:, ENTRY_NS].min()) / 1e3:.1f} us (first entry to last exit); entries spread "
+          f"over {(t[:, ENTRY_NS].max() - t[:, ENTRY_NS].min()) / 1e3:.1f} us, exits over {(t[:, EXIT_NS].max() - t[:, EXIT_NS].min()) / 1e3:.1f} us")
+    if t[:, PREV_EXIT_NS].min() > 0:
+        print(f"last exit of the launch before to first entry of this one: {(t[:, ENTRY_NS].min() - t[:, PREV_EXIT_NS].max()) / 1e3:.2f} us; "
+              f"to last exit of this one: {(t[:, EXIT_NS].max() - t[:, PREV_EXIT_NS].max()) / 1e3:.2f} us")
     print(f"{'milestone':<16}{'median':>9}{'earliest':>10}{'latest':>9}   (us after the CTA's first instruction, {args.sm_mhz:.0f} MHz)")
-    for i, name in enumerate(NAMES):
-        if name in ("entry", "entry_ns", "exit_ns", "num_seg", "num_tiles", "sm_id", "prev_exit_ns"):
-            continue
-        col = t[:, i]
+    ends = t[:, WARP_END:WARP_END + 16]
+    cols = [(name, t[:, i]) for i, name in MILESTONES.items()]
+    cols[-2:-2] = [("first_warp_done", np.where(ends > 0, ends, np.iinfo(np.int64).max).min(axis=1)), ("last_warp_done", ends.max(axis=1))]
+    for name, col in cols:
         ok = col != 0
-        if not ok.any():
-            continue
-        rel = (col[ok] - t[ok, 0]) * us
-        print(f"{name:<16}{np.median(rel):9.2f}{rel.min():10.2f}{rel.max():9.2f}   ({int(ok.sum())} CTAs)")
-    for base, label in ((TEAM_SEG_BASE, "team 0 begins segment"), (SEG_BASE, "epilogue gets segment")):
-        for i in range(6):
-            col = t[:, base + i]
-            ok = col != 0
-            if ok.any():
-                rel = (col[ok] - t[ok, 0]) * us
-                print(f"{label + ' ' + str(i):<26}{np.median(rel):9.2f}{rel.min():10.2f}{rel.max():9.2f}   ({int(ok.sum())} CTAs)")
+        if ok.any():
+            rel = (col[ok] - t[ok, ENTRY]) * us
+            print(f"{name:<16}{np.median(rel):9.2f}{rel.min():10.2f}{rel.max():9.2f}   ({int(ok.sum())} CTAs)")
 
 
 PREFILL_PHASES = (
