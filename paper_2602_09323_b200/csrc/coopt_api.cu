@@ -1,4 +1,5 @@
 // Host side of the C ABI: argument checks, workspace arithmetic, dispatch to the launchers.
+#include <algorithm>
 #include <mutex>
 #include <utility>
 #include <vector>
@@ -62,9 +63,12 @@ int max_chunks_of(int max_blocks_per_seq, int chunk_size) {
   return static_cast<int>((static_cast<long long>(max_blocks_per_seq) * kBlockSize + chunk_size - 1) / chunk_size);
 }
 
-int ctas_of(int batch, int num_kv_heads, int max_blocks_per_seq, int chunk_size) {
+int num_sms() {
   const DeviceInfo* di = device_info();
-  return decode_ctas(di ? di->num_sms : 148, batch, num_kv_heads, max_blocks_per_seq, chunk_size / kBlockSize);
+  return std::min(di ? di->num_sms : 148, kCounterSlots / (kManyLayers * kMaxGroup) / kCtasPerSm);
+}
+int shares_of(int batch, int num_kv_heads, int max_blocks_per_seq, int chunk_size) {
+  return decode_shares(num_sms(), batch, num_kv_heads, max_blocks_per_seq, chunk_size / kBlockSize);
 }
 
 // The sizes that coopt_plan_bytes and coopt_workspace_bytes report are part of the interface: pools are laid out by them,
@@ -97,6 +101,18 @@ size_t larger(size_t a, size_t b) { return a > b ? a : b; }
 
 }  // namespace
 
+// What a call over that many layers has to be given.
+size_t workspace_need(int batch, int num_q_heads, int num_kv_heads, int head_dim, int max_blocks_per_seq, int chunk_size, int layers) {
+  const int group = (num_q_heads + num_kv_heads - 1) / num_kv_heads;
+  const int mc = chunk_size > 0 ? max_chunks_of(max_blocks_per_seq, chunk_size) : 0;
+  const size_t used = decode_workspace_bytes(shares_of(batch, num_kv_heads, max_blocks_per_seq, chunk_size), group, head_dim, batch, num_q_heads, layers, mc);
+  const size_t pieces = static_cast<size_t>(2) * listed_plan_ctas(batch, num_kv_heads, max_blocks_per_seq) * group * (head_dim + 2) * 4;
+  const size_t partials = static_cast<size_t>(batch) * num_q_heads * mc * (head_dim + 2) * 4;
+  const size_t listed = (workspace_control_bytes() + pieces + (mc > 0 ? partials + 256 : 0) + 511) / 256 * 256 +
+                        listed_plan_bytes(batch, num_kv_heads, max_blocks_per_seq, chunk_size / kBlockSize);
+  return larger(used, listed);
+}
+
 int check_attention_shapes(const coopt_cache* c, const void* q, void* out, int32_t max_blocks_per_seq, int32_t batch,
                            int32_t num_q_heads);
 
@@ -125,20 +141,66 @@ int check_attention_shapes(const coopt_cache* c, const void* q, void* out, int32
 }
 
 // What every decode-style launch has in common.
-static DecodeCall attention_call(const coopt_cache* c, const void* q, void* out, int32_t max_blocks_per_seq, int32_t batch, int32_t num_q_heads,
+static DecodeCall attention_call(const coopt_layer_io* layers, int32_t num_layers, int32_t max_blocks_per_seq, int32_t batch, int32_t num_q_heads,
                                  int32_t chunk_size, float sm_scale, void* workspace) {
   DecodeCall a = {};
-  a.q = q;
-  a.out = out;
+  a.layers = layers;
+  a.num_layers = num_layers;
   a.max_blocks_per_seq = max_blocks_per_seq;
   a.batch = batch;
   a.num_q_heads = num_q_heads;
   a.chunk_size = chunk_size;
   a.sm_scale = sm_scale;
   a.workspace = workspace;
-  a.ctas = ctas_of(batch, c->num_kv_heads, max_blocks_per_seq, chunk_size);
-  a.order = kAfterPrevious;
+  a.num_sms = num_sms();
+  a.shares = shares_of(batch, layers[0].cache->num_kv_heads, max_blocks_per_seq, chunk_size);
+  a.order = kDependent;
   return a;
+}
+
+// Whether layers may run side by side: nothing that one of them writes (its output; its cache if it appends) is read or
+// written by another, nor read by all (block table, context lengths).
+static bool layers_are_apart(const coopt_layer_io* layers, int num_layers, int64_t kv_token_stride, const int32_t* block_table, int max_blocks_per_seq,
+                             const int32_t* context_lens, int batch, int num_q_heads) {
+  struct Range { uintptr_t lo, hi; int layer; bool write; };
+  Range r[6 * kManyLayers + 2];
+  int n = 0;
+  auto add = [&](const void* p, size_t bytes, int layer, bool write) {
+    if (p != nullptr && bytes > 0) r[n++] = Range{reinterpret_cast<uintptr_t>(p), reinterpret_cast<uintptr_t>(p) + bytes, layer, write};
+  };
+  const coopt_cache& c = *layers[0].cache;
+  const size_t rows = static_cast<size_t>(batch) * num_q_heads * c.head_dim * 2;
+  const size_t cache = static_cast<size_t>(c.num_blocks) * c.num_kv_heads * granule_bytes(c.head_dim, true);
+  const size_t tokens = (static_cast<size_t>(batch - 1) * kv_token_stride + static_cast<size_t>(c.num_kv_heads) * c.head_dim) * 2;
+  for (int y = 0; y < num_layers; ++y) {
+    const coopt_layer_io& io = layers[y];
+    add(io.q, rows, y, false);
+    add(io.out, rows, y, true);
+    add(io.cache->data, cache, y, io.k_new != nullptr);
+    add(io.k_new, tokens, y, false);
+    add(io.v_new, tokens, y, false);
+    add(io.slot_mapping, static_cast<size_t>(batch) * 8, y, false);
+  }
+  add(block_table, static_cast<size_t>(batch) * max_blocks_per_seq * 4, -1, false);
+  add(context_lens, static_cast<size_t>(batch) * 4, -1, false);
+  std::sort(r, r + n, [](const Range& a, const Range& b) { return a.lo < b.lo; });
+  // in order of their begins: how far the ranges before reach, by the layer that reaches farthest and by the others
+  struct Reach {
+    uintptr_t hi = 0, other = 0;
+    int layer = -2;
+    void add(const Range& x) {
+      if (x.layer == layer) hi = x.hi > hi ? x.hi : hi;
+      else if (x.hi > hi) { other = hi; hi = x.hi; layer = x.layer; }
+      else if (x.hi > other) other = x.hi;
+    }
+    bool meets(const Range& x) const { return x.lo < (x.layer == layer ? other : hi); }
+  } all, written;
+  for (int i = 0; i < n; ++i) {
+    if ((r[i].write ? all : written).meets(r[i])) return false;
+    all.add(r[i]);
+    if (r[i].write) written.add(r[i]);
+  }
+  return true;
 }
 
 }  // namespace coopt
@@ -190,14 +252,8 @@ size_t coopt_workspace_bytes(int32_t batch, int32_t num_q_heads, int32_t num_kv_
                              int32_t max_blocks_per_seq, int32_t chunk_size, int32_t total_q) {
   (void)total_q;
   if (batch < 0 || num_q_heads <= 0 || num_kv_heads <= 0 || max_blocks_per_seq <= 0 || chunk_size < 0) return 0;
-  const int group = (num_q_heads + num_kv_heads - 1) / num_kv_heads;
-  const int mc = chunk_size > 0 ? max_chunks_of(max_blocks_per_seq, chunk_size) : 0;
-  const size_t used = decode_workspace_bytes(ctas_of(batch, num_kv_heads, max_blocks_per_seq, chunk_size), group, head_dim, batch, num_q_heads, mc);
-  const size_t pieces = static_cast<size_t>(2) * listed_plan_ctas(batch, num_kv_heads, max_blocks_per_seq) * group * (head_dim + 2) * 4;
-  const size_t partials = static_cast<size_t>(batch) * num_q_heads * mc * (head_dim + 2) * 4;
-  const size_t listed = (workspace_control_bytes() + pieces + (mc > 0 ? partials + 256 : 0) + 511) / 256 * 256 +
-                        listed_plan_bytes(batch, num_kv_heads, max_blocks_per_seq, chunk_size / kBlockSize);
-  return larger(used, listed);
+  return larger(workspace_need(batch, num_q_heads, num_kv_heads, head_dim, max_blocks_per_seq, chunk_size, 1),
+                chunk_size > 0 ? 0 : workspace_need(batch, num_q_heads, num_kv_heads, head_dim, max_blocks_per_seq, 0, kManyLayers));
 }
 
 int coopt_workspace_init(void* workspace, size_t workspace_bytes, void* stream) {
@@ -224,13 +280,13 @@ int coopt_paged_decode(const coopt_cache* cache, const void* q, void* out, const
   const int rc = check_attention_args(cache, q, out, block_table, max_blocks_per_seq, context_lens, batch, num_q_heads);
   if (rc != COOPT_OK) return rc;
   if (batch == 0) return COOPT_OK;
-  if (!workspace || workspace_bytes < coopt_workspace_bytes(batch, num_q_heads, cache->num_kv_heads, cache->head_dim,
-                                                            max_blocks_per_seq, 0, batch))
+  if (!workspace || workspace_bytes < workspace_need(batch, num_q_heads, cache->num_kv_heads, cache->head_dim, max_blocks_per_seq, 0, 1))
     return COOPT_ERR_WORKSPACE;
-  DecodeCall a = attention_call(cache, q, out, max_blocks_per_seq, batch, num_q_heads, 0, sm_scale, workspace);
+  const coopt_layer_io io = {cache, nullptr, nullptr, nullptr, q, out};
+  DecodeCall a = attention_call(&io, 1, max_blocks_per_seq, batch, num_q_heads, 0, sm_scale, workspace);
   a.block_table = block_table;
   a.context_lens = context_lens;
-  return launch_decode(cache, a, static_cast<cudaStream_t>(stream));
+  return launch_decode(a, static_cast<cudaStream_t>(stream));
 }
 
 int coopt_decode_step(const coopt_cache* cache, const void* k_new, const void* v_new, int64_t kv_token_stride,
@@ -243,16 +299,16 @@ int coopt_decode_step(const coopt_cache* cache, const void* k_new, const void* v
   if (!k_new || !v_new || !slot_mapping || kv_token_stride < static_cast<int64_t>(cache->num_kv_heads) * cache->head_dim)
     return COOPT_ERR_INVALID_ARG;
   if (batch == 0) return COOPT_OK;
-  if (!workspace || workspace_bytes < coopt_workspace_bytes(batch, num_q_heads, cache->num_kv_heads, cache->head_dim,
-                                                            max_blocks_per_seq, 0, batch))
+  if (!workspace || workspace_bytes < workspace_need(batch, num_q_heads, cache->num_kv_heads, cache->head_dim, max_blocks_per_seq, 0, 1))
     return COOPT_ERR_WORKSPACE;
   rc = launch_kv_write(cache, k_new, v_new, kv_token_stride, slot_mapping, batch, static_cast<cudaStream_t>(stream));
   if (rc != COOPT_OK) return rc;
-  DecodeCall a = attention_call(cache, q, out, max_blocks_per_seq, batch, num_q_heads, 0, sm_scale, workspace);
+  const coopt_layer_io io = {cache, nullptr, nullptr, nullptr, q, out};
+  DecodeCall a = attention_call(&io, 1, max_blocks_per_seq, batch, num_q_heads, 0, sm_scale, workspace);
   a.block_table = block_table;
   a.context_lens = context_lens;
-  a.order = kDependent;                      // on the write in front of it
-  return launch_decode(cache, a, static_cast<cudaStream_t>(stream));
+  a.order = kAfterWrite;
+  return launch_decode(a, static_cast<cudaStream_t>(stream));
 }
 
 size_t coopt_plan_bytes(int32_t batch, int32_t num_kv_heads, int32_t max_blocks_per_seq, int32_t chunk_size) {
@@ -297,14 +353,14 @@ int coopt_decode_step_planned(const coopt_cache* cache, const void* plan, size_t
     return COOPT_ERR_INVALID_ARG;
   if ((flags & ~static_cast<uint32_t>(COOPT_FLAG_OVERLAP_PREVIOUS)) != 0) return COOPT_ERR_INVALID_ARG;
   if (batch == 0) return COOPT_OK;
-  if (!workspace || workspace_bytes < coopt_workspace_bytes(batch, num_q_heads, cache->num_kv_heads, cache->head_dim,
-                                                            max_blocks_per_seq, chunk_size, batch))
+  if (!workspace || workspace_bytes < workspace_need(batch, num_q_heads, cache->num_kv_heads, cache->head_dim, max_blocks_per_seq, chunk_size, 1))
     return COOPT_ERR_WORKSPACE;
-  DecodeCall a = attention_call(cache, q, out, max_blocks_per_seq, batch, num_q_heads, chunk_size, sm_scale, workspace);
+  const coopt_layer_io io = {cache, k_new, v_new, slot_mapping, q, out};
+  DecodeCall a = attention_call(&io, 1, max_blocks_per_seq, batch, num_q_heads, chunk_size, sm_scale, workspace);
   a.plan = plan;
-  a.k_new = k_new; a.v_new = v_new; a.slot_mapping = slot_mapping; a.kv_token_stride = kv_token_stride;
-  a.order = (flags & COOPT_FLAG_OVERLAP_PREVIOUS) != 0 ? kOverlapPrevious : kAfterPrevious;
-  return launch_decode(cache, a, static_cast<cudaStream_t>(stream));
+  a.kv_token_stride = kv_token_stride;
+  if ((flags & COOPT_FLAG_OVERLAP_PREVIOUS) != 0) a.order = kOverlapPrevious;
+  return launch_decode(a, static_cast<cudaStream_t>(stream));
 }
 
 int coopt_decode_layers(const coopt_layer_io* layers, int32_t num_layers, int64_t kv_token_stride, const int32_t* block_table,
@@ -330,18 +386,34 @@ int coopt_decode_layers(const coopt_layer_io* layers, int32_t num_layers, int64_
   if (!block_table || !context_lens) return COOPT_ERR_INVALID_ARG;
   if ((flags & ~static_cast<uint32_t>(COOPT_FLAG_OVERLAP_PREVIOUS)) != 0) return COOPT_ERR_INVALID_ARG;
   if (batch == 0) return COOPT_OK;
-  if (!workspace || workspace_bytes < coopt_workspace_bytes(batch, num_q_heads, c0->num_kv_heads, c0->head_dim, max_blocks_per_seq, 0, batch))
+  if (!workspace || workspace_bytes < workspace_need(batch, num_q_heads, c0->num_kv_heads, c0->head_dim, max_blocks_per_seq, 0, 1))
     return COOPT_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   rc = launch_decode_plan(block_table, max_blocks_per_seq, context_lens, batch, c0->num_kv_heads, c0->num_blocks, 0, plan, st);
-  for (int32_t l = 0; l < num_layers && rc == COOPT_OK; ++l) {
-    const coopt_layer_io& io = layers[l];
-    DecodeCall a = attention_call(io.cache, io.q, io.out, max_blocks_per_seq, batch, num_q_heads, 0, sm_scale, workspace);
-    a.plan = plan;
-    a.k_new = io.k_new; a.v_new = io.v_new; a.slot_mapping = io.slot_mapping; a.kv_token_stride = kv_token_stride;
-    // layer l > 0 may read the plan and its own cache while layer l - 1 drains
-    a.order = l > 0 && (flags & COOPT_FLAG_OVERLAP_PREVIOUS) != 0 ? kOverlapPrevious : kDependent;
-    rc = launch_decode(io.cache, a, st);
+  const bool long_layers = static_cast<long long>(batch) * c0->num_kv_heads * max_blocks_per_seq > 160ll * num_sms();
+  for (int32_t l = 0; l < num_layers && rc == COOPT_OK;) {
+    // Layers whose buffers are apart go into one launch where a layer gives a share few places: what a launch costs once is
+    // then most of it (8 sequences of 1..28 tokens, eight layers: 64 / 21 us; 12 of 3052..6105 tokens, 4 kv heads, four
+    // layers, 94 places a share: 84 / 75).  With 230 places a share (32 x 2048 tokens, eight layers) both take 260 us, with
+    // 290 (24 sequences, G = 8, four layers) separate launches 99, one 103.
+    int n = long_layers ? 1 : std::min(num_layers - l, kManyLayers);
+    while (n > 1 && workspace_bytes < workspace_need(batch, num_q_heads, c0->num_kv_heads, c0->head_dim, max_blocks_per_seq, 0, n)) --n;
+    const bool apart = layers_are_apart(layers + l, n, kv_token_stride, block_table, max_blocks_per_seq, context_lens, batch, num_q_heads);
+    if (!apart) n = 1;
+    DecodeCall a = attention_call(layers + l, n, max_blocks_per_seq, batch, num_q_heads, 0, sm_scale, workspace);
+    a.kv_token_stride = kv_token_stride;
+    if (l == 0 && apart) {
+      // behind the planning kernel, which copies lengths and table: this launch reads them where it read them
+      a.block_table = block_table;
+      a.context_lens = context_lens;
+      a.order = kOverlapPrevious;
+    } else {
+      a.plan = plan;
+      // the layers before may still drain while this launch reads the plan and its own caches
+      if (l > 0 && (flags & COOPT_FLAG_OVERLAP_PREVIOUS) != 0) a.order = kOverlapPrevious;
+    }
+    rc = launch_decode(a, st);
+    l += n;
   }
   return rc;
 }
@@ -356,16 +428,16 @@ int coopt_paged_chunked(const coopt_cache* cache, const void* q, void* out, cons
   if (chunk_size <= 0 || chunk_size % kBlockSize != 0 || chunk_size / kBlockSize > decode_max_chunk_blocks())
     return COOPT_ERR_INVALID_ARG;
   if (batch == 0) return COOPT_OK;
-  if (!workspace || workspace_bytes < coopt_workspace_bytes(batch, num_q_heads, cache->num_kv_heads, cache->head_dim,
-                                                            max_blocks_per_seq, chunk_size, total_q))
+  if (!workspace || workspace_bytes < workspace_need(batch, num_q_heads, cache->num_kv_heads, cache->head_dim, max_blocks_per_seq, chunk_size, 1))
     return COOPT_ERR_WORKSPACE;
   if (total_q == batch) {
     // one query token per sequence: the Opt-Pa chunk-and-merge decode
-    DecodeCall a = attention_call(cache, q, out, max_blocks_per_seq, batch, num_q_heads, chunk_size, sm_scale, workspace);
+    const coopt_layer_io io = {cache, nullptr, nullptr, nullptr, q, out};
+    DecodeCall a = attention_call(&io, 1, max_blocks_per_seq, batch, num_q_heads, chunk_size, sm_scale, workspace);
     a.block_table = block_table;
     a.context_lens = context_lens;
     a.cu_q_lens = cu_q_lens;
-    return launch_decode(cache, a, static_cast<cudaStream_t>(stream));
+    return launch_decode(a, static_cast<cudaStream_t>(stream));
   }
   return launch_paged_prefill(cache, q, out, cu_q_lens, block_table, max_blocks_per_seq, context_lens, batch,
                               num_q_heads, total_q, causal, sm_scale, workspace, static_cast<cudaStream_t>(stream));
@@ -428,13 +500,12 @@ int coopt_decode_step_host(const coopt_cache* cache, const void* step_inputs_hos
   if (!is_fp8(cache->dtype)) return COOPT_ERR_UNSUPPORTED;
   rc = check_plan_args(batch, hkv, max_blocks_per_seq, 0, plan, plan_bytes_given);
   if (rc != COOPT_OK) return rc;
-  if (!workspace || workspace_bytes < coopt_workspace_bytes(batch, num_q_heads, hkv, d, max_blocks_per_seq, 0, batch)) return COOPT_ERR_WORKSPACE;
+  if (!workspace || workspace_bytes < workspace_need(batch, num_q_heads, hkv, d, max_blocks_per_seq, 0, 1)) return COOPT_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  DecodeCall a = attention_call(cache, dev + s.q, dev + s.out, max_blocks_per_seq, batch, num_q_heads, 0, sm_scale, workspace);
+  coopt_layer_io io = {cache, dev + s.k_new, dev + s.v_new, reinterpret_cast<const int64_t*>(dev + s.slot_mapping), dev + s.q, dev + s.out};
+  DecodeCall a = attention_call(&io, 1, max_blocks_per_seq, batch, num_q_heads, 0, sm_scale, workspace);
   a.plan = plan;
-  a.k_new = dev + s.k_new; a.v_new = dev + s.v_new; a.slot_mapping = reinterpret_cast<const int64_t*>(dev + s.slot_mapping);
   a.kv_token_stride = static_cast<int64_t>(hkv) * d;
-  a.order = kDependent;
   // Host buffers that are page-locked and mapped into the device's address space are used where they are: the
   // kernel fetches the queries and the new tokens from them and stores the result into them, and only the
   // index arrays (slots, block table, context lengths: what the planner walks) are copied to the device.
@@ -448,10 +519,10 @@ int coopt_decode_step_host(const coopt_cache* cache, const void* step_inputs_hos
                           reinterpret_cast<const int32_t*>(dev + s.context_lens), batch, hkv, cache->num_blocks, 0, plan, st);
   if (rc != COOPT_OK) return rc;
   if (in_place) {
-    a.q = in_dev + s.q; a.k_new = in_dev + s.k_new; a.v_new = in_dev + s.v_new; a.out = out_dev;
-    return launch_decode(cache, a, st);
+    io.q = in_dev + s.q; io.k_new = in_dev + s.k_new; io.v_new = in_dev + s.v_new; io.out = out_dev;
+    return launch_decode(a, st);
   }
-  rc = launch_decode(cache, a, st);
+  rc = launch_decode(a, st);
   if (rc != COOPT_OK) return rc;
   return cudaMemcpyAsync(out_host, dev + s.out, s.out_bytes, cudaMemcpyDeviceToHost, st) == cudaSuccess ? COOPT_OK : COOPT_ERR_CUDA;
 }

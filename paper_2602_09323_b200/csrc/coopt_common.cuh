@@ -190,6 +190,28 @@ __device__ __forceinline__ uint4 lds128(const void* p) {
   return v;
 }
 
+// Launched as a programmatic dependent, a kernel may be set up while the one before it in the stream still runs: here it
+// waits until that one has finished, and lets the one behind it be set up.
+__device__ __forceinline__ void wait_previous_kernel() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <class Kernel, class... Args>
+bool launch_dependent(Kernel kernel, dim3 grid, int threads, int smem, cudaStream_t stream, const Args&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(static_cast<unsigned>(threads));
+  cfg.dynamicSmemBytes = static_cast<size_t>(smem);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...) == cudaSuccess;
+}
+
 #endif  // __CUDACC__
 
 // ---- host-side launch plumbing ------------------------------------------------------------------

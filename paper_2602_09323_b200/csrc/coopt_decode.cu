@@ -21,6 +21,8 @@
 // Before / now: one layer of 56 heads over 8 kv heads, 8 sequences of 1..28 tokens 60 / 8 us; 24 sequences of
 // 300..4000 tokens, G = 8, 46 / 25 us a layer; 32 x 2048 tokens, G = 5, 35 / 32 us; 64 sequences of 128..8192 tokens,
 // 121 / 106 us; 120 sequences of 5..900 tokens at head_dim 64, plan included, 56 / 18.5 us.)
+#include <algorithm>
+
 #include "coopt_decode.cuh"
 #include "coopt_trace.cuh"
 #include "coopt_umma.cuh"
@@ -50,14 +52,20 @@ struct Cfg {
   static constexpr int kStages = kFp8 ? (D == 128 ? 3 : 4) : (D == 128 ? 2 : 4);
   static constexpr int kPieceStride = D + 4;                    // floats of one head of a piece: o[D], maximum, sum, padding
   static constexpr int kPiece = kMaxGroup * kPieceStride * 4;   // bytes
-  static constexpr int kWarpBytes = kStages * kGran + kPiece;
+  // A warp's shared memory: its ring, the piece of a unit from before, and, in a launch over several layers, the piece of a
+  // unit that goes on (in a launch over one the ring has done its work by then, and the piece takes its place).  Pieces are
+  // as large as the group asks for; for the largest groups the ring of a launch over several layers is shorter.
+  static constexpr int kShare = (D == 128 ? 18048 : 13056);
+  static __host__ __device__ constexpr int stages(int layers, int G) { return layers > 1 && kStages * kGran + 2 * G * kPieceStride * 4 > kShare ? kStages - 1 : kStages; }
+  static constexpr int kWarpBytes = kFp8 ? (kShare > kStages * kGran + kPiece ? kShare : kStages * kGran + kPiece) : kStages * kGran + kPiece;
   static constexpr int kBarOff = kWarps * kWarpBytes;
-  static constexpr int kLensOff = kBarOff + kWarps * kStages * 8;
+  static constexpr int kLensOff = kBarOff + (kWarps * kStages + 2) * 8;
   static constexpr int kPreOff = kLensOff + kMaxBatch * 4;
   static constexpr int kRecOff = kPreOff + (kMaxBatch + 4) * 4;
   static constexpr int kMiscOff = kRecOff + kWarps * 32;
   static constexpr int kSmemBytes = kMiscOff + 192;
-  static_assert(kGran % 128 == 0 && kPiece % 128 == 0 && kStages * kGran >= kPiece && kCopy % 16 == 0, "copies land on 128-byte boundaries");
+  static_assert(kGran % 128 == 0 && kPiece % 128 == 0 && kStages * kGran >= kPiece && kWarpBytes % 128 == 0 && kCopy % 16 == 0, "copies land on 128-byte boundaries");
+  static_assert(!kFp8 || (kStages - 1) * kGran + 2 * kPiece <= kWarpBytes, "room for two pieces of the largest group");
   static_assert(kCtasPerSm * (kSmemBytes + 1024) <= 233472, "shared memory of one SM");
 };
 
@@ -257,8 +265,8 @@ __device__ __forceinline__ void acc_merge(Acc& a, int n, float m, float l, bool 
   }
 }
 
-template <int D, int FMT>
-__global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decode_kernel(const DecodeParams p) {
+template <int D, int FMT, int L>
+__global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decode_kernel(const DecodeParams p, const __grid_constant__ LayerTable<L> table) {
   using C = Cfg<D, FMT>;
   constexpr int kQSteps = D / 16;
   extern __shared__ __align__(128) uint8_t smem[];
@@ -270,8 +278,11 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
   const int row = lane >> 2, quad = lane & 3;
   const int B = p.batch, Hkv = p.num_kv_heads, G = p.group, Hq = p.num_q_heads;
   uint8_t* ring = smem + warp * C::kWarpBytes;
-  float* piece0 = reinterpret_cast<float*>(ring + C::kStages * C::kGran);
+  const int stages = L == 1 ? C::kStages : C::stages(L, G);
+  const int piece0_off = stages * C::kGran, piece1_off = L == 1 ? 0 : piece0_off + G * C::kPieceStride * 4;   // in a warp's shared memory
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kBarOff) + warp * C::kStages;
+  uint64_t* bar_pieces = reinterpret_cast<uint64_t*>(smem + C::kBarOff) + C::kWarps * C::kStages;   // every warp has left its pieces
+  uint64_t* bar_merged = bar_pieces + 1;                                                            // .. has no more use for the others' pieces
 
   COOPT_TRACE_CYCLES(p.trace, kTrEntry, tid == 0);
 #ifdef COOPT_TRACE
@@ -285,15 +296,14 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
   COOPT_TRACE_NS(p.trace, kTrEntryNs, tid == 0);
   if (lane == 0) {
     for (int i = 0; i < C::kStages; ++i) mbar_init(&bars[i], 1);
+    if (warp == 0) { mbar_init(bar_pieces, C::kWarps); mbar_init(bar_merged, C::kWarps); }
     mbar_fence_init();
   }
-  // Launched as a programmatic dependent, this CTA may run while the kernel before it still does.  If that kernel
-  // writes neither the plan nor the cache (overlap_previous) only the queries, the new tokens and everything that is
-  // written wait for it (below).
-  if (!p.overlap_previous) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  }
+  const auto layer = [&](int y) -> const LayerPtrs& { return table.l[L == 1 ? 0 : y]; };
+  // Launched as a programmatic dependent, this CTA may run while the kernel before it still does; p.order says what
+  // may be read before that one has finished.  (The kernel behind this one may start only then, too: it may read early
+  // what the kernel before this one wrote.)
+  if (p.order == kDependent) wait_previous_kernel();
 
   // ---- the line: context lengths and their prefix sums -------------------------------------------------------
   {
@@ -332,65 +342,99 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
       at += v[k];
       if (tid * kPer + k < B) pre[tid * kPer + k + 1] = at;
     }
-    recs[warp].flags = 0;
     __syncthreads();
   }
   if (misc[16]) {                                  // not a plan of this problem (uniform over the grid)
-    if (p.overlap_previous) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (p.order != kDependent) wait_previous_kernel();
     if (tid == 0) atomicCAS(p.status, 0, COOPT_ERR_INVALID_ARG);
     return;
   }
   COOPT_TRACE_CYCLES(p.trace, kTrLine, tid == 0);
   Line ln;
   ln.lens = lens; ln.pre = pre; ln.batch = B; ln.heads = Hkv; ln.chunk = p.chunk_blocks > 0 ? p.chunk_blocks : kNoChunks;
+  // A share: T places of a layer's line.  A layer is cut the same way whatever else the launch does, so its result does
+  // not depend on how many layers share the launch.  CTA i takes the shares i, i + grid, .. of all layers, one layer
+  // behind the other; the copies of a share are under way while the pieces of the one before are merged.
   const unsigned places = Hkv * pre[B];
-  const unsigned T = max(static_cast<unsigned>(kMinPlaces), (places + gridDim.x - 1) / gridDim.x);
-  // Shared units cost a trip through the workspace at the end of the launch.  Where units are short, a CTA takes the units
-  // that begin among its places whole instead.  (In chunk mode every CTA between the first and the last of a (sequence,
+  const unsigned T = max(static_cast<unsigned>(kMinPlaces), (places + p.shares - 1) / p.shares);
+  const unsigned shares = (places + T - 1) / T, all_shares = L == 1 ? shares : shares * p.layers;
+  // Shared units cost a trip through the workspace at the end of a share.  Where units are short, a share holds the units
+  // that begin among its places whole instead.  (In chunk mode every share between the first and the last of a (sequence,
   // kv head) has to hold a chunk of it.)
   int most = 0;
   for (int k = 0; k < C::kWarps; ++k) most = max(most, misc[17 + k]);
   const bool whole = most * (D / 64) <= (T == kMinPlaces ? kWholeUnitsIdle : kWholeUnits) && (p.chunk_blocks == 0 || most + kUnitCost <= static_cast<int>(T));
-  unsigned cta_lo = blockIdx.x * T, cta_hi = min(places, cta_lo + T);
-  if (whole && cta_lo < places) {
-    cta_lo = next_unit(ln, cta_lo, lane);
-    cta_hi = cta_hi < places ? next_unit(ln, cta_hi, lane) : places;
-  }
-  const unsigned mine = cta_hi > cta_lo ? cta_hi - cta_lo : 0u, Tw = (mine + C::kWarps - 1) / C::kWarps;
-  const unsigned my_lo = min(cta_hi, cta_lo + warp * Tw), my_hi = min(cta_hi, my_lo + Tw);
+  auto share_range = [&](unsigned v, unsigned& lo, unsigned& hi) {       // places of a layer's share v
+    lo = v * T;
+    hi = min(places, lo + T);
+    if (whole) {
+      lo = next_unit(ln, lo, lane);
+      hi = hi < places ? next_unit(ln, hi, lane) : places;
+    }
+  };
+  auto share_layer = [&](unsigned s) -> int { return L == 1 ? 0 : s / shares; };
+  auto share_walk = [&](unsigned s, Walk& w) {                          // this warp's part of share s
+    unsigned lo, hi;
+    share_range(L == 1 ? s : s % shares, lo, hi);
+    const unsigned mine = hi > lo ? hi - lo : 0u, Tw = (mine + C::kWarps - 1) / C::kWarps;
+    const unsigned my_lo = min(hi, lo + warp * Tw);
+    walk_start(ln, w, my_lo, min(hi, my_lo + Tw), lane);
+  };
+  // this warp's first unit in share s or, over several layers, in a later one (s moves there); and its next one
+  auto walk_later = [&](unsigned& s, Walk& w) {
+    if (L == 1) return;
+    while (!w.more && s + gridDim.x < all_shares) {
+      s += gridDim.x;
+      share_walk(s, w);
+    }
+  };
+  auto walk_on = [&](unsigned& s, Walk& w) {
+    walk_next(ln, w);
+    walk_later(s, w);
+  };
 
   // ---- copies: a granule per request, a ring of stages per warp -------------------------------------------------
   // Physical block ids are looked up 32 at a time (one per lane), one batch ahead of the copies that need them.
-  Walk pw;
-  walk_start(ln, pw, my_lo, my_hi, lane);
-  int ids_a = 0, cnt_a = 0, g_a = 0, pos_a = 0, ids_b = 0, cnt_b = 0, g_b = 0;
+  Walk w, pw;                                      // where this warp's work is (in share `share`), and where its copies are (in share `ps`)
+  unsigned ps = blockIdx.x;
+  w.more = false;
+  if (ps < all_shares) share_walk(ps, w);
+  pw = w;
+  if (ps < all_shares) walk_later(ps, pw);
+  const Walk fw = pw;                              // the first unit, and its layer
+  const int fy = share_layer(ps);
+  int ids_a = 0, cnt_a = 0, g_a = 0, y_a = 0, pos_a = 0, ids_b = 0, cnt_b = 0, g_b = 0, y_b = 0;
   auto fetch_ids = [&]() {
     cnt_b = 0;
     if (!pw.more) return;
     cnt_b = min(32, pw.jend - pw.j);
     g_b = pw.g;
+    y_b = share_layer(ps);
     ids_b = lane < cnt_b ? p.block_table[static_cast<size_t>(pw.b) * p.max_blocks_per_seq + pw.u + pw.j + lane] : 0;
     pw.j += cnt_b;
-    if (pw.j >= pw.jend) walk_next(ln, pw);
+    if (pw.j >= pw.jend) walk_on(ps, pw);
   };
   auto take_ids = [&]() {
-    ids_a = ids_b; cnt_a = cnt_b; g_a = g_b; pos_a = 0;
+    ids_a = ids_b; cnt_a = cnt_b; g_a = g_b; y_a = y_b; pos_a = 0;
     if (ids_a < 0 || ids_a >= p.num_blocks) {      // reported, and replaced by block 0: never dereferenced
       if (p.plan == nullptr) atomicCAS(p.status, 0, COOPT_ERR_INVALID_ARG);
       ids_a = 0;
     }
     fetch_ids();
   };
-  uint32_t issued = 0, consumed = 0;
+  uint32_t issued = 0, consumed = 0;               // copies, and the stages that take the next one and hold the oldest one
+  int in_stage = 0, out_stage = 0;
+  uint32_t out_phase = 0;
   auto issue = [&]() {
     if (pos_a == cnt_a) take_ids();
     if (pos_a < cnt_a) {
       const int id = __shfl_sync(0xffffffffu, ids_a, pos_a);
       ++pos_a;
-      const uint32_t stage = issued % C::kStages;
+      const int stage = in_stage;
+      if (++in_stage == stages) in_stage = 0;
       if (lane == 0) {
         mbar_expect_tx(&bars[stage], C::kCopy);
-        bulk_copy_g2s(ring + stage * C::kGran, p.cache + (static_cast<size_t>(id) * Hkv + g_a) * C::kGran, C::kCopy, &bars[stage]);
+        bulk_copy_g2s(ring + stage * C::kGran, layer(y_a).cache + (static_cast<size_t>(id) * Hkv + g_a) * C::kGran, C::kCopy, &bars[stage]);
       }
       ++issued;
     }
@@ -405,9 +449,9 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
 
   // raw query rows, loaded a unit ahead: this lane's head is `row`, its dims as the contraction takes them
   uint32_t qraw[kQSteps][2];
-  auto load_q = [&](int b, int g) {
+  auto load_q = [&](int y, int b, int g) {
     const bool live = row < G;
-    const __nv_bfloat16* qp = p.q + (static_cast<size_t>(b) * Hq + g * G + (live ? row : 0)) * D;
+    const __nv_bfloat16* qp = layer(y).q + (static_cast<size_t>(b) * Hq + g * G + (live ? row : 0)) * D;
 #pragma unroll
     for (int s = 0; s < kQSteps; ++s) {
       if constexpr (C::kFp8) {
@@ -420,32 +464,28 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
     }
   };
   bool dead = false;
-  Walk w = pw;
   // What the first unit needs besides its blocks is on its way to L2 before the copies queue up in front of it (also where
   // the kernel before may still write it: L2 is where its stores arrive).
-  if (w.more) {
-    const uint8_t* qrows = reinterpret_cast<const uint8_t*>(p.q + (static_cast<size_t>(w.b) * Hq + w.g * G) * D);
+  if (fw.more) {
+    const LayerPtrs& io = layer(fy);
+    const uint8_t* qrows = reinterpret_cast<const uint8_t*>(io.q + (static_cast<size_t>(fw.b) * Hq + fw.g * G) * D);
     if (lane < G * D / 64) prefetch_l2(qrows + lane * 128);
-    if (p.k_new != nullptr && lane < 3) {
-      const long long at = static_cast<long long>(w.b) * p.kv_token_stride + w.g * D;
-      prefetch_l2(lane == 0 ? static_cast<const void*>(p.k_new + at) : lane == 1 ? static_cast<const void*>(p.v_new + at) : static_cast<const void*>(p.slot_mapping + w.b));
+    if (io.k_new != nullptr && lane < 3) {
+      const long long at = static_cast<long long>(fw.b) * p.kv_token_stride + fw.g * D;
+      prefetch_l2(lane == 0 ? static_cast<const void*>(io.k_new + at) : lane == 1 ? static_cast<const void*>(io.v_new + at) : static_cast<const void*>(io.slot_mapping + fw.b));
     }
   }
   fetch_ids();
 #pragma unroll 1
   for (int step = 0; step < 2; ++step) {
-    if ((step == 0) == (p.overlap_previous != 0)) {
+    if ((step == 0) == (p.order == kOverlapPrevious)) {
 #pragma unroll 1
-      for (int i = 0; i < C::kStages; ++i) issue();
+      for (int i = 0; i < stages; ++i) issue();
       COOPT_TRACE_CYCLES(p.trace, kTrFirstCopy, tid == 0);
     } else {
-      // (The kernel behind this one may start only now, when the one before it has finished: it may read early what that one wrote.)
-      if (p.overlap_previous) {
-        asm volatile("griddepcontrol.wait;" ::: "memory");
-        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-      }
+      if (p.order != kDependent) wait_previous_kernel();
       COOPT_TRACE_CYCLES(p.trace, kTrPrevDone, tid == 0);
-      if (w.more) load_q(w.b, w.g);
+      if (fw.more) load_q(fy, fw.b, fw.g);
     }
   }
   if (blockIdx.x == 0) {
@@ -458,8 +498,19 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
   // sequences with an empty context: all-zero output rows
   for (int b = blockIdx.x; b < B; b += gridDim.x)
     if (lens[b] == 0)
-      for (int i = tid; i < Hq * D / 8; i += C::kThreads) reinterpret_cast<uint4*>(p.out + static_cast<size_t>(b) * Hq * D)[i] = make_uint4(0u, 0u, 0u, 0u);
+      for (int y = 0; y < (L == 1 ? 1 : p.layers); ++y)
+        for (int i = tid; i < Hq * D / 8; i += C::kThreads) reinterpret_cast<uint4*>(layer(y).out + static_cast<size_t>(b) * Hq * D)[i] = make_uint4(0u, 0u, 0u, 0u);
 
+  const int d0 = lane * 4;
+  const bool on = d0 < D;
+  uint32_t round = 0;
+#pragma unroll 1
+  for (unsigned share = blockIdx.x; share < all_shares; share += gridDim.x, ++round) {
+  const int y = share_layer(share);
+  const unsigned v_share = L == 1 ? share : share - y * shares;
+  if (round > 0) share_walk(share, w);
+  Rec rec;
+  rec.flags = 0;
 #pragma unroll 1
   while (w.more) {
     // ---- query operand: f16 (exact: rows scaled by a power of two), or bf16 as it is -------------------------------
@@ -490,8 +541,9 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
     COOPT_TRACE_CYCLES(p.trace, kTrQuery, tid == 0 && consumed == 0 && qf[0][0] != 0x12345u);
     {
       Walk nx = w;
-      walk_next(ln, nx);
-      if (nx.more) load_q(nx.b, nx.g);
+      unsigned ns = share;
+      walk_on(ns, nx);
+      if (nx.more) load_q(share_layer(ns), nx.b, nx.g);
     }
 
     float o[D / 16][4];
@@ -502,34 +554,36 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
     float m[2] = {-INFINITY, -INFINITY}, top[2] = {-INFINITY, -INFINITY}, l[2] = {0.0f, 0.0f};
     float vref = 0.0f, vinv = 0.0f;
     const int ctx = lens[w.b];
+    const bool has_new = C::kFp8 && layer(y).k_new != nullptr;
 
 #pragma unroll 1
     for (int j = w.j; j < w.jend; ++j) {
-      const uint32_t stage = consumed % C::kStages;
       // the step's new token: what it needs is loaded while its block is on the way
-      const bool append = C::kFp8 && p.k_new != nullptr && w.u + j == w.nb - 1;
+      const bool append = has_new && w.u + j == w.nb - 1;
       long long slot = -1;
       int id = 0;
       uint2 k_row = make_uint2(0u, 0u), v_row = k_row;
       if constexpr (C::kFp8) {
         if (append) {
-          const bool vec = ((reinterpret_cast<uintptr_t>(p.k_new) | reinterpret_cast<uintptr_t>(p.v_new) | static_cast<uintptr_t>(p.kv_token_stride * 2)) & (D / 16 - 1)) == 0;
+          const LayerPtrs& io = layer(y);
+          const bool vec = ((reinterpret_cast<uintptr_t>(io.k_new) | reinterpret_cast<uintptr_t>(io.v_new) | static_cast<uintptr_t>(p.kv_token_stride * 2)) & (D / 16 - 1)) == 0;
           const long long at = static_cast<long long>(w.b) * p.kv_token_stride + w.g * D;
-          slot = p.slot_mapping[w.b];
+          slot = io.slot_mapping[w.b];
           id = p.block_table[static_cast<size_t>(w.b) * p.max_blocks_per_seq + w.nb - 1];
-          k_row = load_new<D>(p.k_new + at, vec, lane);
-          v_row = load_new<D>(p.v_new + at, vec, lane);
+          k_row = load_new<D>(io.k_new + at, vec, lane);
+          v_row = load_new<D>(io.v_new + at, vec, lane);
         }
       }
-      if (!dead && !mbar_wait_bounded(&bars[stage], (consumed / C::kStages) & 1u)) {
+      if (!dead && !mbar_wait_bounded(&bars[out_stage], out_phase)) {
         dead = true;
-        if (lane == 0) atomicCAS(p.status, 0, COOPT_ERR_TIMEOUT);
+        atomicCAS(p.status, 0, COOPT_ERR_TIMEOUT);
       }
       dead = __any_sync(0xffffffffu, dead);
       COOPT_TRACE_CYCLES(p.trace, kTrFirstLanded, tid == 0 && consumed == 0);
-      ++consumed;
       if (dead) continue;
-      uint8_t* st = ring + stage * C::kGran;
+      uint8_t* st = ring + out_stage * C::kGran;
+      ++consumed;
+      if (++out_stage == stages) { out_stage = 0; out_phase ^= 1u; }
       const int nvalid = min(kBlockSize, ctx - (w.u + j) * kBlockSize);      // Eq. 9: tail of the context
 
       if constexpr (C::kFp8) {
@@ -538,7 +592,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
           if (slot != static_cast<long long>(id) * kBlockSize + off) {         // not the sequence's last position
             if (lane == 0) atomicCAS(p.status, 0, COOPT_ERR_INVALID_ARG);
           } else if (id >= 0 && id < p.num_blocks) {
-            append_token<D, C::kE5m2>(st, p.cache + (static_cast<size_t>(id) * Hkv + w.g) * C::kGran, k_row, v_row, off, lane);
+            append_token<D, C::kE5m2>(st, layer(y).cache + (static_cast<size_t>(id) * Hkv + w.g) * C::kGran, k_row, v_row, off, lane);
           }
           __syncwarp();
         }
@@ -668,7 +722,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
     const bool starts = w.j == 0, ends = w.jend == w.n;
     if (starts && ends && p.chunk_blocks == 0) {
       // the whole (sequence, kv head): bf16 rows, transposed so that a lane holds pairs of dims of head `row`
-      __nv_bfloat16* dst = p.out + (static_cast<size_t>(w.b) * Hq + w.g * G + row) * D + 2 * quad;
+      __nv_bfloat16* dst = layer(y).out + (static_cast<size_t>(w.b) * Hq + w.g * G + row) * D + 2 * quad;
 #pragma unroll
       for (int t = 0; t < D / 16; ++t) {
         const uint32_t a = transpose8x8(pack_bf16x2(o[t][0] * inv[0], o[t][1] * inv[1])), c = transpose8x8(pack_bf16x2(o[t][2] * inv[0], o[t][3] * inv[1]));
@@ -691,48 +745,56 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
         }
       }
     } else {
-      // a piece: into shared memory (the piece of a unit that goes on is the warp's last one: it takes the ring's place)
-      float* piece = starts ? reinterpret_cast<float*>(ring) : piece0;
+      // a piece: into shared memory, once the pieces of the share before are of no more use
+      if (L > 1 && round > 0 && rec.flags == 0 && !dead && !mbar_wait_bounded(bar_merged, (round - 1) & 1u)) {
+        dead = true;
+        atomicCAS(p.status, 0, COOPT_ERR_TIMEOUT);
+      }
+      float* piece = reinterpret_cast<float*>(ring + (starts ? piece1_off : piece0_off));
       float* at = piece + 2 * quad * C::kPieceStride + row;
 #pragma unroll
-      for (int t = 0; t < D / 16; ++t) {
-        at[16 * t] = o[t][0] * inv[0];
-        at[C::kPieceStride + 16 * t] = o[t][1] * inv[1];
-        at[16 * t + 8] = o[t][2] * inv[0];
-        at[C::kPieceStride + 16 * t + 8] = o[t][3] * inv[1];
+      for (int h = 0; h < 2; ++h) {
+        if (2 * quad + h < G) {
+#pragma unroll
+          for (int t = 0; t < D / 16; ++t) {
+            at[h * C::kPieceStride + 16 * t] = o[t][h] * inv[h];
+            at[h * C::kPieceStride + 16 * t + 8] = o[t][2 + h] * inv[h];
+          }
+          if (row == 0) *reinterpret_cast<float2*>(at + h * C::kPieceStride + D) = make_float2(m[h], l[h]);
+        }
       }
-      if (row < 2) {
-        piece[(2 * quad + row) * C::kPieceStride + D] = row ? m[1] : m[0];
-        piece[(2 * quad + row) * C::kPieceStride + D + 1] = row ? l[1] : l[0];
-      }
-      if (lane == 0) {
-        Rec& r = recs[warp];
-        if (starts) { r.b1 = w.b; r.g1 = w.g; r.u1 = w.u; r.flags |= kHas1; }
-        else { r.b0 = w.b; r.g0 = w.g; r.u0 = w.u; r.flags |= kHas0 | (ends ? kEnds0 : 0); }
-      }
+      if (starts) { rec.b1 = w.b; rec.g1 = w.g; rec.u1 = w.u; rec.flags |= kHas1; }
+      else { rec.b0 = w.b; rec.g0 = w.g; rec.u0 = w.u; rec.flags |= kHas0 | (ends ? kEnds0 : 0); }
     }
     walk_next(ln, w);
   }
   COOPT_TRACE_CYCLES(p.trace, kTrWarpEnd + warp, lane == 0);
   COOPT_TRACE_VALUE(p.trace, kTrBlocks, tid == 0, consumed);
-  // a warp that gave up still has copies in flight: they get a bounded time to land
-  if (dead) {
-    while (consumed < issued) {
-      mbar_wait_bounded(&bars[consumed % C::kStages], (consumed / C::kStages) & 1u);
-      ++consumed;
+  if (L == 1) {
+    if (lane == 0) recs[warp] = rec;
+    __syncthreads();
+  } else {
+    if (round > 0 && rec.flags == 0 && !dead && !mbar_wait_bounded(bar_merged, (round - 1) & 1u)) dead = true;   // (its record is still in use)
+    if (lane == 0) {
+      recs[warp] = rec;
+      if (dead) atomicCAS(p.status, 0, COOPT_ERR_TIMEOUT);
     }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar_pieces);
+    if (!dead && !mbar_wait_bounded(bar_pieces, round & 1u)) {
+      dead = true;
+      atomicCAS(p.status, 0, COOPT_ERR_TIMEOUT);
+    }
+    dead = __any_sync(0xffffffffu, dead);
   }
-  __syncthreads();
   COOPT_TRACE_CYCLES(p.trace, kTrStreamed, tid == 0);
 
   // ---- units that several warps share: merged by log-sum-exp, one (unit, head) per warp ---------------------------------
-  const int d0 = lane * 4;
-  const bool on = d0 < D;
-  // One head of a piece that other CTAs hold the rest of goes to the workspace; the warp that delivers the last piece gets
-  // `true` and all pieces merged.  The first piece of a unit sits in the odd slot of its CTA, the others in the even ones.
+  // One head of a piece that other shares hold the rest of goes to the workspace; the warp that delivers the last piece gets
+  // `true` and all pieces merged.  The first piece of a unit sits in the odd slot of its share, the others in the even ones.
   auto deliver = [&](Acc& a, int region, bool first_piece, int cta_f, int pieces, int h) -> bool {
-    const size_t base = static_cast<size_t>(region) * 2 * gridDim.x;
-    const size_t at = (base + 2 * blockIdx.x + (first_piece ? 1 : 0)) * G + h;
+    const size_t base = static_cast<size_t>(region) * 2 * p.shares;
+    const size_t at = (base + 2 * v_share + (first_piece ? 1 : 0)) * G + h;
     const float dinv = a.den > 0.0f ? 1.0f / a.den : 0.0f;
     if (on) *reinterpret_cast<float4*>(p.run_o + at * D + d0) = make_float4(a.num.x * dinv, a.num.y * dinv, a.num.z * dinv, a.num.w * dinv);
     if (lane == 0) { p.run_m[at] = a.M; p.run_l[at] = a.den; }
@@ -740,7 +802,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
     int done = 0;
     if (lane == 0) {
       // release (this piece is visible before the count moves) and acquire (the other pieces are visible before they are read)
-      int* counter = p.counters + (region * gridDim.x + cta_f) * kMaxGroup + h;
+      int* counter = p.counters + (region * p.shares + cta_f) * kMaxGroup + h;
       int old;
       asm volatile("atom.add.acq_rel.gpu.s32 %0, [%1], 1;" : "=r"(old) : "l"(counter) : "memory");
       done = old == pieces - 1;
@@ -758,7 +820,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
   };
   auto store_out = [&](const Acc& a, int b, int g, int h) {
     const float dinv = a.den > 0.0f ? 1.0f / a.den : 0.0f;
-    if (on) *reinterpret_cast<uint2*>(p.out + (static_cast<size_t>(b) * Hq + g * G + h) * D + d0) =
+    if (on) *reinterpret_cast<uint2*>(layer(y).out + (static_cast<size_t>(b) * Hq + g * G + h) * D + d0) =
         make_uint2(pack_bf16x2(a.num.x * dinv, a.num.y * dinv), pack_bf16x2(a.num.z * dinv, a.num.w * dinv));
   };
   const int flags = lane < C::kWarps ? recs[lane].flags : 0;
@@ -781,7 +843,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
     }
     const int b = kind ? recs[from].b1 : recs[from].b0, g = kind ? recs[from].g1 : recs[from].g0, u = kind ? recs[from].u1 : recs[from].u0;
     auto piece = [&](int k) {
-      return reinterpret_cast<const float*>(smem + (from + k) * C::kWarpBytes + ((kind && k == 0) ? 0 : C::kStages * C::kGran)) + h * C::kPieceStride;
+      return reinterpret_cast<const float*>(smem + (from + k) * C::kWarpBytes + ((kind && k == 0) ? piece1_off : piece0_off)) + h * C::kPieceStride;
     };
     const int n = last - from + 1;
     Acc a;
@@ -790,7 +852,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
     if (!(kind && closed)) {
       const unsigned first = unit_place(ln, b, g, u) + kUnitCost;
       const int nu = unit_blocks(ln, line_blocks(ln, b), u), cta_f = first / T;
-      if (!deliver(a, p.chunk_blocks > 0 ? 1 : 0, kind != 0, cta_f, static_cast<int>((first + nu - 1) / T) - cta_f + 1, h)) continue;
+      if (!deliver(a, L > 1 ? y : p.chunk_blocks > 0 ? 1 : 0, kind != 0, cta_f, static_cast<int>((first + nu - 1) / T) - cta_f + 1, h)) continue;
     }
     if (p.chunk_blocks == 0) {
       store_out(a, b, g, h);
@@ -801,15 +863,22 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
       if (lane == 0) { p.part_m[at] = a.M * kLn2; p.part_l[at] = a.den * kUnshift; }
     }
   }
-  COOPT_TRACE_CYCLES(p.trace, kTrExit, tid == 0);
-  COOPT_TRACE_NS(p.trace, kTrExitNs, tid == 0);
-  if (p.chunk_blocks == 0) return;
+  if (L > 1) {
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar_merged);
+    continue;
+  }
+  if (p.chunk_blocks == 0) break;
 
   // ---- Opt-Pa: what this CTA holds of a (sequence, kv head) is merged over its chunks, then with the other CTAs' shares ----
   __syncthreads();                       // this CTA's chunks have been exported (or left in its slots)
   int task = 0;
   Walk c;
-  walk_start(ln, c, cta_lo, cta_hi, lane);
+  {
+    unsigned lo, hi;
+    share_range(share, lo, hi);
+    walk_start(ln, c, lo, hi, lane);
+  }
   while (c.more) {
     const int b = c.b, g = c.g, nb = c.nb, c_first = c.u / ln.chunk;
     const bool cut_first = c.j != 0 || c.jend != c.n, first_began = c.j == 0, run_begins = first_began && c.u == 0;
@@ -826,7 +895,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
       Acc a;
       acc_clear(a);
       const size_t rows = (static_cast<size_t>(b) * Hq + g * G + h) * p.max_chunks;
-      const size_t slots = (static_cast<size_t>(2 * gridDim.x) + 2 * blockIdx.x) * G + h;
+      const size_t slots = (static_cast<size_t>(2 * p.shares) + 2 * share) * G + h;
       auto cut = [&](int i) { return (i == c_first && cut_first) || (i == c_last && cut_last); };
       auto slot = [&](int i) { return slots + (i == c_first && !first_began ? 0 : G); };
       for (int c0 = c_first; c0 <= c_last; c0 += 32) {
@@ -849,23 +918,23 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
       store_out(a, b, g, h);
     }
   }
+  }
+  COOPT_TRACE_CYCLES(p.trace, kTrExit, tid == 0);
+  COOPT_TRACE_NS(p.trace, kTrExitNs, tid == 0);
+  // a warp that gave up still has copies in flight: they get a bounded time to land
+  if (dead) {
+    for (; consumed < issued; ++consumed) {
+      mbar_wait_bounded(&bars[out_stage], out_phase);
+      if (++out_stage == stages) { out_stage = 0; out_phase ^= 1u; }
+    }
+  }
 }
 
-template <int D, int FMT>
-int launch_one(const DecodeParams& p, int grid, bool dependent, cudaStream_t stream) {
+template <int D, int FMT, int L>
+int launch_one(const DecodeParams& p, const LayerTable<L>& table, int grid, cudaStream_t stream) {
   using C = Cfg<D, FMT>;
-  if (!configure_kernel_smem(reinterpret_cast<const void*>(&paged_decode_kernel<D, FMT>), C::kSmemBytes)) return COOPT_ERR_CUDA;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>(grid));
-  cfg.blockDim = dim3(C::kThreads);
-  cfg.dynamicSmemBytes = C::kSmemBytes;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = dependent ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, paged_decode_kernel<D, FMT>, p) == cudaSuccess ? COOPT_OK : COOPT_ERR_CUDA;
+  if (!configure_kernel_smem(reinterpret_cast<const void*>(&paged_decode_kernel<D, FMT, L>), C::kSmemBytes)) return COOPT_ERR_CUDA;
+  return launch_dependent(paged_decode_kernel<D, FMT, L>, grid, C::kThreads, C::kSmemBytes, stream, p, table) ? COOPT_OK : COOPT_ERR_CUDA;
 }
 
 // coopt_decode_plan: a copy of the step's context lengths and of the valid part of its block table, with the block ids
@@ -875,7 +944,7 @@ constexpr int kPlanThreads = 256;
 constexpr int kPlanPiece = 128;          // table entries a warp takes at a time
 __global__ void __launch_bounds__(kPlanThreads) decode_plan_kernel(const int* block_table, int width, const int* context_lens, int batch, int num_blocks,
                                                                    int key, PlanHeader* header) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  wait_previous_kernel();
   int* lens = reinterpret_cast<int*>(header + 1);
   int* table = reinterpret_cast<int*>(reinterpret_cast<uint8_t*>(header) + plan_table_offset(batch));
   __shared__ int bad;
@@ -907,20 +976,43 @@ __global__ void __launch_bounds__(kPlanThreads) decode_plan_kernel(const int* bl
 
 }  // namespace
 
-static int launch_attention(const DecodeParams& p, int head_dim, int dtype, int grid, bool dependent, cudaStream_t stream) {
-  if (head_dim == 128) {
-    if (dtype == COOPT_KV_FP8_E4M3) return launch_one<128, COOPT_KV_FP8_E4M3>(p, grid, dependent, stream);
-    if (dtype == COOPT_KV_FP8_E5M2) return launch_one<128, COOPT_KV_FP8_E5M2>(p, grid, dependent, stream);
-    return launch_one<128, COOPT_KV_BF16>(p, grid, dependent, stream);
+template <int D, int FMT>
+static int launch_layers(const DecodeParams& p, const coopt_layer_io* io, int grid, cudaStream_t stream) {
+  auto fill = [&](LayerPtrs* l) {
+    for (int y = 0; y < p.layers; ++y) {
+      l[y].cache = static_cast<uint8_t*>(io[y].cache->data);
+      l[y].q = static_cast<const __nv_bfloat16*>(io[y].q);
+      l[y].out = static_cast<__nv_bfloat16*>(io[y].out);
+      l[y].k_new = static_cast<const __nv_bfloat16*>(io[y].k_new);
+      l[y].v_new = static_cast<const __nv_bfloat16*>(io[y].v_new);
+      l[y].slot_mapping = reinterpret_cast<const long long*>(io[y].slot_mapping);
+    }
+  };
+  if constexpr (FMT != COOPT_KV_BF16) {
+    if (p.layers > 1) {
+      LayerTable<kManyLayers> table = {};
+      fill(table.l);
+      return launch_one<D, FMT, kManyLayers>(p, table, grid, stream);
+    }
   }
-  if (dtype == COOPT_KV_FP8_E4M3) return launch_one<64, COOPT_KV_FP8_E4M3>(p, grid, dependent, stream);
-  if (dtype == COOPT_KV_FP8_E5M2) return launch_one<64, COOPT_KV_FP8_E5M2>(p, grid, dependent, stream);
-  return launch_one<64, COOPT_KV_BF16>(p, grid, dependent, stream);
+  LayerTable<1> table;
+  fill(table.l);
+  return launch_one<D, FMT, 1>(p, table, grid, stream);
+}
+static int launch_attention(const DecodeParams& p, const coopt_layer_io* io, int head_dim, int dtype, int grid, cudaStream_t stream) {
+  if (head_dim == 128) {
+    if (dtype == COOPT_KV_FP8_E4M3) return launch_layers<128, COOPT_KV_FP8_E4M3>(p, io, grid, stream);
+    if (dtype == COOPT_KV_FP8_E5M2) return launch_layers<128, COOPT_KV_FP8_E5M2>(p, io, grid, stream);
+    return launch_layers<128, COOPT_KV_BF16>(p, io, grid, stream);
+  }
+  if (dtype == COOPT_KV_FP8_E4M3) return launch_layers<64, COOPT_KV_FP8_E4M3>(p, io, grid, stream);
+  if (dtype == COOPT_KV_FP8_E5M2) return launch_layers<64, COOPT_KV_FP8_E5M2>(p, io, grid, stream);
+  return launch_layers<64, COOPT_KV_BF16>(p, io, grid, stream);
 }
 
-// CTAs of a decode launch, from what the host knows: all that fit the device, or fewer where even full block tables would
-// leave a CTA without its smallest share.  The same on the sizing and the launching side.
-int decode_ctas(int num_sms, int batch, int num_kv_heads, int max_blocks_per_seq, int chunk_blocks) {
+// Shares of a layer (the most it can have), from what the host knows: one for every CTA that fits the device, or fewer
+// where even full block tables would not fill them.  The same on the sizing and the launching side.
+int decode_shares(int num_sms, int batch, int num_kv_heads, int max_blocks_per_seq, int chunk_blocks) {
   const long long units = chunk_blocks > 0 ? (max_blocks_per_seq + chunk_blocks - 1) / chunk_blocks : 1;
   const long long places = static_cast<long long>(batch) * num_kv_heads * (max_blocks_per_seq + units * kUnitCost);
   const long long most = (places + kMinPlaces - 1) / kMinPlaces;
@@ -942,10 +1034,11 @@ static size_t pieces_offset(int batch, int num_q_heads, int head_dim, int max_ch
   const size_t partials = static_cast<size_t>(batch) * num_q_heads * max_chunks * (head_dim + 2) * 4;
   return (workspace_control_bytes() + partials + 255) / 256 * 256;
 }
-static size_t pieces_rows(int ctas, int group, int max_chunks) { return static_cast<size_t>(max_chunks > 0 ? 4 : 2) * ctas * group; }
+// two pieces a share: of every layer of the launch, or (chunk mode) of sequences and of chunks
+static size_t pieces_rows(int shares, int group, int layers, int max_chunks) { return static_cast<size_t>(max_chunks > 0 ? 4 : 2 * layers) * shares * group; }
 
-size_t decode_workspace_bytes(int ctas, int group, int head_dim, int batch, int num_q_heads, int max_chunks) {
-  return (pieces_offset(batch, num_q_heads, head_dim, max_chunks) + pieces_rows(ctas, group, max_chunks) * (head_dim + 2) * 4 + 255) / 256 * 256;
+size_t decode_workspace_bytes(int shares, int group, int head_dim, int batch, int num_q_heads, int layers, int max_chunks) {
+  return (pieces_offset(batch, num_q_heads, head_dim, max_chunks) + pieces_rows(shares, group, layers, max_chunks) * (head_dim + 2) * 4 + 255) / 256 * 256;
 }
 size_t decode_plan_bytes(int batch, int max_blocks_per_seq) {
   return plan_table_offset(batch) + static_cast<size_t>(batch) * max_blocks_per_seq * 4;
@@ -956,16 +1049,17 @@ int launch_decode_plan(const int32_t* block_table, int32_t max_blocks_per_seq, c
   const long long pieces = static_cast<long long>(batch) * ((max_blocks_per_seq + kPlanPiece - 1) / kPlanPiece);
   const long long ctas = (pieces + kPlanThreads / 32 - 1) / (kPlanThreads / 32);
   const int key = plan_key(batch, num_kv_heads, chunk_size / kBlockSize, max_blocks_per_seq, num_blocks);
-  decode_plan_kernel<<<static_cast<unsigned>(ctas < kPlanCtas ? ctas : kPlanCtas), kPlanThreads, 0, stream>>>(
-      block_table, max_blocks_per_seq, context_lens, batch, num_blocks, key, static_cast<PlanHeader*>(plan));
-  return cudaGetLastError() == cudaSuccess ? COOPT_OK : COOPT_ERR_CUDA;
+  return launch_dependent(decode_plan_kernel, static_cast<int>(ctas < kPlanCtas ? ctas : kPlanCtas), kPlanThreads, 0, stream, block_table,
+                          max_blocks_per_seq, context_lens, batch, num_blocks, key, static_cast<PlanHeader*>(plan))
+             ? COOPT_OK
+             : COOPT_ERR_CUDA;
 }
 
-int launch_decode(const coopt_cache* c, const DecodeCall& a, cudaStream_t stream) {
+int launch_decode(const DecodeCall& a, cudaStream_t stream) {
+  const coopt_cache* c = a.layers[0].cache;            // all of one shape
   DecodeParams p = {};
-  p.cache = static_cast<uint8_t*>(c->data);
-  p.q = static_cast<const __nv_bfloat16*>(a.q);
-  p.out = static_cast<__nv_bfloat16*>(a.out);
+  p.layers = a.num_layers;
+  p.shares = a.shares;
   p.block_table = a.block_table;
   p.context_lens = a.context_lens;
   p.cu_q_lens = a.cu_q_lens;
@@ -985,11 +1079,8 @@ int launch_decode(const coopt_cache* c, const DecodeCall& a, cudaStream_t stream
     p.block_table = reinterpret_cast<const int*>(plan + plan_table_offset(a.batch));
     p.plan_key = plan_key(a.batch, c->num_kv_heads, p.chunk_blocks, a.max_blocks_per_seq, c->num_blocks);
   }
-  p.k_new = static_cast<const __nv_bfloat16*>(a.k_new);
-  p.v_new = static_cast<const __nv_bfloat16*>(a.v_new);
-  p.slot_mapping = reinterpret_cast<const long long*>(a.slot_mapping);
   p.kv_token_stride = a.kv_token_stride;
-  p.overlap_previous = a.order == kOverlapPrevious ? 1 : 0;
+  p.order = a.order;
   uint8_t* ws = static_cast<uint8_t*>(a.workspace);
   p.status = reinterpret_cast<int*>(ws);
   p.counters = reinterpret_cast<int*>(ws + kWsHeaderBytes);
@@ -1000,14 +1091,14 @@ int launch_decode(const coopt_cache* c, const DecodeCall& a, cudaStream_t stream
     p.part_m = reinterpret_cast<float*>(ws + m);
     p.part_l = reinterpret_cast<float*>(ws + l);
   }
-  const size_t rows = pieces_rows(a.ctas, p.group, p.max_chunks);
+  const size_t rows = pieces_rows(a.shares, p.group, a.num_layers, p.max_chunks);
   p.run_o = reinterpret_cast<float*>(ws + pieces_offset(a.batch, a.num_q_heads, c->head_dim, p.max_chunks));
   p.run_m = p.run_o + rows * c->head_dim;
   p.run_l = p.run_m + rows;
 #ifdef COOPT_TRACE
   p.trace = trace_buffer();
 #endif
-  return launch_attention(p, c->head_dim, c->dtype, a.ctas, a.order != kAfterPrevious, stream);
+  return launch_attention(p, a.layers, c->head_dim, c->dtype, std::min(kCtasPerSm * a.num_sms, a.shares * a.num_layers), stream);
 }
 
 }  // namespace coopt

@@ -2,12 +2,13 @@
 // the kernel's parameters.
 //
 // Work decomposition (Eq. 9: only the valid blocks of every sequence are listed).  A unit is what one softmax runs
-// over before anything is merged: a (sequence, kv head), or in chunk mode (Opt-Pa) one chunk of one.  All units lie
-// one behind the other on a line, in the order sequence, kv head, chunk; a unit of n blocks takes n + kUnitCost places
+// over before anything is merged: a (sequence, kv head), or in chunk mode (Opt-Pa) one chunk of one.  All units of a layer
+// lie one behind the other on a line, in the order sequence, kv head, chunk; a unit of n blocks takes n + kUnitCost places
 // of it, the extra ones in front, because a unit costs its warp a start and an end (query rows, reduction, store)
-// besides its blocks.  CTA i takes the places [i T, (i + 1) T), warp w of it an equal part of those, and a block
-// belongs to the warp that holds its place.  So every warp has at most two units that it holds only a piece of: the
-// one it starts in the middle of, and the one it does not reach the end of.
+// besides its blocks.  Share i of the line has the places [i T, (i + 1) T); a CTA works through one share, or through one
+// of every layer; warp w takes an equal part of the share's places, and a block belongs to the warp that holds its place.
+// So every warp has at most two units of a share that it holds only a piece of: the one it starts in the middle of, and
+// the one it does not reach the end of.
 #pragma once
 
 #include "coopt_common.cuh"
@@ -17,15 +18,15 @@ namespace coopt {
 constexpr int kMaxBatch = 512;
 constexpr int kMaxGroup = 8;
 constexpr int kMaxChunkBlocks = 2048;
-constexpr int kCounterSlots = 16384;
+constexpr int kCounterSlots = 16384;  // >= kManyLayers * shares * kMaxGroup
 constexpr int kWsHeaderBytes = 256;
 // Measured, us a pass: cost 3 / 5 places 435 / 429 (64 mixed lengths, 4 layers), 103 / 101 (24 sequences, G = 8, 4 layers),
 // 126 / 104 (21 sequences of 2..60 tokens, 8 layers); smallest share 64 / 16 places 20.5 / 16.4 (one sequence of 777
 // tokens), 142 / 102 (7 sequences of 272..544 tokens, 8 layers): where a call cannot fill the device, spreading it wins.
 constexpr int kUnitCost = 5;          // places of the line that a unit takes besides its blocks
 constexpr int kCtasPerSm = 1;
-constexpr int kMinPlaces = 16;        // smallest share of a CTA
-constexpr int kWholeUnits = 32;       // units of at most so many blocks (head_dim 64: twice) are not cut between CTAs
+constexpr int kMinPlaces = 16;        // smallest share
+constexpr int kWholeUnits = 32;       // units of at most so many blocks (head_dim 64: twice) are not cut between shares
 constexpr int kWholeUnitsIdle = 192;  // .. where the call does not fill the device
 constexpr int kNoChunks = 1 << 30;    // "blocks per chunk" of a call without chunks
 
@@ -49,68 +50,82 @@ __host__ __device__ inline int plan_key(int batch, int num_kv_heads, int chunk_b
   return static_cast<int>(h | 1u);
 }
 
-struct DecodeParams {
+// What a layer brings of its own.
+struct LayerPtrs {
   uint8_t* cache;
   const __nv_bfloat16* q;
   __nv_bfloat16* out;
+  // fused append (null when the layer has no new tokens): Algorithm 1 phase 1 for one token per sequence
+  const __nv_bfloat16* k_new;
+  const __nv_bfloat16* v_new;
+  const long long* slot_mapping;
+};
+// A launch serves one layer, or up to kManyLayers whose buffers do not touch each other (every one has room of its own for
+// its pieces in the workspace; what a launch costs once is small against eight layers).
+constexpr int kManyLayers = 8;
+template <int L>
+struct LayerTable {
+  LayerPtrs l[L];
+};
+
+struct DecodeParams {
   const int* block_table;
   const int* context_lens;
   const PlanHeader* plan;  // null: block_table and context_lens are the caller's own and are checked here
   const int* cu_q_lens;    // chunk mode of coopt_paged_chunked: prefix sums of the query tokens (must be 0..batch); else null
   int plan_key;
-  // fused append (null when the call has no new tokens): Algorithm 1 phase 1 for one token per sequence
-  const __nv_bfloat16* k_new;
-  const __nv_bfloat16* v_new;
-  const long long* slot_mapping;
   long long kv_token_stride;
+  int layers;
+  int shares;              // decode_shares(): the most shares a layer can have
   int max_blocks_per_seq;
   int batch, num_q_heads, num_kv_heads, group;
   int num_blocks;
-  int overlap_previous;    // 1: plan and cache were complete before the kernel in front of this one began
+  int order;               // DecodeOrder
   float sm_scale_log2;     // sm_scale * log2(e)
   int chunk_blocks;        // 0 = decode mode
   int max_chunks;
   int* status;
-  int* counters;           // [regions][ctas][kMaxGroup]: pieces delivered, by first CTA and head
+  int* counters;           // [regions][shares][kMaxGroup]: pieces delivered, by first share and head
   float* part_o;           // chunk mode: exported partials [B][Hq][max_chunks][D]
   float* part_m;           // [B][Hq][max_chunks]
   float* part_l;
-  float* run_o;            // pieces that CTAs share: [regions][2 ctas][G][D]; region 0 (sequence, kv head), region 1 (chunk mode) chunks
-  float* run_m;            // [regions][2 ctas][G], base-2 logarithm units
+  float* run_o;            // pieces of units that are cut between shares: [regions][2 shares][G][D]; a region per layer, or (chunk
+                           // mode) region 0 for (sequence, kv head), region 1 for chunks
+  float* run_m;            // [regions][2 shares][G], base-2 logarithm units
   float* run_l;
   unsigned long long* trace;   // time stamps (trace build only; null otherwise)
 };
 
 // ---- host side -------------------------------------------------------------------------------------------------
+// How much of a launch may run while the kernel in front of it in the stream still does.
 enum DecodeOrder {
-  kAfterPrevious = 0,     // an ordinary launch
-  kDependent,             // may be set up while the kernel before it runs, and waits for it before it reads anything
-  kOverlapPrevious        // the plan and the cache were complete before that kernel began: they are read early
+  kDependent,             // nothing but set-up
+  kAfterWrite,            // lengths and block table (or plan) were complete before that kernel began: they are read early
+  kOverlapPrevious        // .. and so was the cache: its first blocks are requested early
 };
 struct DecodeCall {
-  const void* q;
-  void* out;
+  const coopt_layer_io* layers;
+  int32_t num_layers;               // <= kManyLayers
   const int32_t* block_table;       // these two, or a plan
   const int32_t* context_lens;
   const void* plan;
   const int32_t* cu_q_lens;
-  const void* k_new;
-  const void* v_new;
-  const int64_t* slot_mapping;
   int64_t kv_token_stride;
   int32_t max_blocks_per_seq, batch, num_q_heads, chunk_size;
   float sm_scale;
   void* workspace;
-  int ctas;                         // decode_ctas()
+  int shares;                       // decode_shares()
+  int num_sms;
   DecodeOrder order;
 };
-int launch_decode(const coopt_cache* c, const DecodeCall& a, cudaStream_t stream);
+int launch_decode(const DecodeCall& a, cudaStream_t stream);
 int launch_decode_plan(const int32_t* block_table, int32_t max_blocks_per_seq, const int32_t* context_lens, int32_t batch,
                        int32_t num_kv_heads, int32_t num_blocks, int32_t chunk_size, void* plan, cudaStream_t stream);
-int decode_ctas(int num_sms, int batch, int num_kv_heads, int max_blocks_per_seq, int chunk_blocks);
-size_t decode_workspace_bytes(int ctas, int group, int head_dim, int batch, int num_q_heads, int max_chunks);
+int decode_shares(int num_sms, int batch, int num_kv_heads, int max_blocks_per_seq, int chunk_blocks);
+size_t decode_workspace_bytes(int shares, int group, int head_dim, int batch, int num_q_heads, int layers, int max_chunks);
 size_t decode_plan_bytes(int batch, int max_blocks_per_seq);
 size_t workspace_control_bytes();
+size_t workspace_need(int batch, int num_q_heads, int num_kv_heads, int head_dim, int max_blocks_per_seq, int chunk_size, int layers);
 int decode_max_batch();
 int decode_counter_slots();
 int decode_max_chunk_blocks();

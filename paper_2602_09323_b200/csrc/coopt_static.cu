@@ -8,7 +8,7 @@
 // it computes exactly what coopt_paged_decode computes.
 #include <mutex>
 
-#include "coopt_common.cuh"
+#include "coopt_decode.cuh"
 
 namespace {
 
@@ -45,8 +45,7 @@ extern "C" int coopt_paged_decode_static(const coopt_cache* cache, const void* q
   int rc = coopt::check_attention_args(cache, q, out, block_table, max_blocks_per_seq, context_lens, batch, num_q_heads);
   if (rc != COOPT_OK) return rc;
   if (batch == 0) return COOPT_OK;
-  const size_t need = coopt_workspace_bytes(batch, num_q_heads, cache->num_kv_heads, cache->head_dim,
-                                            max_blocks_per_seq, 0, batch);
+  const size_t need = coopt::workspace_need(batch, num_q_heads, cache->num_kv_heads, cache->head_dim, max_blocks_per_seq, 0, 1);
   if (need == 0) return COOPT_ERR_INVALID_ARG;
   if (need > static_cast<size_t>(COOPT_STATIC_SCRATCH_BYTES)) return COOPT_ERR_WORKSPACE;   // beyond the built-in maximum
   void* scratch = nullptr;

@@ -18,6 +18,7 @@ __global__ void __launch_bounds__(kWriteWarps * 32) kv_write_fp8_kernel(WritePar
   __shared__ __align__(16) uint8_t stage[kWriteWarps][part_bytes(D, true)];
   __shared__ Group group;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  wait_previous_kernel();
   if (warp == 0) find_group_warp(p, blockIdx.x, group, lane);
   __syncthreads();
   if (group.n == 0) return;
@@ -36,6 +37,7 @@ __global__ void __launch_bounds__(kWriteWarps * 32, 3) kv_write_fp8_span_kernel(
   __shared__ __align__(16) uint8_t stage[kWriteWarps][part_bytes(D, true)];
   __shared__ Group groups[kSpan];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  wait_previous_kernel();
   for (int w = warp; w < kSpan; w += kWriteWarps) {
     const int tok = blockIdx.x * kSpan + w;
     if (tok < p.num_tokens) find_group_warp(p, tok, groups[w], lane);
@@ -58,6 +60,7 @@ __global__ void __launch_bounds__(kWriteWarps * 32, 3) kv_write_fp8_span_kernel(
 template <int D>
 __global__ void __launch_bounds__(kWriteWarps * 32) kv_write_bf16_kernel(WriteParams p) {
   constexpr int kPerLane = D / 32;
+  wait_previous_kernel();
   const int i = blockIdx.x;
   const int64_t slot = p.slot_mapping[i];
   if (slot < 0) return;                                   // Eq. 5
@@ -94,7 +97,6 @@ int launch_kv_write(const coopt_cache* c, const void* k, const void* v, int64_t 
   p.num_tokens = num_tokens;
   p.num_kv_heads = c->num_kv_heads;
   p.num_blocks = c->num_blocks;
-  const dim3 block(kWriteWarps * 32);
   const bool fp8 = is_fp8(c->dtype), e5m2 = c->dtype == COOPT_KV_FP8_E5M2;
   // FP8: a CTA serves kWriteHeads kv heads (two warps each); bf16: kWriteWarps heads (one warp each)
   const int heads_per_cta = fp8 ? kWriteHeads : kWriteWarps;
@@ -102,20 +104,21 @@ int launch_kv_write(const coopt_cache* c, const void* k, const void* v, int64_t 
   const dim3 grid(num_tokens, head_ctas);
   const dim3 span_grid((num_tokens + kSpan - 1) / kSpan, head_ctas);
   const bool span = fp8 && num_tokens > kSpanThreshold;
+  bool ok;
   if (c->head_dim == 128) {
-    if (span && e5m2) kv_write_fp8_span_kernel<128, true><<<span_grid, block, 0, stream>>>(p);
-    else if (span) kv_write_fp8_span_kernel<128, false><<<span_grid, block, 0, stream>>>(p);
-    else if (e5m2) kv_write_fp8_kernel<128, true><<<grid, block, 0, stream>>>(p);
-    else if (fp8) kv_write_fp8_kernel<128, false><<<grid, block, 0, stream>>>(p);
-    else kv_write_bf16_kernel<128><<<grid, block, 0, stream>>>(p);
+    if (span && e5m2) ok = launch_dependent(kv_write_fp8_span_kernel<128, true>, span_grid, kWriteWarps * 32, 0, stream, p);
+    else if (span) ok = launch_dependent(kv_write_fp8_span_kernel<128, false>, span_grid, kWriteWarps * 32, 0, stream, p);
+    else if (e5m2) ok = launch_dependent(kv_write_fp8_kernel<128, true>, grid, kWriteWarps * 32, 0, stream, p);
+    else if (fp8) ok = launch_dependent(kv_write_fp8_kernel<128, false>, grid, kWriteWarps * 32, 0, stream, p);
+    else ok = launch_dependent(kv_write_bf16_kernel<128>, grid, kWriteWarps * 32, 0, stream, p);
   } else {
-    if (span && e5m2) kv_write_fp8_span_kernel<64, true><<<span_grid, block, 0, stream>>>(p);
-    else if (span) kv_write_fp8_span_kernel<64, false><<<span_grid, block, 0, stream>>>(p);
-    else if (e5m2) kv_write_fp8_kernel<64, true><<<grid, block, 0, stream>>>(p);
-    else if (fp8) kv_write_fp8_kernel<64, false><<<grid, block, 0, stream>>>(p);
-    else kv_write_bf16_kernel<64><<<grid, block, 0, stream>>>(p);
+    if (span && e5m2) ok = launch_dependent(kv_write_fp8_span_kernel<64, true>, span_grid, kWriteWarps * 32, 0, stream, p);
+    else if (span) ok = launch_dependent(kv_write_fp8_span_kernel<64, false>, span_grid, kWriteWarps * 32, 0, stream, p);
+    else if (e5m2) ok = launch_dependent(kv_write_fp8_kernel<64, true>, grid, kWriteWarps * 32, 0, stream, p);
+    else if (fp8) ok = launch_dependent(kv_write_fp8_kernel<64, false>, grid, kWriteWarps * 32, 0, stream, p);
+    else ok = launch_dependent(kv_write_bf16_kernel<64>, grid, kWriteWarps * 32, 0, stream, p);
   }
-  return cudaGetLastError() == cudaSuccess ? COOPT_OK : COOPT_ERR_CUDA;
+  return ok ? COOPT_OK : COOPT_ERR_CUDA;
 }
 
 }  // namespace coopt

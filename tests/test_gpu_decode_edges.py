@@ -56,3 +56,54 @@ def test_chunks_that_warps_and_ctas_share(case, chunk):
         assert np.allclose(m_c[b, h, :n], m, rtol=1e-4, atol=1e-3)
         assert np.allclose(l_c[b, h, :n], l, rtol=5e-3, atol=1e-4)
         assert np.allclose(o_c[b, h, :n], o, rtol=5e-3, atol=2e-2)
+
+
+@pytest.mark.parametrize("hq,hkv,d,lens", [(8, 2, 128, [300, 1, 0, 17, 2048]), (16, 2, 64, [16, 33, 1, 900])])
+@pytest.mark.parametrize("n,how", [(2, "apart"), (3, "chained"), (3, "some append"), (67, "apart"), (2, "one output")])
+def test_layers_in_one_launch_equal_layers_one_by_one(hq, hkv, d, lens, n, how):
+    """Layers whose buffers are apart share a launch; layers that read what another writes must still run in order
+    ("chained": a layer's output is the next one's query; "one output": the last layer's result stays)."""
+    w = workloads.make_workload("layers", lens, hq, hkv, d, seed=n)
+    table, lens_t, B, gen = w.block_table.cuda(), w.context_lens_tensor.cuda(), w.batch, torch.Generator("cuda").manual_seed(n)
+    draw = lambda heads: torch.randn(B, heads, d, generator=gen, device="cuda").to(torch.bfloat16)
+    live = torch.tensor([L > 0 for L in lens], device="cuda")
+    at = torch.tensor([w.kv_offsets[b] + max(L, 1) - 1 for b, L in enumerate(lens)]).clamp(max=w.k.shape[0] - 1)
+    slots = torch.where(live, w.slot_mapping[at].cuda(), torch.full((B,), -1, device="cuda"))
+    hist = np.concatenate([np.arange(w.kv_offsets[b], w.kv_offsets[b] + max(0, L - 1)) for b, L in enumerate(lens)])
+    base = helpers.gpu_fill(w, calls=[hist])
+    qs, outs = [draw(hq) for _ in range(n)], [torch.full((B, hq, d), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(n)]
+    if how == "chained":
+        qs[1:] = outs[:-1]
+    if how == "one output":
+        outs = [outs[0]] * n
+    new = [(draw(hkv), draw(hkv), slots) if how != "some append" or y % 2 else (None, None, None) for y in range(n)]
+
+    def run(together):
+        caches = []
+        for _ in range(n):
+            c = binding.Cache(w.num_blocks, hkv, d)
+            c.data.copy_(base.data)
+            caches.append(c)
+        ws = binding.new_workspace(B, hq, hkv, d, table.shape[1])
+        if together:
+            plan = torch.empty(binding.plan_bytes(B, hkv, table.shape[1]), dtype=torch.uint8, device="cuda")
+            ios = [{"cache": c, "q": q, "out": o, "k_new": k, "v_new": v, "slot_mapping": s} for c, q, o, (k, v, s) in zip(caches, qs, outs, new)]
+            layer_set = binding.LayerSet(ios)
+            layer_set.kv_stride = hkv * d
+            binding.decode_layers(layer_set, table, lens_t, hq, w.sm_scale, plan, ws)
+            # the plan is one that a later launch can use
+            again = binding.decode_step_planned(caches[0], plan, qs[0], table.shape[1], w.sm_scale, ws)
+            assert how != "apart" or torch.equal(again, outs[0])
+        else:
+            for c, q, o, (k, v, s) in zip(caches, qs, outs, new):
+                if k is not None:
+                    binding.kv_write(c, k, v, s)
+                binding.paged_decode(c, q, table, lens_t, w.sm_scale, ws, out=o)
+        torch.cuda.synchronize()
+        assert binding.workspace_status(ws) == 0
+        return [o.clone() for o in outs], [c.data for c in caches]
+
+    (want, want_bytes), (got, got_bytes) = run(False), run(True)
+    for y in range(n):
+        assert torch.equal(want_bytes[y], got_bytes[y]), f"layer {y}: cache bytes"
+        assert torch.equal(got[y], want[y]), f"layer {y}: outputs"
