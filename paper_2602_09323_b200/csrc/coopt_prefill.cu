@@ -1,35 +1,59 @@
-// Chunked prefill against the paged FP8 cache: Eq. 1 with the causal K_{<=t}, Eq. 6
-// dequantisation on load, Eq. 7-8 grouped-query sharing, Eq. 9 valid blocks only, Eq. 10
-// max-subtracted softmax, for runs of several query tokens per sequence.
+// Chunked prefill against the paged FP8 cache on the 5th-generation tensor cores: Eq. 1 with the causal K_{<=t}, Eq. 6
+// dequantisation on load, Eq. 7-8 grouped-query sharing, Eq. 9 valid blocks only, Eq. 10 max-subtracted softmax, for runs
+// of several query tokens per sequence.  head_dim 64 and 128.
 //
-// A CTA owns one (sequence, kv head, tile of consecutive query tokens).  Its 128 rows are the
-// (query token, query head of the group) pairs of the tile, so the K/V stream of the kv head is
-// fetched once for all G heads (Algorithm 2).  The context is walked 64 tokens (four cache
-// blocks) at a time:
-//   1. one lane per block starts a bulk async copy of the granule into a ring of raw stages
-//      (an mbarrier per stage counts the bytes);
-//   2. all threads widen the E4M3 codes of the stage to f16 (exact) into a double-buffered
-//      operand tile laid out in the register order of the matrix instruction;
-//   3. every warp runs S = Q K^T and O += P V for its 16 rows on tensor cores
-//      (mma.sync m16n8k16, f16 operands, fp32 accumulators) with an online softmax in between.
-// The K scale of a block is applied to the logits of its 16 tokens and the V scale is folded
-// into the probabilities, both uniform per block, so the products themselves are exact.
-#include "coopt_common.cuh"
+// A CTA owns one (sequence, kv head) and two tiles of consecutive query tokens.  The 128 rows of a tile are its (query
+// token, query head of the group) pairs, so the K/V stream of the kv head is fetched, and V widened, once for all G heads
+// and both tiles (Algorithm 2).  Per tile and 128 keys (eight cache blocks):
+//     S [128 rows x 128 keys] = Q [128 x D] . Ktile^T       head_dim 128: kind::f8f6f4, the cache codes as they are, Q as
+//                                                           two E4M3 terms of the bf16 query; head_dim 64: kind::f16, Q and
+//                                                           K in f16 (both exact)
+//     O [128 rows x D]       += P [128 x 128 keys] . Vtile  kind::f16: P rounded once to f16 and read from tensor memory, V
+//                                                           codes widened to f16 (exact) in shared memory
+// with fp32 accumulators in tensor memory.  The K scale of a block multiplies the logits of its 16 keys, the V scale goes
+// into the exponent of the probabilities.
+//
+// What bounds it: per tile of 128 x 128 the exponential units need 1,024 cycles of an SM (16 a cycle) and the tensor core
+// 1,024 (head_dim 64: 512).  Both run all the time only if neither waits for the other: a tile is multiplied 64 keys (a
+// half) at a time, the logits of the next half while the half before is in the softmax, and two tiles share the SM.
+// Softmax of a tile: four warps, one row per thread, the row's 64 logits of the half in registers, read once.  It keeps a
+// reference maximum per row that may lag the true one by up to 2^11 (and a V scale reference that a scale may exceed by up
+// to 2^4), so the accumulator in tensor memory is rescaled rarely; f16 probabilities have room for that factor.
+//
+// Tensor memory (512 columns): logits of tile x in columns 64 x .., free again as soon as they are in registers; its
+// probabilities, two f16 to a column, in two buffers of 32 columns from 128 + 64 x; its accumulator from 256 + D x.
+//
+// Warp roles (512 threads):
+//   warps 0-3, 4-7   softmax of tile 0, of tile 1
+//   warps 8-11       widen V (head_dim 64: and K) tiles into f16 operands
+//   warps 12, 13     issue the matrix instructions of tile 0, of tile 1
+//   warp 14          copies: gather requests over the tensor map of the cache
+//   warp 15          what the softmax needs of a tile's block scales, worked out once for all rows
+//
+// Measured: 8 sequences of 4096 cached and 512 new tokens, 40 query heads over 8 kv heads, head_dim 128: 690 -> 450 us (the
+// kernel before: one tile a CTA, two groups of eight warps that took its key tiles in turns, each with an accumulator and
+// widening of its own); prompts of 900..2900 tokens, 32 heads over 8, head_dim 64: 495 -> 220 us (mma.sync).  A half takes
+// about 2,050 cycles for both tiles: exponential units 50 %, tensor core 42 %, the rest the way of a half through its
+// barriers (a hand-over from warp to warp costs about 120 cycles) with two softmax warps a scheduler.
+// Every wait is bounded; a wait that runs out is reported in the status word and all roles leave through the common exit,
+// which frees the tensor memory.
+#include "coopt_umma.cuh"
 
 namespace coopt {
 
 namespace {
 
-constexpr int kPfWarps = 8;
-constexpr int kPfThreads = kPfWarps * 32;
-constexpr int kPfRows = kPfWarps * 16;
-constexpr int kTileBlocks = 4;                         // cache blocks per tile
-constexpr int kTileTokens = kTileBlocks * kBlockSize;  // 64
-constexpr int kRawStages = 3;
+constexpr int kRows = 128;
+constexpr int kThreads = 512;
+constexpr int kWidenWarp = 8, kMmaWarp = 12, kCopyWarp = 14;      // warp 15: scales
+constexpr int kTileBlocks = 8;
+constexpr int kTileKeys = kTileBlocks * kBlockSize;        // 128: what is copied and widened at a time
+constexpr int kHalf = kTileKeys / 2;                       // 64: what is multiplied at a time
 constexpr float kLog2e = 1.4426950408889634f;
+constexpr float kMaxLag = 11.0f;                           // a row's reference may lag its maximum by this much (base-2 logarithm units)
+constexpr float kScaleLag = 16.0f;                         // a V scale may exceed the reference scale by this factor
 
 struct PrefillParams {
-  const uint8_t* cache;
   const __nv_bfloat16* q;
   __nv_bfloat16* out;
   const int* cu_q_lens;
@@ -38,391 +62,632 @@ struct PrefillParams {
   int max_blocks_per_seq;
   int batch, num_q_heads, num_kv_heads, group;
   int num_blocks;
-  int tile_queries;        // query tokens per CTA = 128 / group
+  int tile_queries;        // query tokens per tile = 128 / group
   int causal;
   float sm_scale_log2;
   int* status;
 };
 
 template <int D>
-struct PfCfg {
+struct Cfg {
+  static constexpr bool kWideK = D == 64;                         // K is widened to f16 too
+  static constexpr int kPart = kBlockSize * D;                    // K (or V) codes of one granule
   static constexpr int kGran = granule_bytes(D, true);
-  static constexpr int kRawStage = kTileBlocks * kGran;
-  static constexpr int kConvBlock = 2 * (2 * kBlockSize * D);   // f16 K and V of one block
-  static constexpr int kConvTile = kTileBlocks * kConvBlock;
-  static constexpr int kChunksPerBlock = 2 * D;                 // 16-byte chunks of codes (K then V)
-  static constexpr int kRawOff = 0;
-  static constexpr int kConvOff = kRawOff + kRawStages * kRawStage;
-  static constexpr int kScaleOff = kConvOff + 2 * kConvTile;    // float [2 buffers][4 blocks][2]
-  static constexpr int kBarOff = kScaleOff + 2 * kTileBlocks * 2 * 4;
-  static constexpr int kMiscOff = kBarOff + kRawStages * 8;
-  static constexpr int kSmemBytes = kMiscOff + 32;
+  static constexpr int kCodes = kTileBlocks * kPart;              // K (or V) codes of a tile
+  static constexpr int kKSlot = kCodes + kTileBlocks * kFp8Header;   // K parts, then the eight headers
+  static constexpr int kKSlots = D == 128 ? 3 : 2, kVSlots = 2, kWide = 2, kScaleSlots = 4;
+  static constexpr int kOperand = 128 * D * 2;                    // Q of a tile (two terms of codes, or f16); V^T, or K, of a tile in f16
+  static constexpr int kKOff = 0;
+  static constexpr int kVOff = kKOff + kKSlots * kKSlot;
+  static constexpr int kQOff = kVOff + kVSlots * kCodes;
+  static constexpr int kV16Off = kQOff + 2 * kOperand;
+  static constexpr int kK16Off = kV16Off + kWide * kOperand;
+  static constexpr int kScaleOff = kK16Off + (kWideK ? kWide * kOperand : 0);   // [slot][32]: K scales, log2 of V scale ratios, their inverses, factor, reference
+  static constexpr int kBarOff = kScaleOff + kScaleSlots * 128;
+  static constexpr int kNumBars = 2 * kKSlots + 2 * kVSlots + 4 * kWide + kScaleSlots + 13;
+  static constexpr int kMiscOff = kBarOff + kNumBars * 8;
+  static constexpr int kSmemBytes = kMiscOff + 64;
+  static_assert(kKSlot % 128 == 0 && kVOff % 128 == 0 && kQOff % 128 == 0 && kSmemBytes <= 232448, "shared memory of one CTA");
 };
 
-__device__ __forceinline__ float quad_max(float x) {
-  x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, 1));
-  return fmaxf(x, __shfl_xor_sync(0xffffffffu, x, 2));
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
+               ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
+                 "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory");
 }
-__device__ __forceinline__ float quad_sum(float x) {
-  x += __shfl_xor_sync(0xffffffffu, x, 1);
-  return x + __shfl_xor_sync(0xffffffffu, x, 2);
-}
-template <int D>
-__global__ void __launch_bounds__(kPfThreads, 1) paged_prefill_kernel(const PrefillParams p) {
-  using C = PfCfg<D>;
-  constexpr int kKSteps = D / 16, kNTiles = D / 8;
-  extern __shared__ __align__(128) uint8_t smem[];
-  uint8_t* raw = smem + C::kRawOff;
-  uint8_t* conv = smem + C::kConvOff;
-  float* tile_scales = reinterpret_cast<float*>(smem + C::kScaleOff);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kBarOff);
-  int* misc = reinterpret_cast<int*>(smem + C::kMiscOff);   // [0] sequence, [1] first query of the tile
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int quad = lane & 3;
+// Four codes -> four f16 (exact).  Two cycles of a scheduler per conversion of two codes; integer instructions for the same
+// (shift, mask, sign) take 14 cycles per four codes.
+template <bool kE5m2>
+__device__ __forceinline__ uint2 widen4(uint32_t w) {
+  if (kE5m2) return make_uint2(e5m2x2_to_f16x2_lo(w), e5m2x2_to_f16x2_hi(w));
+  return make_uint2(e4m3x2_to_f16x2_lo(w), e4m3x2_to_f16x2_hi(w));
+}
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float d;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+// A wait by all lanes of a warp, and an arrival by one of them (behind the others).
+__device__ __forceinline__ bool wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+  return __all_sync(0xffffffffu, wait_bar(bar, parity, abort_flag));
+}
+__device__ __forceinline__ void arrive_one(uint64_t* bar) {
+  asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n @q mbarrier.arrive.shared::cta.b64 _, [%0];\n}" ::"r"(smem_u32(bar)) : "memory");
+}
+
+template <int D, bool kE5m2>
+__global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap map_part,
+                                                                    const __grid_constant__ CUtensorMap map_hdr) {
+  using C = Cfg<D>;
+  extern __shared__ __align__(128) uint8_t smem[];
+  float* scales = reinterpret_cast<float*>(smem + C::kScaleOff);
+  uint64_t* bar_kfull = reinterpret_cast<uint64_t*>(smem + C::kBarOff);   // K parts and headers of a tile have landed
+  uint64_t* bar_kfree = bar_kfull + C::kKSlots;         // .. are of no more use: to the scale warp, and to both tiles' products (or the widening warps)
+  uint64_t* bar_vfull = bar_kfree + C::kKSlots;         // V parts of a tile have landed
+  uint64_t* bar_vfree = bar_vfull + C::kVSlots;         // .. have been widened
+  uint64_t* bar_v16full = bar_vfree + C::kVSlots;       // V operand ready
+  uint64_t* bar_v16free = bar_v16full + C::kWide;       // .. both tiles' products with it are done
+  uint64_t* bar_k16full = bar_v16free + C::kWide;       // the same of K
+  uint64_t* bar_k16free = bar_k16full + C::kWide;
+  uint64_t* bar_scale = bar_k16free + C::kWide;         // the softmax's share of a tile's scales is ready
+  uint64_t* bar_sfull = bar_scale + C::kScaleSlots;     // [tile] logits of a half are in tensor memory (and the tile's scales ready)
+  uint64_t* bar_sfree = bar_sfull + 2;                  // [tile] .. and now in registers
+  uint64_t* bar_pfull = bar_sfree + 2;                  // [tile][buffer] its probabilities are in tensor memory
+  uint64_t* bar_pv = bar_pfull + 4;                     // [tile] its product with V is done
+  uint64_t* bar_out = bar_pv + 2;                       // [tile] .. and it was the tile's last
+  uint64_t* bar_q = bar_out + 2;                        // the query operands are in shared memory
+  int* misc = reinterpret_cast<int*>(smem + C::kMiscOff);   // [0] sequence, [1] first query, [2] abort flag, [3] tensor memory
+  volatile int* abort_flag = misc + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(misc + 3);
+
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;      // (the warp in a uniform register)
   const int G = p.group, Hq = p.num_q_heads, Hkv = p.num_kv_heads;
   const int g = blockIdx.y;
   const int TQ = p.tile_queries;
 
-  // ---- which (sequence, query tile) is this CTA's ----------------------------------------------
   if (tid == 0) {
-    int left = blockIdx.x, found = -1, q0 = 0;
-    for (int b = 0; b < p.batch; ++b) {
-      const int n = max(0, p.cu_q_lens[b + 1] - p.cu_q_lens[b]);
-      const int nt = (n + TQ - 1) / TQ;
-      if (left < nt) { found = b; q0 = (nt - 1 - left) * TQ; break; }   // late (long) tiles first
-      left -= nt;
+    *abort_flag = 0;
+    for (int i = 0; i < C::kKSlots; ++i) { mbar_init(&bar_kfull[i], 1); mbar_init(&bar_kfree[i], C::kWideK ? 5 : 3); }
+    for (int i = 0; i < C::kVSlots; ++i) { mbar_init(&bar_vfull[i], 1); mbar_init(&bar_vfree[i], 4); }
+    for (int i = 0; i < C::kWide; ++i) {
+      mbar_init(&bar_v16full[i], 4); mbar_init(&bar_v16free[i], 2);
+      mbar_init(&bar_k16full[i], 4); mbar_init(&bar_k16free[i], 2);
     }
-    misc[0] = found;
-    misc[1] = q0;
-    for (int i = 0; i < kRawStages; ++i) mbar_init(&bars[i], 1);
+    for (int i = 0; i < C::kScaleSlots; ++i) mbar_init(&bar_scale[i], 1);
+    mbar_init(bar_q, 8);
+    for (int i = 0; i < 4; ++i) mbar_init(&bar_pfull[i], 4);
+    for (int i = 0; i < 2; ++i) { mbar_init(&bar_sfull[i], 2); mbar_init(&bar_sfree[i], 4); mbar_init(&bar_pv[i], 1); mbar_init(&bar_out[i], 1); }
     mbar_fence_init();
   }
+  if (warp == kMmaWarp) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (tid == kCopyWarp * 32) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&map_part) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&map_hdr) : "memory");
+  }
+  wait_previous_kernel();
+
+  // ---- which (sequence, pair of query tiles) is this CTA's: late (long) ones of a sequence first -------------------------
+  if (warp == 0) {
+    int left = blockIdx.x, found = -1, q0 = 0;
+    for (int b0 = 0; b0 < p.batch && found < 0; b0 += 32) {
+      const int b = b0 + lane;
+      const int n = b < p.batch ? max(0, p.cu_q_lens[b + 1] - p.cu_q_lens[b]) : 0;
+      const int nt = (n + 2 * TQ - 1) / (2 * TQ);
+      int upto = nt;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, upto, o);
+        if (lane >= o) upto += t;
+      }
+      const unsigned in = __ballot_sync(0xffffffffu, upto > left);
+      if (in) {
+        const int l = __ffs(in) - 1;
+        found = b0 + l;
+        q0 = (__shfl_sync(0xffffffffu, upto, l) - 1 - left) * 2 * TQ;
+      } else {
+        left -= __shfl_sync(0xffffffffu, upto, 31);
+      }
+    }
+    if (lane == 0) { misc[0] = found; misc[1] = q0; }
+  }
+  tc_fence_before();
   __syncthreads();
-  const int b = misc[0];
-  if (b < 0) return;
-  const int q0 = misc[1];
-  const int row_base = p.cu_q_lens[b];
-  const int n_new = p.cu_q_lens[b + 1] - row_base;
-  const int nq = min(TQ, n_new - q0);
-  const int L = max(0, min(p.context_lens[b], p.max_blocks_per_seq * kBlockSize));
-  // last position any row of the tile may see (Eq. 1: K_{<=t})
-  const int kv_end = p.causal ? max(0, min(L, L - n_new + q0 + nq)) : L;
-  const int n_tiles = (kv_end + kTileTokens - 1) / kTileTokens;
-  const int n_blocks = (kv_end + kBlockSize - 1) / kBlockSize;
-
-  // ---- the two rows of this lane ------------------------------------------------------------------
-  const int r0 = warp * 16 + (lane >> 2), r1 = r0 + 8;
-  const int qi0 = r0 / G, qi1 = r1 / G;
-  const bool live0 = qi0 < nq, live1 = qi1 < nq;
-  const size_t grow0 = static_cast<size_t>(row_base + q0 + (live0 ? qi0 : 0)) * Hq + g * G + (live0 ? r0 % G : 0);
-  const size_t grow1 = static_cast<size_t>(row_base + q0 + (live1 ? qi1 : 0)) * Hq + g * G + (live1 ? r1 % G : 0);
-  // index of the last visible token of each row; -1 hides everything
-  int lim0 = -1, lim1 = -1;
-  if (live0) lim0 = p.causal ? min(L - 1, L - n_new + q0 + qi0) : L - 1;
-  if (live1) lim1 = p.causal ? min(L - 1, L - n_new + q0 + qi1) : L - 1;
-  int warp_min_lim = min(lim0, lim1);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) warp_min_lim = min(warp_min_lim, __shfl_xor_sync(0xffffffffu, warp_min_lim, o));
-
-  // ---- producer state (warp 0, lanes 0..3: one cache block each) --------------------------------
-  const int* trow = p.block_table + static_cast<size_t>(b) * p.max_blocks_per_seq;
-  int issued = 0;
-  int next_id = 0;
-  auto load_id = [&](int tile) {
-    const int j = tile * kTileBlocks + lane;
-    if (warp == 0 && lane < kTileBlocks && j < n_blocks) {
-      int id = trow[j];
-      if (id < 0 || id >= p.num_blocks) { atomicCAS(p.status, 0, COOPT_ERR_INVALID_ARG); id = 0; }
-      next_id = id;
-    }
-  };
-  auto issue = [&]() {   // warp 0 only: copies of tile `issued` into its ring stage
-    const int tile = issued;
-    const int stage = tile % kRawStages;
-    const int nb = min(kTileBlocks, n_blocks - tile * kTileBlocks);
-    if (lane == 0) {
-      fence_proxy_async();
-      mbar_expect_tx(&bars[stage], nb * C::kGran);
-    }
-    __syncwarp();
-    if (lane < nb) {
-      const uint8_t* src = p.cache + (static_cast<size_t>(next_id) * Hkv + g) * C::kGran;
-      bulk_copy_g2s(raw + stage * C::kRawStage + lane * C::kGran, src, C::kGran, &bars[stage]);
-    }
-    load_id(tile + 1);
-  };
-  if (warp == 0) load_id(0);
-  for (int s = 0; s < kRawStages && s < n_tiles; ++s) {
-    if (warp == 0) issue();
-    ++issued;
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  const int b = misc[0], q0 = misc[1];
+  int row_base = 0, n_new = 0, L = 0;
+  if (b >= 0) {
+    row_base = p.cu_q_lens[b];
+    n_new = p.cu_q_lens[b + 1] - row_base;
+    L = max(0, min(p.context_lens[b], p.max_blocks_per_seq * kBlockSize));
   }
+  // keys that any row of tile x may see (Eq. 1: K_{<=t}), and tiles of keys
+  auto tile_queries = [&](int x) { return max(0, min(TQ, n_new - q0 - x * TQ)); };
+  auto tile_keys = [&](int x) {
+    const int nq = tile_queries(x);
+    return nq == 0 ? 0 : p.causal ? max(0, min(L, L - n_new + q0 + x * TQ + nq)) : L;
+  };
+  const int kv_end = max(tile_keys(0), tile_keys(1));
+  const int n_blocks = (kv_end + kBlockSize - 1) / kBlockSize, n_tiles = (kv_end + kTileKeys - 1) / kTileKeys;
 
-  // ---- query fragments: bf16 -> f16 after an exact power-of-two scaling per row ----------------
-  uint32_t qa[kKSteps][4];
-  float qs0 = p.sm_scale_log2, qs1 = p.sm_scale_log2;
-  {
-    uint32_t w0[kKSteps][2], w1[kKSteps][2];
-    // k-step s of the instruction covers dims 16s..16s+15; its logical k positions 2c, 2c+1 (registers
-    // a0/a1 and b0) stand for dims 16s + 4c + {0, 1}, positions 2c+8, 2c+9 (a2/a3 and b1) for dims
-    // 16s + 4c + {2, 3}: the order in which a 16-byte chunk of the cache's K part splits over a quad
-    const __nv_bfloat16* qp0 = p.q + grow0 * D + 4 * quad;
-    const __nv_bfloat16* qp1 = p.q + grow1 * D + 4 * quad;
-    float am0 = 0.0f, am1 = 0.0f;
+  // softmax groups: this thread's row r of tile x
+  const int x = warp >> 2, r = tid & (kRows - 1);
+  const int qi = r / G;
+  const bool live = x < 2 && qi < tile_queries(x);
+  const size_t grow = static_cast<size_t>(row_base + q0 + x * TQ + (live ? qi : 0)) * Hq + g * G + (live ? r % G : 0);
+  uint32_t pend_mask = 0, pend_par = 0;                 // copy lane: the latest phase expected of every slot it has filled
+
+  if (n_tiles == 0) {
+    // no such tile, or nothing visible: all-zero rows
+    if (live)
+      for (int d = 0; d < D; d += 8) *reinterpret_cast<uint4*>(p.out + grow * D + d) = make_uint4(0u, 0u, 0u, 0u);
+  } else if (warp < 8) {
+    // ================= softmax: one row per thread ===================================================================
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 168;");
+    const uint32_t lane_base = static_cast<uint32_t>(warp & 3) * 32u << 16;
+    const uint32_t s_cols = tmem + kHalf * x + lane_base, p_cols = tmem + 2 * kHalf + kHalf * x + lane_base, o_cols = tmem + 256 + D * x + lane_base;
+    // ---- row r of the query operand
+    float qscale = 0.0f;       // logits of this row = tensor-memory value * qscale * K scale of the block
+    {
+      uint32_t amax = 0;
+      const uint4* src = reinterpret_cast<const uint4*>(p.q + grow * D);
+      if (live) {
+#pragma unroll 8
+        for (int c = 0; c < D / 8; ++c) {
+          const uint4 v = src[c];
+          const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-    for (int s = 0; s < kKSteps; ++s)
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        w0[s][e] = live0 ? *reinterpret_cast<const uint32_t*>(qp0 + 16 * s + 2 * e) : 0u;
-        w1[s][e] = live1 ? *reinterpret_cast<const uint32_t*>(qp1 + 16 * s + 2 * e) : 0u;
-        am0 = fmaxf(am0, fmaxf(fabsf(bf16_lo(w0[s][e])), fabsf(bf16_hi(w0[s][e]))));
-        am1 = fmaxf(am1, fmaxf(fabsf(bf16_lo(w1[s][e])), fabsf(bf16_hi(w1[s][e]))));
+          for (int e = 0; e < 4; ++e) amax = max(amax, max((w[e] << 16) & 0x7FFFFFFFu, w[e] & 0x7FFF0000u));   // |bf16| as fp32 bits
+        }
       }
-    am0 = quad_max(am0);
-    am1 = quad_max(am1);
-    auto pow2 = [](float amax, float& up, float& down) {
+      // the row scaled by a power of two into [128, 256), undone on the logits
       int k2 = 0;
-      if (amax > 0.0f) k2 = max(-64, min(64, 134 - static_cast<int>((__float_as_uint(amax) >> 23) & 0xFF)));
-      up = __uint_as_float(static_cast<uint32_t>(k2 + 127) << 23);
-      down = __uint_as_float(static_cast<uint32_t>(127 - k2) << 23);
-    };
-    float up0, dn0, up1, dn1;
-    pow2(am0, up0, dn0);
-    pow2(am1, up1, dn1);
-    qs0 *= dn0;
-    qs1 *= dn1;
+      if (amax != 0u) k2 = max(-64, min(64, 134 - static_cast<int>((amax >> 23) & 0xFF)));
+      qscale = p.sm_scale_log2 * __uint_as_float(static_cast<uint32_t>(127 - k2) << 23);
+      const float up = __uint_as_float(static_cast<uint32_t>(k2 + 127) << 23);
+      uint8_t* qrow = smem + C::kQOff + x * C::kOperand + (r & 7) * 16;
+#pragma unroll 2
+      for (int c = 0; c < D / 16; ++c) {                  // 16 elements
+        const uint4 a = live ? src[2 * c] : make_uint4(0u, 0u, 0u, 0u), e4 = live ? src[2 * c + 1] : make_uint4(0u, 0u, 0u, 0u);
+        const uint32_t w[8] = {a.x, a.y, a.z, a.w, e4.x, e4.y, e4.z, e4.w};
+        if constexpr (C::kWideK) {
+          // f16 (exact)
+          uint32_t h[8];
 #pragma unroll
-    for (int s = 0; s < kKSteps; ++s) {
-      qa[s][0] = pack_f16x2(bf16_lo(w0[s][0]) * up0, bf16_hi(w0[s][0]) * up0);
-      qa[s][1] = pack_f16x2(bf16_lo(w1[s][0]) * up1, bf16_hi(w1[s][0]) * up1);
-      qa[s][2] = pack_f16x2(bf16_lo(w0[s][1]) * up0, bf16_hi(w0[s][1]) * up0);
-      qa[s][3] = pack_f16x2(bf16_lo(w1[s][1]) * up1, bf16_hi(w1[s][1]) * up1);
-    }
-  }
-
-  float m0 = -INFINITY, m1 = -INFINITY, l0 = 0.0f, l1 = 0.0f, vref = 0.0f;
-  float o[kNTiles][4];
-#pragma unroll
-  for (int t = 0; t < kNTiles; ++t)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) o[t][e] = 0.0f;
-
-  bool failed = false;
-#pragma unroll 1
-  for (int tile = 0; tile < n_tiles; ++tile) {
-    const int stage = tile % kRawStages;
-    const uint32_t parity = (tile / kRawStages) & 1u;
-    const bool ok = mbar_wait_bounded(&bars[stage], parity);
-    const int buf = tile & 1;
-    uint8_t* cv = conv + buf * C::kConvTile;
-    const int nb = min(kTileBlocks, n_blocks - tile * kTileBlocks);
-
-    // ---- widen the stage's codes to f16 and put them in the register order of mma.m16n8k16 --------
-    // A 16-byte chunk of the K part is one token x 16 dims, of the V part one dim x 16 tokens; either
-    // way it feeds the four lanes of one quad with two registers each.
-    if (ok) {
-      const uint8_t* rs = raw + stage * C::kRawStage;
-#pragma unroll
-      for (int c = tid; c < kTileBlocks * C::kChunksPerBlock; c += kPfThreads) {
-        const int jb = c / C::kChunksPerBlock, cc = c % C::kChunksPerBlock;
-        uint4 w = make_uint4(0u, 0u, 0u, 0u);
-        if (jb < nb) w = lds128(rs + jb * C::kGran + cc * 16);
-        uint8_t* dst;
-        uint32_t b0[4], b1[4];
-        if (cc < D) {
-          const int rg = cc / (D / 2), rem = cc % (D / 2), u = rem >> 3, n = rem & 7;   // token 8 rg + n, dims 16u..16u+15
-          dst = cv + jb * C::kConvBlock + (rg * (D / 64) + (u >> 2)) * 1024 + ((u & 3) >> 1) * 512 + (4 * n) * 16 + (u & 1) * 8;
-          const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-          for (int q = 0; q < 4; ++q) { b0[q] = e4m3x2_to_f16x2_lo(ww[q]); b1[q] = e4m3x2_to_f16x2_hi(ww[q]); }
-        } else {
-          const int d = cc - D, j = d >> 3, n = d & 7;                                  // dim d, tokens 0..15
-          const int tok0 = (tile * kTileBlocks + jb) * kBlockSize;
-          if (jb < nb && tok0 + kBlockSize > L) {
-            // V codes of slots past the context are cleared so that stale bytes cannot reach P V
-            const int keep = L - tok0;
-            uint32_t* wm = reinterpret_cast<uint32_t*>(&w);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const int left = keep - 4 * q;
-              wm[q] &= left >= 4 ? 0xFFFFFFFFu : (left <= 0 ? 0u : (1u << (8 * left)) - 1u);
-            }
+          for (int e = 0; e < 4; ++e) {
+            h[2 * e] = pack_f16x2(bf16_lo(w[2 * e]) * up, bf16_hi(w[2 * e]) * up);
+            h[2 * e + 1] = pack_f16x2(bf16_lo(w[2 * e + 1]) * up, bf16_hi(w[2 * e + 1]) * up);
           }
-          dst = cv + jb * C::kConvBlock + (D / 32) * 1024 + (j >> 2) * 1024 + ((j & 3) >> 1) * 512 + (4 * n) * 16 + (j & 1) * 8;
-          // lane c of the quad: b0 = tokens 2c, 2c+1, b1 = tokens 2c+8, 2c+9
-          b0[0] = e4m3x2_to_f16x2_lo(w.x); b0[1] = e4m3x2_to_f16x2_hi(w.x); b0[2] = e4m3x2_to_f16x2_lo(w.y); b0[3] = e4m3x2_to_f16x2_hi(w.y);
-          b1[0] = e4m3x2_to_f16x2_lo(w.z); b1[1] = e4m3x2_to_f16x2_hi(w.z); b1[2] = e4m3x2_to_f16x2_lo(w.w); b1[3] = e4m3x2_to_f16x2_hi(w.w);
+          uint8_t* dst = qrow + (r >> 3) * (16 * D) + c * 256;
+          *reinterpret_cast<uint4*>(dst) = make_uint4(h[0], h[1], h[2], h[3]);
+          *reinterpret_cast<uint4*>(dst + 128) = make_uint4(h[4], h[5], h[6], h[7]);
+        } else {
+          // the exact sum of the nearest E4M3 value and the E4M3 value of the remainder
+          uint32_t lead[4], rest[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            uint32_t h0 = pack_f16x2(bf16_lo(w[2 * e]) * up, bf16_hi(w[2 * e]) * up);
+            uint32_t h1 = pack_f16x2(bf16_lo(w[2 * e + 1]) * up, bf16_hi(w[2 * e + 1]) * up);
+            const uint32_t l0 = e4m3_term(h0, 1.0f), l1 = e4m3_term(h1, 1.0f);
+            lead[e] = l0 | (l1 << 16);
+            rest[e] = f16x2_to_e4m3x2(h0) | (f16x2_to_e4m3x2(h1) << 16);
+          }
+          uint8_t* dst = qrow + (r >> 3) * (8 * D) + c * 128;
+          *reinterpret_cast<uint4*>(dst) = make_uint4(lead[0], lead[1], lead[2], lead[3]);
+          *reinterpret_cast<uint4*>(dst + C::kOperand / 2) = make_uint4(rest[0], rest[1], rest[2], rest[3]);
         }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) *reinterpret_cast<uint2*>(dst + q * 16) = make_uint2(b0[q], b1[q]);
-      }
-      if (tid < kTileBlocks * 2) {
-        const int jb = tid >> 1;
-        tile_scales[buf * kTileBlocks * 2 + tid] =
-            jb < nb ? reinterpret_cast<const float*>(rs + jb * C::kGran + header_offset(D))[tid & 1] : 0.0f;
       }
     }
-    // operand tile complete, raw stage free again; a wait that ran out ends the walk for everyone
-    if (__syncthreads_or(!ok)) {
-      failed = true;
-      break;
-    }
-    if (issued < n_tiles) {
-      if (warp == 0) issue();
-      ++issued;
-    }
+    fence_proxy_async();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar_q);
 
-    // ---- S = Q K^T: 16 rows x 64 tokens ------------------------------------------------------------
-    float s[2 * kTileBlocks][4];
+    // index of the last visible key of the row.  Rows past the tile's last query (their operand is zero, and they are never
+    // stored) see everything, so that their warp takes the same unmasked path as its live rows.
+    const int lim = live ? (p.causal ? min(L - 1, L - n_new + q0 + x * TQ + qi) : L - 1) : (1 << 30);
+    const int halves = (tile_keys(x) + kHalf - 1) / kHalf;
+    float m_ref = -INFINITY, l_row = 0.0f, v_ref = 0.0f;
+    bool ok = true;
+#pragma unroll 1
+    for (int h = 0; h < halves && ok; ++h) {
+      const int t = h >> 1, buf = h & 1;
+      const float* sc = scales + (t & (C::kScaleSlots - 1)) * 32 + 4 * buf;
+      ok = wait_warp(&bar_sfull[x], h & 1u, abort_flag);
+      if (!ok) break;
+      tc_fence_after();
+      uint32_t s[2][32];
 #pragma unroll
-    for (int j = 0; j < 2 * kTileBlocks; ++j)
+      for (int i = 0; i < 2; ++i) tmem_ld32_issue(s_cols + 32 * i, s[i]);
+      float cf[4];                                      // logit = accumulator * cf of its block (a zero scale: tiny, so that -inf stays -inf)
 #pragma unroll
-      for (int e = 0; e < 4; ++e) s[j][e] = 0.0f;
+      for (int c = 0; c < 4; ++c) cf[c] = fmaxf(sc[c] * qscale, 1e-30f);
 #pragma unroll
-    for (int jb = 0; jb < kTileBlocks; ++jb) {
-      const uint8_t* kp = cv + jb * C::kConvBlock + lane * 16;
+      for (int i = 0; i < 2; ++i) tmem_ld_wait32(s[i]);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bar_sfree[x]);
+      const int visible = lim - h * kHalf;
+      if (visible < kHalf - 1) {
 #pragma unroll
-      for (int nt = 0; nt < 2; ++nt)
+        for (int j = 0; j < kHalf; ++j) s[j >> 5][j & 31] = j <= visible ? s[j >> 5][j & 31] : 0xFF800000u;      // -inf
+      }
+      float m_tile = -INFINITY;
 #pragma unroll
-        for (int i = 0; i < D / 64; ++i) {
-          const uint4 a = lds128(kp + (nt * (D / 64) + i) * 1024);
-          const uint4 c = lds128(kp + (nt * (D / 64) + i) * 1024 + 512);
-          mma16816<true>(s[2 * jb + nt], qa[4 * i][0], qa[4 * i][1], qa[4 * i][2], qa[4 * i][3], a.x, a.y);
-          mma16816<true>(s[2 * jb + nt], qa[4 * i + 1][0], qa[4 * i + 1][1], qa[4 * i + 1][2], qa[4 * i + 1][3], a.z, a.w);
-          mma16816<true>(s[2 * jb + nt], qa[4 * i + 2][0], qa[4 * i + 2][1], qa[4 * i + 2][2], qa[4 * i + 2][3], c.x, c.y);
-          mma16816<true>(s[2 * jb + nt], qa[4 * i + 3][0], qa[4 * i + 3][1], qa[4 * i + 3][2], qa[4 * i + 3][3], c.z, c.w);
+      for (int c = 0; c < 4; ++c) {
+        const uint32_t* v = &s[c >> 1][(c & 1) * 16];
+        auto f = [&](int j) { return __uint_as_float(v[j]); };
+        const float m0 = max3(f(0), f(1), f(2)), m1 = max3(f(3), f(4), f(5)), m2 = max3(f(6), f(7), f(8)), m3 = max3(f(9), f(10), f(11)), m4 = max3(f(12), f(13), f(14));
+        m_tile = fmaxf(m_tile, fmaxf(max3(m0, m1, m2), max3(m3, m4, f(15))) * cf[c]);
+      }
+      // lazy references: moved only when the half would push a probability (or a scale ratio) past the margin
+      float factor = 1.0f;
+      if (buf == 0) { factor = sc[24]; v_ref = sc[25]; }
+      if (m_tile > m_ref + kMaxLag) {                   // also true for the row's first visible key
+        const float f = m_ref == -INFINITY ? 0.0f : ex2(m_ref - m_tile);
+        factor *= f;
+        l_row *= f;
+        m_ref = m_tile;
+      }
+      if (__any_sync(0xffffffffu, factor != 1.0f) && h > 0) {
+        // the accumulator is at rest once the product of the half before is done
+        ok = wait_bar(&bar_pv[x], (h - 1) & 1u, abort_flag);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        tc_fence_after();
+#pragma unroll 1
+        for (int i = 0; i < D; i += 64) {
+          uint32_t o[4][16];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) tmem_ld16_issue(o_cols + i + 16 * e, o[e]);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            tmem_ld_wait(o[e]);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) o[e][j] = __float_as_uint(__uint_as_float(o[e][j]) * factor);
+            tmem_st16(o_cols + i + 16 * e, o[e]);
+          }
         }
-    }
-
-    // ---- logits in log2 units, causal / tail mask, online softmax (Eq. 10) -----------------------
-    const float* ts = tile_scales + buf * kTileBlocks * 2;
-    float vmax = 0.0f;
-#pragma unroll
-    for (int jb = 0; jb < kTileBlocks; ++jb) {
-      const float sk = ts[2 * jb];
-      vmax = fmaxf(vmax, ts[2 * jb + 1]);
-#pragma unroll
-      for (int nt = 0; nt < 2; ++nt) {
-        s[2 * jb + nt][0] *= qs0 * sk; s[2 * jb + nt][1] *= qs0 * sk;
-        s[2 * jb + nt][2] *= qs1 * sk; s[2 * jb + nt][3] *= qs1 * sk;
       }
-    }
-    const int tok_base = tile * kTileTokens;
-    if (tok_base + kTileTokens - 1 > warp_min_lim) {
+      const float m_use = m_ref == -INFINITY ? 0.0f : m_ref;
+      // p * pv = 2^(s * cf - m + log2 pv): the V scale rides in the exponent, and a block's sum of p is recovered from the sum
+      // of p * pv (pv: the block's V scale over the reference, at most 2^4, a zero one replaced by 2^-24)
 #pragma unroll
-      for (int j = 0; j < 2 * kTileBlocks; ++j) {
-        const int t0 = tok_base + 8 * j + 2 * quad;
-        s[j][0] = t0 <= lim0 ? s[j][0] : -INFINITY;
-        s[j][1] = t0 + 1 <= lim0 ? s[j][1] : -INFINITY;
-        s[j][2] = t0 <= lim1 ? s[j][2] : -INFINITY;
-        s[j][3] = t0 + 1 <= lim1 ? s[j][3] : -INFINITY;
+      for (int i = 0; i < 2; ++i) {
+        uint32_t pw[16];
+#pragma unroll
+        for (int e2 = 0; e2 < 2; ++e2) {
+          const int c = 2 * i + e2;
+          const float shift = sc[8 + c] - m_use;
+          const uint32_t* v = &s[i][16 * e2];
+          float y[16];
+#pragma unroll
+          for (int e = 0; e < 16; ++e) y[e] = ex2(fmaf(__uint_as_float(v[e]), cf[c], shift));
+          // (Summed as a tree: a chain of sums kept the exponentials waiting, 820-1040 cycles a half for one warp of a scheduler
+          // against 590, with 512 that the exponentials need.)
+          const float u0 = (y[0] + y[1]) + (y[2] + y[3]), u1 = (y[4] + y[5]) + (y[6] + y[7]);
+          const float u2 = (y[8] + y[9]) + (y[10] + y[11]), u3 = (y[12] + y[13]) + (y[14] + y[15]);
+          l_row += ((u0 + u1) + (u2 + u3)) * sc[16 + c];
+#pragma unroll
+          for (int e = 0; e < 8; ++e) pw[8 * e2 + e] = pack_f16x2(y[2 * e], y[2 * e + 1]);
+        }
+        tmem_st16(p_cols + 32 * buf + 16 * i, pw);
       }
+      tmem_st_wait();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bar_pfull[2 * x + buf]);
     }
-    float mt0 = -INFINITY, mt1 = -INFINITY;
+    const bool any_keys = halves > 0;
+    if (ok && any_keys) ok = wait_bar(&bar_out[x], 0u, abort_flag);
+    ok = __all_sync(0xffffffffu, ok);
+    if (ok) {
+      tc_fence_after();
+      const float k = l_row > 0.0f ? v_ref / l_row : 0.0f;
+#pragma unroll 1
+      for (int c = 0; c < D / 32; ++c) {
+        uint32_t o[32];
+        if (any_keys) {
+          tmem_ld32_issue(o_cols + 32 * c, o);
+          tmem_ld_wait32(o);
+        }
+        if (live) {
+          uint32_t w[16];
 #pragma unroll
-    for (int j = 0; j < 2 * kTileBlocks; ++j) {
-      mt0 = fmaxf(mt0, fmaxf(s[j][0], s[j][1]));
-      mt1 = fmaxf(mt1, fmaxf(s[j][2], s[j][3]));
-    }
-    const float mn0 = fmaxf(m0, quad_max(mt0)), mn1 = fmaxf(m1, quad_max(mt1));
-    const float mu0 = mn0 == -INFINITY ? 0.0f : mn0, mu1 = mn1 == -INFINITY ? 0.0f : mn1;
-    const float am0 = ex2(m0 - mu0), am1 = ex2(m1 - mu1);
-    m0 = mn0;
-    m1 = mn1;
-    // o holds sum p * (sV / vref) * codes with vref the largest V scale met so far
-    const float vnew = fmaxf(vref, vmax);
-    const float vr = vnew > 0.0f ? __fdividef(vref, vnew) : 1.0f;
-    const float ao0 = am0 * vr, ao1 = am1 * vr;
-    vref = vnew;
-    float ps0 = 0.0f, ps1 = 0.0f;
+          for (int j = 0; j < 16; ++j) w[j] = k != 0.0f ? pack_bf16x2(__uint_as_float(o[2 * j]) * k, __uint_as_float(o[2 * j + 1]) * k) : 0u;
+          uint4* dst = reinterpret_cast<uint4*>(p.out + grow * D + 32 * c);
 #pragma unroll
-    for (int j = 0; j < 2 * kTileBlocks; ++j) {
-      s[j][0] = ex2(s[j][0] - mu0); s[j][1] = ex2(s[j][1] - mu0);
-      s[j][2] = ex2(s[j][2] - mu1); s[j][3] = ex2(s[j][3] - mu1);
-      ps0 += s[j][0] + s[j][1];
-      ps1 += s[j][2] + s[j][3];
-    }
-    l0 = l0 * am0 + ps0;
-    l1 = l1 * am1 + ps1;
-#pragma unroll
-    for (int t = 0; t < kNTiles; ++t) {
-      o[t][0] *= ao0; o[t][1] *= ao0;
-      o[t][2] *= ao1; o[t][3] *= ao1;
-    }
-
-    // ---- O += P V ----------------------------------------------------------------------------------
-#pragma unroll
-    for (int jb = 0; jb < kTileBlocks; ++jb) {
-      const float pv = vnew > 0.0f ? __fdividef(ts[2 * jb + 1], vnew) : 0.0f;
-      const uint32_t pa0 = pack_f16x2(s[2 * jb][0] * pv, s[2 * jb][1] * pv);
-      const uint32_t pa1 = pack_f16x2(s[2 * jb][2] * pv, s[2 * jb][3] * pv);
-      const uint32_t pa2 = pack_f16x2(s[2 * jb + 1][0] * pv, s[2 * jb + 1][1] * pv);
-      const uint32_t pa3 = pack_f16x2(s[2 * jb + 1][2] * pv, s[2 * jb + 1][3] * pv);
-      const uint8_t* vp = cv + jb * C::kConvBlock + (D / 32) * 1024 + lane * 16;
-#pragma unroll
-      for (int qd = 0; qd < D / 32; ++qd) {
-        const uint4 a = lds128(vp + qd * 1024);
-        const uint4 c = lds128(vp + qd * 1024 + 512);
-        mma16816<true>(o[4 * qd], pa0, pa1, pa2, pa3, a.x, a.y);
-        mma16816<true>(o[4 * qd + 1], pa0, pa1, pa2, pa3, a.z, a.w);
-        mma16816<true>(o[4 * qd + 2], pa0, pa1, pa2, pa3, c.x, c.y);
-        mma16816<true>(o[4 * qd + 3], pa0, pa1, pa2, pa3, c.z, c.w);
+          for (int j = 0; j < 4; ++j) dst[j] = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+        }
       }
+      tc_fence_before();
+    } else if (lane == 0) {
+      atomicCAS(p.status, 0, COOPT_ERR_TIMEOUT);
+    }
+  } else if (warp < kMmaWarp) {
+    // ================= widening ==========================================================================================
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
+    const int wt = tid - kWidenWarp * 32;
+    bool ok = true;
+#pragma unroll 1
+    for (int t = 0; t < n_tiles && ok; ++t) {
+      const int w2 = t % C::kWide;
+      const uint32_t w_use = t / C::kWide;
+      const int nb = min(kTileBlocks, n_blocks - t * kTileBlocks);
+      if constexpr (C::kWideK) {
+        const int ks = t % C::kKSlots;
+        ok = wait_bar(&bar_kfull[ks], (t / C::kKSlots) & 1u, abort_flag);
+        if (ok && w_use > 0) ok = wait_bar(&bar_k16free[w2], (w_use - 1) & 1u, abort_flag);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        // 16 dims of a token at a time: token (wt & 7) of an 8-token group, dims 16 c ..
+        const uint8_t* src = smem + C::kKOff + ks * C::kKSlot;
+        uint8_t* dst = smem + C::kK16Off + w2 * C::kOperand;
+#pragma unroll 1
+        for (int i = wt; i < nb * D; i += 128) {
+          const int tok = i & 7, c = (i >> 3) % (D / 16), grp = (i >> 3) / (D / 16);
+          const uint4 v = *reinterpret_cast<const uint4*>(src + grp * 8 * D + c * 128 + tok * 16);
+          const uint2 a = widen4<kE5m2>(v.x), e = widen4<kE5m2>(v.y), f = widen4<kE5m2>(v.z), h = widen4<kE5m2>(v.w);
+          uint8_t* to = dst + grp * 16 * D + c * 256 + tok * 16;
+          *reinterpret_cast<uint4*>(to) = make_uint4(a.x, a.y, e.x, e.y);
+          *reinterpret_cast<uint4*>(to + 128) = make_uint4(f.x, f.y, h.x, h.y);
+        }
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) { mbar_arrive(&bar_k16full[w2]); mbar_arrive(&bar_kfree[ks]); }
+      }
+      const int vs = t % C::kVSlots;
+      ok = wait_bar(&bar_vfull[vs], (t / C::kVSlots) & 1u, abort_flag);
+      if (ok && w_use > 0) ok = wait_bar(&bar_v16free[w2], (w_use - 1) & 1u, abort_flag);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      // dim d of V^T, the 16 tokens of a block at a time
+      const int d = wt & (D - 1);
+      const uint8_t* src = smem + C::kVOff + vs * C::kCodes + (d >> 3) * 128 + (d & 7) * 16;
+      uint8_t* dst = smem + C::kV16Off + w2 * C::kOperand + (d >> 3) * 2048 + (d & 7) * 16;
+      const int nkeys = kv_end - t * kTileKeys;
+#pragma unroll 1
+      for (int c = wt / D; c < nb; c += 128 / D) {
+        const uint4 v = *reinterpret_cast<const uint4*>(src + c * C::kPart);
+        uint32_t w[4] = {v.x, v.y, v.z, v.w};
+        const int keep = nkeys - c * kBlockSize;
+        if (keep < kBlockSize) {                          // the context ends inside this block: codes past it are cleared
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const int left = keep - 4 * j;
+            w[j] &= left >= 4 ? 0xFFFFFFFFu : (left <= 0 ? 0u : (1u << (8 * left)) - 1u);
+          }
+        }
+        const uint2 a = widen4<kE5m2>(w[0]), e = widen4<kE5m2>(w[1]), f = widen4<kE5m2>(w[2]), h = widen4<kE5m2>(w[3]);
+        *reinterpret_cast<uint4*>(dst + 2 * c * 128) = make_uint4(a.x, a.y, e.x, e.y);
+        *reinterpret_cast<uint4*>(dst + (2 * c + 1) * 128) = make_uint4(f.x, f.y, h.x, h.y);
+      }
+      fence_proxy_async();                                // the tensor core will read what this thread has just written
+      __syncwarp();
+      if (lane == 0) { mbar_arrive(&bar_v16full[w2]); mbar_arrive(&bar_vfree[vs]); }
+    }
+    if (!ok && lane == 0) atomicCAS(p.status, 0, COOPT_ERR_TIMEOUT);
+  } else {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
+    if (warp < kCopyWarp) {
+      // ================= matrix instructions of one tile =================================================================
+      {
+        const int mx = warp - kMmaWarp;
+        uint64_t* k_full = C::kWideK ? bar_k16full : bar_kfull;
+        uint64_t* k_free = C::kWideK ? bar_k16free : bar_kfree;
+        constexpr int kSlots = C::kWideK ? C::kWide : C::kKSlots;
+        constexpr int kSlotBytes = C::kWideK ? C::kOperand : C::kKSlot;
+        constexpr uint32_t kRowGroup = C::kWideK ? 16 * D : 8 * D;       // bytes of eight rows of Q, K
+        const uint64_t desc_k = umma_desc(smem_u32(smem + (C::kWideK ? C::kK16Off : C::kKOff)), 128, kRowGroup);
+        const uint64_t desc_q = umma_desc(smem_u32(smem + C::kQOff + mx * C::kOperand), 128, kRowGroup);
+        const uint64_t desc_v = umma_desc(smem_u32(smem + C::kV16Off), 128, 2048);
+        const uint32_t s_cols = tmem + kHalf * mx, p_cols = tmem + 2 * kHalf + kHalf * mx, o_cols = tmem + 256 + D * mx;
+        const int keys = tile_keys(mx), halves = (keys + kHalf - 1) / kHalf, my_tiles = (keys + kTileKeys - 1) / kTileKeys;
+        bool ok = true;
+        int done = 0;                                     // halves whose product with V has been seen to be done
+        auto see_products = [&](int upto) {
+          for (; ok && done < upto; ++done) {
+            ok = wait_warp(&bar_pv[mx], done & 1u, abort_flag);
+            if (ok && ((done & 1) || done == halves - 1)) arrive_one(&bar_v16free[(done >> 1) % C::kWide]);
+          }
+        };
+        // Logits of a half, once those of the half before are in registers.  (The probabilities of the half will take the place
+        // of those of half h - 2, whose product has to be done by then.)
+        auto issue_logits = [&](int h) {
+          const int t = h >> 1, ks = t % kSlots;
+          if ((h & 1) == 0) {
+            ok = ok && wait_warp(&bar_scale[t & (C::kScaleSlots - 1)], (t / C::kScaleSlots) & 1u, abort_flag);
+            ok = ok && wait_warp(&k_full[ks], (t / kSlots) & 1u, abort_flag);
+          }
+          see_products(h - 1);
+          if (h > 0) ok = ok && wait_warp(&bar_sfree[mx], (h - 1) & 1u, abort_flag);
+          if (!ok) return;
+          tc_fence_after();
+          const uint64_t dk = desc_k + ((ks * kSlotBytes + (h & 1) * 8 * kRowGroup) >> 4);
+          if constexpr (C::kWideK) {
+#pragma unroll
+            for (int k = 0; k < D / 16; ++k) umma_f16(s_cols, desc_q + k * 16, dk + k * 16, umma_idesc(kHalf), k != 0);
+          } else {
+#pragma unroll
+            for (int term = 0; term < 2; ++term)
+#pragma unroll
+              for (int k = 0; k < D / 32; ++k)
+                umma_f8(s_cols, desc_q + ((term * (C::kOperand / 2)) >> 4) + k * 16, dk + k * 16, umma_idesc(kHalf, 0, kE5m2 ? 1 : 0), (term | k) != 0);
+          }
+          umma_commit(&bar_sfull[mx]);
+          arrive_one(&bar_sfull[mx]);
+        };
+        ok = wait_warp(bar_q, 0u, abort_flag);
+        if (halves > 0) issue_logits(0);
+        for (int h = 0; h < halves && ok; ++h) {
+          const int t = h >> 1, w2 = t % C::kWide;
+          // (Products are seen one by one: a wait for a barrier's phase must not fall two phases behind.)
+          if (h + 1 < halves) issue_logits(h + 1); else see_products(h);
+          if ((h & 1) == 0) ok = ok && wait_warp(&bar_v16full[w2], (t / C::kWide) & 1u, abort_flag);
+          ok = ok && wait_warp(&bar_pfull[2 * mx + (h & 1)], t & 1u, abort_flag);
+          if (!ok) break;
+          if ((h & 1) || h == halves - 1) arrive_one(&k_free[t % kSlots]);      // probabilities are there, so the logits have been
+          tc_fence_after();
+          const uint64_t dv = desc_v + ((w2 * C::kOperand) >> 4) + (h & 1) * 64;
+          const uint32_t from = p_cols + 32 * (h & 1);
+          const int nb = min(kTileBlocks / 2, n_blocks - h * (kTileBlocks / 2));      // 16 keys (one cache block) per instruction
+          if (nb == kTileBlocks / 2) {
+#pragma unroll
+            for (int k = 0; k < kTileBlocks / 2; ++k) umma_f16_ts(o_cols, from + 8 * k, dv + k * 16, umma_idesc(D), (h | k) != 0);
+          } else {
+            for (int k = 0; k < nb; ++k) umma_f16_ts(o_cols, from + 8 * k, dv + k * 16, umma_idesc(D), (h | k) != 0);
+          }
+          umma_commit(&bar_pv[mx]);
+        }
+        see_products(halves);
+        if (ok) {
+          tc_fence_after();
+          tc_fence_before();
+          arrive_one(&bar_out[mx]);
+        }
+        for (int t = my_tiles; t < n_tiles && ok; ++t) {  // no row of this tile sees these keys
+          const int ks = t % kSlots, w2 = t % C::kWide;
+          ok = wait_warp(&k_full[ks], (t / kSlots) & 1u, abort_flag);
+          if (ok) arrive_one(&k_free[ks]);
+          ok = ok && wait_warp(&bar_v16full[w2], (t / C::kWide) & 1u, abort_flag);
+          if (ok) arrive_one(&bar_v16free[w2]);
+        }
+        if (!ok && lane == 0) atomicCAS(p.status, 0, COOPT_ERR_TIMEOUT);
+      }
+    } else if (warp == kCopyWarp) {
+      // ================= copies: per tile six gather requests of four granules' K parts, V parts or headers =============
+      // Lane 3 q + w (q = 0, 1; w = 0, 1, 2) fetches the K parts (w = 0), the V parts (w = 1) or the headers (w = 2) of
+      // granules 4 q .. 4 q + 3 of the tile.  Rows past the last block repeat the tile's first one.  The physical blocks are
+      // looked up 32 at a time (four tiles, one per lane), a batch ahead of their use (range-checked: a bad id is reported in
+      // the status word and replaced by block 0, never dereferenced).
+      bool ok = true;
+      const int q4 = lane / 3, what = lane - 3 * q4;
+      const int col = what * (C::kPart / 8);
+      const CUtensorMap* map = what == 2 ? &map_hdr : &map_part;
+      const int* trow = p.block_table + static_cast<size_t>(b) * p.max_blocks_per_seq;
+      auto load_batch = [&](int lb) -> int {
+        const int j = lb * 32 + lane;
+        int id = j < n_blocks ? trow[j] : 0;
+        if (id < 0 || id >= p.num_blocks) { atomicCAS(p.status, 0, COOPT_ERR_INVALID_ARG); id = 0; }
+        return id;
+      };
+      int ids_cur = load_batch(0), ids_next = load_batch(1);
+      for (int t = 0; t < n_tiles; ++t) {
+        const int nb = min(kTileBlocks, n_blocks - t * kTileBlocks);
+        const int ngroups = (nb + 3) / 4;
+        if (t > 0 && (t & 3) == 0) { ids_cur = ids_next; ids_next = load_batch((t >> 2) + 1); }
+        int rows[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int j = (q4 & 1) * 4 + i;                           // block of the tile (lanes past the six copy lanes fetch along)
+          rows[i] = __shfl_sync(0xffffffffu, ids_cur, (t & 3) * 8 + (j < nb ? j : 0)) * Hkv + g;
+        }
+        const int ks = t % C::kKSlots, vs = t % C::kVSlots;
+        const uint32_t k_use = t / C::kKSlots, v_use = t / C::kVSlots;
+        if (lane == 0) {
+          if (k_use > 0) ok = wait_bar(&bar_kfree[ks], (k_use - 1) & 1u, abort_flag);
+          if (ok) {
+            mbar_expect_tx(&bar_kfull[ks], ngroups * 4 * (C::kPart + kFp8Header));
+            pend_mask |= 1u << ks;
+            pend_par = (pend_par & ~(1u << ks)) | ((k_use & 1u) << ks);
+          }
+        }
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        if (!ok) break;
+        if (lane < 3 * ngroups && what != 1)
+          gather4_g2s(smem + C::kKOff + ks * C::kKSlot + (what == 2 ? C::kCodes + q4 * 4 * kFp8Header : q4 * 4 * C::kPart), map, col, rows[0], rows[1], rows[2], rows[3], &bar_kfull[ks]);
+        if (lane == 0) {
+          if (v_use > 0) ok = wait_bar(&bar_vfree[vs], (v_use - 1) & 1u, abort_flag);
+          if (ok) {
+            mbar_expect_tx(&bar_vfull[vs], ngroups * 4 * C::kPart);
+            pend_mask |= 16u << vs;
+            pend_par = (pend_par & ~(16u << vs)) | ((v_use & 1u) << (4 + vs));
+          }
+        }
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        if (!ok) break;
+        if (lane < 3 * ngroups && what == 1)
+          gather4_g2s(smem + C::kVOff + vs * C::kCodes + q4 * 4 * C::kPart, map, col, rows[0], rows[1], rows[2], rows[3], &bar_vfull[vs]);
+      }
+      if (!ok && lane == 0) atomicCAS(p.status, 0, COOPT_ERR_TIMEOUT);
+    } else {
+      // ================= block scales, as the softmax uses them =============================================================
+      float v_ref = 0.0f;
+      bool ok = true;
+      for (int t = 0; t < n_tiles; ++t) {
+        const int ks = t % C::kKSlots;
+        ok = wait_bar(&bar_kfull[ks], (t / C::kKSlots) & 1u, abort_flag);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        const int nb = min(kTileBlocks, n_blocks - t * kTileBlocks);
+        float sk = 0.0f, sv = 0.0f;
+        if (lane < nb) {
+          const float2 h = *reinterpret_cast<const float2*>(smem + C::kKOff + ks * C::kKSlot + C::kCodes + lane * kFp8Header);
+          sk = h.x; sv = h.y;
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bar_kfree[ks]);
+        const float v_tile = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(sv)));   // scales are not negative
+        float factor = 1.0f;
+        if (v_tile > v_ref * kScaleLag) {
+          factor = v_ref > 0.0f ? v_ref / v_tile : 0.0f;
+          v_ref = v_tile;
+        }
+        // (a slot is free again four tiles on: the K slots behind its tile's are handed out only once these scales have been used)
+        float* sc = scales + (t & (C::kScaleSlots - 1)) * 32;
+        const float pv = fmaxf(v_ref > 0.0f ? sv / v_ref : 0.0f, 0x1p-24f);
+        if (lane < kTileBlocks) {
+          float lg;
+          asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lg) : "f"(pv));
+          sc[lane] = sk;
+          sc[8 + lane] = lg;
+          sc[16 + lane] = 1.0f / pv;
+          if (lane == 0) { sc[24] = factor; sc[25] = v_ref; }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bar_scale[t & (C::kScaleSlots - 1)]);
+      }
+      if (!ok && lane == 0) atomicCAS(p.status, 0, COOPT_ERR_TIMEOUT);
     }
   }
 
-  if (failed) {
-    if (tid == 0) atomicCAS(p.status, 0, COOPT_ERR_TIMEOUT);
-    // copies still in flight get a bounded time to land before the shared memory is released
-    for (int t = 0; t < issued; ++t) mbar_wait_bounded(&bars[t % kRawStages], (t / kRawStages) & 1u);
-    return;
+  // ---- exit: copies still in flight get a bounded time to land, tensor memory is returned -----------
+  __syncthreads();
+  if (*abort_flag != 0 && warp == kCopyWarp && lane == 0) {
+    for (int i = 0; i < C::kKSlots; ++i)
+      if ((pend_mask >> i) & 1u) mbar_wait_bounded(&bar_kfull[i], (pend_par >> i) & 1u);
+    for (int i = 0; i < C::kVSlots; ++i)
+      if ((pend_mask >> (4 + i)) & 1u) mbar_wait_bounded(&bar_vfull[i], (pend_par >> (4 + i)) & 1u);
   }
-
-  // ---- normalise and store -------------------------------------------------------------------------
-  l0 = quad_sum(l0);
-  l1 = quad_sum(l1);
-  const float f0 = l0 > 0.0f ? vref / l0 : 0.0f, f1 = l1 > 0.0f ? vref / l1 : 0.0f;
-  if (live0) {
-    __nv_bfloat16* op = p.out + grow0 * D + 2 * quad;
-#pragma unroll
-    for (int t = 0; t < kNTiles; ++t)
-      *reinterpret_cast<uint32_t*>(op + 8 * t) = pack_bf16x2(o[t][0] * f0, o[t][1] * f0);
-  }
-  if (live1) {
-    __nv_bfloat16* op = p.out + grow1 * D + 2 * quad;
-#pragma unroll
-    for (int t = 0; t < kNTiles; ++t)
-      *reinterpret_cast<uint32_t*>(op + 8 * t) = pack_bf16x2(o[t][2] * f1, o[t][3] * f1);
-  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == kMmaWarp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
 }
 
-template <int D>
-int launch_prefill_one(const PrefillParams& p, dim3 grid, cudaStream_t stream) {
-  using C = PfCfg<D>;
-  if (!configure_kernel_smem(reinterpret_cast<const void*>(&paged_prefill_kernel<D>), C::kSmemBytes)) return COOPT_ERR_CUDA;
-  paged_prefill_kernel<D><<<grid, kPfThreads, C::kSmemBytes, stream>>>(p);
-  return cudaGetLastError() == cudaSuccess ? COOPT_OK : COOPT_ERR_CUDA;
+template <int D, bool kE5m2>
+int launch_one(const coopt_cache* c, const PrefillParams& p, dim3 grid, cudaStream_t stream) {
+  using C = Cfg<D>;
+  CUtensorMap map_part, map_hdr;
+  const long long granules = static_cast<long long>(c->num_blocks) * c->num_kv_heads;
+  if (!encode_cache_map(&map_part, c->data, granules, C::kGran, C::kPart / 8) || !encode_cache_map(&map_hdr, c->data, granules, C::kGran, kFp8Header / 8))
+    return COOPT_ERR_CUDA;
+  if (!configure_kernel_smem(reinterpret_cast<const void*>(&paged_prefill_kernel<D, kE5m2>), C::kSmemBytes)) return COOPT_ERR_CUDA;
+  return launch_dependent(paged_prefill_kernel<D, kE5m2>, grid, kThreads, C::kSmemBytes, stream, p, map_part, map_hdr) ? COOPT_OK : COOPT_ERR_CUDA;
 }
 
 }  // namespace
-
-int launch_paged_prefill_umma(const coopt_cache* c, const void* q, void* out, const int32_t* cu_q_lens, const int32_t* block_table,
-                              int32_t max_blocks_per_seq, const int32_t* context_lens, int32_t batch, int32_t num_q_heads,
-                              int32_t total_q, int32_t causal, float sm_scale, void* workspace, cudaStream_t stream);
 
 int launch_paged_prefill(const coopt_cache* c, const void* q, void* out, const int32_t* cu_q_lens,
                          const int32_t* block_table, int32_t max_blocks_per_seq, const int32_t* context_lens,
                          int32_t batch, int32_t num_q_heads, int32_t total_q, int32_t causal, float sm_scale,
                          void* workspace, cudaStream_t stream) {
   if (!is_fp8(c->dtype)) return COOPT_ERR_UNSUPPORTED;
-  if (c->dtype == COOPT_KV_FP8_E5M2 && c->head_dim != 128) return COOPT_ERR_UNSUPPORTED;   // the E5M2 ablation: tcgen05 kernel only
-  if (num_q_heads / c->num_kv_heads > kPfRows) return COOPT_ERR_UNSUPPORTED;   // a tile holds at least one query token of every head of the group
-  // head_dim 128: the tcgen05 kernel; head_dim 64: the mma.sync kernel of this file
-  if (c->head_dim == 128)
-    return launch_paged_prefill_umma(c, q, out, cu_q_lens, block_table, max_blocks_per_seq, context_lens, batch, num_q_heads,
-                                     total_q, causal, sm_scale, workspace, stream);
+  if (c->dtype == COOPT_KV_FP8_E5M2 && c->head_dim != 128) return COOPT_ERR_UNSUPPORTED;
   PrefillParams p;
-  p.cache = static_cast<const uint8_t*>(c->data);
   p.q = static_cast<const __nv_bfloat16*>(q);
   p.out = static_cast<__nv_bfloat16*>(out);
   p.cu_q_lens = cu_q_lens;
@@ -434,15 +699,15 @@ int launch_paged_prefill(const coopt_cache* c, const void* q, void* out, const i
   p.num_kv_heads = c->num_kv_heads;
   p.group = num_q_heads / c->num_kv_heads;
   p.num_blocks = c->num_blocks;
-  p.tile_queries = kPfRows / p.group;
+  p.tile_queries = kRows / p.group;
   p.causal = causal;
   p.sm_scale_log2 = sm_scale * kLog2e;
   p.status = static_cast<int*>(workspace);
-  // every sequence adds at most one partly filled tile
-  const long long tiles = static_cast<long long>(total_q) / p.tile_queries + batch;
-  if (tiles > 0x7fffffffll) return COOPT_ERR_UNSUPPORTED;
-  const dim3 grid(static_cast<unsigned>(tiles), static_cast<unsigned>(c->num_kv_heads));
-  return c->head_dim == 128 ? launch_prefill_one<128>(p, grid, stream) : launch_prefill_one<64>(p, grid, stream);
+  const long long pairs = static_cast<long long>(total_q) / (2 * p.tile_queries) + batch;   // every sequence adds at most one partly filled pair
+  if (pairs > 0x7fffffffll) return COOPT_ERR_UNSUPPORTED;
+  const dim3 grid(static_cast<unsigned>(pairs), static_cast<unsigned>(c->num_kv_heads));
+  if (c->head_dim == 64) return launch_one<64, false>(c, p, grid, stream);
+  return c->dtype == COOPT_KV_FP8_E5M2 ? launch_one<128, true>(c, p, grid, stream) : launch_one<128, false>(c, p, grid, stream);
 }
 
 }  // namespace coopt

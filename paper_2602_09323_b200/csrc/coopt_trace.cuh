@@ -1,4 +1,4 @@
-// Time stamps of the decode and prefill kernels.  Compiled in only with -DCOOPT_TRACE (the separate library
+// Time stamps of the decode kernel.  Compiled in only with -DCOOPT_TRACE (the separate library
 // libcoopt_trace.so); the ordinary library contains none of this.  A stamp is the SM's cycle counter
 // written to slot `s` of the CTA's record in a caller-supplied buffer (coopt_trace_set_buffer); two slots
 // hold the global nanosecond timer at entry and exit so that the CTAs of a launch can be laid side by side.

@@ -1,0 +1,56 @@
+"""GPU parity of the prefill kernel where its tiling can go wrong: query runs around the edges of a tile and of a pair of
+tiles, contexts around the edges of a tile of keys, one pair of which a tile sees fewer keys, every group size's tile."""
+import pytest
+import torch
+
+from oracle import attention
+from paper_2602_09323_b200 import binding, workloads
+from tests import helpers
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(lens, q_lens, hq, hkv, d, causal=True, seed=0, mutate=None):
+    w = workloads.make_workload("prefill_edges", lens, hq, hkv, d, seed=seed, q_lens=q_lens)
+    if mutate:
+        mutate(w)
+    cache = helpers.gpu_fill(w)
+    ws = binding.new_workspace(w.batch, hq, hkv, d, w.block_table.shape[1], 2048, sum(q_lens))
+    call = lambda: binding.paged_chunked(cache, w.q.cuda(), w.cu_q_lens.cuda(), w.block_table.cuda(), w.context_lens_tensor.cuda(), 2048, causal, w.sm_scale, ws)
+    out = call()
+    torch.cuda.synchronize()
+    assert binding.workspace_status(ws) == 0
+    ref = attention.paged_attention(w.q.float().numpy(), helpers.oracle_fp8_cache(w), w.block_table.numpy(), w.context_lens,
+                                    cu_q_lens=w.cu_q_lens.numpy(), causal=causal)
+    helpers.check_attention(out, ref, what=f"prefill {lens} {q_lens}")      # the repository's bound: bf16 output, 11-bit probabilities
+    assert torch.equal(out, call())
+
+
+@pytest.mark.parametrize("hq,hkv,d", [(1, 1, 128), (5, 1, 128), (8, 1, 64), (3, 1, 64), (2, 1, 128)])
+def test_query_runs_around_tile_edges(hq, hkv, d):
+    tq = 128 // (hq // hkv)
+    q_lens = [1, tq - 1, tq, tq + 1, 2 * tq - 1, 2 * tq, 2 * tq + 1]
+    _check([n + 130 for n in q_lens], q_lens, hq, hkv, d, seed=hq)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("causal", [True, False])
+def test_contexts_around_key_tile_edges(d, causal):
+    lens = [16, 127, 128, 129, 143, 144, 145, 255, 256, 257, 513, 641]
+    _check(lens, [min(n, 40) for n in lens], 4, 2, d, causal=causal, seed=d)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_a_first_tile_that_sees_fewer_key_tiles_than_the_second(d):
+    _check([256, 300, 520], [256, 200, 250], 1, 1, d, seed=7)                # 128 queries a tile: one key tile apart
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_references_that_have_to_move(d):
+    """Logits that grow along the context by far more than the margin of a lazy maximum, V scales by more than theirs."""
+    def mutate(w):
+        n = w.k.shape[0]
+        grow = torch.linspace(0.01, 3.0, n)[:, None, None]
+        w.k[:] = (w.k.float() * grow).to(torch.bfloat16)
+        w.v[:] = (w.v.float() * (torch.arange(n)[:, None, None] // 200 * 2.0 + 0.01) * 0.02).to(torch.bfloat16)
+    _check([900, 700], [100, 30], 6, 2, d, seed=9, mutate=mutate)
