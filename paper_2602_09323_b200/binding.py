@@ -127,12 +127,19 @@ def _check(status: int, what: str) -> None:
         raise CooptError(status, what)
 
 
-def _stream() -> ctypes.c_void_p:
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+# A call of a small problem is as long as its way through this file (10 us for a kernel of 2), so what every call does is
+# kept cheap: the current stream's handle without a Stream object around it, addresses as plain integers (the argument
+# types convert them), dtypes compared by identity.
+_BF16, _I32, _I64 = torch.bfloat16, torch.int32, torch.int64
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
-
-def _ptr(t: torch.Tensor) -> ctypes.c_void_p:
-    return ctypes.c_void_p(t.data_ptr())
+if _current_device is not None and _raw_stream is not None:
+    def _stream() -> int:
+        return _raw_stream(_current_device())
+else:
+    def _stream() -> int:
+        return torch.cuda.current_stream().cuda_stream
 
 
 class Cache:
@@ -148,9 +155,10 @@ class Cache:
         self.num_blocks, self.num_kv_heads, self.head_dim, self.dtype = num_blocks, num_kv_heads, head_dim, dtype
         self.granule_bytes = lib.coopt_granule_bytes(head_dim, dtype)
         self.desc = coopt_cache(self.data.data_ptr(), num_blocks, num_kv_heads, head_dim, BLOCK_SIZE, dtype)
+        self._ref = ctypes.byref(self.desc)
 
     def ref(self):
-        return ctypes.byref(self.desc)
+        return self._ref
 
 
 def cache_offset(cache: Cache, block: int, kv_head: int, which: int, token: int, dim: int) -> int:
@@ -163,12 +171,15 @@ def scale_offset(cache: Cache, block: int, kv_head: int, which: int) -> int:
 
 def kv_write(cache: Cache, k: torch.Tensor, v: torch.Tensor, slot_mapping: torch.Tensor) -> None:
     """coopt_kv_write: k, v bf16 [T, Hkv, D] (token stride taken from the tensor), slots int64 [T]."""
-    assert k.dtype == torch.bfloat16 and v.dtype == torch.bfloat16 and slot_mapping.dtype == torch.int64
+    assert k.dtype is _BF16 and v.dtype is _BF16 and slot_mapping.dtype is _I64
     assert k.is_cuda and v.is_cuda and slot_mapping.is_cuda and slot_mapping.is_contiguous()
-    assert k.shape == v.shape and k.stride() == v.stride() and k.stride(2) == 1 and k.stride(1) == k.shape[2]
-    st = load_library().coopt_kv_write(cache.ref(), _ptr(k), _ptr(v), k.stride(0) if k.shape[0] > 1 else k.shape[1] * k.shape[2],
-                                       _ptr(slot_mapping), k.shape[0], _stream())
-    _check(st, "coopt_kv_write")
+    stride = k.stride()
+    tokens, heads, dim = k.shape
+    assert v.shape == k.shape and stride == v.stride() and stride[2] == 1 and stride[1] == dim
+    st = load_library().coopt_kv_write(cache.ref(), k.data_ptr(), v.data_ptr(), stride[0] if tokens > 1 else heads * dim,
+                                       slot_mapping.data_ptr(), tokens, _stream())
+    if st != 0:
+        _check(st, "coopt_kv_write")
 
 
 def workspace_bytes(batch: int, num_q_heads: int, num_kv_heads: int, head_dim: int, max_blocks_per_seq: int,
@@ -178,7 +189,7 @@ def workspace_bytes(batch: int, num_q_heads: int, num_kv_heads: int, head_dim: i
 
 
 def workspace_init(workspace: torch.Tensor) -> None:
-    _check(load_library().coopt_workspace_init(_ptr(workspace), workspace.numel(), _stream()), "coopt_workspace_init")
+    _check(load_library().coopt_workspace_init(workspace.data_ptr(), workspace.numel(), _stream()), "coopt_workspace_init")
 
 
 def new_workspace(batch: int, num_q_heads: int, num_kv_heads: int, head_dim: int, max_blocks_per_seq: int,
@@ -198,13 +209,14 @@ def workspace_status(workspace: torch.Tensor) -> int:
 def paged_decode(cache: Cache, q: torch.Tensor, block_table: torch.Tensor, context_lens: torch.Tensor,
                  sm_scale: float, workspace: torch.Tensor, out: Optional[torch.Tensor] = None) -> torch.Tensor:
     """coopt_paged_decode: q bf16 [B, Hq, D] -> out bf16 [B, Hq, D]."""
-    assert q.dtype == torch.bfloat16 and q.is_contiguous() and q.is_cuda
-    assert block_table.dtype == torch.int32 and block_table.is_contiguous() and context_lens.dtype == torch.int32
+    assert q.dtype is _BF16 and q.is_contiguous() and q.is_cuda
+    assert block_table.dtype is _I32 and block_table.is_contiguous() and context_lens.dtype is _I32
     if out is None:
         out = torch.empty_like(q)
-    st = load_library().coopt_paged_decode(cache.ref(), _ptr(q), _ptr(out), _ptr(block_table), block_table.shape[1],
-                                           _ptr(context_lens), q.shape[0], q.shape[1], float(sm_scale),
-                                           _ptr(workspace), workspace.numel(), _stream())
+    batch, heads, _ = q.shape
+    st = load_library().coopt_paged_decode(cache.ref(), q.data_ptr(), out.data_ptr(), block_table.data_ptr(), block_table.shape[1],
+                                           context_lens.data_ptr(), batch, heads, float(sm_scale),
+                                           workspace.data_ptr(), workspace.numel(), _stream())
     _check(st, "coopt_paged_decode")
     return out
 
@@ -213,14 +225,14 @@ def decode_step(cache: Cache, k_new: torch.Tensor, v_new: torch.Tensor, slot_map
                 block_table: torch.Tensor, context_lens: torch.Tensor, sm_scale: float, workspace: torch.Tensor,
                 out: Optional[torch.Tensor] = None) -> torch.Tensor:
     """coopt_decode_step: the new token of every sequence written, then decode attention, as one call."""
-    assert q.dtype == torch.bfloat16 and q.is_contiguous() and block_table.dtype == torch.int32 and block_table.is_contiguous()
-    assert k_new.dtype == torch.bfloat16 and v_new.dtype == torch.bfloat16 and k_new.is_contiguous() and v_new.is_contiguous()
-    assert slot_mapping.dtype == torch.int64 and context_lens.dtype == torch.int32
+    assert q.dtype is _BF16 and q.is_contiguous() and block_table.dtype is _I32 and block_table.is_contiguous()
+    assert k_new.dtype is _BF16 and v_new.dtype is _BF16 and k_new.is_contiguous() and v_new.is_contiguous()
+    assert slot_mapping.dtype is _I64 and context_lens.dtype is _I32
     if out is None:
         out = torch.empty_like(q)
-    st = load_library().coopt_decode_step(cache.ref(), _ptr(k_new), _ptr(v_new), k_new.shape[1] * k_new.shape[2], _ptr(slot_mapping),
-                                          _ptr(q), _ptr(out), _ptr(block_table), block_table.shape[1], _ptr(context_lens),
-                                          q.shape[0], q.shape[1], float(sm_scale), _ptr(workspace), workspace.numel(), _stream())
+    st = load_library().coopt_decode_step(cache.ref(), k_new.data_ptr(), v_new.data_ptr(), k_new.shape[1] * k_new.shape[2], slot_mapping.data_ptr(),
+                                          q.data_ptr(), out.data_ptr(), block_table.data_ptr(), block_table.shape[1], context_lens.data_ptr(),
+                                          q.shape[0], q.shape[1], float(sm_scale), workspace.data_ptr(), workspace.numel(), _stream())
     _check(st, "coopt_decode_step")
     return out
 
@@ -232,13 +244,13 @@ def plan_bytes(batch: int, num_kv_heads: int, max_blocks_per_seq: int, chunk_siz
 def decode_plan(block_table: torch.Tensor, context_lens: torch.Tensor, num_kv_heads: int, num_blocks: int,
                 chunk_size: int = 0, plan: Optional[torch.Tensor] = None) -> torch.Tensor:
     """coopt_decode_plan: the step's work decomposition, into ``plan`` (allocated here if not given)."""
-    assert block_table.dtype == torch.int32 and block_table.is_contiguous() and block_table.is_cuda
-    assert context_lens.dtype == torch.int32 and context_lens.is_cuda
+    assert block_table.dtype is _I32 and block_table.is_contiguous() and block_table.is_cuda
+    assert context_lens.dtype is _I32 and context_lens.is_cuda
     batch, width = block_table.shape
     if plan is None:
         plan = torch.empty(plan_bytes(batch, num_kv_heads, width, chunk_size), dtype=torch.uint8, device=block_table.device)
-    st = load_library().coopt_decode_plan(_ptr(block_table), width, _ptr(context_lens), batch, num_kv_heads, num_blocks,
-                                          int(chunk_size), _ptr(plan), plan.numel(), _stream())
+    st = load_library().coopt_decode_plan(block_table.data_ptr(), width, context_lens.data_ptr(), batch, num_kv_heads, num_blocks,
+                                          int(chunk_size), plan.data_ptr(), plan.numel(), _stream())
     _check(st, "coopt_decode_plan")
     return plan
 
@@ -248,19 +260,18 @@ def decode_step_planned(cache: Cache, plan: torch.Tensor, q: torch.Tensor, max_b
                         slot_mapping: Optional[torch.Tensor] = None, chunk_size: int = 0, flags: int = 0,
                         out: Optional[torch.Tensor] = None) -> torch.Tensor:
     """coopt_decode_step_planned: append (if k_new, v_new, slot_mapping are given) and attend in one launch."""
-    assert q.dtype == torch.bfloat16 and q.is_contiguous() and q.is_cuda
+    assert q.dtype is _BF16 and q.is_contiguous() and q.is_cuda
     stride = 0
     if k_new is not None:
-        assert k_new.dtype == torch.bfloat16 and v_new.dtype == torch.bfloat16 and k_new.is_contiguous() and v_new.is_contiguous()
-        assert slot_mapping.dtype == torch.int64 and slot_mapping.is_contiguous()
+        assert k_new.dtype is _BF16 and v_new.dtype is _BF16 and k_new.is_contiguous() and v_new.is_contiguous()
+        assert slot_mapping.dtype is _I64 and slot_mapping.is_contiguous()
         stride = k_new.shape[1] * k_new.shape[2]
     if out is None:
         out = torch.empty_like(q)
-    null = ctypes.c_void_p(None)
     st = load_library().coopt_decode_step_planned(
-        cache.ref(), _ptr(plan), plan.numel(), _ptr(k_new) if k_new is not None else null,
-        _ptr(v_new) if v_new is not None else null, stride, _ptr(slot_mapping) if slot_mapping is not None else null,
-        _ptr(q), _ptr(out), max_blocks_per_seq, q.shape[0], q.shape[1], int(chunk_size), float(sm_scale), _ptr(workspace),
+        cache.ref(), plan.data_ptr(), plan.numel(), k_new.data_ptr() if k_new is not None else None,
+        v_new.data_ptr() if v_new is not None else None, stride, slot_mapping.data_ptr() if slot_mapping is not None else None,
+        q.data_ptr(), out.data_ptr(), max_blocks_per_seq, q.shape[0], q.shape[1], int(chunk_size), float(sm_scale), workspace.data_ptr(),
         workspace.numel(), int(flags), _stream())
     _check(st, "coopt_decode_step_planned")
     return out
@@ -287,9 +298,9 @@ class LayerSet:
 def decode_layers(layer_set: LayerSet, block_table: torch.Tensor, context_lens: torch.Tensor, num_q_heads: int,
                   sm_scale: float, plan: torch.Tensor, workspace: torch.Tensor, flags: int = 0) -> None:
     """coopt_decode_layers: one plan, then one fused step per layer, enqueued back to back."""
-    st = load_library().coopt_decode_layers(layer_set.array, len(layer_set.array), layer_set.kv_stride, _ptr(block_table),
-                                            block_table.shape[1], _ptr(context_lens), block_table.shape[0], num_q_heads,
-                                            float(sm_scale), _ptr(plan), plan.numel(), _ptr(workspace), workspace.numel(),
+    st = load_library().coopt_decode_layers(layer_set.array, len(layer_set.array), layer_set.kv_stride, block_table.data_ptr(),
+                                            block_table.shape[1], context_lens.data_ptr(), block_table.shape[0], num_q_heads,
+                                            float(sm_scale), plan.data_ptr(), plan.numel(), workspace.data_ptr(), workspace.numel(),
                                             int(flags), _stream())
     _check(st, "coopt_decode_layers")
 
@@ -299,12 +310,12 @@ def paged_decode_static(cache: Cache, q: torch.Tensor, block_table: torch.Tensor
     """coopt_paged_decode_static: as ``paged_decode`` but the scratch memory is the fixed array inside
     the library, for callers that cannot allocate a workspace (see the header).  ``out`` is still the
     caller's; pass one in if even the output must not be allocated here."""
-    assert q.dtype == torch.bfloat16 and q.is_contiguous() and q.is_cuda
-    assert block_table.dtype == torch.int32 and block_table.is_contiguous() and context_lens.dtype == torch.int32
+    assert q.dtype is _BF16 and q.is_contiguous() and q.is_cuda
+    assert block_table.dtype is _I32 and block_table.is_contiguous() and context_lens.dtype is _I32
     if out is None:
         out = torch.empty_like(q)
-    st = load_library().coopt_paged_decode_static(cache.ref(), _ptr(q), _ptr(out), _ptr(block_table),
-                                                  block_table.shape[1], _ptr(context_lens), q.shape[0], q.shape[1],
+    st = load_library().coopt_paged_decode_static(cache.ref(), q.data_ptr(), out.data_ptr(), block_table.data_ptr(),
+                                                  block_table.shape[1], context_lens.data_ptr(), q.shape[0], q.shape[1],
                                                   float(sm_scale), _stream())
     _check(st, "coopt_paged_decode_static")
     return out
@@ -314,15 +325,15 @@ def paged_chunked(cache: Cache, q: torch.Tensor, cu_q_lens: torch.Tensor, block_
                   context_lens: torch.Tensor, chunk_size: int, causal: bool, sm_scale: float,
                   workspace: torch.Tensor, out: Optional[torch.Tensor] = None) -> torch.Tensor:
     """coopt_paged_chunked: q bf16 [total_q, Hq, D]; cu_q_lens int32 [B + 1] on the device."""
-    assert q.dtype == torch.bfloat16 and q.is_contiguous() and q.is_cuda
-    assert block_table.dtype == torch.int32 and block_table.is_contiguous()
-    assert cu_q_lens.dtype == torch.int32 and context_lens.dtype == torch.int32
+    assert q.dtype is _BF16 and q.is_contiguous() and q.is_cuda
+    assert block_table.dtype is _I32 and block_table.is_contiguous()
+    assert cu_q_lens.dtype is _I32 and context_lens.dtype is _I32
     if out is None:
         out = torch.empty_like(q)
     batch = context_lens.shape[0]
-    st = load_library().coopt_paged_chunked(cache.ref(), _ptr(q), _ptr(out), _ptr(cu_q_lens), _ptr(block_table),
-                                            block_table.shape[1], _ptr(context_lens), batch, q.shape[1], q.shape[0],
-                                            int(chunk_size), int(bool(causal)), float(sm_scale), _ptr(workspace),
+    st = load_library().coopt_paged_chunked(cache.ref(), q.data_ptr(), out.data_ptr(), cu_q_lens.data_ptr(), block_table.data_ptr(),
+                                            block_table.shape[1], context_lens.data_ptr(), batch, q.shape[1], q.shape[0],
+                                            int(chunk_size), int(bool(causal)), float(sm_scale), workspace.data_ptr(),
                                             workspace.numel(), _stream())
     _check(st, "coopt_paged_chunked")
     return out
@@ -365,7 +376,7 @@ def decode_step_host(cache: Cache, step_inputs: torch.Tensor, out: torch.Tensor,
     (page-locked ones are read and written in place by the kernel, pageable ones go through copies); asynchronous:
     ``out`` holds the result once the stream has been synchronised."""
     assert not step_inputs.is_cuda and step_inputs.is_contiguous() and not out.is_cuda and out.is_contiguous()
-    st = load_library().coopt_decode_step_host(cache.ref(), _ptr(step_inputs), _ptr(out), max_blocks_per_seq, out.shape[0],
-                                               num_q_heads, float(sm_scale), _ptr(staging), staging.numel(), _ptr(plan),
-                                               plan.numel(), _ptr(workspace), workspace.numel(), _stream())
+    st = load_library().coopt_decode_step_host(cache.ref(), step_inputs.data_ptr(), out.data_ptr(), max_blocks_per_seq, out.shape[0],
+                                               num_q_heads, float(sm_scale), staging.data_ptr(), staging.numel(), plan.data_ptr(),
+                                               plan.numel(), workspace.data_ptr(), workspace.numel(), _stream())
     _check(st, "coopt_decode_step_host")
