@@ -27,32 +27,121 @@ __global__ void __launch_bounds__(kWriteWarps * 32) kv_write_fp8_kernel(WritePar
   write_part<D, kBlockSize, kE5m2>(p, group, h, warp & 1, stage[warp], lane);
 }
 
-// FP8, many tokens (prefill chunks, bulk fills): one CTA per (kSpan consecutive tokens, kWriteHeads
-// kv heads).  Every warp settles one token of the span in the same memory trip; the groups found
-// (one per 16 tokens in a contiguous fill) are then served by all warps.
-constexpr int kSpan = 4 * kWriteWarps;  // a contiguous fill starts a group every 16 tokens: every CTA finds one
+// The K part (which = 0) or the V part (which = 1) of a block that is written whole: its 16 tokens follow one another in the
+// call from `tok` on, in order, rows aligned for the loads below.  The same scale rule and the same value for every number
+// that is stored as write_part (which takes the blocks that are not whole).  One warp; lane l has dims l D/32 .. of all 16
+// tokens in registers.  K goes through shared memory (st, 16 D bytes; 16-byte pieces swizzled so that neither side meets a
+// bank twice) and leaves as whole lines, V is in order in registers and leaves as 32-byte pieces.
+// False if the scale is outside of the range that the reciprocal serves: nothing has been written then.
+template <int D, bool kE5m2>
+__device__ __forceinline__ bool write_whole_part(const WriteParams& p, int blk, int tok, int h, int which, uint8_t* st, int lane) {
+  constexpr int kPart = part_bytes(D, true), kPerLane = D / 32, kWords = kPerLane / 2;
+  uint32_t raw[kBlockSize][kWords];
+  const __nv_bfloat16* row = (which == 0 ? p.k : p.v) + static_cast<int64_t>(tok) * p.token_stride + h * D + lane * kPerLane;
+#pragma unroll
+  for (int t = 0; t < kBlockSize; ++t) load_row<kPerLane, true>(row + t * p.token_stride, raw[t]);
+  uint32_t top = 0;
+#pragma unroll
+  for (int t = 0; t < kBlockSize; ++t)
+#pragma unroll
+    for (int e = 0; e < kWords; ++e) asm("max.xorsign.abs.bf16x2 %0, %0, %1;" : "+r"(top) : "r"(raw[t][e]));
+  // (magnitudes of bf16 values order like their patterns)
+  const uint32_t am = __reduce_max_sync(0xffffffffu, max((top << 16) & 0x7FFFFFFFu, top & 0x7FFF0000u));
+  const float s = __fdiv_rn(__uint_as_float(am), kE5m2 ? kE5m2Max : kE4m3Max);
+  if (!(s >= 0x1p-40f && s <= 0x1p40f)) return false;
+  // x / s, correctly rounded (Markstein: r = RN(1 / s), q0 = RN(x r), RN(q0 + (x - s q0) r)).  With the residual taken as
+  // s q0 - x a zero keeps the sign of x.
+  const float r = __frcp_rn(s);
+  auto quotient = [&](int t, int e) -> float {
+    const float x = (e & 1) ? bf16_hi(raw[t][e >> 1]) : bf16_lo(raw[t][e >> 1]);
+    const float q0 = __fmul_rn(x, r);
+    return __fmaf_rn(-__fmaf_rn(s, q0, -x), r, q0);
+  };
+  uint8_t* gran = p.cache + (static_cast<size_t>(blk) * p.num_kv_heads + h) * granule_bytes(D, true);
+  uint8_t* part = gran + which * kPart;
+  if (which == 0) {
+    constexpr int kChunks = D / 16;                       // 16-byte pieces of a token
+    auto place = [&](int t, int c) { return t * D + (c ^ (D == 128 ? t & 7 : (t >> 1) & 3)) * 16; };
+#pragma unroll
+    for (int t = 0; t < kBlockSize; ++t) {
+      uint8_t* dst = st + place(t, lane * kPerLane / 16) + lane * kPerLane % 16;
+      if constexpr (kPerLane == 4)
+        *reinterpret_cast<uint32_t*>(dst) = f32x2_to_codes<kE5m2>(quotient(t, 0), quotient(t, 1)) | (f32x2_to_codes<kE5m2>(quotient(t, 2), quotient(t, 3)) << 16);
+      else
+        *reinterpret_cast<uint16_t*>(dst) = static_cast<uint16_t>(f32x2_to_codes<kE5m2>(quotient(t, 0), quotient(t, 1)));
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < kPart / 512; ++i) {
+      const int o = i * 32 + lane, t = (o / (8 * kChunks)) * 8 + (o & 7), c = (o >> 3) % kChunks;
+      reinterpret_cast<uint4*>(part)[o] = *reinterpret_cast<const uint4*>(st + place(t, c));
+    }
+    __syncwarp();                                         // (the staging area may be written again)
+  } else {
+#pragma unroll
+    for (int e = 0; e < kPerLane; e += 2) {               // two dims: 2 x 16 bytes in a row
+      uint32_t w[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int d = e + (k >> 2), t = 4 * (k & 3);
+        w[k] = f32x2_to_codes<kE5m2>(quotient(t, d), quotient(t + 1, d)) | (f32x2_to_codes<kE5m2>(quotient(t + 2, d), quotient(t + 3, d)) << 16);
+      }
+      asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(part + (lane * kPerLane + e) * 16), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]),
+                   "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
+    }
+  }
+  float* header = reinterpret_cast<float*>(gran + header_offset(D));
+  if (lane == 0) header[which] = s;
+  if (which == 0 && lane < 6) header[2 + lane] = 0.0f;
+  return true;
+}
+
+// FP8, many tokens (prefill chunks, bulk fills): one CTA per (kSpan consecutive tokens, kWriteHeads kv heads), a warp per
+// (kv head, K | V).  Every warp finds the span's groups by itself: no warp waits for another.
+// Bound by memory: 65,536 tokens of 8 heads x 128 (403 MB) in 65.9 us, 6.1 TB/s.  Before blocks written whole had a path of
+// their own it was 112.6 us, bound by the integer pipe (10.6 instructions a value: look-ups of rows and groups, signs put
+// back after the division, stores of K words eight lanes to a bank).
+constexpr int kSpan = 32;
 constexpr int kSpanThreshold = 512;     // calls with more tokens than this take the span kernel
 template <int D, bool kE5m2>
-__global__ void __launch_bounds__(kWriteWarps * 32, 3) kv_write_fp8_span_kernel(WriteParams p) {
+__global__ void __launch_bounds__(kWriteWarps * 32, 4) kv_write_fp8_span_kernel(WriteParams p) {
   __shared__ __align__(16) uint8_t stage[kWriteWarps][part_bytes(D, true)];
-  __shared__ Group groups[kSpan];
+  __shared__ Group groups[kWriteWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int h = blockIdx.y * kWriteHeads + (warp >> 1), which = warp & 1;
   wait_previous_kernel();
-  for (int w = warp; w < kSpan; w += kWriteWarps) {
-    const int tok = blockIdx.x * kSpan + w;
-    if (tok < p.num_tokens) find_group_warp(p, tok, groups[w], lane);
-    else if (lane == 0) groups[w].n = 0;
-  }
-  __syncthreads();
-  unsigned leaders = 0;
-#pragma unroll
-  for (int w = 0; w < kSpan; ++w) leaders |= (groups[w].n > 0 ? 1u : 0u) << w;
-  const int h = blockIdx.y * kWriteHeads + (warp >> 1);
   if (h >= p.num_kv_heads) return;
-  while (leaders) {
-    const int w = __ffs(leaders) - 1;
-    leaders &= leaders - 1;
-    write_part<D, kBlockSize, kE5m2>(p, groups[w], h, warp & 1, stage[warp], lane);
+  // the slots of the span, of the token before it, and of the 32 tokens behind it
+  const int base = blockIdx.x * kSpan;
+  auto slot_of = [&](int i) -> int64_t { return i >= 0 && i < p.num_tokens ? p.slot_mapping[i] : -1; };
+  const int64_t s0 = slot_of(base + lane), s1 = slot_of(base + 32 + lane), before = slot_of(base - 1);
+  const int64_t s0_up = __shfl_up_sync(0xffffffffu, s0, 1), s0_last = __shfl_sync(0xffffffffu, s0, 31), s1_up = __shfl_up_sync(0xffffffffu, s1, 1);
+  const int64_t s0_prev = lane == 0 ? before : s0_up, s1_prev = lane == 0 ? s0_last : s1_up;
+  // bit i: token base + i follows the token before it into the next offset of the same block
+  const unsigned long long follows = __ballot_sync(0xffffffffu, s0 >= 0 && s0_prev >= 0 && s0 == s0_prev + 1 && (s0 % kBlockSize) != 0) |
+                                     static_cast<unsigned long long>(__ballot_sync(0xffffffffu, s1 >= 0 && s1_prev >= 0 && s1 == s1_prev + 1 && (s1 % kBlockSize) != 0)) << 32;
+  const bool begins = s0 >= 0 && s0 % kBlockSize == 0 && s0 / kBlockSize < p.num_blocks;
+  // a block written whole begins with its first slot and 15 tokens follow it in order (the precondition of the call, a
+  // block's tokens being consecutive, leaves no other token of it)
+  unsigned whole = __ballot_sync(0xffffffffu, begins && ((follows >> (lane + 1)) & 0x7FFFull) == 0x7FFFull);
+  // tokens that may lead any other group: all that do not follow into a block (a skipped token may stand between them and
+  // the one they follow: find_group_warp looks closer)
+  unsigned others = __ballot_sync(0xffffffffu, s0 >= 0 && !((follows >> lane) & 1ull)) & ~whole;
+  const bool aligned = ((reinterpret_cast<uintptr_t>(which == 0 ? p.k : p.v) | static_cast<uintptr_t>(p.token_stride * 2)) & (D / 16 - 1)) == 0;
+  if (!aligned) { others |= whole; whole = 0; }
+  while (whole) {
+    const int w = __ffs(whole) - 1;
+    whole &= whole - 1;
+    const int blk = static_cast<int>(__shfl_sync(0xffffffffu, s0, w) / kBlockSize);
+    if (!write_whole_part<D, kE5m2>(p, blk, base + w, h, which, stage[warp], lane)) others |= 1u << w;
+  }
+  while (others) {
+    const int w = __ffs(others) - 1;
+    others &= others - 1;
+    find_group_warp(p, base + w, groups[warp], lane);
+    __syncwarp();
+    if (groups[warp].n > 0) write_part<D, kBlockSize, kE5m2>(p, groups[warp], h, which, stage[warp], lane);
+    __syncwarp();
   }
 }
 
