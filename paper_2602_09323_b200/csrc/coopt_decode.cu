@@ -40,7 +40,7 @@ constexpr float kShift = 8.0f, kUnshift = 1.0f / 256.0f;          // probabiliti
 template <int D, int FMT>
 struct Cfg {
   static constexpr bool kFp8 = FMT != COOPT_KV_BF16;
-  static constexpr bool kE5m2 = FMT == COOPT_KV_FP8_E5M2;
+  [[maybe_unused]] static constexpr bool kE5m2 = FMT == COOPT_KV_FP8_E5M2;
   // A warp needs time for a block (about 1 us from landing to the next wait), so many warps are wanted, with at least two
   // blocks in flight each.  head_dim 128: 12 warps x 3 blocks against 16 x 2 (which spill), 14 x 2 and 10 x 4: 423 / 430 /
   // 423 / 427 us (64 sequences of 128..8192 tokens, four layers), 99 / 101 / 105 / 109 us (24 sequences, G = 8, four
@@ -315,10 +315,10 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
 #pragma unroll
     for (int k = 0; k < kPer; ++k) {
       const int b = tid * kPer + k;
-      int L = b < B ? p.context_lens[b] : 0;
-      L = max(0, min(L, p.max_blocks_per_seq * kBlockSize));
-      if (b < B) lens[b] = L;
-      const int nb = (L + kBlockSize - 1) / kBlockSize;
+      int len = b < B ? p.context_lens[b] : 0;
+      len = max(0, min(len, p.max_blocks_per_seq * kBlockSize));
+      if (b < B) lens[b] = len;
+      const int nb = (len + kBlockSize - 1) / kBlockSize;
       const int units = nb == 0 ? 0 : (chunk == kNoChunks ? 1 : (nb + chunk - 1) / chunk);
       v[k] = nb + units * kUnitCost;
       sum += v[k];
@@ -382,10 +382,11 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
   };
   // this warp's first unit in share s or, over several layers, in a later one (s moves there); and its next one
   auto walk_later = [&](unsigned& s, Walk& w) {
-    if (L == 1) return;
-    while (!w.more && s + gridDim.x < all_shares) {
-      s += gridDim.x;
-      share_walk(s, w);
+    if constexpr (L > 1) {
+      while (!w.more && s + gridDim.x < all_shares) {
+        s += gridDim.x;
+        share_walk(s, w);
+      }
     }
   };
   auto walk_on = [&](unsigned& s, Walk& w) {
@@ -503,6 +504,14 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
 
   const int d0 = lane * 4;
   const bool on = d0 < D;
+  // A warp of a launch over several layers whose wait has run out leaves without another word to the others (its record may
+  // still be in use, and an arrival ahead of its time would complete a phase that others have not reached): their waits for
+  // it run out in turn.
+  auto give_up = [&]() -> bool {
+    dead = __any_sync(0xffffffffu, dead);
+    if (dead && lane == 0) atomicCAS(p.status, 0, COOPT_ERR_TIMEOUT);
+    return dead;
+  };
   uint32_t round = 0;
 #pragma unroll 1
   for (unsigned share = blockIdx.x; share < all_shares; share += gridDim.x, ++round) {
@@ -746,9 +755,9 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
       }
     } else {
       // a piece: into shared memory, once the pieces of the share before are of no more use
-      if (L > 1 && round > 0 && rec.flags == 0 && !dead && !mbar_wait_bounded(bar_merged, (round - 1) & 1u)) {
-        dead = true;
-        atomicCAS(p.status, 0, COOPT_ERR_TIMEOUT);
+      if (L > 1) {
+        if (round > 0 && rec.flags == 0 && !dead && !mbar_wait_bounded(bar_merged, (round - 1) & 1u)) dead = true;
+        if (give_up()) break;
       }
       float* piece = reinterpret_cast<float*>(ring + (starts ? piece1_off : piece0_off));
       float* at = piece + 2 * quad * C::kPieceStride + row;
@@ -775,17 +784,12 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
     __syncthreads();
   } else {
     if (round > 0 && rec.flags == 0 && !dead && !mbar_wait_bounded(bar_merged, (round - 1) & 1u)) dead = true;   // (its record is still in use)
-    if (lane == 0) {
-      recs[warp] = rec;
-      if (dead) atomicCAS(p.status, 0, COOPT_ERR_TIMEOUT);
-    }
+    if (give_up()) break;
+    if (lane == 0) recs[warp] = rec;
     __syncwarp();
     if (lane == 0) mbar_arrive(bar_pieces);
-    if (!dead && !mbar_wait_bounded(bar_pieces, round & 1u)) {
-      dead = true;
-      atomicCAS(p.status, 0, COOPT_ERR_TIMEOUT);
-    }
-    dead = __any_sync(0xffffffffu, dead);
+    if (!mbar_wait_bounded(bar_pieces, round & 1u)) dead = true;
+    if (give_up()) break;
   }
   COOPT_TRACE_CYCLES(p.trace, kTrStreamed, tid == 0);
 
