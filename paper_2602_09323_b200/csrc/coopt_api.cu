@@ -13,7 +13,7 @@ int launch_kv_write(const coopt_cache* c, const void* k, const void* v, int64_t 
 int launch_paged_prefill(const coopt_cache* c, const void* q, void* out, const int32_t* cu_q_lens,
                          const int32_t* block_table, int32_t max_blocks_per_seq, const int32_t* context_lens,
                          int32_t batch, int32_t num_q_heads, int32_t total_q, int32_t causal, float sm_scale,
-                         void* workspace, cudaStream_t stream);
+                         void* workspace, int num_sms, cudaStream_t stream);
 const DeviceInfo* device_info() {
   static DeviceInfo info[64];
   static bool known[64] = {};
@@ -440,7 +440,7 @@ int coopt_paged_chunked(const coopt_cache* cache, const void* q, void* out, cons
     return launch_decode(a, static_cast<cudaStream_t>(stream));
   }
   return launch_paged_prefill(cache, q, out, cu_q_lens, block_table, max_blocks_per_seq, context_lens, batch,
-                              num_q_heads, total_q, causal, sm_scale, workspace, static_cast<cudaStream_t>(stream));
+                              num_q_heads, total_q, causal, sm_scale, workspace, num_sms(), static_cast<cudaStream_t>(stream));
 }
 
 namespace {

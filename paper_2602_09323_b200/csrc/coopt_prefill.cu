@@ -15,13 +15,14 @@
 //
 // What bounds it: per tile of 128 x 128 the exponential units need 1,024 cycles of an SM (16 a cycle) and the tensor core
 // 1,024 (head_dim 64: 512).  Both run all the time only if neither waits for the other: a tile is multiplied 64 keys (a
-// half) at a time, the logits of the next half while the half before is in the softmax, and two tiles share the SM.
+// half) at a time, the logits two halves ahead of the softmax (one ahead, waiting for registers to take them: 447 us against
+// 439), and two tiles share the SM.
 // Softmax of a tile: four warps, one row per thread, the row's 64 logits of the half in registers, read once.  It keeps a
 // reference maximum per row that may lag the true one by up to 2^11 (and a V scale reference that a scale may exceed by up
 // to 2^4), so the accumulator in tensor memory is rescaled rarely; f16 probabilities have room for that factor.
 //
-// Tensor memory (512 columns): logits of tile x in columns 64 x .., free again as soon as they are in registers; its
-// probabilities, two f16 to a column, in two buffers of 32 columns from 128 + 64 x; its accumulator from 256 + D x.
+// Tensor memory (512 columns): logits of tile x in two buffers of 64 columns from 128 x, the half's probabilities, two f16
+// to a column, in the same place once the logits are in registers; its accumulator from 256 + D x.
 //
 // Warp roles (512 threads):
 //   warps 0-3, 4-7   softmax of tile 0, of tile 1
@@ -30,11 +31,12 @@
 //   warp 14          copies: gather requests over the tensor map of the cache
 //   warp 15          what the softmax needs of a tile's block scales, worked out once for all rows
 //
-// Measured: 8 sequences of 4096 cached and 512 new tokens, 40 query heads over 8 kv heads, head_dim 128: 690 -> 450 us (the
+// Measured: 8 sequences of 4096 cached and 512 new tokens, 40 query heads over 8 kv heads, head_dim 128: 690 -> 430 us (the
 // kernel before: one tile a CTA, two groups of eight warps that took its key tiles in turns, each with an accumulator and
-// widening of its own); prompts of 900..2900 tokens, 32 heads over 8, head_dim 64: 495 -> 220 us (mma.sync).  A half takes
-// about 2,050 cycles for both tiles: exponential units 50 %, tensor core 42 %, the rest the way of a half through its
-// barriers (a hand-over from warp to warp costs about 120 cycles) with two softmax warps a scheduler.
+// widening of its own); prompts of 900..2900 tokens, 32 heads over 8, head_dim 64: 495 -> 187 us (mma.sync).  A half takes
+// about 1,850 cycles for both tiles: exponential units and issue slots 48 % each, tensor core 61 %, none of them alone (with
+// half the exponentials left out 12 % less time, with half the products of Q 4 %; four softmax warps a scheduler, two threads
+// to a row, took 453 us); a CTA's start and end take 15,000 cycles (head_dim 64: 10,000).
 // Every wait is bounded; a wait that runs out is reported in the status word and all roles leave through the common exit,
 // which frees the tensor memory.
 #include "coopt_umma.cuh"
@@ -64,6 +66,7 @@ struct PrefillParams {
   int num_blocks;
   int tile_queries;        // query tokens per tile = 128 / group
   int causal;
+  int by_length;           // more CTAs than the device holds at a time: the long ones first
   float sm_scale_log2;
   int* status;
 };
@@ -132,19 +135,17 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
   uint64_t* bar_k16full = bar_v16free + C::kWide;       // the same of K
   uint64_t* bar_k16free = bar_k16full + C::kWide;
   uint64_t* bar_scale = bar_k16free + C::kWide;         // the softmax's share of a tile's scales is ready
-  uint64_t* bar_sfull = bar_scale + C::kScaleSlots;     // [tile] logits of a half are in tensor memory (and the tile's scales ready)
-  uint64_t* bar_sfree = bar_sfull + 2;                  // [tile] .. and now in registers
-  uint64_t* bar_pfull = bar_sfree + 2;                  // [tile][buffer] its probabilities are in tensor memory
+  uint64_t* bar_sfull = bar_scale + C::kScaleSlots;     // [tile][buffer] logits of a half are in tensor memory (and the tile's scales ready)
+  uint64_t* bar_pfull = bar_sfull + 4;                  // [tile][buffer] its probabilities are, in their place
   uint64_t* bar_pv = bar_pfull + 4;                     // [tile] its product with V is done
   uint64_t* bar_out = bar_pv + 2;                       // [tile] .. and it was the tile's last
   uint64_t* bar_q = bar_out + 2;                        // the query operands are in shared memory
-  int* misc = reinterpret_cast<int*>(smem + C::kMiscOff);   // [0] sequence, [1] first query, [2] abort flag, [3] tensor memory
+  int* misc = reinterpret_cast<int*>(smem + C::kMiscOff);   // [0] sequence, [1] first query, [2] abort flag, [3] tensor memory, [4] first row, [5] rows, [6] context of the sequence, [7] kv head
   volatile int* abort_flag = misc + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(misc + 3);
 
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;      // (the warp in a uniform register)
   const int G = p.group, Hq = p.num_q_heads, Hkv = p.num_kv_heads;
-  const int g = blockIdx.y;
   const int TQ = p.tile_queries;
 
   if (tid == 0) {
@@ -157,8 +158,8 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
     }
     for (int i = 0; i < C::kScaleSlots; ++i) mbar_init(&bar_scale[i], 1);
     mbar_init(bar_q, 8);
-    for (int i = 0; i < 4; ++i) mbar_init(&bar_pfull[i], 4);
-    for (int i = 0; i < 2; ++i) { mbar_init(&bar_sfull[i], 2); mbar_init(&bar_sfree[i], 4); mbar_init(&bar_pv[i], 1); mbar_init(&bar_out[i], 1); }
+    for (int i = 0; i < 4; ++i) { mbar_init(&bar_sfull[i], 2); mbar_init(&bar_pfull[i], 4); }
+    for (int i = 0; i < 2; ++i) { mbar_init(&bar_pv[i], 1); mbar_init(&bar_out[i], 1); }
     mbar_fence_init();
   }
   if (warp == kMmaWarp) {
@@ -171,41 +172,87 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
   }
   wait_previous_kernel();
 
-  // ---- which (sequence, pair of query tiles) is this CTA's: late (long) ones of a sequence first -------------------------
+  // softmax groups: this thread's row r of tile x
+  const int x = warp >> 2, r = tid & (kRows - 1), qi = r / G, qh = r - qi * G;
+  // ---- which (sequence, kv head, pair of query tiles) is this CTA's --------------------------------------------------------
+  // Pairs with many keys to go through come first, over all sequences, so that the last CTAs to start are short ones.  How
+  // many is a pair's level (in pairs of queries: what fits into the tokens up to it), and levels are taken an eighth of the
+  // highest at a time: within that, the pairs of a (sequence, kv head) are neighbours and read its cache from L2 together.
+  // (Sequence after sequence, prompts of 900..2900 tokens took 204 us, 24 sequences of 105..3158 tokens 115; in this order
+  // 187 and 94; 8 sequences of 4096 + 512 tokens take 427 and 431 us, 443 level by level.)
   if (warp == 0) {
-    int left = blockIdx.x, found = -1, q0 = 0;
-    for (int b0 = 0; b0 < p.batch && found < 0; b0 += 32) {
-      const int b = b0 + lane;
-      const int n = b < p.batch ? max(0, p.cu_q_lens[b + 1] - p.cu_q_lens[b]) : 0;
-      const int nt = (n + 2 * TQ - 1) / (2 * TQ);
-      int upto = nt;
+    constexpr int kPer = 4, kBands = 8;
+    int left = blockIdx.x, found = -1, g = 0, q0 = 0, first = 0, count = 0, ctx = 0;
+    const int W = 2 * TQ;
+    auto sequence = [&](int b, int& from, int& n, int& c) {
+      from = b < p.batch ? p.cu_q_lens[b] : 0;
+      n = b < p.batch ? max(0, p.cu_q_lens[b + 1] - from) : 0;
+      c = b < p.batch ? max(0, min(p.context_lens[b], p.max_blocks_per_seq * kBlockSize)) : 0;
+    };
+    // this CTA among those of 32 sequences, of which lane l's has the pairs [last - m + 1, last]
+    auto look = [&](int b0, int m, int last, int from, int n, int c) {
+      int upto = m * Hkv;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const int t = __shfl_up_sync(0xffffffffu, upto, o);
         if (lane >= o) upto += t;
       }
       const unsigned in = __ballot_sync(0xffffffffu, upto > left);
-      if (in) {
-        const int l = __ffs(in) - 1;
-        found = b0 + l;
-        q0 = (__shfl_sync(0xffffffffu, upto, l) - 1 - left) * 2 * TQ;
-      } else {
-        left -= __shfl_sync(0xffffffffu, upto, 31);
+      if (in == 0) { left -= __shfl_sync(0xffffffffu, upto, 31); return; }
+      const int l = __ffs(in) - 1;
+      m = __shfl_sync(0xffffffffu, m, l);
+      left -= __shfl_sync(0xffffffffu, upto, l) - m * Hkv;
+      found = b0 + l;
+      g = left / m;
+      q0 = (__shfl_sync(0xffffffffu, last, l) - left % m) * W;
+      first = __shfl_sync(0xffffffffu, from, l);
+      count = __shfl_sync(0xffffffffu, n, l);
+      ctx = __shfl_sync(0xffffffffu, c, l);
+    };
+    if (p.by_length && p.batch <= 32 * kPer) {
+      int from[kPer], n[kPer], c[kPer], pairs[kPer], end[kPer], top = 0;
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) {
+        sequence(32 * i + lane, from[i], n[i], c[i]);
+        pairs[i] = (n[i] + W - 1) / W;
+        end[i] = max(0, c[i] - n[i]) / W + pairs[i];
+        top = max(top, end[i]);
+      }
+      const int width = max(1, (__reduce_max_sync(0xffffffffu, top) + kBands - 1) / kBands);
+      auto above = [&](int i, int v) { return max(0, min(pairs[i], end[i] - v * width)); };      // pairs of band v and higher ones
+      int band = kBands - 1;
+#pragma unroll 1
+      for (; band >= 0; --band) {
+        int k = 0;
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) k += above(i, band);
+        if (static_cast<int>(__reduce_add_sync(0xffffffffu, k)) * Hkv > left) break;
+      }
+      if (band >= 0) {
+        int k = 0;
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) k += above(i, band + 1);
+        left -= static_cast<int>(__reduce_add_sync(0xffffffffu, k)) * Hkv;
+#pragma unroll
+        for (int i = 0; i < kPer; ++i)
+          if (found < 0) look(32 * i, above(i, band) - above(i, band + 1), pairs[i] - 1 - above(i, band + 1), from[i], n[i], c[i]);
+      }
+    } else {
+      // all CTAs start at once, or so many sequences that each is short against the whole: one after the other, each from its end
+      for (int b0 = 0; b0 < p.batch && found < 0; b0 += 32) {
+        int from, n, c;
+        sequence(b0 + lane, from, n, c);
+        const int pairs = (n + W - 1) / W;
+        look(b0, pairs, pairs - 1, from, n, c);
       }
     }
-    if (lane == 0) { misc[0] = found; misc[1] = q0; }
+    if (lane == 0) { misc[0] = found; misc[1] = q0; misc[4] = first; misc[5] = count; misc[6] = ctx; misc[7] = g; }
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  const int b = misc[0], q0 = misc[1];
-  int row_base = 0, n_new = 0, L = 0;
-  if (b >= 0) {
-    row_base = p.cu_q_lens[b];
-    n_new = p.cu_q_lens[b + 1] - row_base;
-    L = max(0, min(p.context_lens[b], p.max_blocks_per_seq * kBlockSize));
-  }
+  const int b = misc[0], q0 = misc[1], row_base = misc[4], n_new = misc[5], L = misc[6], g = misc[7];
   // keys that any row of tile x may see (Eq. 1: K_{<=t}), and tiles of keys
   auto tile_queries = [&](int x) { return max(0, min(TQ, n_new - q0 - x * TQ)); };
   auto tile_keys = [&](int x) {
@@ -215,11 +262,8 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
   const int kv_end = max(tile_keys(0), tile_keys(1));
   const int n_blocks = (kv_end + kBlockSize - 1) / kBlockSize, n_tiles = (kv_end + kTileKeys - 1) / kTileKeys;
 
-  // softmax groups: this thread's row r of tile x
-  const int x = warp >> 2, r = tid & (kRows - 1);
-  const int qi = r / G;
   const bool live = x < 2 && qi < tile_queries(x);
-  const size_t grow = static_cast<size_t>(row_base + q0 + x * TQ + (live ? qi : 0)) * Hq + g * G + (live ? r % G : 0);
+  const size_t grow = static_cast<size_t>(row_base + q0 + x * TQ + (live ? qi : 0)) * Hq + g * G + (live ? qh : 0);
   uint32_t pend_mask = 0, pend_par = 0;                 // copy lane: the latest phase expected of every slot it has filled
 
   if (n_tiles == 0) {
@@ -230,87 +274,94 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
     // ================= softmax: one row per thread ===================================================================
     asm volatile("setmaxnreg.inc.sync.aligned.u32 168;");
     const uint32_t lane_base = static_cast<uint32_t>(warp & 3) * 32u << 16;
-    const uint32_t s_cols = tmem + kHalf * x + lane_base, p_cols = tmem + 2 * kHalf + kHalf * x + lane_base, o_cols = tmem + 256 + D * x + lane_base;
-    // ---- row r of the query operand
+    const uint32_t s_cols = tmem + 2 * kHalf * x + lane_base, o_cols = tmem + 4 * kHalf + D * x + lane_base;
+    // ---- the query operand of the warp's 32 rows, eight at a time: a lane has every fourth 16 bytes of one of them.  The bf16
+    // rows come into the operand's own place first.  (Loops that are not unrolled: code that a CTA runs once is bound by the
+    // fetch of its instructions, about four cycles each.  A row per lane and all of it unrolled: 12,000 cycles, head_dim 64
+    // 5,500.)
+    const int row_off = live ? qi * Hq + qh : -1;      // from the tile's first row
+    const size_t tile_row = static_cast<size_t>(row_base + q0 + x * TQ) * Hq + g * G;
     float qscale = 0.0f;       // logits of this row = tensor-memory value * qscale * K scale of the block
     {
-      uint32_t amax = 0;
-      const uint4* src = reinterpret_cast<const uint4*>(p.q + grow * D);
-      if (live) {
-#pragma unroll 8
-        for (int c = 0; c < D / 8; ++c) {
-          const uint4 v = src[c];
-          const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+      constexpr int kOctet = (C::kWideK ? 16 : 8) * D;    // eight rows of the operand (head_dim 128: of one term)
+      const int row = lane & 7, at = lane >> 3;
+      uint8_t* operand = smem + C::kQOff + x * C::kOperand + (warp & 3) * 4 * kOctet;
+      auto raw = [&](int o, int k) { return operand + o * kOctet + (32 * (C::kWideK ? k : k & 1) + lane) * 16 + (k >> 1) * (C::kWideK ? 0 : C::kOperand / 2); };
+#pragma unroll 1
+      for (int o = 0; o < 4; ++o) {
+        const int off = __shfl_sync(0xffffffffu, row_off, 8 * o + row);
+        const __nv_bfloat16* src = p.q + (tile_row + max(off, 0)) * D + at * 8;
 #pragma unroll
-          for (int e = 0; e < 4; ++e) amax = max(amax, max((w[e] << 16) & 0x7FFFFFFFu, w[e] & 0x7FFF0000u));   // |bf16| as fp32 bits
-        }
+        for (int k = 0; k < D / 32; ++k)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(raw(o, k))), "l"(src + 32 * k), "r"(off >= 0 ? 16 : 0) : "memory");
       }
-      // the row scaled by a power of two into [128, 256), undone on the logits
-      int k2 = 0;
-      if (amax != 0u) k2 = max(-64, min(64, 134 - static_cast<int>((amax >> 23) & 0xFF)));
-      qscale = p.sm_scale_log2 * __uint_as_float(static_cast<uint32_t>(127 - k2) << 23);
-      const float up = __uint_as_float(static_cast<uint32_t>(k2 + 127) << 23);
-      uint8_t* qrow = smem + C::kQOff + x * C::kOperand + (r & 7) * 16;
-#pragma unroll 2
-      for (int c = 0; c < D / 16; ++c) {                  // 16 elements
-        const uint4 a = live ? src[2 * c] : make_uint4(0u, 0u, 0u, 0u), e4 = live ? src[2 * c + 1] : make_uint4(0u, 0u, 0u, 0u);
-        const uint32_t w[8] = {a.x, a.y, a.z, a.w, e4.x, e4.y, e4.z, e4.w};
-        if constexpr (C::kWideK) {
-          // f16 (exact)
-          uint32_t h[8];
+      asm volatile("cp.async.wait_all;" ::: "memory");
+#pragma unroll 1
+      for (int o = 0; o < 4; ++o) {
+        uint4 q[D / 32];
+        uint32_t m = 0;
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            h[2 * e] = pack_f16x2(bf16_lo(w[2 * e]) * up, bf16_hi(w[2 * e]) * up);
-            h[2 * e + 1] = pack_f16x2(bf16_lo(w[2 * e + 1]) * up, bf16_hi(w[2 * e + 1]) * up);
-          }
-          uint8_t* dst = qrow + (r >> 3) * (16 * D) + c * 256;
-          *reinterpret_cast<uint4*>(dst) = make_uint4(h[0], h[1], h[2], h[3]);
-          *reinterpret_cast<uint4*>(dst + 128) = make_uint4(h[4], h[5], h[6], h[7]);
-        } else {
-          // the exact sum of the nearest E4M3 value and the E4M3 value of the remainder
-          uint32_t lead[4], rest[4];
+        for (int k = 0; k < D / 32; ++k) {
+          q[k] = *reinterpret_cast<const uint4*>(raw(o, k));
+          m = __vmaxu2(m, __vmaxu2(__vmaxu2(q[k].x & 0x7FFF7FFFu, q[k].y & 0x7FFF7FFFu), __vmaxu2(q[k].z & 0x7FFF7FFFu, q[k].w & 0x7FFF7FFFu)));
+        }
+        m = __vmaxu2(m, __shfl_xor_sync(0xffffffffu, m, 8));
+        m = __vmaxu2(m, __shfl_xor_sync(0xffffffffu, m, 16));
+        const uint32_t amax = max(m << 16, m & 0xFFFF0000u);             // |bf16| as fp32 bits
+        // the row scaled by a power of two into [128, 256), undone on the logits
+        int k2 = 0;
+        if (amax != 0u) k2 = max(-64, min(64, 134 - static_cast<int>((amax >> 23) & 0xFF)));
+        const float up = __uint_as_float(static_cast<uint32_t>(k2 + 127) << 23);
+        const float down = __shfl_sync(0xffffffffu, p.sm_scale_log2 * __uint_as_float(static_cast<uint32_t>(127 - k2) << 23), row);
+        if (at == o) qscale = down;
+        __syncwarp();
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            uint32_t h0 = pack_f16x2(bf16_lo(w[2 * e]) * up, bf16_hi(w[2 * e]) * up);
-            uint32_t h1 = pack_f16x2(bf16_lo(w[2 * e + 1]) * up, bf16_hi(w[2 * e + 1]) * up);
-            const uint32_t l0 = e4m3_term(h0, 1.0f), l1 = e4m3_term(h1, 1.0f);
-            lead[e] = l0 | (l1 << 16);
-            rest[e] = f16x2_to_e4m3x2(h0) | (f16x2_to_e4m3x2(h1) << 16);
+        for (int k = 0; k < D / 32; ++k) {                // eight elements
+          const uint32_t w[4] = {q[k].x, q[k].y, q[k].z, q[k].w};
+          uint32_t h[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) h[e] = pack_f16x2(bf16_lo(w[e]) * up, bf16_hi(w[e]) * up);
+          uint8_t* dst = operand + o * kOctet + row * 16;
+          if constexpr (C::kWideK) {
+            *reinterpret_cast<uint4*>(dst + (at + 4 * k) * 128) = make_uint4(h[0], h[1], h[2], h[3]);      // f16 (exact)
+          } else {
+            // the exact sum of the nearest E4M3 value and the E4M3 value of the remainder
+            uint32_t lead[4], rest[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) { lead[e] = e4m3_term(h[e], 1.0f); rest[e] = f16x2_to_e4m3x2(h[e]); }
+            dst += ((at + 4 * k) >> 1) * 128 + (at & 1) * 8;
+            *reinterpret_cast<uint2*>(dst) = make_uint2(lead[0] | (lead[1] << 16), lead[2] | (lead[3] << 16));
+            *reinterpret_cast<uint2*>(dst + C::kOperand / 2) = make_uint2(rest[0] | (rest[1] << 16), rest[2] | (rest[3] << 16));
           }
-          uint8_t* dst = qrow + (r >> 3) * (8 * D) + c * 128;
-          *reinterpret_cast<uint4*>(dst) = make_uint4(lead[0], lead[1], lead[2], lead[3]);
-          *reinterpret_cast<uint4*>(dst + C::kOperand / 2) = make_uint4(rest[0], rest[1], rest[2], rest[3]);
         }
       }
     }
     fence_proxy_async();
     __syncwarp();
-    if (lane == 0) mbar_arrive(bar_q);
+    arrive_one(bar_q);
 
     // index of the last visible key of the row.  Rows past the tile's last query (their operand is zero, and they are never
     // stored) see everything, so that their warp takes the same unmasked path as its live rows.
     const int lim = live ? (p.causal ? min(L - 1, L - n_new + q0 + x * TQ + qi) : L - 1) : (1 << 30);
     const int halves = (tile_keys(x) + kHalf - 1) / kHalf;
-    float m_ref = -INFINITY, l_row = 0.0f, v_ref = 0.0f;
+    float m_ref = -INFINITY, m_use = 0.0f, l_row = 0.0f, v_ref = 0.0f;      // m_use: m_ref, or 0 before the first visible key
     bool ok = true;
 #pragma unroll 1
     for (int h = 0; h < halves && ok; ++h) {
       const int t = h >> 1, buf = h & 1;
       const float* sc = scales + (t & (C::kScaleSlots - 1)) * 32 + 4 * buf;
-      ok = wait_warp(&bar_sfull[x], h & 1u, abort_flag);
+      ok = wait_warp(&bar_sfull[2 * x + buf], t & 1u, abort_flag);
       if (!ok) break;
       tc_fence_after();
       uint32_t s[2][32];
 #pragma unroll
-      for (int i = 0; i < 2; ++i) tmem_ld32_issue(s_cols + 32 * i, s[i]);
-      float cf[4];                                      // logit = accumulator * cf of its block (a zero scale: tiny, so that -inf stays -inf)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) cf[c] = fmaxf(sc[c] * qscale, 1e-30f);
+      for (int i = 0; i < 2; ++i) tmem_ld32_issue(s_cols + kHalf * buf + 32 * i, s[i]);
+      const float4 sk = *reinterpret_cast<const float4*>(sc), lg = *reinterpret_cast<const float4*>(sc + 8), inv = *reinterpret_cast<const float4*>(sc + 16);
+      const float v_factor = buf == 0 ? sc[24] : 1.0f;
+      // logit = accumulator * cf of its block (a zero scale: tiny, so that -inf stays -inf)
+      const float cf[4] = {fmaxf(sk.x * qscale, 1e-30f), fmaxf(sk.y * qscale, 1e-30f), fmaxf(sk.z * qscale, 1e-30f), fmaxf(sk.w * qscale, 1e-30f)};
 #pragma unroll
       for (int i = 0; i < 2; ++i) tmem_ld_wait32(s[i]);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&bar_sfree[x]);
       const int visible = lim - h * kHalf;
       if (visible < kHalf - 1) {
 #pragma unroll
@@ -324,36 +375,38 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
         const float m0 = max3(f(0), f(1), f(2)), m1 = max3(f(3), f(4), f(5)), m2 = max3(f(6), f(7), f(8)), m3 = max3(f(9), f(10), f(11)), m4 = max3(f(12), f(13), f(14));
         m_tile = fmaxf(m_tile, fmaxf(max3(m0, m1, m2), max3(m3, m4, f(15))) * cf[c]);
       }
-      // lazy references: moved only when the half would push a probability (or a scale ratio) past the margin
-      float factor = 1.0f;
-      if (buf == 0) { factor = sc[24]; v_ref = sc[25]; }
-      if (m_tile > m_ref + kMaxLag) {                   // also true for the row's first visible key
-        const float f = m_ref == -INFINITY ? 0.0f : ex2(m_ref - m_tile);
-        factor *= f;
-        l_row *= f;
-        m_ref = m_tile;
-      }
-      if (__any_sync(0xffffffffu, factor != 1.0f) && h > 0) {
-        // the accumulator is at rest once the product of the half before is done
-        ok = wait_bar(&bar_pv[x], (h - 1) & 1u, abort_flag);
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok) break;
-        tc_fence_after();
+      // lazy references: moved only when the half would push a probability (or a scale ratio) past the margin, so that the common
+      // way through a half is one vote
+      const bool move = m_tile > m_ref + kMaxLag;       // also true for the row's first visible key
+      if (__any_sync(0xffffffffu, move || v_factor != 1.0f)) {
+        float factor = v_factor;
+        if (v_factor != 1.0f) v_ref = sc[25];
+        if (move) {
+          const float f = m_ref == -INFINITY ? 0.0f : ex2(m_ref - m_tile);
+          factor *= f;
+          l_row *= f;
+          m_ref = m_use = m_tile;
+        }
+        if (h > 0) {
+          // the accumulator is at rest once the product of the half before is done
+          ok = wait_warp(&bar_pv[x], (h - 1) & 1u, abort_flag);
+          if (!ok) break;
+          tc_fence_after();
 #pragma unroll 1
-        for (int i = 0; i < D; i += 64) {
-          uint32_t o[4][16];
+          for (int i = 0; i < D; i += 64) {
+            uint32_t o[4][16];
 #pragma unroll
-          for (int e = 0; e < 4; ++e) tmem_ld16_issue(o_cols + i + 16 * e, o[e]);
+            for (int e = 0; e < 4; ++e) tmem_ld16_issue(o_cols + i + 16 * e, o[e]);
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            tmem_ld_wait(o[e]);
+            for (int e = 0; e < 4; ++e) {
+              tmem_ld_wait(o[e]);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) o[e][j] = __float_as_uint(__uint_as_float(o[e][j]) * factor);
-            tmem_st16(o_cols + i + 16 * e, o[e]);
+              for (int j = 0; j < 16; ++j) o[e][j] = __float_as_uint(__uint_as_float(o[e][j]) * factor);
+              tmem_st16(o_cols + i + 16 * e, o[e]);
+            }
           }
         }
       }
-      const float m_use = m_ref == -INFINITY ? 0.0f : m_ref;
       // p * pv = 2^(s * cf - m + log2 pv): the V scale rides in the exponent, and a block's sum of p is recovered from the sum
       // of p * pv (pv: the block's V scale over the reference, at most 2^4, a zero one replaced by 2^-24)
 #pragma unroll
@@ -362,7 +415,7 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
 #pragma unroll
         for (int e2 = 0; e2 < 2; ++e2) {
           const int c = 2 * i + e2;
-          const float shift = sc[8 + c] - m_use;
+          const float shift = (c == 0 ? lg.x : c == 1 ? lg.y : c == 2 ? lg.z : lg.w) - m_use;
           const uint32_t* v = &s[i][16 * e2];
           float y[16];
 #pragma unroll
@@ -371,16 +424,16 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
           // against 590, with 512 that the exponentials need.)
           const float u0 = (y[0] + y[1]) + (y[2] + y[3]), u1 = (y[4] + y[5]) + (y[6] + y[7]);
           const float u2 = (y[8] + y[9]) + (y[10] + y[11]), u3 = (y[12] + y[13]) + (y[14] + y[15]);
-          l_row += ((u0 + u1) + (u2 + u3)) * sc[16 + c];
+          l_row += ((u0 + u1) + (u2 + u3)) * (c == 0 ? inv.x : c == 1 ? inv.y : c == 2 ? inv.z : inv.w);
 #pragma unroll
           for (int e = 0; e < 8; ++e) pw[8 * e2 + e] = pack_f16x2(y[2 * e], y[2 * e + 1]);
         }
-        tmem_st16(p_cols + 32 * buf + 16 * i, pw);
+        tmem_st16(s_cols + kHalf * buf + 16 * i, pw);
       }
       tmem_st_wait();
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&bar_pfull[2 * x + buf]);
+      arrive_one(&bar_pfull[2 * x + buf]);
     }
     const bool any_keys = halves > 0;
     if (ok && any_keys) ok = wait_bar(&bar_out[x], 0u, abort_flag);
@@ -388,6 +441,11 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
     if (ok) {
       tc_fence_after();
       const float k = l_row > 0.0f ? v_ref / l_row : 0.0f;
+      // The rows go through shared memory, where the tile's query operand was (its products are done): 16 bytes of a row at
+      // (chunk ^ row).
+      constexpr int kLanes = D / 8, kRowsAt = 32 / kLanes;  // lanes of a row, rows at a time
+      const int at = lane % kLanes, at_row = lane / kLanes;
+      uint8_t* rows = smem + C::kQOff + x * C::kOperand + (warp & 3) * 32 * D * 2;
 #pragma unroll 1
       for (int c = 0; c < D / 32; ++c) {
         uint32_t o[32];
@@ -395,14 +453,19 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
           tmem_ld32_issue(o_cols + 32 * c, o);
           tmem_ld_wait32(o);
         }
-        if (live) {
-          uint32_t w[16];
+        uint32_t w[16];
 #pragma unroll
-          for (int j = 0; j < 16; ++j) w[j] = k != 0.0f ? pack_bf16x2(__uint_as_float(o[2 * j]) * k, __uint_as_float(o[2 * j + 1]) * k) : 0u;
-          uint4* dst = reinterpret_cast<uint4*>(p.out + grow * D + 32 * c);
+        for (int j = 0; j < 16; ++j) w[j] = k != 0.0f ? pack_bf16x2(__uint_as_float(o[2 * j]) * k, __uint_as_float(o[2 * j + 1]) * k) : 0u;
 #pragma unroll
-          for (int j = 0; j < 4; ++j) dst[j] = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
-        }
+        for (int j = 0; j < 4; ++j)
+          *reinterpret_cast<uint4*>(rows + lane * D * 2 + ((4 * c + j) ^ (lane & (kLanes - 1))) * 16) = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+      }
+      __syncwarp();
+#pragma unroll 4
+      for (int i = 0; i < kLanes; ++i) {
+        const int row = kRowsAt * i + at_row, off = __shfl_sync(0xffffffffu, row_off, row);
+        if (off >= 0)
+          *reinterpret_cast<uint4*>(p.out + (tile_row + off) * D + at * 8) = *reinterpret_cast<const uint4*>(rows + row * D * 2 + (at ^ (row & (kLanes - 1))) * 16);
       }
       tc_fence_before();
     } else if (lane == 0) {
@@ -485,7 +548,7 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
         const uint64_t desc_k = umma_desc(smem_u32(smem + (C::kWideK ? C::kK16Off : C::kKOff)), 128, kRowGroup);
         const uint64_t desc_q = umma_desc(smem_u32(smem + C::kQOff + mx * C::kOperand), 128, kRowGroup);
         const uint64_t desc_v = umma_desc(smem_u32(smem + C::kV16Off), 128, 2048);
-        const uint32_t s_cols = tmem + kHalf * mx, p_cols = tmem + 2 * kHalf + kHalf * mx, o_cols = tmem + 256 + D * mx;
+        const uint32_t s_cols = tmem + 2 * kHalf * mx, o_cols = tmem + 4 * kHalf + D * mx;
         const int keys = tile_keys(mx), halves = (keys + kHalf - 1) / kHalf, my_tiles = (keys + kTileKeys - 1) / kTileKeys;
         bool ok = true;
         int done = 0;                                     // halves whose product with V has been seen to be done
@@ -495,45 +558,42 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
             if (ok && ((done & 1) || done == halves - 1)) arrive_one(&bar_v16free[(done >> 1) % C::kWide]);
           }
         };
-        // Logits of a half, once those of the half before are in registers.  (The probabilities of the half will take the place
-        // of those of half h - 2, whose product has to be done by then.)
+        // Logits of a half, where those of half h - 2 and then its probabilities were: its product is done.
         auto issue_logits = [&](int h) {
           const int t = h >> 1, ks = t % kSlots;
           if ((h & 1) == 0) {
             ok = ok && wait_warp(&bar_scale[t & (C::kScaleSlots - 1)], (t / C::kScaleSlots) & 1u, abort_flag);
             ok = ok && wait_warp(&k_full[ks], (t / kSlots) & 1u, abort_flag);
           }
-          see_products(h - 1);
-          if (h > 0) ok = ok && wait_warp(&bar_sfree[mx], (h - 1) & 1u, abort_flag);
           if (!ok) return;
           tc_fence_after();
           const uint64_t dk = desc_k + ((ks * kSlotBytes + (h & 1) * 8 * kRowGroup) >> 4);
+          const uint32_t to = s_cols + kHalf * (h & 1);
           if constexpr (C::kWideK) {
 #pragma unroll
-            for (int k = 0; k < D / 16; ++k) umma_f16(s_cols, desc_q + k * 16, dk + k * 16, umma_idesc(kHalf), k != 0);
+            for (int k = 0; k < D / 16; ++k) umma_f16(to, desc_q + k * 16, dk + k * 16, umma_idesc(kHalf), k != 0);
           } else {
 #pragma unroll
             for (int term = 0; term < 2; ++term)
 #pragma unroll
               for (int k = 0; k < D / 32; ++k)
-                umma_f8(s_cols, desc_q + ((term * (C::kOperand / 2)) >> 4) + k * 16, dk + k * 16, umma_idesc(kHalf, 0, kE5m2 ? 1 : 0), (term | k) != 0);
+                umma_f8(to, desc_q + ((term * (C::kOperand / 2)) >> 4) + k * 16, dk + k * 16, umma_idesc(kHalf, 0, kE5m2 ? 1 : 0), (term | k) != 0);
           }
-          umma_commit(&bar_sfull[mx]);
-          arrive_one(&bar_sfull[mx]);
+          umma_commit(&bar_sfull[2 * mx + (h & 1)]);
+          arrive_one(&bar_sfull[2 * mx + (h & 1)]);
         };
         ok = wait_warp(bar_q, 0u, abort_flag);
         if (halves > 0) issue_logits(0);
+        if (halves > 1) issue_logits(1);
         for (int h = 0; h < halves && ok; ++h) {
           const int t = h >> 1, w2 = t % C::kWide;
-          // (Products are seen one by one: a wait for a barrier's phase must not fall two phases behind.)
-          if (h + 1 < halves) issue_logits(h + 1); else see_products(h);
           if ((h & 1) == 0) ok = ok && wait_warp(&bar_v16full[w2], (t / C::kWide) & 1u, abort_flag);
           ok = ok && wait_warp(&bar_pfull[2 * mx + (h & 1)], t & 1u, abort_flag);
           if (!ok) break;
           if ((h & 1) || h == halves - 1) arrive_one(&k_free[t % kSlots]);      // probabilities are there, so the logits have been
           tc_fence_after();
           const uint64_t dv = desc_v + ((w2 * C::kOperand) >> 4) + (h & 1) * 64;
-          const uint32_t from = p_cols + 32 * (h & 1);
+          const uint32_t from = s_cols + kHalf * (h & 1);
           const int nb = min(kTileBlocks / 2, n_blocks - h * (kTileBlocks / 2));      // 16 keys (one cache block) per instruction
           if (nb == kTileBlocks / 2) {
 #pragma unroll
@@ -542,8 +602,10 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
             for (int k = 0; k < nb; ++k) umma_f16_ts(o_cols, from + 8 * k, dv + k * 16, umma_idesc(D), (h | k) != 0);
           }
           umma_commit(&bar_pv[mx]);
+          // (Products are seen one by one: a wait for a barrier's phase must not fall two phases behind.)
+          see_products(h + 1);
+          if (h + 2 < halves) issue_logits(h + 2);
         }
-        see_products(halves);
         if (ok) {
           tc_fence_after();
           tc_fence_before();
@@ -684,7 +746,7 @@ int launch_one(const coopt_cache* c, const PrefillParams& p, dim3 grid, cudaStre
 int launch_paged_prefill(const coopt_cache* c, const void* q, void* out, const int32_t* cu_q_lens,
                          const int32_t* block_table, int32_t max_blocks_per_seq, const int32_t* context_lens,
                          int32_t batch, int32_t num_q_heads, int32_t total_q, int32_t causal, float sm_scale,
-                         void* workspace, cudaStream_t stream) {
+                         void* workspace, int num_sms, cudaStream_t stream) {
   if (!is_fp8(c->dtype)) return COOPT_ERR_UNSUPPORTED;
   if (c->dtype == COOPT_KV_FP8_E5M2 && c->head_dim != 128) return COOPT_ERR_UNSUPPORTED;
   PrefillParams p;
@@ -704,8 +766,9 @@ int launch_paged_prefill(const coopt_cache* c, const void* q, void* out, const i
   p.sm_scale_log2 = sm_scale * kLog2e;
   p.status = static_cast<int*>(workspace);
   const long long pairs = static_cast<long long>(total_q) / (2 * p.tile_queries) + batch;   // every sequence adds at most one partly filled pair
-  if (pairs > 0x7fffffffll) return COOPT_ERR_UNSUPPORTED;
-  const dim3 grid(static_cast<unsigned>(pairs), static_cast<unsigned>(c->num_kv_heads));
+  if (pairs * c->num_kv_heads > 0x7fffffffll) return COOPT_ERR_UNSUPPORTED;
+  const dim3 grid(static_cast<unsigned>(pairs * c->num_kv_heads));
+  p.by_length = pairs * c->num_kv_heads > num_sms ? 1 : 0;
   if (c->head_dim == 64) return launch_one<64, false>(c, p, grid, stream);
   return c->dtype == COOPT_KV_FP8_E5M2 ? launch_one<128, true>(c, p, grid, stream) : launch_one<128, false>(c, p, grid, stream);
 }

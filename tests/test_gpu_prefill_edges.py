@@ -54,3 +54,15 @@ def test_references_that_have_to_move(d):
         w.k[:] = (w.k.float() * grow).to(torch.bfloat16)
         w.v[:] = (w.v.float() * (torch.arange(n)[:, None, None] // 200 * 2.0 + 0.01) * 0.02).to(torch.bfloat16)
     _check([900, 700], [100, 30], 6, 2, d, seed=9, mutate=mutate)
+
+
+@pytest.mark.parametrize("batch", [3, 33, 128, 129])
+def test_more_tiles_than_the_device_holds_ragged(batch):
+    """Every (sequence, kv head, pair of tiles) is found once in the order of lengths, with sequences whose runs are empty or
+    longer than their context's start, on both sides of the number of sequences that are ordered."""
+    g = torch.Generator().manual_seed(batch)
+    lens = [int(n) for n in torch.randint(1, 260, (batch,), generator=g)]
+    q_lens = [0 if i % 7 == 3 else max(1, n - (37 * i) % 90) for i, n in enumerate(lens)]
+    if batch == 3:
+        lens, q_lens = [700, 40, 1500], [690, 40, 900]
+    _check(lens, q_lens, 32, 4, 64, seed=batch)
