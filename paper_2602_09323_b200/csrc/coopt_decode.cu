@@ -19,8 +19,14 @@
 // CTA and a plan of every CTA's blocks made by a kernel of its own.  The tensor core was 21 % busy with columns that
 // are mostly padding, and what bounded the launch were the hand-overs between its roles, per unit and at both ends.
 // Before / now: one layer of 56 heads over 8 kv heads, 8 sequences of 1..28 tokens 60 / 8 us; 24 sequences of
-// 300..4000 tokens, G = 8, 46 / 25 us a layer; 32 x 2048 tokens, G = 5, 35 / 32 us; 64 sequences of 128..8192 tokens,
-// 121 / 106 us; 120 sequences of 5..900 tokens at head_dim 64, plan included, 56 / 18.5 us.)
+// 300..4000 tokens, G = 8, 46 / 23 us a layer; 32 x 2048 tokens, G = 5, 35 / 30 us; 64 sequences of 128..8192 tokens,
+// 121 / 105 us; 120 sequences of 5..900 tokens at head_dim 64, plan included, 56 / 17 us.)
+//
+// A launch of 32 x 2048 tokens streams at 6.4 TB/s from its first copies, 3 us after a CTA's first instruction, to the end
+// of its last block, 5 us before the CTA's last; code that runs once costs about four cycles an instruction to fetch.
+// Registers are what the loop over blocks is short of: the walk of the copies waits in shared memory, and the query rows of
+// a unit are fetched when it starts (eight layers of 21 sequences of 2..60 tokens: 49 / 43.6 us; prefetching the rows into
+// registers at the end of the unit before instead: 49.5).
 #include <algorithm>
 
 #include "coopt_decode.cuh"
@@ -63,7 +69,8 @@ struct Cfg {
   static constexpr int kPreOff = kLensOff + kMaxBatch * 4;
   static constexpr int kRecOff = kPreOff + (kMaxBatch + 4) * 4;
   static constexpr int kMiscOff = kRecOff + kWarps * 32;
-  static constexpr int kSmemBytes = kMiscOff + 192;
+  static constexpr int kCopyWalkOff = kMiscOff + 192;           // a walk per warp: where its copies are
+  static constexpr int kSmemBytes = kCopyWalkOff + kWarps * 64;
   static_assert(kGran % 128 == 0 && kPiece % 128 == 0 && kStages * kGran >= kPiece && kWarpBytes % 128 == 0 && kCopy % 16 == 0, "copies land on 128-byte boundaries");
   static_assert(!kFp8 || (kStages - 1) * kGran + 2 * kPiece <= kWarpBytes, "room for two pieces of the largest group");
   static_assert(kCtasPerSm * (kSmemBytes + 1024) <= 233472, "shared memory of one SM");
@@ -101,6 +108,7 @@ struct Walk {
   unsigned base, end;
   bool more;
 };
+static_assert(sizeof(Walk) <= 48, "shared memory layout");
 __device__ __forceinline__ void walk_range(Walk& w, unsigned x) {
   w.j = max(0, static_cast<int>(x - w.base) - kUnitCost);
   w.jend = min(w.n, static_cast<int>(w.end - w.base) - kUnitCost);
@@ -396,16 +404,23 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
 
   // ---- copies: a granule per request, a ring of stages per warp -------------------------------------------------
   // Physical block ids are looked up 32 at a time (one per lane), one batch ahead of the copies that need them.
-  Walk w, pw;                                      // where this warp's work is (in share `share`), and where its copies are (in share `ps`)
+  Walk w;                                          // where this warp's work is (in share `share`), and where its copies are (in share `ps`)
   unsigned ps = blockIdx.x;
   w.more = false;
   if (ps < all_shares) share_walk(ps, w);
-  pw = w;
-  if (ps < all_shares) walk_later(ps, pw);
-  const Walk fw = pw;                              // the first unit, and its layer
+  Walk fw = w;
+  if (ps < all_shares) walk_later(ps, fw);                              // the first unit, and its layer
   const int fy = share_layer(ps);
   int ids_a = 0, cnt_a = 0, g_a = 0, y_a = 0, pos_a = 0, ids_b = 0, cnt_b = 0, g_b = 0, y_b = 0;
+  auto prefetch_q = [&](int y, int b, int g) {
+    if (lane < G * D / 64) prefetch_l2(reinterpret_cast<const uint8_t*>(layer(y).q + (static_cast<size_t>(b) * Hq + g * G) * D) + lane * 128);
+  };
+  // (The walk of the copies is looked at once in 32 blocks: it waits in shared memory, not in registers.)
+  Walk* copy_walk = reinterpret_cast<Walk*>(smem + C::kCopyWalkOff + warp * 64);
+  unsigned* copy_share = reinterpret_cast<unsigned*>(copy_walk) + 12;
   auto fetch_ids = [&]() {
+    Walk pw = *copy_walk;
+    unsigned ps = *copy_share;
     cnt_b = 0;
     if (!pw.more) return;
     cnt_b = min(32, pw.jend - pw.j);
@@ -413,7 +428,13 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
     y_b = share_layer(ps);
     ids_b = lane < cnt_b ? p.block_table[static_cast<size_t>(pw.b) * p.max_blocks_per_seq + pw.u + pw.j + lane] : 0;
     pw.j += cnt_b;
-    if (pw.j >= pw.jend) walk_on(ps, pw);
+    if (pw.j >= pw.jend) {
+      walk_on(ps, pw);
+      if (pw.more) prefetch_q(share_layer(ps), pw.b, pw.g);
+    }
+    __syncwarp();
+    if (lane == 0) { *copy_walk = pw; *copy_share = ps; }
+    __syncwarp();
   };
   auto take_ids = [&]() {
     ids_a = ids_b; cnt_a = cnt_b; g_a = g_b; y_a = y_b; pos_a = 0;
@@ -448,7 +469,9 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
   const int tok0 = C::kFp8 ? 4 * (row >> 1) + (row & 1) : row;       // token of this lane's logits 0 and 1; 2 and 3: tok0 + kTokStep
   constexpr int kTokStep = C::kFp8 ? 2 : 8;
 
-  // raw query rows, loaded a unit ahead: this lane's head is `row`, its dims as the contraction takes them
+  // raw query rows: this lane's head is `row`, its dims as the contraction takes them.  (The first unit's are requested ahead of
+  // its blocks; those of later units come from L2, where they have been requested with the unit's first block ids: registers
+  // that hold them through the unit before cost more than the trip.)
   uint32_t qraw[kQSteps][2];
   auto load_q = [&](int y, int b, int g) {
     const bool live = row < G;
@@ -469,13 +492,14 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
   // the kernel before may still write it: L2 is where its stores arrive).
   if (fw.more) {
     const LayerPtrs& io = layer(fy);
-    const uint8_t* qrows = reinterpret_cast<const uint8_t*>(io.q + (static_cast<size_t>(fw.b) * Hq + fw.g * G) * D);
-    if (lane < G * D / 64) prefetch_l2(qrows + lane * 128);
+    prefetch_q(fy, fw.b, fw.g);
     if (io.k_new != nullptr && lane < 3) {
       const long long at = static_cast<long long>(fw.b) * p.kv_token_stride + fw.g * D;
       prefetch_l2(lane == 0 ? static_cast<const void*>(io.k_new + at) : lane == 1 ? static_cast<const void*>(io.v_new + at) : static_cast<const void*>(io.slot_mapping + fw.b));
     }
   }
+  if (lane == 0) { *copy_walk = fw; *copy_share = ps; }
+  __syncwarp();
   fetch_ids();
 #pragma unroll 1
   for (int step = 0; step < 2; ++step) {
@@ -504,14 +528,6 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
 
   const int d0 = lane * 4;
   const bool on = d0 < D;
-  // A warp of a launch over several layers whose wait has run out leaves without another word to the others (its record may
-  // still be in use, and an arrival ahead of its time would complete a phase that others have not reached): their waits for
-  // it run out in turn.
-  auto give_up = [&]() -> bool {
-    dead = __any_sync(0xffffffffu, dead);
-    if (dead && lane == 0) atomicCAS(p.status, 0, COOPT_ERR_TIMEOUT);
-    return dead;
-  };
   uint32_t round = 0;
 #pragma unroll 1
   for (unsigned share = blockIdx.x; share < all_shares; share += gridDim.x, ++round) {
@@ -522,6 +538,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
   rec.flags = 0;
 #pragma unroll 1
   while (w.more) {
+    if (consumed != 0) load_q(y, w.b, w.g);
     // ---- query operand: f16 (exact: rows scaled by a power of two), or bf16 as it is -------------------------------
     uint32_t qf[kQSteps][2];
     float qs[2];                                   // logit scale of heads 2 quad, 2 quad + 1
@@ -548,13 +565,6 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
       qs[0] = qs[1] = p.sm_scale_log2;
     }
     COOPT_TRACE_CYCLES(p.trace, kTrQuery, tid == 0 && consumed == 0 && qf[0][0] != 0x12345u);
-    {
-      Walk nx = w;
-      unsigned ns = share;
-      walk_on(ns, nx);
-      if (nx.more) load_q(share_layer(ns), nx.b, nx.g);
-    }
-
     float o[D / 16][4];
 #pragma unroll
     for (int t = 0; t < D / 16; ++t)
@@ -585,7 +595,6 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
       }
       if (!dead && !mbar_wait_bounded(&bars[out_stage], out_phase)) {
         dead = true;
-        atomicCAS(p.status, 0, COOPT_ERR_TIMEOUT);
       }
       dead = __any_sync(0xffffffffu, dead);
       COOPT_TRACE_CYCLES(p.trace, kTrFirstLanded, tid == 0 && consumed == 0);
@@ -755,10 +764,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
       }
     } else {
       // a piece: into shared memory, once the pieces of the share before are of no more use
-      if (L > 1) {
-        if (round > 0 && rec.flags == 0 && !dead && !mbar_wait_bounded(bar_merged, (round - 1) & 1u)) dead = true;
-        if (give_up()) break;
-      }
+      if (L > 1 && round > 0 && rec.flags == 0 && !dead && !mbar_wait_bounded(bar_merged, (round - 1) & 1u)) dead = true;
       float* piece = reinterpret_cast<float*>(ring + (starts ? piece1_off : piece0_off));
       float* at = piece + 2 * quad * C::kPieceStride + row;
 #pragma unroll
@@ -784,55 +790,73 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
     __syncthreads();
   } else {
     if (round > 0 && rec.flags == 0 && !dead && !mbar_wait_bounded(bar_merged, (round - 1) & 1u)) dead = true;   // (its record is still in use)
-    if (give_up()) break;
-    if (lane == 0) recs[warp] = rec;
-    __syncwarp();
-    if (lane == 0) mbar_arrive(bar_pieces);
-    if (!mbar_wait_bounded(bar_pieces, round & 1u)) dead = true;
-    if (give_up()) break;
+    // A warp whose wait has run out leaves without another word to the others (its record may still be in use, and an arrival
+    // ahead of its time would complete a phase that others have not reached): their waits for it run out in turn.
+    dead = __any_sync(0xffffffffu, dead);
+    if (dead) break;
+    if (lane == 0) {
+      recs[warp] = rec;
+      mbar_arrive(bar_pieces);
+    }
+    dead = !mbar_wait_bounded(bar_pieces, round & 1u);
+    dead = __any_sync(0xffffffffu, dead);
+    if (dead) break;
   }
   COOPT_TRACE_CYCLES(p.trace, kTrStreamed, tid == 0);
 
   // ---- units that several warps share: merged by log-sum-exp, one (unit, head) per warp ---------------------------------
-  // One head of a piece that other shares hold the rest of goes to the workspace; the warp that delivers the last piece gets
-  // `true` and all pieces merged.  The first piece of a unit sits in the odd slot of its share, the others in the even ones.
-  auto deliver = [&](Acc& a, int region, bool first_piece, int cta_f, int pieces, int h) -> bool {
-    const size_t base = static_cast<size_t>(region) * 2 * p.shares;
-    const size_t at = (base + 2 * v_share + (first_piece ? 1 : 0)) * G + h;
+  // A head of a piece that other shares hold the rest of goes to the workspace, and is counted; who counts the last one takes
+  // them all and finishes the unit.  The first piece of a unit lies in the odd slot of its share, the others in the even ones.
+  auto slot_of = [&](int region, int cta, bool first, int h) -> size_t { return ((static_cast<size_t>(region) * p.shares + cta) * 2 + (first ? 1 : 0)) * G + h; };
+  auto leave_piece = [&](const Acc& a, size_t at) {
     const float dinv = a.den > 0.0f ? 1.0f / a.den : 0.0f;
     if (on) *reinterpret_cast<float4*>(p.run_o + at * D + d0) = make_float4(a.num.x * dinv, a.num.y * dinv, a.num.z * dinv, a.num.w * dinv);
     if (lane == 0) { p.run_m[at] = a.M; p.run_l[at] = a.den; }
-    __syncwarp();
-    int done = 0;
-    if (lane == 0) {
-      // release (this piece is visible before the count moves) and acquire (the other pieces are visible before they are read)
-      int* counter = p.counters + (region * p.shares + cta_f) * kMaxGroup + h;
-      int old;
-      asm volatile("atom.add.acq_rel.gpu.s32 %0, [%1], 1;" : "=r"(old) : "l"(counter) : "memory");
-      done = old == pieces - 1;
-      if (done) *counter = 0;            // ready for the next call
-    }
-    if (!__shfl_sync(0xffffffffu, done, 0)) return false;
+  };
+  auto count_piece = [&](int region, int cta_f, int pieces, int h) -> bool {      // one lane, behind the others' stores
+    // release (this piece is visible before the count moves) and acquire (the other pieces are visible before they are read)
+    int* counter = p.counters + (region * p.shares + cta_f) * kMaxGroup + h;
+    int old;
+    asm volatile("atom.add.acq_rel.gpu.s32 %0, [%1], 1;" : "=r"(old) : "l"(counter) : "memory");
+    if (old != pieces - 1) return false;
+    *counter = 0;                        // ready for the next call
+    return true;
+  };
+  auto take_pieces = [&](Acc& a, int region, int cta_f, int pieces, int h) {
     acc_clear(a);
-    auto slot = [&](int c) -> size_t { return (base + 2 * (cta_f + c) + (c == 0 ? 1 : 0)) * G + h; };
     for (int c0 = 0; c0 < pieces; c0 += 32) {
       const int n = min(32, pieces - c0);
+      auto slot = [&](int c) { return slot_of(region, cta_f + c, c == 0, h); };
       const float m = lane < n ? __ldcg(p.run_m + slot(c0 + lane)) : 0.0f, l = lane < n ? __ldcg(p.run_l + slot(c0 + lane)) : 0.0f;
       acc_merge<true>(a, n, m, l, on, [&](int k) { return p.run_o + slot(c0 + k) * D + d0; });
     }
-    return true;
   };
   auto store_out = [&](const Acc& a, int b, int g, int h) {
     const float dinv = a.den > 0.0f ? 1.0f / a.den : 0.0f;
     if (on) *reinterpret_cast<uint2*>(layer(y).out + (static_cast<size_t>(b) * Hq + g * G + h) * D + d0) =
         make_uint2(pack_bf16x2(a.num.x * dinv, a.num.y * dinv), pack_bf16x2(a.num.z * dinv, a.num.w * dinv));
   };
+  auto finish = [&](const Acc& a, int b, int g, int h, int u) {
+    if (p.chunk_blocks == 0) {
+      store_out(a, b, g, h);
+    } else {
+      const size_t at = (static_cast<size_t>(b) * Hq + g * G + h) * p.max_chunks + u / ln.chunk;
+      const float dinv = a.den > 0.0f ? 1.0f / a.den : 0.0f;
+      if (on) *reinterpret_cast<float4*>(p.part_o + at * D + d0) = make_float4(a.num.x * dinv, a.num.y * dinv, a.num.z * dinv, a.num.w * dinv);
+      if (lane == 0) { p.part_m[at] = a.M * kLn2; p.part_l[at] = a.den * kUnshift; }
+    }
+  };
+  const int region = L > 1 ? y : p.chunk_blocks > 0 ? 1 : 0;
   const int flags = lane < C::kWarps ? recs[lane].flags : 0;
   const unsigned has0 = __ballot_sync(0xffffffffu, flags & kHas0), ends0 = __ballot_sync(0xffffffffu, flags & kEnds0), has1 = __ballot_sync(0xffffffffu, flags & kHas1);
   // a chain: the warps that hold pieces of one unit, the first of them `from` (kind 0: the unit began in another CTA)
   const int chains = static_cast<int>(has0 & 1u) + __popc(has1);
+  // What a warp's tasks leave in the workspace is counted at once, lane i for task i: the trips there and back (about 2 us)
+  // are made side by side.
+  static_assert((C::kWarps + 1) * kMaxGroup <= 32 * C::kWarps, "a task per lane");
+  int left_cta = 0, left_pieces = 0, left_b = 0, left_gh = 0, left_u = 0;
 #pragma unroll 1
-  for (int task = warp; task < chains * G; task += C::kWarps) {
+  for (int task = warp, i = 0; task < chains * G; task += C::kWarps, ++i) {
     const int ci = task / G, h = task - ci * G;
     const int kind = (has0 & 1u) && ci == 0 ? 0 : 1;
     unsigned rest = has1;
@@ -856,22 +880,25 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
     if (!(kind && closed)) {
       const unsigned first = unit_place(ln, b, g, u) + kUnitCost;
       const int nu = unit_blocks(ln, line_blocks(ln, b), u), cta_f = first / T;
-      if (!deliver(a, L > 1 ? y : p.chunk_blocks > 0 ? 1 : 0, kind != 0, cta_f, static_cast<int>((first + nu - 1) / T) - cta_f + 1, h)) continue;
+      leave_piece(a, slot_of(region, v_share, kind != 0, h));
+      if (lane == i) { left_cta = cta_f; left_pieces = static_cast<int>((first + nu - 1) / T) - cta_f + 1; left_b = b; left_gh = g * G + h; left_u = u; }
+      continue;
     }
-    if (p.chunk_blocks == 0) {
-      store_out(a, b, g, h);
-    } else {
-      const size_t at = (static_cast<size_t>(b) * Hq + g * G + h) * p.max_chunks + u / ln.chunk;
-      const float dinv = a.den > 0.0f ? 1.0f / a.den : 0.0f;
-      if (on) *reinterpret_cast<float4*>(p.part_o + at * D + d0) = make_float4(a.num.x * dinv, a.num.y * dinv, a.num.z * dinv, a.num.w * dinv);
-      if (lane == 0) { p.part_m[at] = a.M * kLn2; p.part_l[at] = a.den * kUnshift; }
-    }
+    finish(a, b, g, h, u);
   }
-  if (L > 1) {
+  {
     __syncwarp();
-    if (lane == 0) mbar_arrive(bar_merged);
-    continue;
+    if (L > 1 && lane == 0) mbar_arrive(bar_merged);
+    unsigned last = __ballot_sync(0xffffffffu, left_pieces > 0 && count_piece(region, left_cta, left_pieces, left_gh % G));
+#pragma unroll 1
+    for (; last != 0; last &= last - 1) {
+      const int i = __ffs(last) - 1, gh = __shfl_sync(0xffffffffu, left_gh, i), g = gh / G;
+      Acc a;
+      take_pieces(a, region, __shfl_sync(0xffffffffu, left_cta, i), __shfl_sync(0xffffffffu, left_pieces, i), gh - g * G);
+      finish(a, __shfl_sync(0xffffffffu, left_b, i), g, gh - g * G, __shfl_sync(0xffffffffu, left_u, i));
+    }
   }
+  if (L > 1) continue;
   if (p.chunk_blocks == 0) break;
 
   // ---- Opt-Pa: what this CTA holds of a (sequence, kv head) is merged over its chunks, then with the other CTAs' shares ----
@@ -917,7 +944,11 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
         const unsigned first = unit_place(ln, b, g, 0) + (whole ? 0 : kUnitCost);
         const unsigned last = unit_place(ln, b, g, u_last) + (whole ? 0 : kUnitCost + (nb - u_last) - 1);
         const int cta_f = first / T;
-        if (!deliver(a, 0, run_begins, cta_f, static_cast<int>(last / T) - cta_f + 1, h)) continue;
+        const int pieces = static_cast<int>(last / T) - cta_f + 1;
+        leave_piece(a, slot_of(0, share, run_begins, h));
+        __syncwarp();
+        if (!__shfl_sync(0xffffffffu, lane == 0 && count_piece(0, cta_f, pieces, h), 0)) continue;
+        take_pieces(a, 0, cta_f, pieces, h);
       }
       store_out(a, b, g, h);
     }
@@ -927,6 +958,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
   COOPT_TRACE_NS(p.trace, kTrExitNs, tid == 0);
   // a warp that gave up still has copies in flight: they get a bounded time to land
   if (dead) {
+    if (lane == 0) atomicCAS(p.status, 0, COOPT_ERR_TIMEOUT);
     for (; consumed < issued; ++consumed) {
       mbar_wait_bounded(&bars[out_stage], out_phase);
       if (++out_stage == stages) { out_stage = 0; out_phase ^= 1u; }
