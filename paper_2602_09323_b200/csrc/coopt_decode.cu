@@ -382,11 +382,24 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
   };
   auto share_layer = [&](unsigned s) -> int { return L == 1 ? 0 : s / shares; };
   auto share_walk = [&](unsigned s, Walk& w) {                          // this warp's part of share s
-    unsigned lo, hi;
-    share_range(L == 1 ? s : s % shares, lo, hi);
-    const unsigned mine = hi > lo ? hi - lo : 0u, Tw = (mine + C::kWarps - 1) / C::kWarps;
-    const unsigned my_lo = min(hi, lo + warp * Tw);
-    walk_start(ln, w, my_lo, min(hi, my_lo + Tw), lane);
+    // (Three look-ups at most, in a loop: code that a CTA runs once is bound by the fetch of its instructions.)
+    unsigned lo = (L == 1 ? s : s % shares) * T, hi = min(places, lo + T), x = lo;
+    w.more = false;
+#pragma unroll 1
+    for (int step = whole ? 0 : 2; step < 3; ++step) {
+      if (step == 1) x = hi;
+      if (step == 2) {
+        const unsigned mine = hi > lo ? hi - lo : 0u, Tw = (mine + C::kWarps - 1) / C::kWarps;
+        x = min(hi, lo + warp * Tw);
+        w.end = min(hi, x + Tw);
+        if (x >= w.end) return;
+      }
+      if (x < places) walk_unit(ln, w, x, lane);
+      const unsigned next = x >= places || w.base == x ? x : w.base + w.n + kUnitCost;
+      if (step == 0) lo = next;
+      if (step == 1) hi = next;
+    }
+    walk_range(w, x);
   };
   // this warp's first unit in share s or, over several layers, in a later one (s moves there); and its next one
   auto walk_later = [&](unsigned& s, Walk& w) {
