@@ -393,9 +393,9 @@ int coopt_decode_layers(const coopt_layer_io* layers, int32_t num_layers, int64_
   const bool long_layers = static_cast<long long>(batch) * c0->num_kv_heads * max_blocks_per_seq > 256ll * num_sms();
   for (int32_t l = 0; l < num_layers && rc == COOPT_OK;) {
     // Layers whose buffers are apart go into one launch where a layer gives a share few places: what a launch costs once is
-    // then much of it (8 sequences of 1..28 tokens, eight layers: 64 / 19 us; 32 x 2048 tokens, 230 places a share: 249 / 241).
-    // With 290 places (24 sequences, G = 8, four layers) separate launches take 92 us, one 95: a ring of two blocks a warp is
-    // all that the pieces of eight heads leave room for there.
+    // then much of it (8 sequences of 1..28 tokens, eight layers: 64 / 10 us; 32 x 2048 tokens, 230 places a share: 249 / 230).
+    // With 290 places (24 sequences, G = 8, four layers) separate launches and one take 92 us: a ring of two blocks a warp is all
+    // that the pieces of eight heads leave room for there.
     int n = long_layers ? 1 : std::min(num_layers - l, kManyLayers);
     while (n > 1 && workspace_bytes < workspace_need(batch, num_q_heads, c0->num_kv_heads, c0->head_dim, max_blocks_per_seq, 0, n)) --n;
     const bool apart = layers_are_apart(layers + l, n, kv_token_stride, block_table, max_blocks_per_seq, context_lens, batch, num_q_heads);

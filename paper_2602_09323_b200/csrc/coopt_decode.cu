@@ -18,9 +18,9 @@
 // (The kernel before this one ran the contractions on tcgen05.mma, 128 tokens at a time, with two softmax teams per
 // CTA and a plan of every CTA's blocks made by a kernel of its own.  The tensor core was 21 % busy with columns that
 // are mostly padding, and what bounded the launch were the hand-overs between its roles, per unit and at both ends.
-// Before / now: one layer of 56 heads over 8 kv heads, 8 sequences of 1..28 tokens 60 / 8 us; 24 sequences of
-// 300..4000 tokens, G = 8, 46 / 23 us a layer; 32 x 2048 tokens, G = 5, 35 / 30 us; 64 sequences of 128..8192 tokens,
-// 121 / 105 us; 120 sequences of 5..900 tokens at head_dim 64, plan included, 56 / 17 us.)
+// Before / now: one layer of 56 heads over 8 kv heads, 8 sequences of 1..28 tokens 60 / 7.5 us; 24 sequences of
+// 300..4000 tokens, G = 8, 46 / 23 us a layer; 32 x 2048 tokens, G = 5, 35 / 29 us; 64 sequences of 128..8192 tokens,
+// 121 / 104 us; 120 sequences of 5..900 tokens at head_dim 64, plan included, 56 / 17 us.)
 //
 // A launch of 32 x 2048 tokens streams at 6.4 TB/s from its first copies, 3 us after a CTA's first instruction, to the end
 // of its last block, 5 us before the CTA's last; code that runs once costs about four cycles an instruction to fetch.
@@ -364,14 +364,28 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
   // not depend on how many layers share the launch.  CTA i takes the shares i, i + grid, .. of all layers, one layer
   // behind the other; the copies of a share are under way while the pieces of the one before are merged.
   const unsigned places = Hkv * pre[B];
-  const unsigned T = max(static_cast<unsigned>(kMinPlaces), (places + p.shares - 1) / p.shares);
-  const unsigned shares = (places + T - 1) / T, all_shares = L == 1 ? shares : shares * p.layers;
+  unsigned T = max(static_cast<unsigned>(kMinPlaces), (places + p.shares - 1) / p.shares);
   // Shared units cost a trip through the workspace at the end of a share.  Where units are short, a share holds the units
   // that begin among its places whole instead.  (In chunk mode every share between the first and the last of a (sequence,
   // kv head) has to hold a chunk of it.)
   int most = 0;
   for (int k = 0; k < C::kWarps; ++k) most = max(most, misc[17 + k]);
   const bool whole = most * (D / 64) <= (T == kMinPlaces ? kWholeUnitsIdle : kWholeUnits) && (p.chunk_blocks == 0 || most + kUnitCost <= static_cast<int>(T));
+  // Where they are very short, a warp holds whole what begins among its places, and nothing is merged.  Nor does a unit's
+  // result depend on the shares then: they are made as large as it takes for every CTA to have one at most.
+  const bool solo = whole && p.chunk_blocks == 0 && most <= kSoloUnits;
+  if (L > 1 && solo) {
+    const unsigned m = max(1u, gridDim.x / p.layers);
+    T = max(T, (places + m - 1) / m);
+  }
+  const unsigned shares = (places + T - 1) / T, all_shares = L == 1 ? shares : shares * p.layers;
+  // What is looked at seldom waits in shared memory, a copy for every warp, and not in registers that the loop over blocks
+  // needs: the walk of the copies (once in 32 blocks), its share, and how shares are cut.
+  Walk* copy_walk = reinterpret_cast<Walk*>(smem + C::kCopyWalkOff + warp * 64);
+  unsigned* copy_share = reinterpret_cast<unsigned*>(copy_walk) + 12;
+  volatile unsigned* cut = copy_share + 1;                              // [0] bit 0: whole, bit 1: solo; [1] T
+  if (lane == 0) { cut[0] = (whole ? 1u : 0u) | (solo ? 2u : 0u); cut[1] = T; }
+  __syncwarp();
   auto share_range = [&](unsigned v, unsigned& lo, unsigned& hi) {       // places of a layer's share v
     lo = v * T;
     hi = min(places, lo + T);
@@ -383,15 +397,22 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
   auto share_layer = [&](unsigned s) -> int { return L == 1 ? 0 : s / shares; };
   auto share_walk = [&](unsigned s, Walk& w) {                          // this warp's part of share s
     // (Three look-ups at most, in a loop: code that a CTA runs once is bound by the fetch of its instructions.)
+    const unsigned T = cut[1], mode = cut[0];
+    const bool solo = (mode & 2u) != 0;
     unsigned lo = (L == 1 ? s : s % shares) * T, hi = min(places, lo + T), x = lo;
     w.more = false;
+    if (solo) {
+      const unsigned Tw = (T + C::kWarps - 1) / C::kWarps;
+      x = min(hi, lo + warp * Tw);
+      hi = min(hi, x + Tw);
+    }
 #pragma unroll 1
-    for (int step = whole ? 0 : 2; step < 3; ++step) {
+    for (int step = (mode & 1u) != 0 ? 0 : 2; step < 3; ++step) {
       if (step == 1) x = hi;
       if (step == 2) {
         const unsigned mine = hi > lo ? hi - lo : 0u, Tw = (mine + C::kWarps - 1) / C::kWarps;
-        x = min(hi, lo + warp * Tw);
-        w.end = min(hi, x + Tw);
+        x = solo ? lo : min(hi, lo + warp * Tw);
+        w.end = solo ? hi : min(hi, x + Tw);
         if (x >= w.end) return;
       }
       if (x < places) walk_unit(ln, w, x, lane);
@@ -428,9 +449,6 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
   auto prefetch_q = [&](int y, int b, int g) {
     if (lane < G * D / 64) prefetch_l2(reinterpret_cast<const uint8_t*>(layer(y).q + (static_cast<size_t>(b) * Hq + g * G) * D) + lane * 128);
   };
-  // (The walk of the copies is looked at once in 32 blocks: it waits in shared memory, not in registers.)
-  Walk* copy_walk = reinterpret_cast<Walk*>(smem + C::kCopyWalkOff + warp * 64);
-  unsigned* copy_share = reinterpret_cast<unsigned*>(copy_walk) + 12;
   auto fetch_ids = [&]() {
     Walk pw = *copy_walk;
     unsigned ps = *copy_share;
@@ -798,6 +816,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
   }
   COOPT_TRACE_CYCLES(p.trace, kTrWarpEnd + warp, lane == 0);
   COOPT_TRACE_VALUE(p.trace, kTrBlocks, tid == 0, consumed);
+  if ((cut[0] & 2u) != 0) break;         // solo: one share a CTA
   if (L == 1) {
     if (lane == 0) recs[warp] = rec;
     __syncthreads();

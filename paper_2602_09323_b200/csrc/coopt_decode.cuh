@@ -28,6 +28,10 @@ constexpr int kCtasPerSm = 1;
 constexpr int kMinPlaces = 16;        // smallest share
 constexpr int kWholeUnits = 32;       // units of at most so many blocks (head_dim 64: twice) are not cut between shares
 constexpr int kWholeUnitsIdle = 192;  // .. where the call does not fill the device
+// Units of at most so many blocks are not cut between warps either.  Eight layers of 40 sequences, 4 kv heads, us against units
+// spread over a CTA's warps: 1 block 10.6 / 27.6, 4 blocks 13.6 / 44, 8 blocks 17.5 / 65; one layer: 8.8 / 8.8, 11.7 / 10.5,
+// 14.0 / 10.5.
+constexpr int kSoloUnits = 4;
 constexpr int kNoChunks = 1 << 30;    // "blocks per chunk" of a call without chunks
 
 // A plan: header, the clamped context lengths int32[batch] (padded to 16 bytes), the block table

@@ -107,3 +107,9 @@ def test_layers_in_one_launch_equal_layers_one_by_one(hq, hkv, d, lens, n, how):
     for y in range(n):
         assert torch.equal(want_bytes[y], got_bytes[y]), f"layer {y}: cache bytes"
         assert torch.equal(got[y], want[y]), f"layer {y}: outputs"
+
+
+@pytest.mark.parametrize("lens", [[64, 0, 1, 49, 16], [1 + i % 64 for i in range(300)], [65, 3, 64]])
+@pytest.mark.parametrize("hq,hkv,d,n", [(8, 8, 128, 8), (10, 2, 64, 3)])
+def test_layers_of_units_around_the_most_that_a_warp_holds_whole(hq, hkv, d, n, lens):
+    test_layers_in_one_launch_equal_layers_one_by_one(hq, hkv, d, lens, n, "apart")
