@@ -102,6 +102,7 @@ __device__ __forceinline__ int unit_blocks(const Line& ln, int nb, int u) { retu
 
 // A walk over the units of the places [x, end): unit (b, g, first block u, n blocks), of which the blocks [j, jend)
 // (counted from u) belong to the walker.
+constexpr int kSomeEmpty = 1 << 28;      // added to a length: a sequence's context is empty
 struct Walk {
   int b, g, nb, u, n;
   int j, jend;
@@ -318,7 +319,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
     constexpr int kPer = (kMaxBatch + C::kThreads - 1) / C::kThreads;
     const int chunk = p.chunk_blocks > 0 ? p.chunk_blocks : kNoChunks;
     unsigned v[kPer], sum = 0;
-    int most = 0, key = p.plan_key;
+    int most = 0, empty = 0, key = p.plan_key;
     if (tid == 0 && p.plan != nullptr) key = p.plan->key;
 #pragma unroll
     for (int k = 0; k < kPer; ++k) {
@@ -331,8 +332,9 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
       v[k] = nb + units * kUnitCost;
       sum += v[k];
       most = max(most, min(nb, chunk));
+      if (b < B && nb == 0) empty = kSomeEmpty;
     }
-    most = __reduce_max_sync(0xffffffffu, most);
+    most = __reduce_max_sync(0xffffffffu, most + empty);
     unsigned inc = sum;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -369,7 +371,12 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
   // that begin among its places whole instead.  (In chunk mode every share between the first and the last of a (sequence,
   // kv head) has to hold a chunk of it.)
   int most = 0;
-  for (int k = 0; k < C::kWarps; ++k) most = max(most, misc[17 + k]);
+  bool none_empty = true;
+  for (int k = 0; k < C::kWarps; ++k) {
+    const int m = misc[17 + k];
+    none_empty = none_empty && m < kSomeEmpty;
+    most = max(most, m & (kSomeEmpty - 1));
+  }
   const bool whole = most * (D / 64) <= (T == kMinPlaces ? kWholeUnitsIdle : kWholeUnits) && (p.chunk_blocks == 0 || most + kUnitCost <= static_cast<int>(T));
   // Where they are very short, a warp holds whole what begins among its places, and nothing is merged.  Nor does a unit's
   // result depend on the shares then: they are made as large as it takes for every CTA to have one at most.
@@ -378,13 +385,17 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
     const unsigned m = max(1u, gridDim.x / p.layers);
     T = max(T, (places + m - 1) / m);
   }
-  const unsigned shares = (places + T - 1) / T, all_shares = L == 1 ? shares : shares * p.layers;
+  // Where a layer does not fill the device, its shares are its units: as many at a time as there are CTAs, of whichever layer.
+  // (Three layers of 17 sequences of 854 tokens, two kv heads: 35.4 us with shares of 16 places, most of them empty and the
+  // others unevenly spread over the CTAs, 14.1 so; eight of 7 sequences of 272..544 tokens, four kv heads: 29.7 / 20.5.)
+  const bool by_unit = whole && !solo && p.chunk_blocks == 0 && T == kMinPlaces && none_empty && B * Hkv <= p.shares;
+  const unsigned shares = by_unit ? B * Hkv : (places + T - 1) / T, all_shares = L == 1 ? shares : shares * p.layers;
   // What is looked at seldom waits in shared memory, a copy for every warp, and not in registers that the loop over blocks
   // needs: the walk of the copies (once in 32 blocks), its share, and how shares are cut.
   Walk* copy_walk = reinterpret_cast<Walk*>(smem + C::kCopyWalkOff + warp * 64);
   unsigned* copy_share = reinterpret_cast<unsigned*>(copy_walk) + 12;
-  volatile unsigned* cut = copy_share + 1;                              // [0] bit 0: whole, bit 1: solo; [1] T
-  if (lane == 0) { cut[0] = (whole ? 1u : 0u) | (solo ? 2u : 0u); cut[1] = T; }
+  volatile unsigned* cut = copy_share + 1;                              // [0] bit 0: whole, bit 1: solo, bit 2: by unit; [1] T
+  if (lane == 0) { cut[0] = by_unit ? 4u : (whole ? 1u : 0u) | (solo ? 2u : 0u); cut[1] = T; }
   __syncwarp();
   auto share_range = [&](unsigned v, unsigned& lo, unsigned& hi) {       // places of a layer's share v
     lo = v * T;
@@ -399,8 +410,14 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
     // (Three look-ups at most, in a loop: code that a CTA runs once is bound by the fetch of its instructions.)
     const unsigned T = cut[1], mode = cut[0];
     const bool solo = (mode & 2u) != 0;
-    unsigned lo = (L == 1 ? s : s % shares) * T, hi = min(places, lo + T), x = lo;
+    const unsigned v = L == 1 ? s : s % shares;
+    unsigned lo = v * T, hi = min(places, lo + T), x = lo;
     w.more = false;
+    if ((mode & 4u) != 0) {
+      const unsigned b = v / Hkv, head = pre[b + 1] - pre[b];
+      lo = Hkv * pre[b] + (v - b * Hkv) * head;
+      hi = lo + head;
+    }
     if (solo) {
       const unsigned Tw = (T + C::kWarps - 1) / C::kWarps;
       x = min(hi, lo + warp * Tw);

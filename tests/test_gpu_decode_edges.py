@@ -113,3 +113,10 @@ def test_layers_in_one_launch_equal_layers_one_by_one(hq, hkv, d, lens, n, how):
 @pytest.mark.parametrize("hq,hkv,d,n", [(8, 8, 128, 8), (10, 2, 64, 3)])
 def test_layers_of_units_around_the_most_that_a_warp_holds_whole(hq, hkv, d, n, lens):
     test_layers_in_one_launch_equal_layers_one_by_one(hq, hkv, d, lens, n, "apart")
+
+
+@pytest.mark.parametrize("lens", [[70, 300, 900, 3072], [80, 176, 3073], [70, 0, 300], [200] * 74])
+@pytest.mark.parametrize("d,n", [(128, 5), (64, 2)])
+def test_layers_whose_shares_are_their_units(d, n, lens):
+    """On both sides of the longest unit that is held whole, with an empty context, and with as many units as there are CTAs."""
+    test_layers_in_one_launch_equal_layers_one_by_one(6, 2, d, lens, n, "apart")
