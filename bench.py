@@ -274,11 +274,11 @@ def run_other_workload(args):
         # flops each.  The peak for that mix is the harmonic combination of the measured sustained bf16 rate (f16 has
         # the same nominal rate) and twice that rate for E4M3 (nominal fp8 : bf16 ratio): 4/3 of the bf16 rate.
         # `achieved` counts the attention's own flops (4 D per visible (query, key, head)), not the extra instructions
-        # of the second query term and of the second walk.
+        # of the second query term.
         bf16_peak = peaks["bf16_tflops_sustained"] if peaks else 1400.0
         peak = bf16_peak * 4.0 / 3.0
         achieved = flops / (kernel_ms * 1e-3) / 1e12
-        roofline = {"bound": "tensor", "kernel": "paged_prefill_umma_kernel", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+        roofline = {"bound": "tensor", "kernel": "paged_prefill_kernel<128>", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                     "frac": achieved / peak,
                     "peak_source": ("measured sustained bf16 x 4/3 (half the flops on E4M3 operands at twice the bf16 rate, "
                                     "half on f16 operands)" if peaks else "fallback x 4/3"),
@@ -289,7 +289,7 @@ def run_other_workload(args):
         algo = kv_bytes + 2 * q.numel() * 2 + blocks * 4 + B * 4
         peak = peaks["hbm_gbs"] if peaks else FALLBACK_HBM_GBS
         achieved = algo / (kernel_ms * 1e-3) / 1e9
-        kern = "paged_decode_kernel<128> (bf16, mma.sync)" if esize == 2 else "paged_decode_umma_kernel<128,16>"
+        kern = "paged_decode_kernel<128> (bf16)" if esize == 2 else "paged_decode_kernel<128>"
         roofline = {"bound": "hbm", "kernel": kern, "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                     "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)" if peaks else "fallback",
                     "algorithmic_bytes_per_launch": algo, "kernel_us": kernel_ms * 1e3, "traffic": None}
@@ -587,7 +587,7 @@ def main():
     kernel_ms = kernel_b2b_ms
     achieved = algo / (kernel_ms * 1e-3) / 1e9
     clocks = sampler.summary()
-    roofline = {"bound": "hbm", "kernel": "paged_decode_umma_kernel<128,16> (append + attention in one launch)",
+    roofline = {"bound": "hbm", "kernel": "paged_decode_kernel<128> (append + attention in one launch)",
                 "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak, "peak_source": peak_src,
                 "frac_of_nominal_8TBs": achieved / 8000.0,
                 "algorithmic_bytes_per_launch": algo, "kernel_us": kernel_ms * 1e3,
@@ -602,7 +602,7 @@ def main():
     cpu = cpu_baseline(args.cpu_seconds) if world == 1 and args.cpu_seconds > 0 else None
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps, "warmup": warmup,
             "ms_per_step": ms / args.steps, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-            "dtype": "fp8_e4m3 (cache, query and probability terms on tcgen05), f32 accumulate", "data": "synthetic",
+            "dtype": "fp8_e4m3 cache, f16 operands (codes and queries exact) on mma.sync, f32 accumulate", "data": "synthetic",
             "config": {"workload": WORKLOAD, "layers_rotated": NL,
                        "l2": "inputs larger than L2: %d layer caches of %.0f MB visited round-robin" % (NL, algo / 1e6),
                        "step": "coopt_decode_step_planned (one launch: the new token of every sequence written, then attention); "
@@ -708,13 +708,13 @@ def run_layers(args):
     best = res["overlap_previous"]
     line = {"metric": METRIC, "value": BATCH * NL / (best["ms_per_model_step"] * 1e-3), "unit": UNIT, "n_gpus": 1, "steps": steps,
             "warmup": warmup, "ms_per_step": best["ms_per_model_step"], "higher_is_better": True, "scaling": "weak",
-            "vs_baseline": None, "dtype": "fp8_e4m3 (cache, query and probability terms on tcgen05), f32 accumulate",
+            "vs_baseline": None, "dtype": "fp8_e4m3 cache, f16 operands (codes and queries exact) on mma.sync, f32 accumulate",
             "data": "synthetic",
-            "config": {"workload": "llama13b_40layers: " + WORKLOAD, "layers": NL, "step": "coopt_decode_layers: one plan + 40 fused "
-                       "launches per model step; value counts 40 x 32 attention-layer tokens per step",
+            "config": {"workload": "llama13b_40layers: " + WORKLOAD, "layers": NL, "step": "coopt_decode_layers: one plan and a launch for every "
+                       "eight layers per model step; value counts 40 x 32 attention-layer tokens per step",
                        "l2": "40 layer caches of 135 MB visited in turn"},
-            "gpu_launches": steps * (NL + 1), "clocks": sampler.summary(), "e2e": None,
-            "roofline": {"bound": "hbm", "kernel": "paged_decode_umma_kernel<128,16>", "achieved": best["achieved_gbs"], "peak": peak,
+            "gpu_launches": steps * (1 + (NL + 7) // 8), "clocks": sampler.summary(), "e2e": None,
+            "roofline": {"bound": "hbm", "kernel": "paged_decode_kernel<128>", "achieved": best["achieved_gbs"], "peak": peak,
                          "unit": "GB/s", "frac": best["frac_of_measured_peak"], "algorithmic_bytes_per_launch": algo,
                          "kernel_us": best["us_per_layer"], "traffic": None},
             "layers": res, "cpu_baseline": None}
@@ -723,7 +723,7 @@ def run_layers(args):
 
 # dram__bytes_read.sum + dram__bytes_write.sum of one decode launch on this workload, from the
 # ncu capture summarised under profiles/ (None while the kernel is newer than the capture).
-DRAM_TRAFFIC_PER_LAUNCH = 140057856 + 5144320   # dram__bytes_read.sum + dram__bytes_write.sum of one launch (profiles/)
+DRAM_TRAFFIC_PER_LAUNCH = 139022592 + 5901312   # dram__bytes_read.sum + dram__bytes_write.sum of one launch (profiles/)
 
 if __name__ == "__main__":
     main()

@@ -139,7 +139,7 @@ int coopt_paged_decode(const coopt_cache* cache, const void* q, void* out, const
  * COOPT_STATIC_SCRATCH_BYTES inside the library; every device that loads the library holds
  * that much memory until the process exits.  The call itself allocates nothing.
  *   - Arguments as coopt_paged_decode, minus the workspace.
- *   - Problems whose coopt_workspace_bytes(..., chunk_size = 0) exceeds
+ *   - Problems whose pieces of one layer need more than
  *     COOPT_STATIC_SCRATCH_BYTES are refused with COOPT_ERR_WORKSPACE before anything is
  *     enqueued (the LLaMA-13B decode shape needs about 0.8 MB).
  *   - The first call on a device looks up the array's device address; make that first call
@@ -201,9 +201,9 @@ int coopt_decode_step(const coopt_cache* cache, const void* k_new, const void* v
  * Planned decode: the work decomposition of a decode step depends only on the context lengths and the
  * block table, which every layer of a model shares within one step (the decode loop of Section 2 visits
  * the same sequences once per layer; Eq. 9's valid blocks are the same in each).  coopt_decode_plan
- * computes it once -- every CTA's share of the (sequence, kv head, block) list with the physical block
- * ids looked up and range-checked -- and coopt_decode_step_planned / coopt_decode_layers read it in
- * every launch instead of working it out again.
+ * checks and copies what it follows from -- the lengths, and the valid part of the block table with its
+ * ids range-checked -- once, and coopt_decode_step_planned / coopt_decode_layers read that in every launch;
+ * every CTA works out its own share of the (sequence, kv head, block) list.
  *
  * coopt_plan_bytes      bytes of a plan buffer for these shapes (host arithmetic; 0 for bad arguments).
  * coopt_decode_plan     fills `plan` (DEVICE, 16-byte aligned, >= coopt_plan_bytes) on `stream`.
@@ -223,9 +223,9 @@ int coopt_decode_plan(const int32_t* block_table, int32_t max_blocks_per_seq, co
 /*
  * coopt_decode_step_planned -- Algorithm 1 in ONE launch: phase 1 (the new token of every sequence is
  * compressed to FP8 and stored, Eq. 5 skip rule, dynamic per-block scales exactly as coopt_kv_write) and
- * phase 2 with Algorithms 2-3 (attention over the updated cache, exactly as coopt_paged_decode).  The CTA
- * whose share of the plan holds the last block of a (sequence, kv head) writes that sequence's new token
- * into it before its copy engine requests the block; no other CTA reads that block.
+ * phase 2 with Algorithms 2-3 (attention over the updated cache, exactly as coopt_paged_decode).  The warp
+ * that holds the last block of a (sequence, kv head) adds that sequence's new token to it in shared memory
+ * and stores the block back; no other warp reads that block.
  *   plan                       DEVICE, made by coopt_decode_plan for the same batch, num_kv_heads,
  *                              max_blocks_per_seq, chunk_size and num_blocks (a mismatch is reported as
  *                              COOPT_ERR_INVALID_ARG in the workspace status word and the launch does nothing)
@@ -251,12 +251,13 @@ int coopt_decode_step_planned(const coopt_cache* cache, const void* plan, size_t
 
 /*
  * coopt_decode_layers -- the decode loop of Section 2 over the layers of a model for one step: one plan,
- * then one coopt_decode_step_planned launch per layer, enqueued back to back on `stream`.
+ * then the layers' fused steps, enqueued back to back on `stream`: a launch per layer, or one for up to eight
+ * layers whose buffers are apart where a layer is small.  Results are those of one call per layer.
  *   layers        HOST array of num_layers entries; every pointer inside is DEVICE memory: the layer's cache
  *                 (all of one shape), its new token's k/v and slots (all NULL = no append), its q and out
  *   block_table, context_lens, plan, workspace   shared by all layers
- *   flags         COOPT_FLAG_OVERLAP_PREVIOUS lets layer l + 1 start while layer l drains (its copy engine
- *                 reads only the plan and its own cache until layer l has finished)
+ *   flags         COOPT_FLAG_OVERLAP_PREVIOUS lets layer l + 1 start while layer l drains (it reads only the
+ *                 plan and its own cache until layer l has finished)
  * Errors: as the calls it makes; every argument of every layer is checked before anything is launched.
  */
 typedef struct coopt_layer_io {

@@ -92,13 +92,6 @@ __device__ __forceinline__ void gather4_g2s(void* dst, const CUtensorMap* map, i
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-// Named barrier `id` over `count` threads, carrying an OR reduction of a per-thread flag.
-__device__ __forceinline__ bool barrier_or(int id, int count, bool flag) {
-  uint32_t r;
-  asm volatile("{\n .reg .pred p, q;\n setp.ne.b32 p, %3, 0;\n barrier.cta.red.or.pred q, %1, %2, p;\n selp.u32 %0, 1, 0, q;\n}"
-               : "=r"(r) : "r"(id), "r"(count), "r"(static_cast<uint32_t>(flag)) : "memory");
-  return r != 0;
-}
 // Bounded wait that also gives up when another role has already given up.  try_wait lets the hardware
 // park the warp, so waiting warps do not take issue slots from the two single-lane roles that share
 // their schedulers.  The clock and the abort flag are looked at once in 256 unsuccessful tries.

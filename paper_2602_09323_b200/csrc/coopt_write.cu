@@ -24,7 +24,7 @@ __global__ void __launch_bounds__(kWriteWarps * 32) kv_write_fp8_kernel(WritePar
   if (group.n == 0) return;
   const int h = blockIdx.y * kWriteHeads + (warp >> 1);
   if (h >= p.num_kv_heads) return;
-  write_part<D, kBlockSize, kE5m2>(p, group, h, warp & 1, stage[warp], lane);
+  write_part<D, kE5m2>(p, group, h, warp & 1, stage[warp], lane);
 }
 
 // The K part (which = 0) or the V part (which = 1) of a block that is written whole: its 16 tokens follow one another in the
@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(kWriteWarps * 32, 4) kv_write_fp8_span_kernel(
     others &= others - 1;
     find_group_warp(p, base + w, groups[warp], lane);
     __syncwarp();
-    if (groups[warp].n > 0) write_part<D, kBlockSize, kE5m2>(p, groups[warp], h, which, stage[warp], lane);
+    if (groups[warp].n > 0) write_part<D, kE5m2>(p, groups[warp], h, which, stage[warp], lane);
     __syncwarp();
   }
 }

@@ -134,13 +134,13 @@ __device__ __forceinline__ float row_elem(const uint32_t (&w)[kWords], int e) {
 // granule: it stages the part in shared memory (st, 16 * D bytes), applies the scale rule, and
 // writes the part back with 16-byte stores.  A group that fills the whole block in order needs no
 // resident codes; its V part goes from registers straight to memory.
-// kTok bounds the group's size: 16 for the write kernels, 1 for the fused decode step (one new token per
-// sequence); the arithmetic is the same instruction for instruction, so both give the same bytes.
+// (The fused decode step adds its one token by the same rule in its own code, append_token.)
 // kE5m2 selects the code format (the E5M2 ablation): encoder, decoder and the format's largest value.
-template <int D, int kTok = kBlockSize, bool kE5m2 = false>
+template <int D, bool kE5m2>
 __device__ __forceinline__ void write_part(const WriteParams& p, const Group& g, int h, int which, uint8_t* st, int lane) {
   constexpr int kPart = part_bytes(D, true);          // 16 * D bytes
   constexpr int kPerLane = D / 32;                    // dims handled by one lane
+  constexpr int kTok = kBlockSize;
   const int n = g.n;
   bool fresh = false, full = (n == kBlockSize);
 #pragma unroll
@@ -169,7 +169,7 @@ __device__ __forceinline__ void write_part(const WriteParams& p, const Group& g,
   uint32_t raw[kTok][kPerLane / 2];
   const __nv_bfloat16* rows = src + h * D + lane * kPerLane;
   // a whole block of tokens that follow one another in the call (a bulk fill): no look-up of the rows
-  const bool in_a_row = kTok > 1 && n == kTok && g.tok[kTok - 1] - g.tok[0] == kTok - 1;
+  const bool in_a_row = n == kTok && g.tok[kTok - 1] - g.tok[0] == kTok - 1;
   if (vec && in_a_row) {
     const __nv_bfloat16* r0 = rows + static_cast<int64_t>(g.tok[0]) * p.token_stride;
 #pragma unroll
@@ -230,7 +230,7 @@ __device__ __forceinline__ void write_part(const WriteParams& p, const Group& g,
   };
 
   auto encode = [&](auto scaled, auto scaled_k, bool k_signs_from_x) {
-    if (kTok == kBlockSize && full && which == 1) {
+    if (full && which == 1) {
       // V of a whole block: the 16 tokens of one dim are 16 consecutive bytes of the part
 #pragma unroll
       for (int e = 0; e < kPerLane; ++e) {
