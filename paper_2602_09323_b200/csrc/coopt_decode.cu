@@ -380,7 +380,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
   const bool whole = most * (D / 64) <= (T == kMinPlaces ? kWholeUnitsIdle : kWholeUnits) && (p.chunk_blocks == 0 || most + kUnitCost <= static_cast<int>(T));
   // Where they are very short, a warp holds whole what begins among its places, and nothing is merged.  Nor does a unit's
   // result depend on the shares then: they are made as large as it takes for every CTA to have one at most.
-  const bool solo = whole && p.chunk_blocks == 0 && most <= kSoloUnits;
+  const bool solo = whole && p.chunk_blocks == 0 && most <= p.solo_blocks;
   if (L > 1 && solo) {
     const unsigned m = max(1u, gridDim.x / p.layers);
     T = max(T, (places + m - 1) / m);
@@ -1154,6 +1154,7 @@ int launch_decode(const DecodeCall& a, cudaStream_t stream) {
   p.num_kv_heads = c->num_kv_heads;
   p.group = a.num_q_heads / c->num_kv_heads;
   p.num_blocks = c->num_blocks;
+  p.solo_blocks = std::max(kSoloUnits, std::min(kSoloMost, a.batch * c->num_kv_heads / kSoloShare));
   p.sm_scale_log2 = a.sm_scale * kLog2e;
   p.chunk_blocks = a.chunk_size / kBlockSize;
   p.max_chunks = a.chunk_size > 0 ? static_cast<int>((static_cast<long long>(a.max_blocks_per_seq) * kBlockSize + a.chunk_size - 1) / a.chunk_size) : 0;

@@ -32,6 +32,10 @@ constexpr int kWholeUnitsIdle = 192;  // .. where the call does not fill the dev
 // spread over a CTA's warps: 1 block 10.6 / 27.6, 4 blocks 13.6 / 44, 8 blocks 17.5 / 65; one layer: 8.8 / 8.8, 11.7 / 10.5,
 // 14.0 / 10.5.
 constexpr int kSoloUnits = 4;
+// .. or of more, the more units there are to keep the warps busy: one block for every kSoloShare units, at most kSoloMost.
+// (Four kv heads, eight layers / one, cut between warps and not: 160 sequences of 10 blocks 112 / 16.5 and 53 / 16.9 us, 400 of
+// 10 blocks 181 / 26.5 and 126 / 22.2, 400 of 1..16 blocks 175 / 25.8 and 112 / 30.0, 80 of 12 blocks 96 / 14.2 and 41 / 19.8.)
+constexpr int kSoloShare = 48, kSoloMost = 12;
 constexpr int kNoChunks = 1 << 30;    // "blocks per chunk" of a call without chunks
 
 // A plan: header, the clamped context lengths int32[batch] (padded to 16 bytes), the block table
@@ -84,6 +88,7 @@ struct DecodeParams {
   int max_blocks_per_seq;
   int batch, num_q_heads, num_kv_heads, group;
   int num_blocks;
+  int solo_blocks;         // units of at most so many blocks are held whole by a warp
   int order;               // DecodeOrder
   float sm_scale_log2;     // sm_scale * log2(e)
   int chunk_blocks;        // 0 = decode mode

@@ -109,7 +109,8 @@ def test_layers_in_one_launch_equal_layers_one_by_one(hq, hkv, d, lens, n, how):
         assert torch.equal(got[y], want[y]), f"layer {y}: outputs"
 
 
-@pytest.mark.parametrize("lens", [[64, 0, 1, 49, 16], [1 + i % 64 for i in range(300)], [65, 3, 64]])
+@pytest.mark.parametrize("lens", [[64, 0, 1, 49, 16], [1 + i % 64 for i in range(300)], [65, 3, 64], [1 + 7 * i % 192 for i in range(288)],
+                                  [1 + 7 * i % 193 for i in range(193)]])
 @pytest.mark.parametrize("hq,hkv,d,n", [(8, 8, 128, 8), (10, 2, 64, 3)])
 def test_layers_of_units_around_the_most_that_a_warp_holds_whole(hq, hkv, d, n, lens):
     test_layers_in_one_launch_equal_layers_one_by_one(hq, hkv, d, lens, n, "apart")
