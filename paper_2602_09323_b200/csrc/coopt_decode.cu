@@ -102,7 +102,7 @@ __device__ __forceinline__ int unit_blocks(const Line& ln, int nb, int u) { retu
 
 // A walk over the units of the places [x, end): unit (b, g, first block u, n blocks), of which the blocks [j, jend)
 // (counted from u) belong to the walker.
-constexpr int kSomeEmpty = 1 << 28;      // added to a length: a sequence's context is empty
+constexpr int kSomeEmpty = 1 << 28;      // added to a warp's longest unit: a sequence's context is empty
 struct Walk {
   int b, g, nb, u, n;
   int j, jend;
@@ -319,7 +319,8 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
     constexpr int kPer = (kMaxBatch + C::kThreads - 1) / C::kThreads;
     const int chunk = p.chunk_blocks > 0 ? p.chunk_blocks : kNoChunks;
     unsigned v[kPer], sum = 0;
-    int most = 0, empty = 0, key = p.plan_key;
+    int most = 0, key = p.plan_key;
+    bool empty = false;
     if (tid == 0 && p.plan != nullptr) key = p.plan->key;
 #pragma unroll
     for (int k = 0; k < kPer; ++k) {
@@ -332,9 +333,9 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
       v[k] = nb + units * kUnitCost;
       sum += v[k];
       most = max(most, min(nb, chunk));
-      if (b < B && nb == 0) empty = kSomeEmpty;
+      empty = empty || (b < B && nb == 0);
     }
-    most = __reduce_max_sync(0xffffffffu, most + empty);
+    most = __reduce_max_sync(0xffffffffu, most) + (__any_sync(0xffffffffu, empty) ? kSomeEmpty : 0);
     unsigned inc = sum;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {

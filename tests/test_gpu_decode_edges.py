@@ -58,6 +58,24 @@ def test_chunks_that_warps_and_ctas_share(case, chunk):
         assert np.allclose(o_c[b, h, :n], o, rtol=5e-3, atol=2e-2)
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("lens,hkv,chunk", [([0, 0, 9000], 2, 512), ([9000, 0, 0, 9000, 1], 2, 512), ([0, 0, 9000, 0], 2, 512),
+                                            ([0, 0, 131072, 131072], 1, 2048)])
+def test_chunks_longer_than_a_share_beside_empty_contexts(lens, hkv, chunk, d):
+    """The longest chunk counts whatever else is empty: every row is stored, and no piece is left counted for a later call."""
+    w = workloads.make_workload("empties", lens, 2 * hkv, hkv, d, seed=d)
+    cache, kv = helpers.gpu_fill(w), helpers.oracle_fp8_cache(w)
+    ws = binding.new_workspace(w.batch, 2 * hkv, hkv, d, w.block_table.shape[1], chunk, w.batch)
+    for now in (lens, [L * 3 // 5 for L in lens]):
+        out = torch.full(w.q.shape, float("nan"), dtype=torch.bfloat16, device="cuda")
+        binding.paged_chunked(cache, w.q.cuda(), w.cu_q_lens.cuda(), w.block_table.cuda(), torch.tensor(now, dtype=torch.int32).cuda(), chunk, True, w.sm_scale, ws, out=out)
+        torch.cuda.synchronize()
+        assert binding.workspace_status(ws) == 0
+        assert not ws[256:256 + 4 * 16384].any(), "piece counters"
+        ref, _ = attention.paged_attention_chunked(w.q.float().numpy(), kv, w.block_table.numpy(), now, chunk)
+        helpers.check_attention(out, ref, what=f"{now} chunk {chunk}")
+
+
 @pytest.mark.parametrize("hq,hkv,d,lens", [(8, 2, 128, [300, 1, 0, 17, 2048]), (16, 2, 64, [16, 33, 1, 900])])
 @pytest.mark.parametrize("n,how", [(2, "apart"), (3, "chained"), (3, "some append"), (67, "apart"), (2, "one output")])
 def test_layers_in_one_launch_equal_layers_one_by_one(hq, hkv, d, lens, n, how):
