@@ -844,6 +844,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
     // ahead of its time would complete a phase that others have not reached): their waits for it run out in turn.
     dead = __any_sync(0xffffffffu, dead);
     if (dead) break;
+    __syncwarp();                        // every lane's part of the pieces is there (a vote orders no memory)
     if (lane == 0) {
       recs[warp] = rec;
       mbar_arrive(bar_pieces);
@@ -940,6 +941,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
     __syncwarp();
     if (L > 1 && lane == 0) mbar_arrive(bar_merged);
     unsigned last = __ballot_sync(0xffffffffu, left_pieces > 0 && count_piece(region, left_cta, left_pieces, left_gh % G));
+    __syncwarp();                        // the others' pieces, which a lane has acquired, are there for all lanes
 #pragma unroll 1
     for (; last != 0; last &= last - 1) {
       const int i = __ffs(last) - 1, gh = __shfl_sync(0xffffffffu, left_gh, i), g = gh / G;
@@ -998,6 +1000,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
         leave_piece(a, slot_of(0, share, run_begins, h));
         __syncwarp();
         if (!__shfl_sync(0xffffffffu, lane == 0 && count_piece(0, cta_f, pieces, h), 0)) continue;
+        __syncwarp();
         take_pieces(a, 0, cta_f, pieces, h);
       }
       store_out(a, b, g, h);

@@ -660,6 +660,7 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
         }
         ok = __shfl_sync(0xffffffffu, ok, 0);
         if (!ok) break;
+        __syncwarp();                                     // what lane 0 has waited for holds for the lanes that copy
         if (lane < 3 * ngroups && what != 1)
           gather4_g2s(smem + C::kKOff + ks * C::kKSlot + (what == 2 ? C::kCodes + q4 * 4 * kFp8Header : q4 * 4 * C::kPart), map, col, rows[0], rows[1], rows[2], rows[3], &bar_kfull[ks]);
         if (lane == 0) {
@@ -672,6 +673,7 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
         }
         ok = __shfl_sync(0xffffffffu, ok, 0);
         if (!ok) break;
+        __syncwarp();                                     // what lane 0 has waited for holds for the lanes that copy
         if (lane < 3 * ngroups && what == 1)
           gather4_g2s(smem + C::kVOff + vs * C::kCodes + q4 * 4 * C::kPart, map, col, rows[0], rows[1], rows[2], rows[3], &bar_vfull[vs]);
       }

@@ -139,3 +139,10 @@ def test_layers_of_units_around_the_most_that_a_warp_holds_whole(hq, hkv, d, n, 
 def test_layers_whose_shares_are_their_units(d, n, lens):
     """On both sides of the longest unit that is held whole, with an empty context, and with as many units as there are CTAs."""
     test_layers_in_one_launch_equal_layers_one_by_one(6, 2, d, lens, n, "apart")
+
+
+@pytest.mark.parametrize("hq,hkv,d", [(16, 2, 128), (10, 2, 64)])
+def test_pieces_of_many_rounds_are_read_behind_their_writers(hq, hkv, d):
+    """Eight layers a launch whose units are cut between all warps and CTAs, again and again: the same bits every time."""
+    for _ in range(4):
+        test_layers_in_one_launch_equal_layers_one_by_one(hq, hkv, d, [1500 + 61 * i for i in range(16)], 8, "apart")
