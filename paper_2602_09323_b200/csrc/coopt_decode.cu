@@ -27,6 +27,8 @@
 // Registers are what the loop over blocks is short of: the walk of the copies waits in shared memory, and the query rows of
 // a unit are fetched when it starts (eight layers of 21 sequences of 2..60 tokens: 49 / 43.6 us; prefetching the rows into
 // registers at the end of the unit before instead: 49.5).
+#include <float.h>
+
 #include <algorithm>
 
 #include "coopt_decode.cuh"
@@ -713,11 +715,12 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
           m[h] = mn;
           l[h] *= f[h];
         }
-        if (grow) {
-          const float fv = vref * (1.0f / sv);
+        if (grow) {                                // (a reference is a normal number: its reciprocal is one then, too)
+          const float vnew = fmaxf(sv, FLT_MIN);
+          vinv = 1.0f / vnew;
+          const float fv = vref * vinv;
           f[0] *= fv; f[1] *= fv;
-          vref = sv;
-          vinv = 1.0f / sv;
+          vref = vnew;
         }
 #pragma unroll
         for (int t = 0; t < D / 16; ++t) { o[t][0] *= f[0]; o[t][1] *= f[1]; o[t][2] *= f[0]; o[t][3] *= f[1]; }
@@ -773,6 +776,15 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
     }
 
     // ---- end of the unit (or of this warp's piece of it) ----------------------------------------------------------------
+    if constexpr (C::kFp8) {
+      if (__builtin_expect(vref < 0x1p-64f && vref > 0.0f, 0)) {      // (vref / l would lose bits among the subnormals)
+#pragma unroll
+        for (int t = 0; t < D / 16; ++t)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) o[t][e] *= 0x1p-64f;
+        vref *= 0x1p64f;
+      }
+    }
     float inv[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {

@@ -146,3 +146,33 @@ def test_pieces_of_many_rounds_are_read_behind_their_writers(hq, hkv, d):
     """Eight layers a launch whose units are cut between all warps and CTAs, again and again: the same bits every time."""
     for _ in range(4):
         test_layers_in_one_launch_equal_layers_one_by_one(hq, hkv, d, [1500 + 61 * i for i in range(16)], 8, "apart")
+
+
+def _tiny_values(lens, fmt, d, spans):
+    """A workload without outlier channels whose V is N(0, 1) times 2^-124 (a block's scale is then below 2^-128, whose
+    reciprocal is not a number of 32 bits) at the positions ``spans`` of every sequence."""
+    w = workloads.make_workload("tiny", lens, 6, 2, d, seed=d + len(lens), outliers=False)
+    for b, L in enumerate(lens):
+        for lo, hi in spans:
+            rows = slice(w.kv_offsets[b] + min(lo, L), w.kv_offsets[b] + min(hi, L))
+            w.v[rows] = (w.v[rows].float() * 2.0 ** -124).to(torch.bfloat16)
+    kv = helpers.oracle_fp8_cache(w) if fmt == "e4m3" else (*helpers.oracle_fp8_cache(w, fmt=e5m2), e5m2)
+    return w, helpers.gpu_fill(w, dtype=binding.KV_FP8_E4M3 if fmt == "e4m3" else binding.KV_FP8_E5M2), kv
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("fmt", ["e4m3", "e5m2"])
+@pytest.mark.parametrize("lens", [[40, 16, 700, 3000], [9, 64, 33] * 40])
+def test_v_scales_whose_reciprocal_overflows(lens, fmt, d):
+    """Tiny blocks in front of, between and behind ordinary ones count for nothing beside them, and alone they keep their
+    values: bf16 rounding (2^-9 of the result, or half of 2^-133 among subnormals) plus 11 bits of probabilities."""
+    w, cache, kv = _tiny_values(lens, fmt, d, [(0, 32), (64, 80), (1500, 2000)])
+    ref = attention.paged_attention(w.q.float().numpy(), kv, w.block_table.numpy(), w.context_lens)
+    out, _ = helpers.gpu_decode(w, cache)
+    helpers.check_attention(out, ref, what=f"tiny blocks {fmt}")
+    helpers.check_attention(helpers.gpu_decode(w, cache, chunk_size=32)[0], ref, what=f"tiny blocks in chunks {fmt}")
+    w, cache, kv = _tiny_values(lens, fmt, d, [(0, 1 << 20)])
+    ref = attention.paged_attention(w.q.float().numpy(), kv, w.block_table.numpy(), w.context_lens)
+    got = helpers.gpu_decode(w, cache)[0].double().cpu().numpy()
+    bound = 2.0 ** -8 * np.abs(ref) + 2.0 ** -134 + 2.0 ** -11 * float(w.v.float().abs().max())
+    assert np.all(np.abs(got - ref) <= bound), np.max(np.abs(got - ref) / bound)
