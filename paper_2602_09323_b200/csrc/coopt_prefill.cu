@@ -311,8 +311,9 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
         // the row scaled by a power of two into [128, 256), undone on the logits
         int k2 = 0;
         if (amax != 0u) k2 = max(-64, min(64, 134 - static_cast<int>((amax >> 23) & 0xFF)));
-        const float up = __uint_as_float(static_cast<uint32_t>(k2 + 127) << 23);
-        const float down = __shfl_sync(0xffffffffu, p.sm_scale_log2 * __uint_as_float(static_cast<uint32_t>(127 - k2) << 23), row);
+        // (and by the logits' sign: their scale is not negative from here on)
+        const float up = copysignf(__uint_as_float(static_cast<uint32_t>(k2 + 127) << 23), p.sm_scale_log2);
+        const float down = __shfl_sync(0xffffffffu, fabsf(p.sm_scale_log2) * __uint_as_float(static_cast<uint32_t>(127 - k2) << 23), row);
         if (at == o) qscale = down;
         __syncwarp();
 #pragma unroll
@@ -358,7 +359,7 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
       for (int i = 0; i < 2; ++i) tmem_ld32_issue(s_cols + kHalf * buf + 32 * i, s[i]);
       const float4 sk = *reinterpret_cast<const float4*>(sc), lg = *reinterpret_cast<const float4*>(sc + 8), inv = *reinterpret_cast<const float4*>(sc + 16);
       const float v_factor = buf == 0 ? sc[24] : 1.0f;
-      // logit = accumulator * cf of its block (a zero scale: tiny, so that -inf stays -inf)
+      // logit = accumulator * cf of its block (a zero scale: tiny, so that -inf stays -inf; none is negative)
       const float cf[4] = {fmaxf(sk.x * qscale, 1e-30f), fmaxf(sk.y * qscale, 1e-30f), fmaxf(sk.z * qscale, 1e-30f), fmaxf(sk.w * qscale, 1e-30f)};
 #pragma unroll
       for (int i = 0; i < 2; ++i) tmem_ld_wait32(s[i]);

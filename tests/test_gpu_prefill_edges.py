@@ -66,3 +66,24 @@ def test_more_tiles_than_the_device_holds_ragged(batch):
     if batch == 3:
         lens, q_lens = [700, 40, 1500], [690, 40, 900]
     _check(lens, q_lens, 32, 4, 64, seed=batch)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("sm_scale", [-0.0625, -1.0, 0.0])
+def test_a_logit_scale_that_is_not_positive(d, sm_scale):
+    """As in decode: the logits are scaled by what the caller gives, its sign included, which is the same as -q and the other
+    sign.  (A scale of 1 is not held against the oracle: at head_dim 128 a logit's error is up to sm_scale 2^-17 max|q| sum|k|,
+    here 2^-17 * 60 * 130 = 0.06 of a probability; of 1/16, 0.004.)"""
+    w = workloads.make_workload("negative", [300, 140, 17], 6, 2, d, seed=d, q_lens=[100, 33, 17])
+    cache, ws = helpers.gpu_fill(w), binding.new_workspace(w.batch, 6, 2, d, w.block_table.shape[1], 2048, 150)
+    for causal in (True, False):
+        call = lambda q, s: binding.paged_chunked(cache, q, w.cu_q_lens.cuda(), w.block_table.cuda(), w.context_lens_tensor.cuda(), 2048, causal, s, ws)
+        out = call(w.q.cuda(), sm_scale)
+        torch.cuda.synchronize()
+        assert binding.workspace_status(ws) == 0
+        assert torch.equal(out, call(-w.q.cuda(), -sm_scale))
+        if sm_scale == -1.0:
+            continue
+        ref = attention.paged_attention(w.q.float().numpy(), helpers.oracle_fp8_cache(w), w.block_table.numpy(), w.context_lens,
+                                        cu_q_lens=w.cu_q_lens.numpy(), causal=causal, sm_scale=sm_scale)
+        helpers.check_attention(out, ref, what=f"prefill, logits times {sm_scale}")
