@@ -2,7 +2,7 @@
 // dequantisation on load, Eq. 7-8 grouped-query sharing, Eq. 9 valid blocks only, Eq. 10 max-subtracted softmax, for runs
 // of several query tokens per sequence.  head_dim 64 and 128.
 //
-// A CTA owns one (sequence, kv head) and two tiles of consecutive query tokens.  The 128 rows of a tile are its (query
+// A CTA owns one (sequence, kv head) and two tiles of consecutive query tokens (or one, where all CTAs start at once).  The 128 rows of a tile are its (query
 // token, query head of the group) pairs, so the K/V stream of the kv head is fetched, and V widened, once for all G heads
 // and both tiles (Algorithm 2).  Per tile and 128 keys (eight cache blocks):
 //     S [128 rows x 128 keys] = Q [128 x D] . Ktile^T       head_dim 128: kind::f8f6f4, the cache codes as they are, Q as
@@ -65,6 +65,7 @@ struct PrefillParams {
   int batch, num_q_heads, num_kv_heads, group;
   int num_blocks;
   int tile_queries;        // query tokens per tile = 128 / group
+  int tiles;               // of a CTA: 2, or 1
   int causal;
   int by_length;           // more CTAs than the device holds at a time: the long ones first
   float sm_scale_log2;
@@ -183,7 +184,7 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
   if (warp == 0) {
     constexpr int kPer = 4, kBands = 8;
     int left = blockIdx.x, found = -1, g = 0, q0 = 0, first = 0, count = 0, ctx = 0;
-    const int W = 2 * TQ;
+    const int W = p.tiles * TQ;
     auto sequence = [&](int b, int& from, int& n, int& c) {
       from = b < p.batch ? p.cu_q_lens[b] : 0;
       n = b < p.batch ? max(0, p.cu_q_lens[b + 1] - from) : 0;
@@ -254,7 +255,7 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
   const uint32_t tmem = *tmem_slot;
   const int b = misc[0], q0 = misc[1], row_base = misc[4], n_new = misc[5], L = misc[6], g = misc[7];
   // keys that any row of tile x may see (Eq. 1: K_{<=t}), and tiles of keys
-  auto tile_queries = [&](int x) { return max(0, min(TQ, n_new - q0 - x * TQ)); };
+  auto tile_queries = [&](int x) { return x < p.tiles ? max(0, min(TQ, n_new - q0 - x * TQ)) : 0; };
   auto tile_keys = [&](int x) {
     const int nq = tile_queries(x);
     return nq == 0 ? 0 : p.causal ? max(0, min(L, L - n_new + q0 + x * TQ + nq)) : L;
@@ -768,7 +769,13 @@ int launch_paged_prefill(const coopt_cache* c, const void* q, void* out, const i
   p.causal = causal;
   p.sm_scale_log2 = sm_scale * kLog2e;
   p.status = static_cast<int*>(workspace);
-  const long long pairs = static_cast<long long>(total_q) / (2 * p.tile_queries) + batch;   // every sequence adds at most one partly filled pair
+  auto most = [&](int tiles) { return static_cast<long long>(total_q) / (tiles * p.tile_queries) + batch; };   // every sequence adds at most one that is partly filled
+  // A CTA with one tile takes about 0.73 of the time of one with two (the tensor core and the exponential units are less busy,
+  // and so nothing waits as long), but twice as many are needed: one tile as long as all of them start at once.  (One sequence,
+  // 40 heads over 8, head_dim 128: 256 new tokens behind 8000 139.5 us with two / 108.6 with one, 512 behind 8000, which
+  // would be 168 CTAs, 151 with two; 8 heads over 1, 128 behind 32000 508 / 370, 2048 alone 42.1 / 32.6.)
+  p.tiles = most(1) * c->num_kv_heads <= num_sms ? 1 : 2;
+  const long long pairs = most(p.tiles);
   if (pairs * c->num_kv_heads > 0x7fffffffll) return COOPT_ERR_UNSUPPORTED;
   const dim3 grid(static_cast<unsigned>(pairs * c->num_kv_heads));
   p.by_length = pairs * c->num_kv_heads > num_sms ? 1 : 0;

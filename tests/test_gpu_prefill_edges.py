@@ -87,3 +87,22 @@ def test_a_logit_scale_that_is_not_positive(d, sm_scale):
         ref = attention.paged_attention(w.q.float().numpy(), helpers.oracle_fp8_cache(w), w.block_table.numpy(), w.context_lens,
                                         cu_q_lens=w.cu_q_lens.numpy(), causal=causal, sm_scale=sm_scale)
         helpers.check_attention(out, ref, what=f"prefill, logits times {sm_scale}")
+
+
+@pytest.mark.parametrize("hq,hkv,d", [(16, 16, 128), (60, 12, 128), (96, 12, 64)])
+def test_query_runs_around_the_edges_of_pairs_of_tiles(hq, hkv, d):
+    """As test_query_runs_around_tile_edges, with so many kv heads that a CTA has two tiles."""
+    test_query_runs_around_tile_edges(hq, hkv, d)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_a_first_tile_of_a_pair_that_sees_fewer_key_tiles_than_the_second(d):
+    _check([256, 300, 520], [256, 200, 250], 20, 20, d, seed=7)
+
+
+@pytest.mark.parametrize("more", [0, 1])
+@pytest.mark.parametrize("d", [64, 128])
+def test_on_both_sides_of_as_many_tiles_as_multiprocessors(d, more):
+    """16 queries a tile; the launch reckons with one tile more than the sequence fills."""
+    n = 16 * (torch.cuda.get_device_properties(0).multi_processor_count - 1 + more)
+    _check([n + 5], [n], 8, 1, d, seed=more)
