@@ -96,14 +96,20 @@ __device__ __forceinline__ bool write_whole_part(const WriteParams& p, int blk, 
   return true;
 }
 
-// FP8, many tokens (prefill chunks, bulk fills): one CTA per (kSpan consecutive tokens, kWriteHeads kv heads), a warp per
-// (kv head, K | V).  Every warp finds the span's groups by itself: no warp waits for another.
+// FP8, many tokens (prefill chunks, bulk fills): one CTA (kShared: several) per (kSpan consecutive tokens, kWriteHeads kv
+// heads), a warp per (kv head, K | V).  Every warp finds the span's groups by itself: no warp waits for another.
 // Bound by memory: 65,536 tokens of 8 heads x 128 (403 MB) in 65.9 us, 6.1 TB/s.  Before blocks written whole had a path of
 // their own it was 112.6 us, bound by the integer pipe (10.6 instructions a value: look-ups of rows and groups, signs put
 // back after the division, stores of K words eight lanes to a bank).
 constexpr int kSpan = 32;
 constexpr int kSpanThreshold = 512;     // calls with more tokens than this take the span kernel
-template <int D, bool kE5m2>
+// Groups that are not whole blocks take a warp 2 us each, one after the other (head_dim 128: the kernel's registers are what
+// whole blocks want).  Where spans are few, several CTAs share one: as many as bring the launch to 8 CTAs an SM (6 at head_dim
+// 64, where a group is shorter), a power of two, kSpanSplit at most.  300 sequences of 2 tokens 41.1 -> 8.7 us, 128 of 7 28.5 ->
+// 8.4, 300 of 7 29.2 -> 15.8, 300 of 13 tokens 19.8 -> 16.8 (with 6 CTAs an SM, which shares by two there, 23.5); calls whose
+// spans are not shared have a kernel without the choice (30,000 tokens of one kv head 6.6 us, 6.8 with it).
+constexpr int kSpanSplit = 16;
+template <int D, bool kE5m2, bool kShared>
 __global__ void __launch_bounds__(kWriteWarps * 32, 4) kv_write_fp8_span_kernel(WriteParams p) {
   __shared__ __align__(16) uint8_t stage[kWriteWarps][part_bytes(D, true)];
   __shared__ Group groups[kWriteWarps];
@@ -129,6 +135,11 @@ __global__ void __launch_bounds__(kWriteWarps * 32, 4) kv_write_fp8_span_kernel(
   unsigned others = __ballot_sync(0xffffffffu, s0 >= 0 && !((follows >> lane) & 1ull)) & ~whole;
   const bool aligned = ((reinterpret_cast<uintptr_t>(which == 0 ? p.k : p.v) | static_cast<uintptr_t>(p.token_stride * 2)) & (D / 16 - 1)) == 0;
   if (!aligned) { others |= whole; whole = 0; }
+  if constexpr (kShared) {                 // this CTA's part of the span's groups
+    const unsigned mine = __ballot_sync(0xffffffffu, (__popc((whole | others) & ((1u << lane) - 1u)) & (gridDim.z - 1)) == blockIdx.z);
+    whole &= mine;
+    others &= mine;
+  }
   while (whole) {
     const int w = __ffs(whole) - 1;
     whole &= whole - 1;
@@ -191,21 +202,23 @@ int launch_kv_write(const coopt_cache* c, const void* k, const void* v, int64_t 
   const int heads_per_cta = fp8 ? kWriteHeads : kWriteWarps;
   const int head_ctas = (c->num_kv_heads + heads_per_cta - 1) / heads_per_cta;
   const dim3 grid(num_tokens, head_ctas);
-  const dim3 span_grid((num_tokens + kSpan - 1) / kSpan, head_ctas);
+  const long long spans = (static_cast<long long>(num_tokens) + kSpan - 1) / kSpan * head_ctas;
+  const DeviceInfo* di = device_info();
+  int split = 1;
+  while (2 * split <= kSpanSplit && 2 * split * spans <= (c->head_dim == 128 ? 8 : 6) * (di ? di->num_sms : 148)) split *= 2;
+  const dim3 span_grid((num_tokens + kSpan - 1) / kSpan, head_ctas, split);
   const bool span = fp8 && num_tokens > kSpanThreshold;
+  const auto launch = [&](auto kernel, dim3 ctas) { return launch_dependent(kernel, ctas, kWriteWarps * 32, 0, stream, p); };
+  const auto launch_fp8 = [&](auto few, auto many, auto shared) { return !span ? launch(few, grid) : split > 1 ? launch(shared, span_grid) : launch(many, span_grid); };
   bool ok;
   if (c->head_dim == 128) {
-    if (span && e5m2) ok = launch_dependent(kv_write_fp8_span_kernel<128, true>, span_grid, kWriteWarps * 32, 0, stream, p);
-    else if (span) ok = launch_dependent(kv_write_fp8_span_kernel<128, false>, span_grid, kWriteWarps * 32, 0, stream, p);
-    else if (e5m2) ok = launch_dependent(kv_write_fp8_kernel<128, true>, grid, kWriteWarps * 32, 0, stream, p);
-    else if (fp8) ok = launch_dependent(kv_write_fp8_kernel<128, false>, grid, kWriteWarps * 32, 0, stream, p);
-    else ok = launch_dependent(kv_write_bf16_kernel<128>, grid, kWriteWarps * 32, 0, stream, p);
+    if (e5m2) ok = launch_fp8(kv_write_fp8_kernel<128, true>, kv_write_fp8_span_kernel<128, true, false>, kv_write_fp8_span_kernel<128, true, true>);
+    else if (fp8) ok = launch_fp8(kv_write_fp8_kernel<128, false>, kv_write_fp8_span_kernel<128, false, false>, kv_write_fp8_span_kernel<128, false, true>);
+    else ok = launch(kv_write_bf16_kernel<128>, grid);
   } else {
-    if (span && e5m2) ok = launch_dependent(kv_write_fp8_span_kernel<64, true>, span_grid, kWriteWarps * 32, 0, stream, p);
-    else if (span) ok = launch_dependent(kv_write_fp8_span_kernel<64, false>, span_grid, kWriteWarps * 32, 0, stream, p);
-    else if (e5m2) ok = launch_dependent(kv_write_fp8_kernel<64, true>, grid, kWriteWarps * 32, 0, stream, p);
-    else if (fp8) ok = launch_dependent(kv_write_fp8_kernel<64, false>, grid, kWriteWarps * 32, 0, stream, p);
-    else ok = launch_dependent(kv_write_bf16_kernel<64>, grid, kWriteWarps * 32, 0, stream, p);
+    if (e5m2) ok = launch_fp8(kv_write_fp8_kernel<64, true>, kv_write_fp8_span_kernel<64, true, false>, kv_write_fp8_span_kernel<64, true, true>);
+    else if (fp8) ok = launch_fp8(kv_write_fp8_kernel<64, false>, kv_write_fp8_span_kernel<64, false, false>, kv_write_fp8_span_kernel<64, false, true>);
+    else ok = launch(kv_write_bf16_kernel<64>, grid);
   }
   return ok ? COOPT_OK : COOPT_ERR_CUDA;
 }

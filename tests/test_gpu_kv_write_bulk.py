@@ -48,3 +48,11 @@ def test_bulk_write_bit_exact(d, fmt, hkv, how):
     kw = {"fmt": e5m2} if fmt == "e5m2" else {}
     kv_cache.kv_write(codes, scales, k.float().numpy(), v.float().numpy(), slots.numpy(), **kw)
     helpers.check_cache_bit_exact(cache, codes, scales, what=how)
+
+
+@pytest.mark.parametrize("d,hkv,sequences,run", [(128, 1, 270, 2), (128, 1, 300, 13), (64, 5, 200, 7), (64, 5, 400, 13), (128, 5, 400, 11), (128, 4, 800, 20), (64, 1, 1500, 13)])
+def test_short_runs_of_many_sequences_in_two_calls(d, hkv, sequences, run):
+    """Spans that 16, 8, 4, 2 CTAs share and that one CTA has alone; the second call finds codes in the blocks."""
+    w = workloads.make_workload("runs", [2 * run] * sequences, hkv, hkv, d, seed=run)
+    first = np.concatenate([np.arange(o, o + run) for o in w.kv_offsets])
+    helpers.check_cache_bit_exact(helpers.gpu_fill(w, calls=[first, first + run]), *helpers.oracle_fp8_cache(w, calls=[first, first + run]))
