@@ -58,6 +58,7 @@ struct Cfg {
   static constexpr int kGran = granule_bytes(D, kFp8);
   static constexpr int kCopy = kFp8 ? 2 * kBlockSize * D + kFp8Header : kGran;   // bytes of a granule that are read
   static constexpr int kStages = kFp8 ? (D == 128 ? 3 : 4) : (D == 128 ? 2 : 4);
+  static constexpr int kWholeIdle = kFp8 ? kWholeUnitsIdle : kWholeUnitsIdleBf16 * (D / 64);
   static constexpr int kPieceStride = D + 4;                    // floats of one head of a piece: o[D], maximum, sum, padding
   static constexpr int kPiece = kMaxGroup * kPieceStride * 4;   // bytes
   // A warp's shared memory: its ring, the piece of a unit from before, and, in a launch over several layers, the piece of a
@@ -380,7 +381,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
     none_empty = none_empty && m < kSomeEmpty;
     most = max(most, m & (kSomeEmpty - 1));
   }
-  const bool whole = most * (D / 64) <= (T == kMinPlaces ? kWholeUnitsIdle : kWholeUnits) && (p.chunk_blocks == 0 || most + kUnitCost <= static_cast<int>(T));
+  const bool whole = most * (D / 64) <= (T == kMinPlaces ? C::kWholeIdle : kWholeUnits) && (p.chunk_blocks == 0 || most + kUnitCost <= static_cast<int>(T));
   // Where they are very short, a warp holds whole what begins among its places, and nothing is merged.  Nor does a unit's
   // result depend on the shares then: they are made as large as it takes for every CTA to have one at most.
   const bool solo = whole && p.chunk_blocks == 0 && most <= p.solo_blocks;

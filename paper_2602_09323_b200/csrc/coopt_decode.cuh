@@ -26,8 +26,18 @@ constexpr int kWsHeaderBytes = 256;
 constexpr int kUnitCost = 5;          // places of the line that a unit takes besides its blocks
 constexpr int kCtasPerSm = 1;
 constexpr int kMinPlaces = 16;        // smallest share
-constexpr int kWholeUnits = 32;       // units of at most so many blocks (head_dim 64: twice) are not cut between shares
-constexpr int kWholeUnitsIdle = 192;  // .. where the call does not fill the device
+// Units of at most so many blocks at head_dim 64, half as many at 128, are not cut between shares.  (Device full, not cut / cut:
+// 64 sequences of up to 16 and 24 blocks, 40 heads over 8, head_dim 128 15.4 / 16.7 and 16.6 / 18.2 us; 130 of up to 32, 16 over
+// 4, head_dim 64 15.5 / 17.2.)
+constexpr int kWholeUnits = 32;
+// .. where the call does not fill the device.  One layer alone would have the line at 40 blocks (one sequence, 40 heads over 8,
+// head_dim 128, 32 / 48 / 96 blocks: 10.2 / 11.8 / 16.0 us not cut, 10.5 / 10.5 / 10.9 cut; head_dim 64, 32 / 48 / 96 / 192: 9.2 /
+// 10.3 / 13.4 / 18.4 and 10.3 / 10.3 / 10.9 / 11.9), but a layer is cut the same way alone and in a launch over several, where
+// units that are not cut win throughout (eight layers of four sequences of 64 blocks 25.5 / 77.9; of one of 96 17.4 / 32.2).
+constexpr int kWholeUnitsIdle = 192;
+// .. and of a bf16 cache, which has no launch over several layers: blocks at either head dim.  (One sequence, 8 heads, head_dim
+// 128, 32 / 48 / 64 blocks: 9.0 / 10.5 / 11.8 us not cut, 9.4 / 9.6 / 10.2 cut; head_dim 64: 8.6 / 9.7 / 10.8 and 9.0 / 9.3 / 10.0.)
+constexpr int kWholeUnitsIdleBf16 = 40;
 // Units of at most so many blocks are not cut between warps either.  Eight layers of 40 sequences, 4 kv heads, us against units
 // spread over a CTA's warps: 1 block 10.6 / 27.6, 4 blocks 13.6 / 44, 8 blocks 17.5 / 65; one layer: 8.8 / 8.8, 11.7 / 10.5,
 // 14.0 / 10.5.

@@ -176,3 +176,13 @@ def test_v_scales_whose_reciprocal_overflows(lens, fmt, d):
     got = helpers.gpu_decode(w, cache)[0].double().cpu().numpy()
     bound = 2.0 ** -8 * np.abs(ref) + 2.0 ** -134 + 2.0 ** -11 * float(w.v.float().abs().max())
     assert np.all(np.abs(got - ref) <= bound), np.max(np.abs(got - ref) / bound)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("lens", [[640], [641], [640, 0, 300], [639, 657]])
+def test_bf16_units_around_the_longest_that_are_not_cut(lens, d):
+    w = workloads.make_workload("bf16", lens, 6, 2, d, seed=lens[0])
+    kv = kv_cache.new_cache_bf16(w.num_blocks, 2, d)
+    kv_cache.kv_write_bf16(kv, w.k.float().numpy(), w.v.float().numpy(), w.slot_mapping.numpy())
+    out, _ = helpers.gpu_decode(w, helpers.gpu_fill(w, dtype=binding.KV_BF16))
+    helpers.check_attention(out, attention.paged_attention(w.q.float().numpy(), kv, w.block_table.numpy(), w.context_lens), what=f"bf16 {lens}")
