@@ -800,7 +800,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
       }
     }
     const bool starts = w.j == 0, ends = w.jend == w.n;
-    if (starts && ends && p.chunk_blocks == 0) {
+    if (starts && ends && w.n == w.nb) {
       // the whole (sequence, kv head): bf16 rows, transposed so that a lane holds pairs of dims of head `row`
       __nv_bfloat16* dst = layer(y).out + (static_cast<size_t>(w.b) * Hq + w.g * G + row) * D + 2 * quad;
 #pragma unroll
@@ -811,7 +811,8 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
           *reinterpret_cast<uint32_t*>(dst + 16 * t + 8) = c;
         }
       }
-    } else if (starts && ends) {
+    }
+    if (starts && ends && p.chunk_blocks > 0) {
       // a whole chunk: exported
       const size_t rows = static_cast<size_t>(p.max_chunks);
       const size_t at = (static_cast<size_t>(w.b) * Hq + w.g * G + 2 * quad) * rows + w.u / ln.chunk;
@@ -824,7 +825,8 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
           if (row == 0) { p.part_m[at + h * rows] = m[h] * kLn2; p.part_l[at + h * rows] = l[h] * kUnshift; }
         }
       }
-    } else {
+    }
+    if (!(starts && ends)) {
       // a piece: into shared memory, once the pieces of the share before are of no more use
       if (L > 1 && round > 0 && rec.flags == 0 && !dead && !mbar_wait_bounded(bar_merged, (round - 1) & 1u)) dead = true;
       float* piece = reinterpret_cast<float*>(ring + (starts ? piece1_off : piece0_off));
@@ -901,9 +903,8 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
         make_uint2(pack_bf16x2(a.num.x * dinv, a.num.y * dinv), pack_bf16x2(a.num.z * dinv, a.num.w * dinv));
   };
   auto finish = [&](const Acc& a, int b, int g, int h, int u) {
-    if (p.chunk_blocks == 0) {
-      store_out(a, b, g, h);
-    } else {
+    if (p.chunk_blocks == 0 || line_blocks(ln, b) <= ln.chunk) store_out(a, b, g, h);
+    if (p.chunk_blocks > 0) {
       const size_t at = (static_cast<size_t>(b) * Hq + g * G + h) * p.max_chunks + u / ln.chunk;
       const float dinv = a.den > 0.0f ? 1.0f / a.den : 0.0f;
       if (on) *reinterpret_cast<float4*>(p.part_o + at * D + d0) = make_float4(a.num.x * dinv, a.num.y * dinv, a.num.z * dinv, a.num.w * dinv);
@@ -986,6 +987,9 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
       run_ends = c.u + c.n >= nb && c.jend == c.n;
       walk_next(ln, c);
     } while (c.more && c.b == b && c.g == g);
+    // A single chunk has been stored with its export.  (16 heads over 4, head_dim 64, bf16, one sequence of 300 tokens in a chunk
+    // of 2048: 14.1 us read back and merged, 11.0 so.)
+    if (nb <= ln.chunk) continue;
     for (int h = 0; h < G; ++h, ++task) {
       if (task % C::kWarps != warp) continue;
       Acc a;

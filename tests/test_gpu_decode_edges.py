@@ -186,3 +186,24 @@ def test_bf16_units_around_the_longest_that_are_not_cut(lens, d):
     kv_cache.kv_write_bf16(kv, w.k.float().numpy(), w.v.float().numpy(), w.slot_mapping.numpy())
     out, _ = helpers.gpu_decode(w, helpers.gpu_fill(w, dtype=binding.KV_BF16))
     helpers.check_attention(out, attention.paged_attention(w.q.float().numpy(), kv, w.block_table.numpy(), w.context_lens), what=f"bf16 {lens}")
+
+
+@pytest.mark.parametrize("d,fmt", [(64, "e4m3"), (128, "e4m3"), (64, "bf16"), (128, "bf16")])
+@pytest.mark.parametrize("chunk", [512, 2048, 32768])
+def test_a_context_in_a_single_chunk_beside_longer_ones(chunk, d, fmt):
+    """Whole in a warp, shared by warps, shared by CTAs: output and exported partials."""
+    w = workloads.make_workload("one chunk", [9000, 1, 512, 513, 0, 2048, 30, 2049], 6, 2, d, seed=chunk + d)
+    if fmt == "bf16":
+        kv = kv_cache.new_cache_bf16(w.num_blocks, 2, d)
+        kv_cache.kv_write_bf16(kv, w.k.float().numpy(), w.v.float().numpy(), w.slot_mapping.numpy())
+    else:
+        kv = helpers.oracle_fp8_cache(w)
+    out, ws = helpers.gpu_decode(w, helpers.gpu_fill(w, dtype=binding.KV_BF16 if fmt == "bf16" else binding.KV_FP8_E4M3), chunk_size=chunk)
+    ref, partials = attention.paged_attention_chunked(w.q.float().numpy(), kv, w.block_table.numpy(), w.context_lens, chunk)
+    helpers.check_attention(out, ref, what=f"chunk {chunk} {fmt}")
+    o_c, m_c, l_c = (t.cpu().numpy() for t in binding.chunk_partials(ws, w.batch, 6, d, w.block_table.shape[1], chunk))
+    for (b, h), (m, l, o) in partials.items():          # bounds as above
+        n = len(m)
+        assert np.allclose(m_c[b, h, :n], m, rtol=1e-4, atol=1e-3)
+        assert np.allclose(l_c[b, h, :n], l, rtol=5e-3, atol=1e-4)
+        assert np.allclose(o_c[b, h, :n], o, rtol=5e-3, atol=2e-2)
