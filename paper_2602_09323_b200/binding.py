@@ -173,10 +173,10 @@ def kv_write(cache: Cache, k: torch.Tensor, v: torch.Tensor, slot_mapping: torch
     """coopt_kv_write: k, v bf16 [T, Hkv, D] (token stride taken from the tensor), slots int64 [T]."""
     assert k.dtype is _BF16 and v.dtype is _BF16 and slot_mapping.dtype is _I64
     assert k.is_cuda and v.is_cuda and slot_mapping.is_cuda and slot_mapping.is_contiguous()
-    stride = k.stride()
-    tokens, heads, dim = k.shape
-    assert v.shape == k.shape and stride == v.stride() and stride[2] == 1 and stride[1] == dim
-    st = load_library().coopt_kv_write(cache.ref(), k.data_ptr(), v.data_ptr(), stride[0] if tokens > 1 else heads * dim,
+    stride, shape = k.stride(), k.shape
+    tokens = shape[0]
+    assert v.shape == shape and stride == v.stride() and stride[2] == 1 and stride[1] == shape[2]
+    st = load_library().coopt_kv_write(cache.ref(), k.data_ptr(), v.data_ptr(), stride[0] if tokens > 1 else shape[1] * shape[2],
                                        slot_mapping.data_ptr(), tokens, _stream())
     if st != 0:
         _check(st, "coopt_kv_write")
@@ -213,9 +213,9 @@ def paged_decode(cache: Cache, q: torch.Tensor, block_table: torch.Tensor, conte
     assert block_table.dtype is _I32 and block_table.is_contiguous() and context_lens.dtype is _I32
     if out is None:
         out = torch.empty_like(q)
-    batch, heads, _ = q.shape
+    shape = q.shape
     st = load_library().coopt_paged_decode(cache.ref(), q.data_ptr(), out.data_ptr(), block_table.data_ptr(), block_table.shape[1],
-                                           context_lens.data_ptr(), batch, heads, float(sm_scale),
+                                           context_lens.data_ptr(), shape[0], shape[1], float(sm_scale),
                                            workspace.data_ptr(), workspace.numel(), _stream())
     _check(st, "coopt_paged_decode")
     return out

@@ -207,3 +207,14 @@ def test_a_context_in_a_single_chunk_beside_longer_ones(chunk, d, fmt):
         assert np.allclose(m_c[b, h, :n], m, rtol=1e-4, atol=1e-3)
         assert np.allclose(l_c[b, h, :n], l, rtol=5e-3, atol=1e-4)
         assert np.allclose(o_c[b, h, :n], o, rtol=5e-3, atol=2e-2)
+
+
+def test_views_with_a_further_dimension_are_taken_as_before():
+    w = workloads.make_workload("views", [40, 17], 4, 2, 64, seed=5)
+    plain, cache = helpers.gpu_fill(w), binding.Cache(w.num_blocks, 2, 64)
+    binding.kv_write(cache, w.k.cuda()[..., None], w.v.cuda()[..., None], w.slot_mapping.cuda())
+    assert torch.equal(cache.data, plain.data)
+    out, ws = helpers.gpu_decode(w, cache)
+    q = w.q.cuda().view(w.batch, 4, 2, 32)
+    again = binding.paged_decode(cache, q, w.block_table.cuda(), w.context_lens_tensor.cuda(), w.sm_scale, ws)
+    assert again.shape == q.shape and torch.equal(again.view_as(out), out)
