@@ -139,9 +139,11 @@ int coopt_paged_decode(const coopt_cache* cache, const void* q, void* out, const
  * COOPT_STATIC_SCRATCH_BYTES inside the library; every device that loads the library holds
  * that much memory until the process exits.  The call itself allocates nothing.
  *   - Arguments as coopt_paged_decode, minus the workspace.
- *   - Problems whose pieces of one layer need more than
- *     COOPT_STATIC_SCRATCH_BYTES are refused with COOPT_ERR_WORKSPACE before anything is
- *     enqueued (the LLaMA-13B decode shape needs about 0.8 MB).
+ *   - Refused with COOPT_ERR_WORKSPACE before anything is enqueued: problems for which the
+ *     smallest workspace that coopt_paged_decode takes is larger than
+ *     COOPT_STATIC_SCRATCH_BYTES (the LLaMA-13B decode shape: about 0.8 MB).  That size follows
+ *     from the arguments alone (batch, heads, head_dim, max_blocks_per_seq); it counts a list of
+ *     every block that the block table has room for, which is more than the call now writes.
  *   - The first call on a device looks up the array's device address; make that first call
  *     outside any stream capture.
  *   - All calls on a device share the array.  Each call clears the control words on `stream`

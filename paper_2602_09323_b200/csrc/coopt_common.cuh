@@ -28,11 +28,11 @@ inline bool is_fp8(int dtype) { return dtype == COOPT_KV_FP8_E4M3 || dtype == CO
 //       (t / 8) * 8D + (d / 16) * 128 + (t % 8) * 16 + d % 16
 //   V part (rows = dims, contraction over tokens; i.e. V transposed): token t, dim d at
 //       (d / 8) * 128 + (d % 8) * 16 + t
-// bf16 granule (ablation cache, mma.sync kernel): values permuted so that lane `l` of a warp finds
-// the B-operand registers of mma.m16n8k16 in consecutive 16-byte chunks:
-//   K tile (QK^T: n = token, k = dim):   lane = 4 * (token % 8) + (dim % 8) / 2
-//   V tile (P V : k = token, n = dim):   lane = 4 * (dim % 8)   + (token % 8) / 2
-// a chunk holds two k-steps (K) or two n-tiles (V) of two registers each.
+// bf16 granule (ablation cache): values permuted so that lane `l` of a warp finds the A-operand registers
+// of mma.m16n8k16 in consecutive 16-byte chunks:
+//   K tile (K Q^T:     rows = tokens, contraction over dims):   lane = 4 * (token % 8) + (dim % 8) / 2
+//   V tile (V^T P^T:   rows = dims, contraction over tokens):   lane = 4 * (dim % 8)   + (token % 8) / 2
+// a chunk holds the registers of eight rows for two k-steps (K), or of two times eight rows for one (V).
 
 __host__ __device__ constexpr int granule_bytes(int D, bool fp8) {
   return fp8 ? kFp8Tail + 2 * kBlockSize * D : 2 * kBlockSize * D * 2;

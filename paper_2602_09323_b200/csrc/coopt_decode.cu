@@ -15,12 +15,9 @@
 // multiplies its logits, the V scale goes into the probabilities.  No barrier is met between the first block and the
 // last; pieces of units that warps or CTAs share are merged by log-sum-exp at the end.
 //
-// (The kernel before this one ran the contractions on tcgen05.mma, 128 tokens at a time, with two softmax teams per
-// CTA and a plan of every CTA's blocks made by a kernel of its own.  The tensor core was 21 % busy with columns that
-// are mostly padding, and what bounded the launch were the hand-overs between its roles, per unit and at both ends.
-// Before / now: one layer of 56 heads over 8 kv heads, 8 sequences of 1..28 tokens 60 / 7.5 us; 24 sequences of
-// 300..4000 tokens, G = 8, 46 / 23 us a layer; 32 x 2048 tokens, G = 5, 35 / 29 us; 64 sequences of 128..8192 tokens,
-// 121 / 104 us; 120 sequences of 5..900 tokens at head_dim 64, plan included, 56 / 17 us.)
+// (On tcgen05.mma, 128 tokens at a time, the tensor core was 21 % busy with columns that are mostly padding, and the launch
+// waited for hand-overs between its roles.  On tcgen05 / here: 24 sequences of 300..4000 tokens, G = 8, 46 / 23 us a layer;
+// 32 x 2048 tokens, G = 5, 35 / 29; 64 sequences of 128..8192 tokens 121 / 104; 120 of 5..900, head_dim 64, 56 / 17.)
 //
 // A launch of 32 x 2048 tokens streams at 6.4 TB/s from its first copies, 3 us after a CTA's first instruction, to the end
 // of its last block, 5 us before the CTA's last; code that runs once costs about four cycles an instruction to fetch.

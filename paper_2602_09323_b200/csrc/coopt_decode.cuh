@@ -20,9 +20,10 @@ constexpr int kMaxGroup = 8;
 constexpr int kMaxChunkBlocks = 2048;
 constexpr int kCounterSlots = 16384;  // >= kManyLayers * shares * kMaxGroup
 constexpr int kWsHeaderBytes = 256;
-// Measured, us a pass: cost 3 / 5 places 435 / 429 (64 mixed lengths, 4 layers), 103 / 101 (24 sequences, G = 8, 4 layers),
-// 126 / 104 (21 sequences of 2..60 tokens, 8 layers); smallest share 64 / 16 places 20.5 / 16.4 (one sequence of 777
-// tokens), 142 / 102 (7 sequences of 272..544 tokens, 8 layers): where a call cannot fill the device, spreading it wins.
+// Measured, us a pass: cost 3 / 5 / 8 places 391 / 394 / 390 (64 mixed lengths, 4 layers), 125 / 123 / 121 (24 sequences, G = 8,
+// 4 layers), 235.5 / 231.5 / 239.8 (32 x 2048 tokens, 8 layers); smallest share 8 / 16 / 64 places 12.2 / 12.3 / 16.6 (one
+// sequence of 777 tokens), 11.9 / 11.6 / 15.2 (one of 2000), 13.7 / 13.6 / 15.3 (four of 1600..3000), 20.6 / 20.6 / 18.0 (7 of
+// 272..544 tokens, 8 layers): where a call cannot fill the device, spreading it wins, except in launches over several layers.
 constexpr int kUnitCost = 5;          // places of the line that a unit takes besides its blocks
 constexpr int kCtasPerSm = 1;
 constexpr int kMinPlaces = 16;        // smallest share

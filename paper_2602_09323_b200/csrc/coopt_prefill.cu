@@ -31,9 +31,9 @@
 //   warp 14          copies: gather requests over the tensor map of the cache
 //   warp 15          what the softmax needs of a tile's block scales, worked out once for all rows
 //
-// Measured: 8 sequences of 4096 cached and 512 new tokens, 40 query heads over 8 kv heads, head_dim 128: 690 -> 430 us (the
-// kernel before: one tile a CTA, two groups of eight warps that took its key tiles in turns, each with an accumulator and
-// widening of its own); prompts of 900..2900 tokens, 32 heads over 8, head_dim 64: 495 -> 187 us (mma.sync).  A half takes
+// Measured: 8 sequences of 4096 cached and 512 new tokens, 40 query heads over 8 kv heads, head_dim 128: 430 us (one tile a CTA,
+// its key tiles taken in turns by two groups of eight warps: 690); prompts of 900..2900 tokens, 32 heads over 8, head_dim 64:
+// 187 us (on mma.sync 495).  A half takes
 // about 1,850 cycles for both tiles: exponential units and issue slots 48 % each, tensor core 61 %, none of them alone (with
 // half the exponentials left out 12 % less time, with half the products of Q 4 %; four softmax warps a scheduler, two threads
 // to a row, took 453 us); a CTA's start and end take 15,000 cycles (head_dim 64: 10,000).
