@@ -390,16 +390,11 @@ int coopt_decode_layers(const coopt_layer_io* layers, int32_t num_layers, int64_
     return COOPT_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   rc = launch_decode_plan(block_table, max_blocks_per_seq, context_lens, batch, c0->num_kv_heads, c0->num_blocks, 0, plan, st);
-  const bool long_layers = static_cast<long long>(batch) * c0->num_kv_heads * max_blocks_per_seq > 256ll * num_sms();
   for (int32_t l = 0; l < num_layers && rc == COOPT_OK;) {
-    // Layers whose buffers are apart go into one launch where a layer is small: what a launch costs once is then much of it.
-    // (Eight layers, apart / together: 8 sequences of 1..28 tokens 53 / 11.4 us, 8 x 2048 tokens, G = 5, 118 / 109, 32 x 2048
-    // 248 / 233.)  The line is drawn by the columns of the block table, which is what the host knows: 256 blocks a
-    // multiprocessor if every sequence filled its row.  Beyond it lie calls that gain from a launch together (64 x 2048: 427 /
-    // 408; 64 of 128..8192, four layers, 442 / 424; short sequences in wide tables) and calls that lose (24 of 300..4000, G =
-    // 8, four layers, 120.4 / 123.2, where the pieces of eight heads leave room for a ring of two blocks a warp instead of
-    // three; head_dim 64, 64 of 100..5000, 304 / 317), which their lengths would have to tell apart.
-    int n = long_layers ? 1 : std::min(num_layers - l, kManyLayers);
+    // Layers whose buffers are apart go into one launch, up to eight: what a launch costs once is then shared, and the pieces of a
+    // layer are merged while the blocks of the next are under way.  (Apart / together: eight layers of 8 sequences of 1..28
+    // tokens 53 / 11.4 us; three of 54 of 4072..8144, G = 2, 185 / 171; four of 24 of 300..4000, G = 8, 96.8 / 93.2.)
+    int n = std::min(num_layers - l, kManyLayers);
     while (n > 1 && workspace_bytes < workspace_need(batch, num_q_heads, c0->num_kv_heads, c0->head_dim, max_blocks_per_seq, 0, n)) --n;
     const bool apart = layers_are_apart(layers + l, n, kv_token_stride, block_table, max_blocks_per_seq, context_lens, batch, num_q_heads);
     if (!apart) n = 1;

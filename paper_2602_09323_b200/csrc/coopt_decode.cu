@@ -19,10 +19,16 @@
 // waited for hand-overs between its roles.  On tcgen05 / here: 24 sequences of 300..4000 tokens, G = 8, 46 / 23 us a layer;
 // 32 x 2048 tokens, G = 5, 35 / 29; 64 sequences of 128..8192 tokens 121 / 104; 120 of 5..900, head_dim 64, 56 / 17.)
 //
+// A warp takes two blocks at a time, and their contractions, exponentials and look-ups side by side: one block is a chain of
+// dependent instructions (302 of them, one every 5.9 cycles with three warps a scheduler), and at one block at a time that
+// bounded the stream and not HBM.  One / two, us: 32 x 16384 tokens, G = 5, out of L2 153 / 112, out of HBM 186 / 174; 64 x
+// 4096, head_dim 64, G = 4, out of L2 60 / 48; 64 mixed lengths, four layers, 422 / 399.  (8 warps with 255 registers: 181 for
+// the second figure; two CTAs of 6 warps an SM: the same as one of 12.)
+//
 // A launch of 32 x 2048 tokens streams at 6.4 TB/s from its first copies, 3 us after a CTA's first instruction, to the end
 // of its last block, 5 us before the CTA's last; code that runs once costs about four cycles an instruction to fetch.
-// Registers are what the loop over blocks is short of: the walk of the copies waits in shared memory, and the query rows of
-// a unit are fetched when it starts (eight layers of 21 sequences of 2..60 tokens: 49 / 43.6 us; prefetching the rows into
+// Registers are what the loop over blocks is short of (what it spills goes to L2: all of L1 is shared memory, and 24 bytes cost
+// 4 %): the walks of the copies and of the work wait in shared memory, and the query rows of a unit are fetched when it starts (eight layers of 21 sequences of 2..60 tokens: 49 / 43.6 us; prefetching the rows into
 // registers at the end of the unit before instead: 49.5).
 #include <float.h>
 
@@ -42,37 +48,42 @@ constexpr float kLn2 = 0.6931471805599453f;
 constexpr float kLag = 6.0f;                                      // how far a reference maximum may lag (base-2 logarithm units)
 constexpr float kShift = 8.0f, kUnshift = 1.0f / 256.0f;          // probabilities are carried times 2^kShift: at most 2^14 in f16
 
+constexpr int kMaxSmem = 232448;                                 // of a CTA
+
 template <int D, int FMT>
 struct Cfg {
   static constexpr bool kFp8 = FMT != COOPT_KV_BF16;
   [[maybe_unused]] static constexpr bool kE5m2 = FMT == COOPT_KV_FP8_E5M2;
-  // A warp needs time for a block (about 1 us from landing to the next wait), so many warps are wanted, with at least two
-  // blocks in flight each.  head_dim 128: 12 warps x 3 blocks against 16 x 2 (which spill), 14 x 2 and 10 x 4: 423 / 430 /
-  // 423 / 427 us (64 sequences of 128..8192 tokens, four layers), 99 / 101 / 105 / 109 us (24 sequences, G = 8, four
-  // layers).  head_dim 64: 16 x 4 against 12 x 6: 33 / 36 us (85 x 2002 tokens).  bf16: 8 x 2 (182 registers).
+  // A warp needs time for two blocks (about 1.2 us from landing to the next wait), so many warps are wanted, with at least two
+  // blocks in flight each.  head_dim 128: 12 warps x 3 blocks against 8 x 5 and 10 x 4: 399 / 415 / 421 us (64 sequences of
+  // 128..8192 tokens, four layers); eight layers of 32 x 2048 tokens 226 / 225 / 247.  head_dim 64: 16 x 4 against 12 x 6:
+  // 13.0 / 15.2 us (four sequences of 1595..3191 tokens), 59 / 57 (64 x 4096).  bf16: 8 x 2 (182 registers).
   static constexpr int kWarps = kFp8 ? (D == 128 ? 12 : 16) : 8;
   static constexpr int kThreads = kWarps * 32;
   static constexpr int kGran = granule_bytes(D, kFp8);
   static constexpr int kCopy = kFp8 ? 2 * kBlockSize * D + kFp8Header : kGran;   // bytes of a granule that are read
-  static constexpr int kStages = kFp8 ? (D == 128 ? 3 : 4) : (D == 128 ? 2 : 4);
   static constexpr int kWholeIdle = kFp8 ? kWholeUnitsIdle : kWholeUnitsIdleBf16 * (D / 64);
   static constexpr int kPieceStride = D + 4;                    // floats of one head of a piece: o[D], maximum, sum, padding
   static constexpr int kPiece = kMaxGroup * kPieceStride * 4;   // bytes
   // A warp's shared memory: its ring, the piece of a unit from before, and, in a launch over several layers, the piece of a
   // unit that goes on (in a launch over one the ring has done its work by then, and the piece takes its place).  Pieces are
   // as large as the group asks for; for the largest groups the ring of a launch over several layers is shorter.
-  static constexpr int kShare = (D == 128 ? 18048 : 13056);
-  static __host__ __device__ constexpr int stages(int layers, int G) { return layers > 1 && kStages * kGran + 2 * G * kPieceStride * 4 > kShare ? kStages - 1 : kStages; }
-  static constexpr int kWarpBytes = kFp8 ? (kShare > kStages * kGran + kPiece ? kShare : kStages * kGran + kPiece) : kStages * kGran + kPiece;
+  static constexpr int kFixed = kMaxBatch * 4 + (kMaxBatch + 4) * 4 + 192 + 16 + kWarps * (96 + 128);      // what lies behind the warps' parts
+  static constexpr int kWarpBytes = kFp8 ? (kMaxSmem - kFixed) / kWarps / 128 * 128 : (D == 128 ? 2 : 4) * kGran + kPiece;
+  static constexpr int kStages = (kWarpBytes - kPiece) / kGran;
+  static __host__ __device__ constexpr int stages(int layers, int G) {
+    const int most = (kWarpBytes - 2 * G * kPieceStride * 4) / kGran;
+    return layers > 1 && most < kStages ? most : kStages;
+  }
   static constexpr int kBarOff = kWarps * kWarpBytes;
   static constexpr int kLensOff = kBarOff + (kWarps * kStages + 2) * 8;
   static constexpr int kPreOff = kLensOff + kMaxBatch * 4;
   static constexpr int kRecOff = kPreOff + (kMaxBatch + 4) * 4;
   static constexpr int kMiscOff = kRecOff + kWarps * 32;
-  static constexpr int kCopyWalkOff = kMiscOff + 192;           // a walk per warp: where its copies are
-  static constexpr int kSmemBytes = kCopyWalkOff + kWarps * 64;
+  static constexpr int kCopyWalkOff = kMiscOff + 192;           // walks of a warp: where its copies are, and where its work is
+  static constexpr int kSmemBytes = kCopyWalkOff + kWarps * 128;
   static_assert(kGran % 128 == 0 && kPiece % 128 == 0 && kStages * kGran >= kPiece && kWarpBytes % 128 == 0 && kCopy % 16 == 0, "copies land on 128-byte boundaries");
-  static_assert(!kFp8 || (kStages - 1) * kGran + 2 * kPiece <= kWarpBytes, "room for two pieces of the largest group");
+  static_assert(kStages >= 2 && kStages <= 8 && (!kFp8 || stages(kManyLayers, kMaxGroup) >= 2) && kSmemBytes <= kMaxSmem, "room for copies in flight");
   static_assert(kCtasPerSm * (kSmemBytes + 1024) <= 233472, "shared memory of one SM");
 };
 
@@ -107,9 +118,10 @@ struct Walk {
   int b, g, nb, u, n;
   int j, jend;
   unsigned base, end;
-  bool more;
+  int more;
+  int pad[2];
 };
-static_assert(sizeof(Walk) <= 48, "shared memory layout");
+static_assert(sizeof(Walk) == 48, "shared memory layout");
 __device__ __forceinline__ void walk_range(Walk& w, unsigned x) {
   w.j = max(0, static_cast<int>(x - w.base) - kUnitCost);
   w.jend = min(w.n, static_cast<int>(w.end - w.base) - kUnitCost);
@@ -252,6 +264,15 @@ __device__ __forceinline__ void acc_clear(Acc& a) { a.M = -INFINITY; a.den = 0.0
 template <bool kGlobal, class Rows>
 __device__ __forceinline__ void acc_merge(Acc& a, int n, float m, float l, bool on, Rows rows) {
   constexpr int kUnroll = 4;
+  float4 o[kUnroll];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int k = 0; k < kUnroll; ++k) {
+      const float4* from = reinterpret_cast<const float4*>(rows(min(k0 + k, n - 1)));
+      o[k] = on ? (kGlobal ? __ldcg(from) : *from) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    }
+  };
+  fetch(0);                              // (on their way while the weights are worked out)
   const bool some = l > 0.0f;
   const float top = fmaxf(a.M, ordered_to_f32(__reduce_max_sync(0xffffffffu, f32_to_ordered(some ? m : -INFINITY))));
   const float wgt = some ? l * ex2(m - top) : 0.0f;
@@ -259,25 +280,148 @@ __device__ __forceinline__ void acc_merge(Acc& a, int n, float m, float l, bool 
   a.num.x *= keep; a.num.y *= keep; a.num.z *= keep; a.num.w *= keep;
   a.den = a.den * keep + warp_sum(wgt);
   a.M = top;
-  for (int k0 = 0; k0 < n; k0 += kUnroll) {
-    float4 o[kUnroll];
-#pragma unroll
-    for (int k = 0; k < kUnroll; ++k) {
-      const float4* from = reinterpret_cast<const float4*>(rows(min(k0 + k, n - 1)));
-      o[k] = on ? (kGlobal ? __ldcg(from) : *from) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    }
+#pragma unroll 1
+  for (int k0 = 0;;) {
 #pragma unroll
     for (int k = 0; k < kUnroll; ++k) {
       const float w = k0 + k < n ? __shfl_sync(0xffffffffu, wgt, k0 + k) : 0.0f;
       if (w > 0.0f) { a.num.x += w * o[k].x; a.num.y += w * o[k].y; a.num.z += w * o[k].z; a.num.w += w * o[k].w; }
     }
+    k0 += kUnroll;
+    if (k0 >= n) break;
+    fetch(k0);
   }
 }
 
+// ---- units that several warps share: merged by log-sum-exp, one (unit, head) per warp at a time ---------------------------
+// Pieces of the warps of a CTA lie in shared memory.  A head of a piece that other shares hold the rest of goes to the
+// workspace, and is counted; who counts the last one takes them all and finishes the unit.  The first piece of a unit lies
+// in the odd slot of its share, the others in the even ones.
 template <int D, int FMT, int L>
-__global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decode_kernel(const DecodeParams p, const __grid_constant__ LayerTable<L> table) {
+struct Merge {
+  using C = Cfg<D, FMT>;
+  const DecodeParams& p;
+  const LayerTable<L>& table;
+  Line ln;
+  uint8_t* smem;
+  const Rec* recs;
+  unsigned T;                            // places of a share
+  int piece0_off, piece1_off;            // in a warp's part of shared memory
+  int warp, lane, y;                     // y: the layer
+  // What this warp has left in the workspace, lane i for the i-th piece: they are counted at once, so that the trips there
+  // and back (about 1 us) are made side by side.
+  int left = 0;
+  int left_cta = 0, left_pieces = 0, left_b = 0, left_gh = 0, left_u = 0, left_region = 0;
+
+  __device__ __forceinline__ bool on() const { return lane * 4 < D; }
+  __device__ __forceinline__ size_t slot_of(int region, int cta, bool first, int h) const {
+    return ((static_cast<size_t>(region) * p.shares + cta) * 2 + (first ? 1 : 0)) * p.group + h;
+  }
+  __device__ __forceinline__ void leave_piece(const Acc& a, int region, unsigned share, bool first, int b, int g, int h, int u, int cta_first, int pieces) {
+    const size_t at = slot_of(region, share, first, h);
+    const float dinv = a.den > 0.0f ? 1.0f / a.den : 0.0f;
+    if (on()) *reinterpret_cast<float4*>(p.run_o + at * D + lane * 4) = make_float4(a.num.x * dinv, a.num.y * dinv, a.num.z * dinv, a.num.w * dinv);
+    if (lane == 0) { p.run_m[at] = a.M; p.run_l[at] = a.den; }
+    if (lane == left) { left_cta = cta_first; left_pieces = pieces; left_b = b; left_gh = g * p.group + h; left_u = u; left_region = region; }
+    ++left;
+  }
+  __device__ __forceinline__ bool count_piece() const {      // one lane, behind the others' stores
+    // release (this piece is visible before the count moves) and acquire (the other pieces are visible before they are read)
+    int* counter = p.counters + (left_region * p.shares + left_cta) * kMaxGroup + left_gh % p.group;
+    int old;
+    asm volatile("atom.add.acq_rel.gpu.s32 %0, [%1], 1;" : "=r"(old) : "l"(counter) : "memory");
+    if (old != left_pieces - 1) return false;
+    *counter = 0;                        // ready for the next call
+    return true;
+  }
+  __device__ __forceinline__ void take_pieces(Acc& a, int region, int cta_f, int pieces, int h) const {
+    acc_clear(a);
+#pragma unroll 1
+    for (int c0 = 0; c0 < pieces; c0 += 32) {
+      const int n = min(32, pieces - c0);
+      auto slot = [&](int c) { return slot_of(region, cta_f + c, c == 0, h); };
+      const float m = lane < n ? __ldcg(p.run_m + slot(c0 + lane)) : 0.0f, l = lane < n ? __ldcg(p.run_l + slot(c0 + lane)) : 0.0f;
+      acc_merge<true>(a, n, m, l, on(), [&](int k) { return p.run_o + slot(c0 + k) * D + lane * 4; });
+    }
+  }
+  __device__ __forceinline__ void store_out(const Acc& a, int b, int g, int h) const {
+    const float dinv = a.den > 0.0f ? 1.0f / a.den : 0.0f;
+    if (on()) *reinterpret_cast<uint2*>(table.l[L == 1 ? 0 : y].out + (static_cast<size_t>(b) * p.num_q_heads + g * p.group + h) * D + lane * 4) =
+        make_uint2(pack_bf16x2(a.num.x * dinv, a.num.y * dinv), pack_bf16x2(a.num.z * dinv, a.num.w * dinv));
+  }
+  __device__ __forceinline__ void finish(const Acc& a, int b, int g, int h, int u) const {
+    if (p.chunk_blocks == 0 || line_blocks(ln, b) <= ln.chunk) store_out(a, b, g, h);
+    if (p.chunk_blocks > 0) {
+      const size_t at = (static_cast<size_t>(b) * p.num_q_heads + g * p.group + h) * p.max_chunks + u / ln.chunk;
+      const float dinv = a.den > 0.0f ? 1.0f / a.den : 0.0f;
+      if (on()) *reinterpret_cast<float4*>(p.part_o + at * D + lane * 4) = make_float4(a.num.x * dinv, a.num.y * dinv, a.num.z * dinv, a.num.w * dinv);
+      if (lane == 0) { p.part_m[at] = a.M * kLn2; p.part_l[at] = a.den * kUnshift; }
+    }
+  }
+  // what the warps of this CTA hold of the units of a share
+  __device__ __forceinline__ void local(unsigned share) {
+    const int G = p.group;
+    const int region = L > 1 ? y : p.chunk_blocks > 0 ? 1 : 0;
+    const int flags = lane < C::kWarps ? recs[lane].flags : 0;
+    const unsigned has0 = __ballot_sync(0xffffffffu, flags & kHas0), ends0 = __ballot_sync(0xffffffffu, flags & kEnds0), has1 = __ballot_sync(0xffffffffu, flags & kHas1);
+    // a chain: the warps that hold pieces of one unit, the first of them `from` (kind 0: the unit began in another CTA)
+    const int chains = static_cast<int>(has0 & 1u) + __popc(has1);
+    static_assert((C::kWarps + 1) * kMaxGroup / C::kWarps + 3 <= 32, "a lane for every piece a warp leaves");
+#pragma unroll 1
+    for (int task = warp; task < chains * G; task += C::kWarps) {
+      const int ci = task / G, h = task - ci * G;
+      const int kind = (has0 & 1u) && ci == 0 ? 0 : 1;
+      unsigned rest = has1;
+      for (int k = static_cast<int>(has0 & 1u); k < ci; ++k) rest &= rest - 1;
+      const int from = kind ? __ffs(rest) - 1 : 0;
+      int last = from;
+      bool closed = kind == 0 && (ends0 & 1u);
+      if (!closed) {
+        const int held = __ffs(~(has0 >> (from + 1))) - 1, end = __ffs(ends0 >> (from + 1));
+        closed = end != 0 && end <= held;
+        last = from + (closed ? end : held);
+      }
+      const int b = kind ? recs[from].b1 : recs[from].b0, g = kind ? recs[from].g1 : recs[from].g0, u = kind ? recs[from].u1 : recs[from].u0;
+      auto piece = [&](int k) {
+        return reinterpret_cast<const float*>(smem + (from + k) * C::kWarpBytes + ((kind && k == 0) ? piece1_off : piece0_off)) + h * C::kPieceStride;
+      };
+      const int n = last - from + 1;
+      Acc a;
+      acc_clear(a);
+      acc_merge<false>(a, n, lane < n ? piece(lane)[D] : 0.0f, lane < n ? piece(lane)[D + 1] : 0.0f, on(), [&](int k) { return piece(k) + lane * 4; });
+      if (kind && closed) {
+        finish(a, b, g, h, u);
+      } else {
+        const unsigned first = unit_place(ln, b, g, u) + kUnitCost;
+        const int nu = unit_blocks(ln, line_blocks(ln, b), u), cta_f = first / T;
+        leave_piece(a, region, share, kind != 0, b, g, h, u, cta_f, static_cast<int>((first + nu - 1) / T) - cta_f + 1);
+      }
+    }
+  }
+  // the pieces left in the workspace: counted, and units finished of which they were the last.  (In chunk mode region 0 has
+  // whole (sequence, kv head) pairs, of which the output is due, region 1 chunks.)
+  __device__ __forceinline__ void count_and_finish() const {
+    __syncwarp();
+    unsigned last = __ballot_sync(0xffffffffu, left_pieces > 0 && count_piece());
+    __syncwarp();                        // the others' pieces, which a lane has acquired, are there for all lanes
+#pragma unroll 1
+    for (; last != 0; last &= last - 1) {
+      const int i = __ffs(last) - 1, gh = __shfl_sync(0xffffffffu, left_gh, i), g = gh / p.group, h = gh - g * p.group;
+      const int region = __shfl_sync(0xffffffffu, left_region, i), b = __shfl_sync(0xffffffffu, left_b, i), u = __shfl_sync(0xffffffffu, left_u, i);
+      Acc a;
+      take_pieces(a, region, __shfl_sync(0xffffffffu, left_cta, i), __shfl_sync(0xffffffffu, left_pieces, i), h);
+      if (L == 1 && p.chunk_blocks > 0 && region == 0) store_out(a, b, g, h); else finish(a, b, g, h, u);
+    }
+  }
+};
+
+template <int kBlocks> struct Blocks { static constexpr int kCount = kBlocks; };
+
+template <int D, int FMT, int L>
+__global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decode_kernel(const __grid_constant__ DecodeParams p, const __grid_constant__ LayerTable<L> table) {
   using C = Cfg<D, FMT>;
   constexpr int kQSteps = D / 16;
+  constexpr int N = C::kFp8 ? 2 : 1;     // blocks that a warp takes at a time
   extern __shared__ __align__(128) uint8_t smem[];
   int* lens = reinterpret_cast<int*>(smem + C::kLensOff);
   unsigned* pre = reinterpret_cast<unsigned*>(smem + C::kPreOff);
@@ -393,8 +537,9 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
   const unsigned shares = by_unit ? B * Hkv : (places + T - 1) / T, all_shares = L == 1 ? shares : shares * p.layers;
   // What is looked at seldom waits in shared memory, a copy for every warp, and not in registers that the loop over blocks
   // needs: the walk of the copies (once in 32 blocks), its share, and how shares are cut.
-  Walk* copy_walk = reinterpret_cast<Walk*>(smem + C::kCopyWalkOff + warp * 64);
-  unsigned* copy_share = reinterpret_cast<unsigned*>(copy_walk) + 12;
+  Walk* copy_walk = reinterpret_cast<Walk*>(smem + C::kCopyWalkOff + warp * 128);
+  Walk* work_walk = copy_walk + 1;
+  unsigned* copy_share = reinterpret_cast<unsigned*>(copy_walk) + 24;
   volatile unsigned* cut = copy_share + 1;                              // [0] bit 0: whole, bit 1: solo, bit 2: by unit; [1] T
   if (lane == 0) { cut[0] = by_unit ? 4u : (whole ? 1u : 0u) | (solo ? 2u : 0u); cut[1] = T; }
   __syncwarp();
@@ -463,7 +608,8 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
   Walk fw = w;
   if (ps < all_shares) walk_later(ps, fw);                              // the first unit, and its layer
   const int fy = share_layer(ps);
-  int ids_a = 0, cnt_a = 0, g_a = 0, y_a = 0, pos_a = 0, ids_b = 0, cnt_b = 0, g_b = 0, y_b = 0;
+  const uint8_t* from_a = nullptr;                 // this lane's granule of the batch
+  int cnt_a = 0, pos_a = 0, ids_b = 0, cnt_b = 0, g_b = 0, y_b = 0;
   auto prefetch_q = [&](int y, int b, int g) {
     if (lane < G * D / 64) prefetch_l2(reinterpret_cast<const uint8_t*>(layer(y).q + (static_cast<size_t>(b) * Hq + g * G) * D) + lane * 128);
   };
@@ -486,29 +632,36 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
     __syncwarp();
   };
   auto take_ids = [&]() {
-    ids_a = ids_b; cnt_a = cnt_b; g_a = g_b; y_a = y_b; pos_a = 0;
-    if (ids_a < 0 || ids_a >= p.num_blocks) {      // reported, and replaced by block 0: never dereferenced
+    int id = ids_b;
+    if (id < 0 || id >= p.num_blocks) {            // reported, and replaced by block 0: never dereferenced
       if (p.plan == nullptr) atomicCAS(p.status, 0, COOPT_ERR_INVALID_ARG);
-      ids_a = 0;
+      id = 0;
     }
+    from_a = layer(y_b).cache + (static_cast<size_t>(id) * Hkv + g_b) * C::kGran;
+    cnt_a = cnt_b; pos_a = 0;
     fetch_ids();
   };
   uint32_t issued = 0, consumed = 0;               // copies, and the stages that take the next one and hold the oldest one
   int in_stage = 0, out_stage = 0;
   uint32_t out_phase = 0;
-  auto issue = [&]() {
-    if (pos_a == cnt_a) take_ids();
-    if (pos_a < cnt_a) {
-      const int id = __shfl_sync(0xffffffffu, ids_a, pos_a);
-      ++pos_a;
-      const int stage = in_stage;
-      if (++in_stage == stages) in_stage = 0;
-      if (lane == 0) {
+  // The next `left` copies (fewer at the end): each by the lane that has its granule's address.
+  auto issue = [&](int left) {
+#pragma unroll 1
+    do {
+      if (pos_a == cnt_a) take_ids();
+      const int n = min(left, cnt_a - pos_a), k = lane - pos_a;
+      if (n == 0) return;
+      if (k >= 0 && k < n) {
+        const int stage = in_stage + k < stages ? in_stage + k : in_stage + k - stages;
         mbar_expect_tx(&bars[stage], C::kCopy);
-        bulk_copy_g2s(ring + stage * C::kGran, layer(y_a).cache + (static_cast<size_t>(id) * Hkv + g_a) * C::kGran, C::kCopy, &bars[stage]);
+        bulk_copy_g2s(ring + stage * C::kGran, from_a, C::kCopy, &bars[stage]);
       }
-      ++issued;
-    }
+      pos_a += n;
+      in_stage += n;
+      if (in_stage >= stages) in_stage -= stages;
+      issued += n;
+      left -= n;
+    } while (left > 0);
   };
 
   // ---- per-lane constants of the operand layouts ---------------------------------------------------------------
@@ -554,7 +707,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
   for (int step = 0; step < 2; ++step) {
     if ((step == 0) == (p.order == kOverlapPrevious)) {
 #pragma unroll 1
-      for (int i = 0; i < stages; ++i) issue();
+      for (int i = 0; i < stages; ++i) issue(1);
       COOPT_TRACE_CYCLES(p.trace, kTrFirstCopy, tid == 0);
     } else {
       if (p.order != kDependent) wait_previous_kernel();
@@ -575,16 +728,13 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
       for (int y = 0; y < (L == 1 ? 1 : p.layers); ++y)
         for (int i = tid; i < Hq * D / 8; i += C::kThreads) reinterpret_cast<uint4*>(layer(y).out + static_cast<size_t>(b) * Hq * D)[i] = make_uint4(0u, 0u, 0u, 0u);
 
-  const int d0 = lane * 4;
-  const bool on = d0 < D;
   uint32_t round = 0;
 #pragma unroll 1
   for (unsigned share = blockIdx.x; share < all_shares; share += gridDim.x, ++round) {
   const int y = share_layer(share);
   const unsigned v_share = L == 1 ? share : share - y * shares;
   if (round > 0) share_walk(share, w);
-  Rec rec;
-  rec.flags = 0;
+  int flags = 0;                         // of the pieces this warp leaves (Rec)
 #pragma unroll 1
   while (w.more) {
     if (consumed != 0) load_q(y, w.b, w.g);
@@ -621,85 +771,77 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
       for (int e = 0; e < 4; ++e) o[t][e] = 0.0f;
     float m[2] = {-INFINITY, -INFINITY}, top[2] = {-INFINITY, -INFINITY}, l[2] = {0.0f, 0.0f};
     float vref = 0.0f, vinv = 0.0f;
-    const int ctx = lens[w.b];
-    const bool has_new = C::kFp8 && layer(y).k_new != nullptr;
+    // what the loop over blocks needs of the walk; the rest waits in shared memory
+    const int j_end = w.jend, valid = lens[w.b] - w.u * kBlockSize;            // (the end of the context, counted from the unit's start)
+    if (lane == 0) *work_walk = w;
+    __syncwarp();
 
-#pragma unroll 1
-    for (int j = w.j; j < w.jend; ++j) {
-      // the step's new token: what it needs is loaded while its block is on the way
-      const bool append = has_new && w.u + j == w.nb - 1;
-      long long slot = -1;
-      int id = 0;
-      uint2 k_row = make_uint2(0u, 0u), v_row = k_row;
+    // Some blocks, of which the first `seen` tokens count.
+    auto attend = [&](auto count, uint8_t* const st0, uint8_t* const st1, int seen) {
+      constexpr int kN = decltype(count)::kCount;
+      uint8_t* const st[2] = {st0, st1};
+      // ---- S^T = K Q^T: 16 tokens x 8 heads a block ------------------------------------------------------------------
+      float x[kN][4], sv[kN];
       if constexpr (C::kFp8) {
-        if (append) {
-          const LayerPtrs& io = layer(y);
-          const bool vec = ((reinterpret_cast<uintptr_t>(io.k_new) | reinterpret_cast<uintptr_t>(io.v_new) | static_cast<uintptr_t>(p.kv_token_stride * 2)) & (D / 16 - 1)) == 0;
-          const long long at = static_cast<long long>(w.b) * p.kv_token_stride + w.g * D;
-          slot = io.slot_mapping[w.b];
-          id = p.block_table[static_cast<size_t>(w.b) * p.max_blocks_per_seq + w.nb - 1];
-          k_row = load_new<D>(io.k_new + at, vec, lane);
-          v_row = load_new<D>(io.v_new + at, vec, lane);
+        float sa[kN][4], sb[kN][4];
+        float2 hdr[kN];
+#pragma unroll
+        for (int i = 0; i < kN; ++i) {
+          hdr[i] = *reinterpret_cast<const float2*>(st[i] + header_offset(D));
+#pragma unroll
+          for (int e = 0; e < 4; ++e) sa[i][e] = sb[i][e] = 0.0f;
         }
-      }
-      if (!dead && !mbar_wait_bounded(&bars[out_stage], out_phase)) {
-        dead = true;
-      }
-      dead = __any_sync(0xffffffffu, dead);
-      COOPT_TRACE_CYCLES(p.trace, kTrFirstLanded, tid == 0 && consumed == 0);
-      if (dead) continue;
-      uint8_t* st = ring + out_stage * C::kGran;
-      ++consumed;
-      if (++out_stage == stages) { out_stage = 0; out_phase ^= 1u; }
-      const int nvalid = min(kBlockSize, ctx - (w.u + j) * kBlockSize);      // Eq. 9: tail of the context
-
-      if constexpr (C::kFp8) {
-        if (append && slot >= 0) {                                             // Eq. 5: negative slots are skipped
-          const int off = (ctx - 1) % kBlockSize;
-          if (slot != static_cast<long long>(id) * kBlockSize + off) {         // not the sequence's last position
-            if (lane == 0) atomicCAS(p.status, 0, COOPT_ERR_INVALID_ARG);
-          } else if (id >= 0 && id < p.num_blocks) {
-            append_token<D, C::kE5m2>(st, layer(y).cache + (static_cast<size_t>(id) * Hkv + w.g) * C::kGran, k_row, v_row, off, lane);
-          }
-          __syncwarp();
-        }
-      }
-
-      // ---- S^T = K Q^T: 16 tokens x 8 heads ------------------------------------------------------------------------
-      float sa[4] = {0.0f, 0.0f, 0.0f, 0.0f}, sb[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-      float sk = 1.0f, sv = 1.0f;
-      if constexpr (C::kFp8) {
-        const uint32_t ka = smem_u32(st) + k_lane;
-        const float2 hdr = *reinterpret_cast<const float2*>(st + header_offset(D));
-        sk = hdr.x; sv = hdr.y;
 #pragma unroll
         for (int c = 0; c < D / 32; ++c) {
-          uint32_t r[4];
-          ldmatrix4(ka + c * 256, r);
-          mma16816<true>(sa, codes_lo<C::kE5m2>(r[0]), codes_lo<C::kE5m2>(r[1]), codes_hi<C::kE5m2>(r[0]), codes_hi<C::kE5m2>(r[1]), qf[2 * c][0], qf[2 * c][1]);
-          mma16816<true>(sb, codes_lo<C::kE5m2>(r[2]), codes_lo<C::kE5m2>(r[3]), codes_hi<C::kE5m2>(r[2]), codes_hi<C::kE5m2>(r[3]), qf[2 * c + 1][0], qf[2 * c + 1][1]);
+#pragma unroll
+          for (int i = 0; i < kN; ++i) {
+            uint32_t r[4];
+            ldmatrix4(smem_u32(st[i]) + k_lane + c * 256, r);
+            mma16816<true>(sa[i], codes_lo<C::kE5m2>(r[0]), codes_lo<C::kE5m2>(r[1]), codes_hi<C::kE5m2>(r[0]), codes_hi<C::kE5m2>(r[1]), qf[2 * c][0], qf[2 * c][1]);
+            mma16816<true>(sb[i], codes_lo<C::kE5m2>(r[2]), codes_lo<C::kE5m2>(r[3]), codes_hi<C::kE5m2>(r[2]), codes_hi<C::kE5m2>(r[3]), qf[2 * c + 1][0], qf[2 * c + 1][1]);
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < kN; ++i) {
+          const float k0 = qs[0] * hdr[i].x, k1 = qs[1] * hdr[i].x;
+          sv[i] = hdr[i].y;
+          x[i][0] = (sa[i][0] + sb[i][0]) * k0; x[i][1] = (sa[i][1] + sb[i][1]) * k1;
+          x[i][2] = (sa[i][2] + sb[i][2]) * k0; x[i][3] = (sa[i][3] + sb[i][3]) * k1;
         }
       } else {
-        const uint8_t* kp = st + lane * 16;
+        float sa[4] = {0.0f, 0.0f, 0.0f, 0.0f}, sb[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        const uint8_t* kp = st[0] + lane * 16;
 #pragma unroll
         for (int i = 0; i < D / 32; ++i) {
           const uint4 w0 = lds128(kp + i * 512), w1 = lds128(kp + (D / 32 + i) * 512);
           mma16816<false>(sa, w0.x, w1.x, w0.y, w1.y, qf[2 * i][0], qf[2 * i][1]);
           mma16816<false>(sb, w0.z, w1.z, w0.w, w1.w, qf[2 * i + 1][0], qf[2 * i + 1][1]);
         }
+        sv[0] = 1.0f;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x[0][e] = (sa[e] + sb[e]) * qs[e & 1];
       }
 
       // ---- online softmax (Eq. 10) in base-2 units; the reference maximum is lazy ------------------------------------
-      const float k0 = qs[0] * sk, k1 = qs[1] * sk;
-      float x[4] = {(sa[0] + sb[0]) * k0, (sa[1] + sb[1]) * k1, (sa[2] + sb[2]) * k0, (sa[3] + sb[3]) * k1};
-      if (nvalid < kBlockSize) {
-        if (tok0 >= nvalid) x[0] = x[1] = -INFINITY;
-        if (tok0 + kTokStep >= nvalid) x[2] = x[3] = -INFINITY;
+      if (seen < kN * kBlockSize) {
+#pragma unroll
+        for (int i = 0; i < kN; ++i) {
+          if (tok0 + i * kBlockSize >= seen) x[i][0] = x[i][1] = -INFINITY;
+          if (tok0 + kTokStep + i * kBlockSize >= seen) x[i][2] = x[i][3] = -INFINITY;
+        }
       }
-      const float t0 = fmaxf(x[0], x[2]), t1 = fmaxf(x[1], x[3]);
-      top[0] = fmaxf(top[0], t0);
-      top[1] = fmaxf(top[1], t1);
-      const bool grow = C::kFp8 && sv > vref;
+      float t0 = fmaxf(x[0][0], x[0][2]), t1 = fmaxf(x[0][1], x[0][3]), sv_top = sv[0];
+#pragma unroll
+      for (int i = 1; i < kN; ++i) {
+        t0 = fmaxf(t0, fmaxf(x[i][0], x[i][2]));
+        t1 = fmaxf(t1, fmaxf(x[i][1], x[i][3]));
+        sv_top = fmaxf(sv_top, sv[i]);
+      }
+      if constexpr (L == 1) {                      // (for exported partials)
+        top[0] = fmaxf(top[0], t0);
+        top[1] = fmaxf(top[1], t1);
+      }
+      const bool grow = C::kFp8 && sv_top > vref;
       if (__any_sync(0xffffffffu, t0 > m[0] + kLag || t1 > m[1] + kLag) || grow) {
         float f[2];
 #pragma unroll
@@ -714,7 +856,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
           l[h] *= f[h];
         }
         if (grow) {                                // (a reference is a normal number: its reciprocal is one then, too)
-          const float vnew = fmaxf(sv, FLT_MIN);
+          const float vnew = fmaxf(sv_top, FLT_MIN);
           vinv = 1.0f / vnew;
           const float fv = vref * vinv;
           f[0] *= fv; f[1] *= fv;
@@ -723,41 +865,44 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
 #pragma unroll
         for (int t = 0; t < D / 16; ++t) { o[t][0] *= f[0]; o[t][1] *= f[1]; o[t][2] *= f[0]; o[t][3] *= f[1]; }
       }
-      float pr[4];
       const float b0 = kShift - m[0], b1 = kShift - m[1];
-      pr[0] = ex2(x[0] + b0); pr[1] = ex2(x[1] + b1); pr[2] = ex2(x[2] + b0); pr[3] = ex2(x[3] + b1);
-      l[0] += pr[0] + pr[2];
-      l[1] += pr[1] + pr[3];
+#pragma unroll
+      for (int i = 0; i < kN; ++i) {
+        x[i][0] = ex2(x[i][0] + b0); x[i][1] = ex2(x[i][1] + b1); x[i][2] = ex2(x[i][2] + b0); x[i][3] = ex2(x[i][3] + b1);
+        l[0] += x[i][0] + x[i][2];
+        l[1] += x[i][1] + x[i][3];
+      }
 
       // ---- O^T += V^T P^T -----------------------------------------------------------------------------------------------
       if constexpr (C::kFp8) {
-        const float pv = sv * vinv;
-        const uint32_t p0 = transpose8x8(pack_f16x2(pr[0] * pv, pr[1] * pv)), p1 = transpose8x8(pack_f16x2(pr[2] * pv, pr[3] * pv));
-        const uint32_t va = smem_u32(st) + kBlockSize * D + lane * 16;
-        uint32_t mask = 0xFFFFFFFFu;
-        if (nvalid < kBlockSize) {                 // codes of slots past the context are cleared: they may hold anything
-          const int keep = nvalid - 4 * quad;
-          mask = keep >= 4 ? 0xFFFFFFFFu : keep <= 0 ? 0u : (1u << (8 * keep)) - 1u;
+        uint32_t p0[kN], p1[kN];
+#pragma unroll
+        for (int i = 0; i < kN; ++i) {
+          const float pv = sv[i] * vinv;
+          p0[i] = transpose8x8(pack_f16x2(x[i][0] * pv, x[i][1] * pv));
+          p1[i] = transpose8x8(pack_f16x2(x[i][2] * pv, x[i][3] * pv));
         }
 #pragma unroll
-        for (int i = 0; i < D / 32; ++i) {
-          uint32_t r[4];
-          ldmatrix4(va + i * 512, r);
+        for (int c = 0; c < D / 32; ++c) {
 #pragma unroll
-          for (int e = 0; e < 4; ++e) r[e] &= mask;
-          mma16816<true>(o[2 * i], codes_lo<C::kE5m2>(r[0]), codes_lo<C::kE5m2>(r[1]), codes_hi<C::kE5m2>(r[0]), codes_hi<C::kE5m2>(r[1]), p0, p1);
-          mma16816<true>(o[2 * i + 1], codes_lo<C::kE5m2>(r[2]), codes_lo<C::kE5m2>(r[3]), codes_hi<C::kE5m2>(r[2]), codes_hi<C::kE5m2>(r[3]), p0, p1);
+          for (int i = 0; i < kN; ++i) {
+            uint32_t r[4];
+            ldmatrix4(smem_u32(st[i]) + kBlockSize * D + lane * 16 + c * 512, r);
+            mma16816<true>(o[2 * c], codes_lo<C::kE5m2>(r[0]), codes_lo<C::kE5m2>(r[1]), codes_hi<C::kE5m2>(r[0]), codes_hi<C::kE5m2>(r[1]), p0[i], p1[i]);
+            mma16816<true>(o[2 * c + 1], codes_lo<C::kE5m2>(r[2]), codes_lo<C::kE5m2>(r[3]), codes_hi<C::kE5m2>(r[2]), codes_hi<C::kE5m2>(r[3]), p0[i], p1[i]);
+          }
         }
       } else {
         // bf16 probabilities as a high and a low half (16 bits in all)
+        const float (&pr)[4] = x[0];
         const uint32_t h0 = pack_bf16x2(pr[0], pr[1]), h1 = pack_bf16x2(pr[2], pr[3]);
         const uint32_t e0 = pack_bf16x2(pr[0] - bf16_lo(h0), pr[1] - bf16_hi(h0)), e1 = pack_bf16x2(pr[2] - bf16_lo(h1), pr[3] - bf16_hi(h1));
         const uint32_t p0 = transpose8x8(h0), p1 = transpose8x8(h1), r0 = transpose8x8(e0), r1 = transpose8x8(e1);
-        const uint8_t* vp = st + part_offset(D, false, 1) + lane * 16;
+        const uint8_t* vp = st[0] + part_offset(D, false, 1) + lane * 16;
         uint32_t m0 = 0xFFFFFFFFu, m1 = 0xFFFFFFFFu;
-        if (nvalid < kBlockSize) {
-          m0 = (2 * quad < nvalid ? 0x0000FFFFu : 0u) | (2 * quad + 1 < nvalid ? 0xFFFF0000u : 0u);
-          m1 = (2 * quad + 8 < nvalid ? 0x0000FFFFu : 0u) | (2 * quad + 9 < nvalid ? 0xFFFF0000u : 0u);
+        if (seen < kBlockSize) {
+          m0 = (2 * quad < seen ? 0x0000FFFFu : 0u) | (2 * quad + 1 < seen ? 0xFFFF0000u : 0u);
+          m1 = (2 * quad + 8 < seen ? 0x0000FFFFu : 0u) | (2 * quad + 9 < seen ? 0xFFFF0000u : 0u);
         }
 #pragma unroll
         for (int i = 0; i < D / 16; ++i) {
@@ -766,13 +911,96 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
           mma16816<false>(o[i], v.x & m0, v.z & m0, v.y & m1, v.w & m1, r0, r1);
         }
       }
+    };
+#pragma unroll 1
+    for (int j = w.j; j < j_end && !dead; j += N) {
+      // (The one test that every block meets: whether there is less than a full step of blocks, all of them before the last of the
+      // context.  A block that is not there counts for nothing.)
+      const bool rare = j + N > j_end || (j + N) * kBlockSize >= valid;
+      int n = N, seen = N * kBlockSize;                                      // blocks, and tokens of them (Eq. 9)
+      // the step's new token: what it needs is loaded while its block is on the way
+      bool append = false;
+      long long slot = -1;
+      int id = 0;
+      uint2 k_row = make_uint2(0u, 0u), v_row = k_row;
+      if (rare) {
+        n = min(N, j_end - j);
+        seen = min(valid - j * kBlockSize, n * kBlockSize);
+        if constexpr (C::kFp8) {
+          append = layer(y).k_new != nullptr && (j + n) * kBlockSize >= valid;
+          if (append) {
+            const LayerPtrs& io = layer(y);
+            const bool vec = ((reinterpret_cast<uintptr_t>(io.k_new) | reinterpret_cast<uintptr_t>(io.v_new) | static_cast<uintptr_t>(p.kv_token_stride * 2)) & (D / 16 - 1)) == 0;
+            const long long at = static_cast<long long>(work_walk->b) * p.kv_token_stride + work_walk->g * D;
+            slot = io.slot_mapping[work_walk->b];
+            id = p.block_table[static_cast<size_t>(work_walk->b) * p.max_blocks_per_seq + work_walk->u + (valid - 1) / kBlockSize];
+            k_row = load_new<D>(io.k_new + at, vec, lane);
+            v_row = load_new<D>(io.v_new + at, vec, lane);
+          }
+        }
+      }
+      // the oldest copies in flight
+      uint8_t* st[N];
+      st[0] = ring + out_stage * C::kGran;
+      bool there = mbar_wait_bounded(&bars[out_stage], out_phase);
+      if (++out_stage == stages) { out_stage = 0; out_phase ^= 1u; }
+      if constexpr (N == 2) {
+        st[1] = st[0];
+        if (n == 2) {
+          st[1] = ring + out_stage * C::kGran;
+          there = there && mbar_wait_bounded(&bars[out_stage], out_phase);
+          if (++out_stage == stages) { out_stage = 0; out_phase ^= 1u; }
+        }
+      }
+      dead = !__all_sync(0xffffffffu, there);
+      COOPT_TRACE_CYCLES(p.trace, kTrFirstLanded, tid == 0 && consumed == 0);
+      if (dead) {                                  // (the stages that were waited for stay the oldest)
+        out_stage -= n;
+        if (out_stage < 0) { out_stage += stages; out_phase ^= 1u; }
+        break;
+      }
+      consumed += n;
+      if constexpr (C::kFp8) {
+        if (rare) {
+          uint8_t* const tail = st[n - 1];
+          if (append && slot >= 0) {                                         // Eq. 5: negative slots are skipped
+            const int off = (valid - 1) % kBlockSize;
+            if (slot != static_cast<long long>(id) * kBlockSize + off) {     // not the sequence's last position
+              if (lane == 0) atomicCAS(p.status, 0, COOPT_ERR_INVALID_ARG);
+            } else if (id >= 0 && id < p.num_blocks) {
+              append_token<D, C::kE5m2>(tail, layer(y).cache + (static_cast<size_t>(id) * Hkv + work_walk->g) * C::kGran, k_row, v_row, off, lane);
+            }
+            __syncwarp();
+          }
+          if (seen < n * kBlockSize) {             // V codes of slots past the context are cleared: they may hold anything
+            const int keep = seen - (n - 1) * kBlockSize;
+            auto mask = [&](int word) { return keep >= 4 * word + 4 ? 0xFFFFFFFFu : keep <= 4 * word ? 0u : (1u << (8 * (keep - 4 * word))) - 1u; };
+#pragma unroll
+            for (int i = 0; i < D / 32; ++i) {
+              uint4* row = reinterpret_cast<uint4*>(tail + kBlockSize * D) + i * 32 + lane;      // 16 tokens of a dim
+              const uint4 v = *row;
+              *row = make_uint4(v.x & mask(0), v.y & mask(1), v.z & mask(2), v.w & mask(3));
+            }
+            __syncwarp();
+          }
+        }
+      }
 
-      // ---- the stage goes back to the copy engine ---------------------------------------------------------------------
+      // (A single block by the code for two gives the same result and takes two thirds of the time of two.  A launch over one layer
+      // has no other code: fetching it would cost more.)
+      if constexpr (L > 1 && N == 2) {
+        if (n == 2) attend(Blocks<2>(), st[0], st[N - 1], seen); else attend(Blocks<1>(), st[0], st[0], seen);
+      } else {
+        attend(Blocks<N>(), st[0], st[N - 1], seen);
+      }
+
+      // ---- the stages go back to the copy engine ------------------------------------------------------------------------
       __syncwarp();
-      if (lane == 0) fence_proxy_async();
-      issue();
+      fence_proxy_async();
+      issue(n);
     }
-
+    w = *work_walk;
+    __syncwarp();
     // ---- end of the unit (or of this warp's piece of it) ----------------------------------------------------------------
     if constexpr (C::kFp8) {
       if (__builtin_expect(vref < 0x1p-64f && vref > 0.0f, 0)) {      // (vref / l would lose bits among the subnormals)
@@ -789,7 +1017,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
 #pragma unroll
       for (int s = 4; s <= 16; s <<= 1) l[h] += __shfl_xor_sync(0xffffffffu, l[h], s);
       inv[h] = l[h] > 0.0f ? (C::kFp8 ? vref : 1.0f) / l[h] : 0.0f;      // o and l go by the same reference
-      if (p.chunk_blocks > 0) {                    // exported partials carry the true maximum
+      if (L == 1 && p.chunk_blocks > 0) {          // exported partials carry the true maximum
 #pragma unroll
         for (int s = 4; s <= 16; s <<= 1) top[h] = fmaxf(top[h], __shfl_xor_sync(0xffffffffu, top[h], s));
         l[h] *= ex2(m[h] - top[h]);
@@ -825,7 +1053,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
     }
     if (!(starts && ends)) {
       // a piece: into shared memory, once the pieces of the share before are of no more use
-      if (L > 1 && round > 0 && rec.flags == 0 && !dead && !mbar_wait_bounded(bar_merged, (round - 1) & 1u)) dead = true;
+      if (L > 1 && round > 0 && flags == 0 && !dead) dead = !__all_sync(0xffffffffu, mbar_wait_bounded(bar_merged, (round - 1) & 1u));
       float* piece = reinterpret_cast<float*>(ring + (starts ? piece1_off : piece0_off));
       float* at = piece + 2 * quad * C::kPieceStride + row;
 #pragma unroll
@@ -839,8 +1067,12 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
           if (row == 0) *reinterpret_cast<float2*>(at + h * C::kPieceStride + D) = make_float2(m[h], l[h]);
         }
       }
-      if (starts) { rec.b1 = w.b; rec.g1 = w.g; rec.u1 = w.u; rec.flags |= kHas1; }
-      else { rec.b0 = w.b; rec.g0 = w.g; rec.u0 = w.u; rec.flags |= kHas0 | (ends ? kEnds0 : 0); }
+      if (lane == 0) {
+        Rec& rec = recs[warp];
+        if (starts) { rec.b1 = w.b; rec.g1 = w.g; rec.u1 = w.u; }
+        else { rec.b0 = w.b; rec.g0 = w.g; rec.u0 = w.u; }
+      }
+      flags |= starts ? kHas1 : kHas0 | (ends ? kEnds0 : 0);
     }
     walk_next(ln, w);
   }
@@ -848,17 +1080,17 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
   COOPT_TRACE_VALUE(p.trace, kTrBlocks, tid == 0, consumed);
   if ((cut[0] & 2u) != 0) break;         // solo: one share a CTA
   if (L == 1) {
-    if (lane == 0) recs[warp] = rec;
+    if (lane == 0) recs[warp].flags = flags;
     __syncthreads();
   } else {
-    if (round > 0 && rec.flags == 0 && !dead && !mbar_wait_bounded(bar_merged, (round - 1) & 1u)) dead = true;   // (its record is still in use)
+    if (round > 0 && flags == 0 && !dead && !mbar_wait_bounded(bar_merged, (round - 1) & 1u)) dead = true;   // (its record is still in use)
     // A warp whose wait has run out leaves without another word to the others (its record may still be in use, and an arrival
     // ahead of its time would complete a phase that others have not reached): their waits for it run out in turn.
     dead = __any_sync(0xffffffffu, dead);
     if (dead) break;
     __syncwarp();                        // every lane's part of the pieces is there (a vote orders no memory)
     if (lane == 0) {
-      recs[warp] = rec;
+      recs[warp].flags = flags;
       mbar_arrive(bar_pieces);
     }
     dead = !mbar_wait_bounded(bar_pieces, round & 1u);
@@ -867,102 +1099,15 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
   }
   COOPT_TRACE_CYCLES(p.trace, kTrStreamed, tid == 0);
 
-  // ---- units that several warps share: merged by log-sum-exp, one (unit, head) per warp ---------------------------------
-  // A head of a piece that other shares hold the rest of goes to the workspace, and is counted; who counts the last one takes
-  // them all and finishes the unit.  The first piece of a unit lies in the odd slot of its share, the others in the even ones.
-  auto slot_of = [&](int region, int cta, bool first, int h) -> size_t { return ((static_cast<size_t>(region) * p.shares + cta) * 2 + (first ? 1 : 0)) * G + h; };
-  auto leave_piece = [&](const Acc& a, size_t at) {
-    const float dinv = a.den > 0.0f ? 1.0f / a.den : 0.0f;
-    if (on) *reinterpret_cast<float4*>(p.run_o + at * D + d0) = make_float4(a.num.x * dinv, a.num.y * dinv, a.num.z * dinv, a.num.w * dinv);
-    if (lane == 0) { p.run_m[at] = a.M; p.run_l[at] = a.den; }
-  };
-  auto count_piece = [&](int region, int cta_f, int pieces, int h) -> bool {      // one lane, behind the others' stores
-    // release (this piece is visible before the count moves) and acquire (the other pieces are visible before they are read)
-    int* counter = p.counters + (region * p.shares + cta_f) * kMaxGroup + h;
-    int old;
-    asm volatile("atom.add.acq_rel.gpu.s32 %0, [%1], 1;" : "=r"(old) : "l"(counter) : "memory");
-    if (old != pieces - 1) return false;
-    *counter = 0;                        // ready for the next call
-    return true;
-  };
-  auto take_pieces = [&](Acc& a, int region, int cta_f, int pieces, int h) {
-    acc_clear(a);
-    for (int c0 = 0; c0 < pieces; c0 += 32) {
-      const int n = min(32, pieces - c0);
-      auto slot = [&](int c) { return slot_of(region, cta_f + c, c == 0, h); };
-      const float m = lane < n ? __ldcg(p.run_m + slot(c0 + lane)) : 0.0f, l = lane < n ? __ldcg(p.run_l + slot(c0 + lane)) : 0.0f;
-      acc_merge<true>(a, n, m, l, on, [&](int k) { return p.run_o + slot(c0 + k) * D + d0; });
-    }
-  };
-  auto store_out = [&](const Acc& a, int b, int g, int h) {
-    const float dinv = a.den > 0.0f ? 1.0f / a.den : 0.0f;
-    if (on) *reinterpret_cast<uint2*>(layer(y).out + (static_cast<size_t>(b) * Hq + g * G + h) * D + d0) =
-        make_uint2(pack_bf16x2(a.num.x * dinv, a.num.y * dinv), pack_bf16x2(a.num.z * dinv, a.num.w * dinv));
-  };
-  auto finish = [&](const Acc& a, int b, int g, int h, int u) {
-    if (p.chunk_blocks == 0 || line_blocks(ln, b) <= ln.chunk) store_out(a, b, g, h);
-    if (p.chunk_blocks > 0) {
-      const size_t at = (static_cast<size_t>(b) * Hq + g * G + h) * p.max_chunks + u / ln.chunk;
-      const float dinv = a.den > 0.0f ? 1.0f / a.den : 0.0f;
-      if (on) *reinterpret_cast<float4*>(p.part_o + at * D + d0) = make_float4(a.num.x * dinv, a.num.y * dinv, a.num.z * dinv, a.num.w * dinv);
-      if (lane == 0) { p.part_m[at] = a.M * kLn2; p.part_l[at] = a.den * kUnshift; }
-    }
-  };
-  const int region = L > 1 ? y : p.chunk_blocks > 0 ? 1 : 0;
-  const int flags = lane < C::kWarps ? recs[lane].flags : 0;
-  const unsigned has0 = __ballot_sync(0xffffffffu, flags & kHas0), ends0 = __ballot_sync(0xffffffffu, flags & kEnds0), has1 = __ballot_sync(0xffffffffu, flags & kHas1);
-  // a chain: the warps that hold pieces of one unit, the first of them `from` (kind 0: the unit began in another CTA)
-  const int chains = static_cast<int>(has0 & 1u) + __popc(has1);
-  // What a warp's tasks leave in the workspace is counted at once, lane i for task i: the trips there and back (about 2 us)
-  // are made side by side.
-  static_assert((C::kWarps + 1) * kMaxGroup <= 32 * C::kWarps, "a task per lane");
-  int left_cta = 0, left_pieces = 0, left_b = 0, left_gh = 0, left_u = 0;
-#pragma unroll 1
-  for (int task = warp, i = 0; task < chains * G; task += C::kWarps, ++i) {
-    const int ci = task / G, h = task - ci * G;
-    const int kind = (has0 & 1u) && ci == 0 ? 0 : 1;
-    unsigned rest = has1;
-    for (int k = static_cast<int>(has0 & 1u); k < ci; ++k) rest &= rest - 1;
-    const int from = kind ? __ffs(rest) - 1 : 0;
-    int last = from;
-    bool closed = kind == 0 && (ends0 & 1u);
-    if (!closed) {
-      const int held = __ffs(~(has0 >> (from + 1))) - 1, end = __ffs(ends0 >> (from + 1));
-      closed = end != 0 && end <= held;
-      last = from + (closed ? end : held);
-    }
-    const int b = kind ? recs[from].b1 : recs[from].b0, g = kind ? recs[from].g1 : recs[from].g0, u = kind ? recs[from].u1 : recs[from].u0;
-    auto piece = [&](int k) {
-      return reinterpret_cast<const float*>(smem + (from + k) * C::kWarpBytes + ((kind && k == 0) ? piece1_off : piece0_off)) + h * C::kPieceStride;
-    };
-    const int n = last - from + 1;
-    Acc a;
-    acc_clear(a);
-    acc_merge<false>(a, n, lane < n ? piece(lane)[D] : 0.0f, lane < n ? piece(lane)[D + 1] : 0.0f, on, [&](int k) { return piece(k) + d0; });
-    if (!(kind && closed)) {
-      const unsigned first = unit_place(ln, b, g, u) + kUnitCost;
-      const int nu = unit_blocks(ln, line_blocks(ln, b), u), cta_f = first / T;
-      leave_piece(a, slot_of(region, v_share, kind != 0, h));
-      if (lane == i) { left_cta = cta_f; left_pieces = static_cast<int>((first + nu - 1) / T) - cta_f + 1; left_b = b; left_gh = g * G + h; left_u = u; }
-      continue;
-    }
-    finish(a, b, g, h, u);
-  }
-  {
+  Merge<D, FMT, L> merge{p, table, ln, smem, recs, cut[1], piece0_off, piece1_off, warp, lane, y};
+  merge.local(v_share);
+  if (L > 1 || p.chunk_blocks == 0) {
     __syncwarp();
     if (L > 1 && lane == 0) mbar_arrive(bar_merged);
-    unsigned last = __ballot_sync(0xffffffffu, left_pieces > 0 && count_piece(region, left_cta, left_pieces, left_gh % G));
-    __syncwarp();                        // the others' pieces, which a lane has acquired, are there for all lanes
-#pragma unroll 1
-    for (; last != 0; last &= last - 1) {
-      const int i = __ffs(last) - 1, gh = __shfl_sync(0xffffffffu, left_gh, i), g = gh / G;
-      Acc a;
-      take_pieces(a, region, __shfl_sync(0xffffffffu, left_cta, i), __shfl_sync(0xffffffffu, left_pieces, i), gh - g * G);
-      finish(a, __shfl_sync(0xffffffffu, left_b, i), g, gh - g * G, __shfl_sync(0xffffffffu, left_u, i));
-    }
+    merge.count_and_finish();
+    if (L > 1) continue;
+    break;
   }
-  if (L > 1) continue;
-  if (p.chunk_blocks == 0) break;
 
   // ---- Opt-Pa: what this CTA holds of a (sequence, kv head) is merged over its chunks, then with the other CTAs' shares ----
   __syncthreads();                       // this CTA's chunks have been exported (or left in its slots)
@@ -992,9 +1137,8 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
       Acc a;
       acc_clear(a);
       const size_t rows = (static_cast<size_t>(b) * Hq + g * G + h) * p.max_chunks;
-      const size_t slots = (static_cast<size_t>(2 * p.shares) + 2 * share) * G + h;
       auto cut = [&](int i) { return (i == c_first && cut_first) || (i == c_last && cut_last); };
-      auto slot = [&](int i) { return slots + (i == c_first && !first_began ? 0 : G); };
+      auto slot = [&](int i) { return merge.slot_of(1, share, i != c_first || first_began, h); };
       for (int c0 = c_first; c0 <= c_last; c0 += 32) {
         const int n = min(32, c_last - c0 + 1);
         float m = 0.0f, l = 0.0f;
@@ -1003,23 +1147,20 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
           m = cut(i) ? __ldcg(p.run_m + slot(i)) : __ldcg(p.part_m + rows + i) * kLog2e;
           l = cut(i) ? __ldcg(p.run_l + slot(i)) * kUnshift : __ldcg(p.part_l + rows + i);
         }
-        acc_merge<true>(a, n, m, l, on, [&](int k) { return (cut(c0 + k) ? p.run_o + slot(c0 + k) * D : p.part_o + (rows + c0 + k) * D) + d0; });
+        acc_merge<true>(a, n, m, l, merge.on(), [&](int k) { return (cut(c0 + k) ? p.run_o + slot(c0 + k) * D : p.part_o + (rows + c0 + k) * D) + lane * 4; });
       }
-      if (!(run_begins && run_ends)) {
+      if (run_begins && run_ends) {
+        merge.store_out(a, b, g, h);
+      } else {
         const int u_last = (nb - 1) / ln.chunk * ln.chunk;
         const unsigned first = unit_place(ln, b, g, 0) + (whole ? 0 : kUnitCost);
         const unsigned last = unit_place(ln, b, g, u_last) + (whole ? 0 : kUnitCost + (nb - u_last) - 1);
         const int cta_f = first / T;
-        const int pieces = static_cast<int>(last / T) - cta_f + 1;
-        leave_piece(a, slot_of(0, share, run_begins, h));
-        __syncwarp();
-        if (!__shfl_sync(0xffffffffu, lane == 0 && count_piece(0, cta_f, pieces, h), 0)) continue;
-        __syncwarp();
-        take_pieces(a, 0, cta_f, pieces, h);
+        merge.leave_piece(a, 0, share, run_begins, b, g, h, 0, cta_f, static_cast<int>(last / T) - cta_f + 1);
       }
-      store_out(a, b, g, h);
     }
   }
+  merge.count_and_finish();              // of chunks and of outputs together
   }
   COOPT_TRACE_CYCLES(p.trace, kTrExit, tid == 0);
   COOPT_TRACE_NS(p.trace, kTrExitNs, tid == 0);

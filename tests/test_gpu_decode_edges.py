@@ -218,3 +218,30 @@ def test_views_with_a_further_dimension_are_taken_as_before():
     q = w.q.cuda().view(w.batch, 4, 2, 32)
     again = binding.paged_decode(cache, q, w.block_table.cuda(), w.context_lens_tensor.cuda(), w.sm_scale, ws)
     assert again.shape == q.shape and torch.equal(again.view_as(out), out)
+
+
+@pytest.mark.parametrize("fmt", ["e4m3", "e5m2"])
+@pytest.mark.parametrize("d", [64, 128])
+def test_codes_past_the_context_do_not_count(d, fmt):
+    """Blocks are taken two at a time: contexts that end anywhere in the first or the second of them, alone and behind
+    others, with codes that are no numbers in all slots past the end.  The result is that of a clean cache, bit for bit
+    (a slot past the end counts for nothing), and the cache is left as it is."""
+    lens = [1, 5, 16, 17, 31, 32, 33, 47, 48, 63, 700, 2049]
+    kind = {"e4m3": binding.KV_FP8_E4M3, "e5m2": binding.KV_FP8_E5M2}[fmt]
+    w = workloads.make_workload("past the end", lens, 6, 2, d, seed=d)
+    cache = helpers.gpu_fill(w, dtype=kind)
+    out, ws = helpers.gpu_decode(w, cache)
+    kv = (*helpers.oracle_fp8_cache(w, fmt=e5m2), e5m2) if fmt == "e5m2" else helpers.oracle_fp8_cache(w)
+    helpers.check_attention(out, attention.paged_attention(w.q.float().numpy(), kv, w.block_table.numpy(), w.context_lens), what=f"past the end {fmt}")
+    at = [binding.cache_offset(cache, int(w.block_table[b, (L - 1) // 16]), g, which, t, e)
+          for b, L in enumerate(lens) for g in range(2) for which in (0, 1) for t in range((L - 1) % 16 + 1, 16) for e in range(d)]
+    cache.data[torch.tensor(at, device="cuda")] = 0x7F
+    before = cache.data.clone()
+    table, lens_t = w.block_table.cuda(), w.context_lens_tensor.cuda()
+    assert torch.equal(binding.paged_decode(cache, w.q.cuda(), table, lens_t, w.sm_scale, ws), out)
+    outs = [torch.full_like(out, float("nan")) for _ in range(3)]          # layers in one launch
+    layers = binding.LayerSet([{"cache": cache, "q": w.q.cuda(), "out": o} for o in outs])
+    plan = torch.empty(binding.plan_bytes(w.batch, 2, table.shape[1]), dtype=torch.uint8, device="cuda")
+    binding.decode_layers(layers, table, lens_t, 6, w.sm_scale, plan, ws)
+    assert all(torch.equal(o, out) for o in outs)
+    assert torch.equal(cache.data, before)
