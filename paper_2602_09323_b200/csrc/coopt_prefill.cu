@@ -31,12 +31,14 @@
 //   warp 14          copies: gather requests over the tensor map of the cache
 //   warp 15          what the softmax needs of a tile's block scales, worked out once for all rows
 //
-// Measured: 8 sequences of 4096 cached and 512 new tokens, 40 query heads over 8 kv heads, head_dim 128: 430 us (one tile a CTA,
-// its key tiles taken in turns by two groups of eight warps: 690); prompts of 900..2900 tokens, 32 heads over 8, head_dim 64:
-// 187 us (on mma.sync 495).  A half takes
-// about 1,850 cycles for both tiles: exponential units and issue slots 48 % each, tensor core 61 %, none of them alone (with
-// half the exponentials left out 12 % less time, with half the products of Q 4 %; four softmax warps a scheduler, two threads
-// to a row, took 453 us); a CTA's start and end take 15,000 cycles (head_dim 64: 10,000).
+// Measured: 8 sequences of 4096 cached and 512 new tokens, 40 query heads over 8 kv heads, head_dim 128: 385 us (one tile a CTA,
+// its key tiles taken in turns by two groups of eight warps: 690; the two tiles' exponentials side by side and one fp32
+// operation an instruction: 412); prompts of 900..2900 tokens, 32 heads over 8, head_dim 64: 178 us (on mma.sync 495; 188).  A
+// half takes about 1,700 cycles for both tiles: a softmax warp waits 300 for logits, loads them in 140, has their maximum in
+// 240 more, and is 740 at the exponentials, 512 of which they need; shared memory is busy 1,600 cycles of it at head_dim 128
+// (the products of Q, 64 keys at a time, read 6 KB each).  Half the exponentials left out took 12 % off, half the products of Q
+// 4 %; four softmax warps a scheduler, two threads to a row, took 453 us against 439; a CTA's start and end take 15,000
+// cycles (head_dim 64: 10,000).
 // Every wait is bounded; a wait that runs out is reported in the status word and all roles leave through the common exit,
 // which frees the tensor memory.
 #include "coopt_umma.cuh"
@@ -88,7 +90,7 @@ struct Cfg {
   static constexpr int kK16Off = kV16Off + kWide * kOperand;
   static constexpr int kScaleOff = kK16Off + (kWideK ? kWide * kOperand : 0);   // [slot][32]: K scales, log2 of V scale ratios, their inverses, factor, reference
   static constexpr int kBarOff = kScaleOff + kScaleSlots * 128;
-  static constexpr int kNumBars = 2 * kKSlots + 2 * kVSlots + 4 * kWide + kScaleSlots + 13;
+  static constexpr int kNumBars = 2 * kKSlots + 2 * kVSlots + 4 * kWide + kScaleSlots + 21;
   static constexpr int kMiscOff = kBarOff + kNumBars * 8;
   static constexpr int kSmemBytes = kMiscOff + 64;
   static_assert(kKSlot % 128 == 0 && kVOff % 128 == 0 && kQOff % 128 == 0 && kSmemBytes <= 232448, "shared memory of one CTA");
@@ -107,6 +109,27 @@ template <bool kE5m2>
 __device__ __forceinline__ uint2 widen4(uint32_t w) {
   if (kE5m2) return make_uint2(e5m2x2_to_f16x2_lo(w), e5m2x2_to_f16x2_hi(w));
   return make_uint2(e4m3x2_to_f16x2_lo(w), e4m3x2_to_f16x2_hi(w));
+}
+// Two fp32 operations in one instruction.
+__device__ __forceinline__ uint64_t f32_pair(float a, float b) {
+  uint64_t d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+  return d;
+}
+__device__ __forceinline__ float2 f32_both(uint64_t a) {
+  float2 d;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(a));
+  return d;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
 }
 __device__ __forceinline__ float max3(float a, float b, float c) {
   float d;
@@ -141,6 +164,7 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
   uint64_t* bar_pv = bar_pfull + 4;                     // [tile] its product with V is done
   uint64_t* bar_out = bar_pv + 2;                       // [tile] .. and it was the tile's last
   uint64_t* bar_q = bar_out + 2;                        // the query operands are in shared memory
+  uint64_t* bar_turn = bar_q + 1;                       // [tile][scheduler] the exponentials of a half are done
   int* misc = reinterpret_cast<int*>(smem + C::kMiscOff);   // [0] sequence, [1] first query, [2] abort flag, [3] tensor memory, [4] first row, [5] rows, [6] context of the sequence, [7] kv head
   volatile int* abort_flag = misc + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(misc + 3);
@@ -159,6 +183,7 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
     }
     for (int i = 0; i < C::kScaleSlots; ++i) mbar_init(&bar_scale[i], 1);
     mbar_init(bar_q, 8);
+    for (int i = 0; i < 8; ++i) mbar_init(&bar_turn[i], 1);
     for (int i = 0; i < 4; ++i) { mbar_init(&bar_sfull[i], 2); mbar_init(&bar_pfull[i], 4); }
     for (int i = 0; i < 2; ++i) { mbar_init(&bar_pv[i], 1); mbar_init(&bar_out[i], 1); }
     mbar_fence_init();
@@ -345,7 +370,7 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
     // index of the last visible key of the row.  Rows past the tile's last query (their operand is zero, and they are never
     // stored) see everything, so that their warp takes the same unmasked path as its live rows.
     const int lim = live ? (p.causal ? min(L - 1, L - n_new + q0 + x * TQ + qi) : L - 1) : (1 << 30);
-    const int halves = (tile_keys(x) + kHalf - 1) / kHalf;
+    const int halves = (tile_keys(x) + kHalf - 1) / kHalf, other_halves = (tile_keys(1 - x) + kHalf - 1) / kHalf;
     float m_ref = -INFINITY, m_use = 0.0f, l_row = 0.0f, v_ref = 0.0f;      // m_use: m_ref, or 0 before the first visible key
     bool ok = true;
 #pragma unroll 1
@@ -409,6 +434,12 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
           }
         }
       }
+      // The two softmax warps of a scheduler take turns at the exponentials: tile 0's half h comes behind tile 1's h - 1, tile 1's
+      // behind tile 0's h, as long as the other tile has such a half.  Side by side they would each take twice as long, and then
+      // leave the units idle while both load logits and look for the maximum.
+      const int turn = x == 0 ? h - 1 : h;
+      if (turn >= 0 && turn < other_halves) ok = wait_warp(&bar_turn[4 * (1 - x) + (warp & 3)], turn & 1u, abort_flag);
+      if (!ok) break;
       // p * pv = 2^(s * cf - m + log2 pv): the V scale rides in the exponent, and a block's sum of p is recovered from the sum
       // of p * pv (pv: the block's V scale over the reference, at most 2^4, a zero one replaced by 2^-24)
 #pragma unroll
@@ -419,17 +450,21 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
           const int c = 2 * i + e2;
           const float shift = (c == 0 ? lg.x : c == 1 ? lg.y : c == 2 ? lg.z : lg.w) - m_use;
           const uint32_t* v = &s[i][16 * e2];
-          float y[16];
+          const uint64_t cf2 = f32_pair(cf[c], cf[c]), shift2 = f32_pair(shift, shift);
+          uint64_t y[8];
 #pragma unroll
-          for (int e = 0; e < 16; ++e) y[e] = ex2(fmaf(__uint_as_float(v[e]), cf[c], shift));
+          for (int e = 0; e < 8; ++e) {
+            const float2 t = f32_both(fma2(f32_pair(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1])), cf2, shift2));
+            const float2 q = make_float2(ex2(t.x), ex2(t.y));
+            pw[8 * e2 + e] = pack_f16x2(q.x, q.y);
+            y[e] = f32_pair(q.x, q.y);
+          }
           // (Summed as a tree: a chain of sums kept the exponentials waiting, 820-1040 cycles a half for one warp of a scheduler
           // against 590, with 512 that the exponentials need.)
-          const float u0 = (y[0] + y[1]) + (y[2] + y[3]), u1 = (y[4] + y[5]) + (y[6] + y[7]);
-          const float u2 = (y[8] + y[9]) + (y[10] + y[11]), u3 = (y[12] + y[13]) + (y[14] + y[15]);
-          l_row += ((u0 + u1) + (u2 + u3)) * (c == 0 ? inv.x : c == 1 ? inv.y : c == 2 ? inv.z : inv.w);
-#pragma unroll
-          for (int e = 0; e < 8; ++e) pw[8 * e2 + e] = pack_f16x2(y[2 * e], y[2 * e + 1]);
+          const float2 u = f32_both(add2(add2(add2(y[0], y[1]), add2(y[2], y[3])), add2(add2(y[4], y[5]), add2(y[6], y[7]))));
+          l_row += (u.x + u.y) * (c == 0 ? inv.x : c == 1 ? inv.y : c == 2 ? inv.z : inv.w);
         }
+        if (i == 1) arrive_one(&bar_turn[4 * x + (warp & 3)]);       // (ahead of the store: behind it 394 us, here 385)
         tmem_st16(s_cols + kHalf * buf + 16 * i, pw);
       }
       tmem_st_wait();
