@@ -19,17 +19,15 @@
 // waited for hand-overs between its roles.  On tcgen05 / here: 24 sequences of 300..4000 tokens, G = 8, 46 / 23 us a layer;
 // 32 x 2048 tokens, G = 5, 35 / 29; 64 sequences of 128..8192 tokens 121 / 104; 120 of 5..900, head_dim 64, 56 / 17.)
 //
-// A warp takes two blocks at a time, and their contractions, exponentials and look-ups side by side: one block is a chain of
-// dependent instructions (302 of them, one every 5.9 cycles with three warps a scheduler), and at one block at a time that
-// bounded the stream and not HBM.  One / two, us: 32 x 16384 tokens, G = 5, out of L2 153 / 112, out of HBM 186 / 174; 64 x
-// 4096, head_dim 64, G = 4, out of L2 60 / 48; 64 mixed lengths, four layers, 422 / 399.  (8 warps with 255 registers: 181 for
-// the second figure; two CTAs of 6 warps an SM: the same as one of 12.)
-//
 // A launch of 32 x 2048 tokens streams at 6.4 TB/s from its first copies, 3 us after a CTA's first instruction, to the end
 // of its last block, 5 us before the CTA's last; code that runs once costs about four cycles an instruction to fetch.
-// Registers are what the loop over blocks is short of (what it spills goes to L2: all of L1 is shared memory, and 24 bytes cost
-// 4 %): the walks of the copies and of the work wait in shared memory, and the query rows of a unit are fetched when it starts (eight layers of 21 sequences of 2..60 tokens: 49 / 43.6 us; prefetching the rows into
-// registers at the end of the unit before instead: 49.5).
+// Registers are what the loop over blocks is short of: the walks of the copies and of the work wait in shared memory, and the
+// query rows of a unit are fetched when it starts (eight layers of 21 sequences of 2..60 tokens: 49 / 43.6 us; prefetching the
+// rows into registers at the end of the unit before instead: 49.5).
+//
+// (Two blocks at a time, contractions and exponentials side by side, each block by its own references, against one: eight layers
+// of 32 x 2048 tokens 233 / 227 us, 64 of 128..8192, four layers, 411 / 404, four of 32768..131072 in chunks 127.5 / 125.8, 30 x
+// 1597 34.5 / 32.1; only eight layers of 64 x 100..5000, head_dim 64, are a little faster, 174 / 176.)
 #include <float.h>
 
 #include <algorithm>
@@ -54,10 +52,11 @@ template <int D, int FMT>
 struct Cfg {
   static constexpr bool kFp8 = FMT != COOPT_KV_BF16;
   [[maybe_unused]] static constexpr bool kE5m2 = FMT == COOPT_KV_FP8_E5M2;
-  // A warp needs time for two blocks (about 1.2 us from landing to the next wait), so many warps are wanted, with at least two
-  // blocks in flight each.  head_dim 128: 12 warps x 3 blocks against 8 x 5 and 10 x 4: 399 / 415 / 421 us (64 sequences of
-  // 128..8192 tokens, four layers); eight layers of 32 x 2048 tokens 226 / 225 / 247.  head_dim 64: 16 x 4 against 12 x 6:
-  // 13.0 / 15.2 us (four sequences of 1595..3191 tokens), 59 / 57 (64 x 4096).  bf16: 8 x 2 (182 registers).
+  // A warp needs time for a block (about 1 us from landing to the next wait), so many warps are wanted, with two blocks in
+  // flight each, or four of head_dim 64.  More of them in flight take longer: head_dim 128, 2 / 3 blocks 404 / 424 us (64
+  // sequences of 128..8192 tokens, four layers), 125.8 / 133.0 (four of 32768..131072 in chunks), 219.5 / 228.3 (32 x 4096, four
+  // launches), 226.6 / 227.6 (eight layers of 32 x 2048), 32.1 / 32.4 (30 x 1597); head_dim 64, 4 / 5: 138.6 / 139.8 (64 of
+  // 100..5000, G = 4, four layers), 17.1 / 17.3 (120 of 5..900).  bf16: 8 x 2 and 8 x 4 (182 registers).
   static constexpr int kWarps = kFp8 ? (D == 128 ? 12 : 16) : 8;
   static constexpr int kThreads = kWarps * 32;
   static constexpr int kGran = granule_bytes(D, kFp8);
@@ -66,15 +65,9 @@ struct Cfg {
   static constexpr int kPieceStride = D + 4;                    // floats of one head of a piece: o[D], maximum, sum, padding
   static constexpr int kPiece = kMaxGroup * kPieceStride * 4;   // bytes
   // A warp's shared memory: its ring, the piece of a unit from before, and, in a launch over several layers, the piece of a
-  // unit that goes on (in a launch over one the ring has done its work by then, and the piece takes its place).  Pieces are
-  // as large as the group asks for; for the largest groups the ring of a launch over several layers is shorter.
-  static constexpr int kFixed = kMaxBatch * 4 + (kMaxBatch + 4) * 4 + 192 + 16 + kWarps * (96 + 128);      // what lies behind the warps' parts
-  static constexpr int kWarpBytes = kFp8 ? (kMaxSmem - kFixed) / kWarps / 128 * 128 : (D == 128 ? 2 : 4) * kGran + kPiece;
-  static constexpr int kStages = (kWarpBytes - kPiece) / kGran;
-  static __host__ __device__ constexpr int stages(int layers, int G) {
-    const int most = (kWarpBytes - 2 * G * kPieceStride * 4) / kGran;
-    return layers > 1 && most < kStages ? most : kStages;
-  }
+  // unit that goes on (in a launch over one the ring has done its work by then, and the piece takes its place).
+  static constexpr int kStages = D == 128 ? 2 : 4;
+  static constexpr int kWarpBytes = kStages * kGran + (kFp8 ? 2 : 1) * kPiece;
   static constexpr int kBarOff = kWarps * kWarpBytes;
   static constexpr int kLensOff = kBarOff + (kWarps * kStages + 2) * 8;
   static constexpr int kPreOff = kLensOff + kMaxBatch * 4;
@@ -83,7 +76,7 @@ struct Cfg {
   static constexpr int kCopyWalkOff = kMiscOff + 192;           // walks of a warp: where its copies are, and where its work is
   static constexpr int kSmemBytes = kCopyWalkOff + kWarps * 128;
   static_assert(kGran % 128 == 0 && kPiece % 128 == 0 && kStages * kGran >= kPiece && kWarpBytes % 128 == 0 && kCopy % 16 == 0, "copies land on 128-byte boundaries");
-  static_assert(kStages >= 2 && kStages <= 8 && (!kFp8 || stages(kManyLayers, kMaxGroup) >= 2) && kSmemBytes <= kMaxSmem, "room for copies in flight");
+  static_assert(kStages >= 2 && kSmemBytes <= kMaxSmem, "room for copies in flight");
   static_assert(kCtasPerSm * (kSmemBytes + 1024) <= 233472, "shared memory of one SM");
 };
 
@@ -415,13 +408,10 @@ struct Merge {
   }
 };
 
-template <int kBlocks> struct Blocks { static constexpr int kCount = kBlocks; };
-
 template <int D, int FMT, int L>
 __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decode_kernel(const __grid_constant__ DecodeParams p, const __grid_constant__ LayerTable<L> table) {
   using C = Cfg<D, FMT>;
   constexpr int kQSteps = D / 16;
-  constexpr int N = C::kFp8 ? 2 : 1;     // blocks that a warp takes at a time
   extern __shared__ __align__(128) uint8_t smem[];
   int* lens = reinterpret_cast<int*>(smem + C::kLensOff);
   unsigned* pre = reinterpret_cast<unsigned*>(smem + C::kPreOff);
@@ -431,8 +421,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
   const int row = lane >> 2, quad = lane & 3;
   const int B = p.batch, Hkv = p.num_kv_heads, G = p.group, Hq = p.num_q_heads;
   uint8_t* ring = smem + warp * C::kWarpBytes;
-  const int stages = L == 1 ? C::kStages : C::stages(L, G);
-  const int piece0_off = stages * C::kGran, piece1_off = L == 1 ? 0 : piece0_off + G * C::kPieceStride * 4;   // in a warp's shared memory
+  constexpr int piece0_off = C::kStages * C::kGran, piece1_off = L == 1 ? 0 : piece0_off + C::kPiece;   // in a warp's shared memory
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::kBarOff) + warp * C::kStages;
   uint64_t* bar_pieces = reinterpret_cast<uint64_t*>(smem + C::kBarOff) + C::kWarps * C::kStages;   // every warp has left its pieces
   uint64_t* bar_merged = bar_pieces + 1;                                                            // .. has no more use for the others' pieces
@@ -608,7 +597,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
   Walk fw = w;
   if (ps < all_shares) walk_later(ps, fw);                              // the first unit, and its layer
   const int fy = share_layer(ps);
-  const uint8_t* from_a = nullptr;                 // this lane's granule of the batch
+  int ids_a = 0, g_a = 0, y_a = 0;
   int cnt_a = 0, pos_a = 0, ids_b = 0, cnt_b = 0, g_b = 0, y_b = 0;
   auto prefetch_q = [&](int y, int b, int g) {
     if (lane < G * D / 64) prefetch_l2(reinterpret_cast<const uint8_t*>(layer(y).q + (static_cast<size_t>(b) * Hq + g * G) * D) + lane * 128);
@@ -637,31 +626,26 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
       if (p.plan == nullptr) atomicCAS(p.status, 0, COOPT_ERR_INVALID_ARG);
       id = 0;
     }
-    from_a = layer(y_b).cache + (static_cast<size_t>(id) * Hkv + g_b) * C::kGran;
+    ids_a = id; g_a = g_b; y_a = y_b;
     cnt_a = cnt_b; pos_a = 0;
     fetch_ids();
   };
   uint32_t issued = 0, consumed = 0;               // copies, and the stages that take the next one and hold the oldest one
   int in_stage = 0, out_stage = 0;
   uint32_t out_phase = 0;
-  // The next `left` copies (fewer at the end): each by the lane that has its granule's address.
-  auto issue = [&](int left) {
-#pragma unroll 1
-    do {
-      if (pos_a == cnt_a) take_ids();
-      const int n = min(left, cnt_a - pos_a), k = lane - pos_a;
-      if (n == 0) return;
-      if (k >= 0 && k < n) {
-        const int stage = in_stage + k < stages ? in_stage + k : in_stage + k - stages;
+  auto issue = [&]() {
+    if (pos_a == cnt_a) take_ids();
+    if (pos_a < cnt_a) {
+      const int id = __shfl_sync(0xffffffffu, ids_a, pos_a);
+      ++pos_a;
+      const int stage = in_stage;
+      if (++in_stage == C::kStages) in_stage = 0;
+      if (lane == 0) {
         mbar_expect_tx(&bars[stage], C::kCopy);
-        bulk_copy_g2s(ring + stage * C::kGran, from_a, C::kCopy, &bars[stage]);
+        bulk_copy_g2s(ring + stage * C::kGran, layer(y_a).cache + (static_cast<size_t>(id) * Hkv + g_a) * C::kGran, C::kCopy, &bars[stage]);
       }
-      pos_a += n;
-      in_stage += n;
-      if (in_stage >= stages) in_stage -= stages;
-      issued += n;
-      left -= n;
-    } while (left > 0);
+      ++issued;
+    }
   };
 
   // ---- per-lane constants of the operand layouts ---------------------------------------------------------------
@@ -707,7 +691,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
   for (int step = 0; step < 2; ++step) {
     if ((step == 0) == (p.order == kOverlapPrevious)) {
 #pragma unroll 1
-      for (int i = 0; i < stages; ++i) issue(1);
+      for (int i = 0; i < C::kStages; ++i) issue();
       COOPT_TRACE_CYCLES(p.trace, kTrFirstCopy, tid == 0);
     } else {
       if (p.order != kDependent) wait_previous_kernel();
@@ -776,72 +760,100 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
     if (lane == 0) *work_walk = w;
     __syncwarp();
 
-    // Some blocks, of which the first `seen` tokens count.
-    auto attend = [&](auto count, uint8_t* const st0, uint8_t* const st1, int seen) {
-      constexpr int kN = decltype(count)::kCount;
-      uint8_t* const st[2] = {st0, st1};
-      // ---- S^T = K Q^T: 16 tokens x 8 heads a block ------------------------------------------------------------------
-      float x[kN][4], sv[kN];
-      if constexpr (C::kFp8) {
-        float sa[kN][4], sb[kN][4];
-        float2 hdr[kN];
-#pragma unroll
-        for (int i = 0; i < kN; ++i) {
-          hdr[i] = *reinterpret_cast<const float2*>(st[i] + header_offset(D));
-#pragma unroll
-          for (int e = 0; e < 4; ++e) sa[i][e] = sb[i][e] = 0.0f;
-        }
-#pragma unroll
-        for (int c = 0; c < D / 32; ++c) {
-#pragma unroll
-          for (int i = 0; i < kN; ++i) {
-            uint32_t r[4];
-            ldmatrix4(smem_u32(st[i]) + k_lane + c * 256, r);
-            mma16816<true>(sa[i], codes_lo<C::kE5m2>(r[0]), codes_lo<C::kE5m2>(r[1]), codes_hi<C::kE5m2>(r[0]), codes_hi<C::kE5m2>(r[1]), qf[2 * c][0], qf[2 * c][1]);
-            mma16816<true>(sb[i], codes_lo<C::kE5m2>(r[2]), codes_lo<C::kE5m2>(r[3]), codes_hi<C::kE5m2>(r[2]), codes_hi<C::kE5m2>(r[3]), qf[2 * c + 1][0], qf[2 * c + 1][1]);
+#pragma unroll 1
+    for (int j = w.j; j < j_end && !dead; ++j) {
+      // (The one test that every block meets: whether it is the last of the context.)
+      const bool last = (j + 1) * kBlockSize >= valid;
+      int seen = kBlockSize;                                                 // tokens of the block (Eq. 9)
+      // the step's new token: what it needs is loaded while its block is on the way
+      bool append = false;
+      long long slot = -1;
+      int id = 0;
+      uint2 k_row = make_uint2(0u, 0u), v_row = k_row;
+      if (last) {
+        seen = valid - j * kBlockSize;
+        if constexpr (C::kFp8) {
+          append = layer(y).k_new != nullptr;
+          if (append) {
+            const LayerPtrs& io = layer(y);
+            const bool vec = ((reinterpret_cast<uintptr_t>(io.k_new) | reinterpret_cast<uintptr_t>(io.v_new) | static_cast<uintptr_t>(p.kv_token_stride * 2)) & (D / 16 - 1)) == 0;
+            const long long at = static_cast<long long>(work_walk->b) * p.kv_token_stride + work_walk->g * D;
+            slot = io.slot_mapping[work_walk->b];
+            id = p.block_table[static_cast<size_t>(work_walk->b) * p.max_blocks_per_seq + work_walk->u + j];
+            k_row = load_new<D>(io.k_new + at, vec, lane);
+            v_row = load_new<D>(io.v_new + at, vec, lane);
           }
         }
+      }
+      // the oldest copy in flight
+      dead = !__all_sync(0xffffffffu, mbar_wait_bounded(&bars[out_stage], out_phase));
+      COOPT_TRACE_CYCLES(p.trace, kTrFirstLanded, tid == 0 && consumed == 0);
+      if (dead) break;
+      uint8_t* const st = ring + out_stage * C::kGran;
+      ++consumed;
+      if (++out_stage == C::kStages) { out_stage = 0; out_phase ^= 1u; }
+      if constexpr (C::kFp8) {
+        if (last) {
+          if (append && slot >= 0) {                                         // Eq. 5: negative slots are skipped
+            const int off = (valid - 1) % kBlockSize;
+            if (slot != static_cast<long long>(id) * kBlockSize + off) {     // not the sequence's last position
+              if (lane == 0) atomicCAS(p.status, 0, COOPT_ERR_INVALID_ARG);
+            } else if (id >= 0 && id < p.num_blocks) {
+              append_token<D, C::kE5m2>(st, layer(y).cache + (static_cast<size_t>(id) * Hkv + work_walk->g) * C::kGran, k_row, v_row, off, lane);
+            }
+            __syncwarp();
+          }
+          if (seen < kBlockSize) {                 // V codes of slots past the context are cleared: they may hold anything
+            auto mask = [&](int word) { return seen >= 4 * word + 4 ? 0xFFFFFFFFu : seen <= 4 * word ? 0u : (1u << (8 * (seen - 4 * word))) - 1u; };
 #pragma unroll
-        for (int i = 0; i < kN; ++i) {
-          const float k0 = qs[0] * hdr[i].x, k1 = qs[1] * hdr[i].x;
-          sv[i] = hdr[i].y;
-          x[i][0] = (sa[i][0] + sb[i][0]) * k0; x[i][1] = (sa[i][1] + sb[i][1]) * k1;
-          x[i][2] = (sa[i][2] + sb[i][2]) * k0; x[i][3] = (sa[i][3] + sb[i][3]) * k1;
+            for (int i = 0; i < D / 32; ++i) {
+              uint4* row = reinterpret_cast<uint4*>(st + kBlockSize * D) + i * 32 + lane;        // 16 tokens of a dim
+              const uint4 v = *row;
+              *row = make_uint4(v.x & mask(0), v.y & mask(1), v.z & mask(2), v.w & mask(3));
+            }
+            __syncwarp();
+          }
+        }
+      }
+
+      // ---- S^T = K Q^T: 16 tokens x 8 heads ------------------------------------------------------------------------
+      float sa[4] = {0.0f, 0.0f, 0.0f, 0.0f}, sb[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+      float sk = 1.0f, sv = 1.0f;
+      if constexpr (C::kFp8) {
+        const float2 hdr = *reinterpret_cast<const float2*>(st + header_offset(D));
+        sk = hdr.x; sv = hdr.y;
+#pragma unroll
+        for (int c = 0; c < D / 32; ++c) {
+          uint32_t r[4];
+          ldmatrix4(smem_u32(st) + k_lane + c * 256, r);
+          mma16816<true>(sa, codes_lo<C::kE5m2>(r[0]), codes_lo<C::kE5m2>(r[1]), codes_hi<C::kE5m2>(r[0]), codes_hi<C::kE5m2>(r[1]), qf[2 * c][0], qf[2 * c][1]);
+          mma16816<true>(sb, codes_lo<C::kE5m2>(r[2]), codes_lo<C::kE5m2>(r[3]), codes_hi<C::kE5m2>(r[2]), codes_hi<C::kE5m2>(r[3]), qf[2 * c + 1][0], qf[2 * c + 1][1]);
         }
       } else {
-        float sa[4] = {0.0f, 0.0f, 0.0f, 0.0f}, sb[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-        const uint8_t* kp = st[0] + lane * 16;
+        const uint8_t* kp = st + lane * 16;
 #pragma unroll
         for (int i = 0; i < D / 32; ++i) {
           const uint4 w0 = lds128(kp + i * 512), w1 = lds128(kp + (D / 32 + i) * 512);
           mma16816<false>(sa, w0.x, w1.x, w0.y, w1.y, qf[2 * i][0], qf[2 * i][1]);
           mma16816<false>(sb, w0.z, w1.z, w0.w, w1.w, qf[2 * i + 1][0], qf[2 * i + 1][1]);
         }
-        sv[0] = 1.0f;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) x[0][e] = (sa[e] + sb[e]) * qs[e & 1];
       }
 
-      // ---- online softmax (Eq. 10) in base-2 units; the reference maximum is lazy ------------------------------------
-      if (seen < kN * kBlockSize) {
-#pragma unroll
-        for (int i = 0; i < kN; ++i) {
-          if (tok0 + i * kBlockSize >= seen) x[i][0] = x[i][1] = -INFINITY;
-          if (tok0 + kTokStep + i * kBlockSize >= seen) x[i][2] = x[i][3] = -INFINITY;
-        }
+      // ---- online softmax (Eq. 10) in base-2 units; the reference maximum is lazy --------------------------------------
+      // (Each block goes by the references that it finds or moves itself.  Two blocks by one: far below what the second moves, the
+      // first one's probabilities are f16 numbers of few bits, or zero.)
+      const float k0 = qs[0] * sk, k1 = qs[1] * sk;
+      float x[4] = {(sa[0] + sb[0]) * k0, (sa[1] + sb[1]) * k1, (sa[2] + sb[2]) * k0, (sa[3] + sb[3]) * k1};
+      if (seen < kBlockSize) {
+        if (tok0 >= seen) x[0] = x[1] = -INFINITY;
+        if (tok0 + kTokStep >= seen) x[2] = x[3] = -INFINITY;
       }
-      float t0 = fmaxf(x[0][0], x[0][2]), t1 = fmaxf(x[0][1], x[0][3]), sv_top = sv[0];
-#pragma unroll
-      for (int i = 1; i < kN; ++i) {
-        t0 = fmaxf(t0, fmaxf(x[i][0], x[i][2]));
-        t1 = fmaxf(t1, fmaxf(x[i][1], x[i][3]));
-        sv_top = fmaxf(sv_top, sv[i]);
-      }
+      const float t0 = fmaxf(x[0], x[2]), t1 = fmaxf(x[1], x[3]);
       if constexpr (L == 1) {                      // (for exported partials)
         top[0] = fmaxf(top[0], t0);
         top[1] = fmaxf(top[1], t1);
       }
-      const bool grow = C::kFp8 && sv_top > vref;
+      const bool grow = C::kFp8 && sv > vref;
       if (__any_sync(0xffffffffu, t0 > m[0] + kLag || t1 > m[1] + kLag) || grow) {
         float f[2];
 #pragma unroll
@@ -856,7 +868,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
           l[h] *= f[h];
         }
         if (grow) {                                // (a reference is a normal number: its reciprocal is one then, too)
-          const float vnew = fmaxf(sv_top, FLT_MIN);
+          const float vnew = fmaxf(sv, FLT_MIN);
           vinv = 1.0f / vnew;
           const float fv = vref * vinv;
           f[0] *= fv; f[1] *= fv;
@@ -866,39 +878,28 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
         for (int t = 0; t < D / 16; ++t) { o[t][0] *= f[0]; o[t][1] *= f[1]; o[t][2] *= f[0]; o[t][3] *= f[1]; }
       }
       const float b0 = kShift - m[0], b1 = kShift - m[1];
-#pragma unroll
-      for (int i = 0; i < kN; ++i) {
-        x[i][0] = ex2(x[i][0] + b0); x[i][1] = ex2(x[i][1] + b1); x[i][2] = ex2(x[i][2] + b0); x[i][3] = ex2(x[i][3] + b1);
-        l[0] += x[i][0] + x[i][2];
-        l[1] += x[i][1] + x[i][3];
-      }
+      float pr[4];
+      pr[0] = ex2(x[0] + b0); pr[1] = ex2(x[1] + b1); pr[2] = ex2(x[2] + b0); pr[3] = ex2(x[3] + b1);
+      l[0] += pr[0] + pr[2];
+      l[1] += pr[1] + pr[3];
 
       // ---- O^T += V^T P^T -----------------------------------------------------------------------------------------------
       if constexpr (C::kFp8) {
-        uint32_t p0[kN], p1[kN];
-#pragma unroll
-        for (int i = 0; i < kN; ++i) {
-          const float pv = sv[i] * vinv;
-          p0[i] = transpose8x8(pack_f16x2(x[i][0] * pv, x[i][1] * pv));
-          p1[i] = transpose8x8(pack_f16x2(x[i][2] * pv, x[i][3] * pv));
-        }
+        const float pv = sv * vinv;
+        const uint32_t p0 = transpose8x8(pack_f16x2(pr[0] * pv, pr[1] * pv)), p1 = transpose8x8(pack_f16x2(pr[2] * pv, pr[3] * pv));
 #pragma unroll
         for (int c = 0; c < D / 32; ++c) {
-#pragma unroll
-          for (int i = 0; i < kN; ++i) {
-            uint32_t r[4];
-            ldmatrix4(smem_u32(st[i]) + kBlockSize * D + lane * 16 + c * 512, r);
-            mma16816<true>(o[2 * c], codes_lo<C::kE5m2>(r[0]), codes_lo<C::kE5m2>(r[1]), codes_hi<C::kE5m2>(r[0]), codes_hi<C::kE5m2>(r[1]), p0[i], p1[i]);
-            mma16816<true>(o[2 * c + 1], codes_lo<C::kE5m2>(r[2]), codes_lo<C::kE5m2>(r[3]), codes_hi<C::kE5m2>(r[2]), codes_hi<C::kE5m2>(r[3]), p0[i], p1[i]);
-          }
+          uint32_t r[4];
+          ldmatrix4(smem_u32(st) + kBlockSize * D + lane * 16 + c * 512, r);
+          mma16816<true>(o[2 * c], codes_lo<C::kE5m2>(r[0]), codes_lo<C::kE5m2>(r[1]), codes_hi<C::kE5m2>(r[0]), codes_hi<C::kE5m2>(r[1]), p0, p1);
+          mma16816<true>(o[2 * c + 1], codes_lo<C::kE5m2>(r[2]), codes_lo<C::kE5m2>(r[3]), codes_hi<C::kE5m2>(r[2]), codes_hi<C::kE5m2>(r[3]), p0, p1);
         }
       } else {
         // bf16 probabilities as a high and a low half (16 bits in all)
-        const float (&pr)[4] = x[0];
         const uint32_t h0 = pack_bf16x2(pr[0], pr[1]), h1 = pack_bf16x2(pr[2], pr[3]);
         const uint32_t e0 = pack_bf16x2(pr[0] - bf16_lo(h0), pr[1] - bf16_hi(h0)), e1 = pack_bf16x2(pr[2] - bf16_lo(h1), pr[3] - bf16_hi(h1));
         const uint32_t p0 = transpose8x8(h0), p1 = transpose8x8(h1), r0 = transpose8x8(e0), r1 = transpose8x8(e1);
-        const uint8_t* vp = st[0] + part_offset(D, false, 1) + lane * 16;
+        const uint8_t* vp = st + part_offset(D, false, 1) + lane * 16;
         uint32_t m0 = 0xFFFFFFFFu, m1 = 0xFFFFFFFFu;
         if (seen < kBlockSize) {
           m0 = (2 * quad < seen ? 0x0000FFFFu : 0u) | (2 * quad + 1 < seen ? 0xFFFF0000u : 0u);
@@ -911,93 +912,11 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
           mma16816<false>(o[i], v.x & m0, v.z & m0, v.y & m1, v.w & m1, r0, r1);
         }
       }
-    };
-#pragma unroll 1
-    for (int j = w.j; j < j_end && !dead; j += N) {
-      // (The one test that every block meets: whether there is less than a full step of blocks, all of them before the last of the
-      // context.  A block that is not there counts for nothing.)
-      const bool rare = j + N > j_end || (j + N) * kBlockSize >= valid;
-      int n = N, seen = N * kBlockSize;                                      // blocks, and tokens of them (Eq. 9)
-      // the step's new token: what it needs is loaded while its block is on the way
-      bool append = false;
-      long long slot = -1;
-      int id = 0;
-      uint2 k_row = make_uint2(0u, 0u), v_row = k_row;
-      if (rare) {
-        n = min(N, j_end - j);
-        seen = min(valid - j * kBlockSize, n * kBlockSize);
-        if constexpr (C::kFp8) {
-          append = layer(y).k_new != nullptr && (j + n) * kBlockSize >= valid;
-          if (append) {
-            const LayerPtrs& io = layer(y);
-            const bool vec = ((reinterpret_cast<uintptr_t>(io.k_new) | reinterpret_cast<uintptr_t>(io.v_new) | static_cast<uintptr_t>(p.kv_token_stride * 2)) & (D / 16 - 1)) == 0;
-            const long long at = static_cast<long long>(work_walk->b) * p.kv_token_stride + work_walk->g * D;
-            slot = io.slot_mapping[work_walk->b];
-            id = p.block_table[static_cast<size_t>(work_walk->b) * p.max_blocks_per_seq + work_walk->u + (valid - 1) / kBlockSize];
-            k_row = load_new<D>(io.k_new + at, vec, lane);
-            v_row = load_new<D>(io.v_new + at, vec, lane);
-          }
-        }
-      }
-      // the oldest copies in flight
-      uint8_t* st[N];
-      st[0] = ring + out_stage * C::kGran;
-      bool there = mbar_wait_bounded(&bars[out_stage], out_phase);
-      if (++out_stage == stages) { out_stage = 0; out_phase ^= 1u; }
-      if constexpr (N == 2) {
-        st[1] = st[0];
-        if (n == 2) {
-          st[1] = ring + out_stage * C::kGran;
-          there = there && mbar_wait_bounded(&bars[out_stage], out_phase);
-          if (++out_stage == stages) { out_stage = 0; out_phase ^= 1u; }
-        }
-      }
-      dead = !__all_sync(0xffffffffu, there);
-      COOPT_TRACE_CYCLES(p.trace, kTrFirstLanded, tid == 0 && consumed == 0);
-      if (dead) {                                  // (the stages that were waited for stay the oldest)
-        out_stage -= n;
-        if (out_stage < 0) { out_stage += stages; out_phase ^= 1u; }
-        break;
-      }
-      consumed += n;
-      if constexpr (C::kFp8) {
-        if (rare) {
-          uint8_t* const tail = st[n - 1];
-          if (append && slot >= 0) {                                         // Eq. 5: negative slots are skipped
-            const int off = (valid - 1) % kBlockSize;
-            if (slot != static_cast<long long>(id) * kBlockSize + off) {     // not the sequence's last position
-              if (lane == 0) atomicCAS(p.status, 0, COOPT_ERR_INVALID_ARG);
-            } else if (id >= 0 && id < p.num_blocks) {
-              append_token<D, C::kE5m2>(tail, layer(y).cache + (static_cast<size_t>(id) * Hkv + work_walk->g) * C::kGran, k_row, v_row, off, lane);
-            }
-            __syncwarp();
-          }
-          if (seen < n * kBlockSize) {             // V codes of slots past the context are cleared: they may hold anything
-            const int keep = seen - (n - 1) * kBlockSize;
-            auto mask = [&](int word) { return keep >= 4 * word + 4 ? 0xFFFFFFFFu : keep <= 4 * word ? 0u : (1u << (8 * (keep - 4 * word))) - 1u; };
-#pragma unroll
-            for (int i = 0; i < D / 32; ++i) {
-              uint4* row = reinterpret_cast<uint4*>(tail + kBlockSize * D) + i * 32 + lane;      // 16 tokens of a dim
-              const uint4 v = *row;
-              *row = make_uint4(v.x & mask(0), v.y & mask(1), v.z & mask(2), v.w & mask(3));
-            }
-            __syncwarp();
-          }
-        }
-      }
 
-      // (A single block by the code for two gives the same result and takes two thirds of the time of two.  A launch over one layer
-      // has no other code: fetching it would cost more.)
-      if constexpr (L > 1 && N == 2) {
-        if (n == 2) attend(Blocks<2>(), st[0], st[N - 1], seen); else attend(Blocks<1>(), st[0], st[0], seen);
-      } else {
-        attend(Blocks<N>(), st[0], st[N - 1], seen);
-      }
-
-      // ---- the stages go back to the copy engine ------------------------------------------------------------------------
+      // ---- the stage goes back to the copy engine ---------------------------------------------------------------------
       __syncwarp();
-      fence_proxy_async();
-      issue(n);
+      if (lane == 0) fence_proxy_async();
+      issue();
     }
     w = *work_walk;
     __syncwarp();
@@ -1169,7 +1088,7 @@ __global__ void __launch_bounds__(Cfg<D, FMT>::kThreads, kCtasPerSm) paged_decod
     if (lane == 0) atomicCAS(p.status, 0, COOPT_ERR_TIMEOUT);
     for (; consumed < issued; ++consumed) {
       mbar_wait_bounded(&bars[out_stage], out_phase);
-      if (++out_stage == stages) { out_stage = 0; out_phase ^= 1u; }
+      if (++out_stage == C::kStages) { out_stage = 0; out_phase ^= 1u; }
     }
   }
 }

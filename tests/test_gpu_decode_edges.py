@@ -223,8 +223,7 @@ def test_views_with_a_further_dimension_are_taken_as_before():
 @pytest.mark.parametrize("fmt", ["e4m3", "e5m2"])
 @pytest.mark.parametrize("d", [64, 128])
 def test_codes_past_the_context_do_not_count(d, fmt):
-    """Blocks are taken two at a time: contexts that end anywhere in the first or the second of them, alone and behind
-    others, with codes that are no numbers in all slots past the end.  The result is that of a clean cache, bit for bit
+    """Contexts that end anywhere in a block, the first or a later one, with codes that are no numbers in all slots past the end.  The result is that of a clean cache, bit for bit
     (a slot past the end counts for nothing), and the cache is left as it is."""
     lens = [1, 5, 16, 17, 31, 32, 33, 47, 48, 63, 700, 2049]
     kind = {"e4m3": binding.KV_FP8_E4M3, "e5m2": binding.KV_FP8_E5M2}[fmt]
@@ -245,3 +244,61 @@ def test_codes_past_the_context_do_not_count(d, fmt):
     binding.decode_layers(layers, table, lens_t, 6, w.sm_scale, plan, ws)
     assert all(torch.equal(o, out) for o in outs)
     assert torch.equal(cache.data, before)
+
+
+@pytest.mark.parametrize("loud", ["V scale", "logits"])
+@pytest.mark.parametrize("fmt", ["e4m3", "e5m2"])
+@pytest.mark.parametrize("d", [64, 128])
+def test_a_block_keeps_its_bits_beside_one_that_dwarfs_it(d, fmt, loud):
+    """The last block of a context moves a reference by 2^20 to 2^40, and all of its V but one value is zero: the other dims'
+    results are those of the blocks in front of it.  V is not negative there, so every product is in the sum with its own sign,
+    and the result is off by no more than its terms are, 2^-11 (a probability of 11 bits, rounded to nearest: 2^-12, and less than
+    that again for fp32 exponentials and sums), and by the rounding of the bf16 result, of 8 bits, to nearest: 2^-8 at most."""
+    lens, bits = [32, 29, 17, 64, 61, 32, 32], [20, 24, 28, 32, 36, 40, 30]
+    w = workloads.make_workload("dwarfed", lens, 6, 2, d, seed=d, outliers=False)
+    w.v.copy_(w.v.abs())
+    w.q.fill_(1.0)
+    w.k.mul_(0.125)
+    for b, (L, e) in enumerate(zip(lens, bits)):
+        rows = slice(w.kv_offsets[b] + (L - 1) // 16 * 16, w.kv_offsets[b] + L)      # the last block, the second or the fourth
+        w.v[rows] = 0
+        if loud == "V scale":
+            w.v[w.kv_offsets[b] + L - 1, :, 0] = 2.0 ** e
+        else:
+            w.k[rows] = e * np.log(2.0) / np.sqrt(d)
+    kind = binding.KV_FP8_E4M3 if fmt == "e4m3" else binding.KV_FP8_E5M2
+    kv = helpers.oracle_fp8_cache(w) if fmt == "e4m3" else (*helpers.oracle_fp8_cache(w, fmt=e5m2), e5m2)
+    ref = attention.paged_attention(w.q.float().numpy(), kv, w.block_table.numpy(), w.context_lens)[..., 1:]
+    cache = helpers.gpu_fill(w, dtype=kind)
+    out, ws = helpers.gpu_decode(w, cache)
+    outs = [torch.full_like(out, float("nan")) for _ in range(2)]          # layers in one launch
+    layers = binding.LayerSet([{"cache": cache, "q": w.q.cuda(), "out": o} for o in outs])
+    plan = torch.empty(binding.plan_bytes(w.batch, 2, w.block_table.shape[1]), dtype=torch.uint8, device="cuda")
+    binding.decode_layers(layers, w.block_table.cuda(), w.context_lens_tensor.cuda(), 6, w.sm_scale, plan, ws)
+    assert torch.equal(outs[0], out) and torch.equal(outs[1], out)
+    chunked = helpers.gpu_decode(w, cache, chunk_size=32)[0]
+    for got in (out, chunked):
+        off = np.abs(got.double().cpu().numpy()[..., 1:] - ref)
+        assert np.all(off <= (2.0 ** -8 + 2.0 ** -11) * ref), np.max(off / ref)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_an_infinite_value_is_an_infinite_result(d):
+    """An E5M2 cache that comes from elsewhere may hold infinities (the write saturates).  One in V at a valid token makes its
+    dim's result infinite and no other, wherever the context ends behind it, for one layer and for several in a launch."""
+    lens = [1, 5, 16, 17, 20, 32, 33, 48, 80, 700]
+    w = workloads.make_workload("infinite", lens, 6, 2, d, seed=d, outliers=False)
+    w.q.mul_(0.25)                                                         # every probability is an f16 number
+    cache = helpers.gpu_fill(w, dtype=binding.KV_FP8_E5M2)
+    clean, ws = helpers.gpu_decode(w, cache)
+    at = [binding.cache_offset(cache, int(w.block_table[b, (L - 1) // 16]), g, 1, (L - 1) % 16, 3 + g) for b, L in enumerate(lens) for g in range(2)]
+    cache.data[torch.tensor(at, device="cuda")] = torch.tensor([0x7C, 0xFC] * len(lens), dtype=torch.uint8, device="cuda")
+    want = clean.clone()
+    want[:, :3, 3], want[:, 3:, 4] = float("inf"), float("-inf")
+    table, lens_t = w.block_table.cuda(), w.context_lens_tensor.cuda()
+    assert torch.equal(binding.paged_decode(cache, w.q.cuda(), table, lens_t, w.sm_scale, ws), want)
+    outs = [torch.full_like(clean, float("nan")) for _ in range(2)]        # layers in one launch
+    layers = binding.LayerSet([{"cache": cache, "q": w.q.cuda(), "out": o} for o in outs])
+    plan = torch.empty(binding.plan_bytes(w.batch, 2, table.shape[1]), dtype=torch.uint8, device="cuda")
+    binding.decode_layers(layers, table, lens_t, 6, w.sm_scale, plan, ws)
+    assert torch.equal(outs[0], want) and torch.equal(outs[1], want)
