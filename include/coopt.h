@@ -326,6 +326,16 @@ int coopt_chunk_partials(int32_t batch, int32_t num_q_heads, int32_t head_dim, i
                          int32_t* max_chunks);
 
 /*
+ * coopt_selftest_layers_launch -- diagnostic: for every layer of a coopt_decode_layers call, how many layers its
+ * launch takes and whether that launch may begin ahead of the kernel in front of it (the call's own planning kernel,
+ * for the first).  Host arithmetic only: the pointers are compared, and nothing is enqueued.
+ *   layers_of_launch, early   HOST int32 [num_layers]; the other arguments as for coopt_decode_layers
+ */
+int coopt_selftest_layers_launch(const coopt_layer_io* layers, int32_t num_layers, int64_t kv_token_stride, const int32_t* block_table,
+                                 int32_t max_blocks_per_seq, const int32_t* context_lens, int32_t batch, int32_t num_q_heads,
+                                 size_t workspace_bytes, uint32_t flags, int32_t* layers_of_launch, int32_t* early);
+
+/*
  * coopt_selftest_bounded_wait -- diagnostic: one warp waits on a barrier that never completes, with the
  * same bounded wait every role of the attention kernels uses (a 2 s limit there), and gives up after
  * about limit_ns nanoseconds (1 .. 100,000,000).  The paper has no counterpart.  On return from the

@@ -87,6 +87,9 @@ _SIGNATURES = {
                                            ctypes.c_int32, ctypes.c_void_p, ctypes.c_int32, ctypes.c_int32, ctypes.c_float,
                                            ctypes.c_void_p, ctypes.c_size_t, ctypes.c_void_p, ctypes.c_size_t, ctypes.c_uint32,
                                            ctypes.c_void_p]),
+    "coopt_selftest_layers_launch": (ctypes.c_int, [ctypes.POINTER(coopt_layer_io), ctypes.c_int32, ctypes.c_int64, ctypes.c_void_p,
+                                                    ctypes.c_int32, ctypes.c_void_p, ctypes.c_int32, ctypes.c_int32, ctypes.c_size_t,
+                                                    ctypes.c_uint32, ctypes.c_void_p, ctypes.c_void_p]),
     "coopt_selftest_bounded_wait": (ctypes.c_int, [ctypes.c_uint64, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]),
     "coopt_status_string": (ctypes.c_char_p, [ctypes.c_int]),
     "coopt_version": (ctypes.c_int, []),

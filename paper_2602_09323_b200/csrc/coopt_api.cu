@@ -203,6 +203,25 @@ static bool layers_are_apart(const coopt_layer_io* layers, int num_layers, int64
   return true;
 }
 
+// Layers that the next launch of a coopt_decode_layers call takes, of `left` (of one shape, the first of the call if `first`),
+// and whether it may begin ahead of the kernel before it (the planning kernel, if it is the call's first).
+struct LayersLaunch {
+  int layers;
+  bool early;
+};
+static LayersLaunch next_layers(const coopt_layer_io* layers, int left, bool first, int64_t kv_token_stride, const int32_t* block_table,
+                                int max_blocks_per_seq, const int32_t* context_lens, int batch, int num_q_heads, size_t workspace_bytes, bool overlap) {
+  const coopt_cache& c = *layers[0].cache;
+  // Layers whose buffers are apart go into one launch, up to eight: what a launch costs once is then shared, and the pieces of a
+  // layer are merged while the blocks of the next are under way.  (Apart / together: eight layers of 8 sequences of 1..28
+  // tokens 53 / 11.4 us; three of 54 of 4072..8144, G = 2, 185 / 171; four of 24 of 300..4000, G = 8, 96.8 / 93.2.)
+  int n = std::min(left, kManyLayers);
+  while (n > 1 && workspace_bytes < workspace_need(batch, num_q_heads, c.num_kv_heads, c.head_dim, max_blocks_per_seq, 0, n)) --n;
+  auto apart = [&](int n) { return layers_are_apart(layers, n, kv_token_stride, block_table, max_blocks_per_seq, context_lens, batch, num_q_heads); };
+  if (n > 1 && !apart(n)) n = 1;
+  return {n, first ? n > 1 || apart(1) : overlap};
+}
+
 }  // namespace coopt
 
 using namespace coopt;
@@ -391,29 +410,37 @@ int coopt_decode_layers(const coopt_layer_io* layers, int32_t num_layers, int64_
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   rc = launch_decode_plan(block_table, max_blocks_per_seq, context_lens, batch, c0->num_kv_heads, c0->num_blocks, 0, plan, st);
   for (int32_t l = 0; l < num_layers && rc == COOPT_OK;) {
-    // Layers whose buffers are apart go into one launch, up to eight: what a launch costs once is then shared, and the pieces of a
-    // layer are merged while the blocks of the next are under way.  (Apart / together: eight layers of 8 sequences of 1..28
-    // tokens 53 / 11.4 us; three of 54 of 4072..8144, G = 2, 185 / 171; four of 24 of 300..4000, G = 8, 96.8 / 93.2.)
-    int n = std::min(num_layers - l, kManyLayers);
-    while (n > 1 && workspace_bytes < workspace_need(batch, num_q_heads, c0->num_kv_heads, c0->head_dim, max_blocks_per_seq, 0, n)) --n;
-    const bool apart = layers_are_apart(layers + l, n, kv_token_stride, block_table, max_blocks_per_seq, context_lens, batch, num_q_heads);
-    if (!apart) n = 1;
-    DecodeCall a = attention_call(layers + l, n, max_blocks_per_seq, batch, num_q_heads, 0, sm_scale, workspace);
+    const LayersLaunch next = next_layers(layers + l, num_layers - l, l == 0, kv_token_stride, block_table, max_blocks_per_seq, context_lens, batch,
+                                          num_q_heads, workspace_bytes, (flags & COOPT_FLAG_OVERLAP_PREVIOUS) != 0);
+    DecodeCall a = attention_call(layers + l, next.layers, max_blocks_per_seq, batch, num_q_heads, 0, sm_scale, workspace);
     a.kv_token_stride = kv_token_stride;
-    if (l == 0 && apart) {
+    if (next.early) a.order = kOverlapPrevious;
+    if (l == 0 && next.early) {
       // behind the planning kernel, which copies lengths and table: this launch reads them where it read them
       a.block_table = block_table;
       a.context_lens = context_lens;
-      a.order = kOverlapPrevious;
     } else {
-      a.plan = plan;
-      // the layers before may still drain while this launch reads the plan and its own caches
-      if (l > 0 && (flags & COOPT_FLAG_OVERLAP_PREVIOUS) != 0) a.order = kOverlapPrevious;
+      a.plan = plan;                     // (early: the layers before may still drain while this launch reads the plan and its own caches)
     }
     rc = launch_decode(a, st);
-    l += n;
+    l += next.layers;
   }
   return rc;
+}
+
+int coopt_selftest_layers_launch(const coopt_layer_io* layers, int32_t num_layers, int64_t kv_token_stride, const int32_t* block_table,
+                                 int32_t max_blocks_per_seq, const int32_t* context_lens, int32_t batch, int32_t num_q_heads,
+                                 size_t workspace_bytes, uint32_t flags, int32_t* layers_of_launch, int32_t* early) {
+  if (!layers || num_layers <= 0 || !layers_of_launch || !early) return COOPT_ERR_INVALID_ARG;
+  for (int32_t l = 0; l < num_layers;) {
+    const LayersLaunch next = next_layers(layers + l, num_layers - l, l == 0, kv_token_stride, block_table, max_blocks_per_seq, context_lens, batch,
+                                          num_q_heads, workspace_bytes, (flags & COOPT_FLAG_OVERLAP_PREVIOUS) != 0);
+    for (int32_t k = 0; k < next.layers; ++k, ++l) {
+      layers_of_launch[l] = next.layers;
+      early[l] = next.early ? 1 : 0;
+    }
+  }
+  return COOPT_OK;
 }
 
 int coopt_paged_chunked(const coopt_cache* cache, const void* q, void* out, const int32_t* cu_q_lens,

@@ -128,3 +128,35 @@ def test_sizes_and_host_side_argument_checks(lib):
     assert lib.coopt_paged_chunked(ctypes.byref(good), 0x100, 0x100, 0x100, 0x100, 8, 0x100, 2, 4, 2, 100, 1, 0.1,
                                    0x100, 1 << 30, None) == -1                                           # chunk % 16
     assert lib.coopt_workspace_init(None, 0, None) == -1 and lib.coopt_workspace_init(0x100, 8, None) == -3
+
+
+@pytest.mark.parametrize("width", [8, 640])
+def test_which_layers_share_a_launch_and_which_launches_begin_early(lib, width):
+    """Twelve layers of 64 sequences, 8 kv heads, in a short block table and in a wide one (2,200 blocks a multiprocessor): apart, chained (a
+    layer's output is the next one's query), with an output in the block table, and in the workspace that the library asks for."""
+    n, batch, hq, hkv, d = 12, 64, 40, 8, 128
+    caches = [binding.coopt_cache((1 << 40) + (y << 32), 1000, hkv, d, 16, 0) for y in range(n)]
+    table, lens = 1 << 30, 1 << 31
+
+    def ask(how, flags=0, room=1 << 40):
+        io = (binding.coopt_layer_io * n)()
+        for y in range(n):
+            io[y].cache = ctypes.pointer(caches[y])
+            io[y].q, io[y].out = (1 << 50) + (y << 30), (1 << 51) + (y << 30)
+            if how == "chained" and y:
+                io[y].q = io[y - 1].out
+        if how == "in the table":
+            io[0].out = table
+        took, early = (ctypes.c_int32 * n)(), (ctypes.c_int32 * n)()
+        assert lib.coopt_selftest_layers_launch(io, n, hkv * d, table, width, lens, batch, hq, room, flags, took, early) == 0
+        return list(took), list(early)
+
+    overlap = binding.FLAG_OVERLAP_PREVIOUS
+    assert ask("apart") == ([8] * 8 + [4] * 4, [1] * 8 + [0] * 4)
+    assert ask("apart", overlap) == ([8] * 8 + [4] * 4, [1] * n)
+    assert ask("chained") == ([1] * 8 + [1] * 4, [1] + [0] * 11)          # the first launch begins early all the same
+    assert ask("chained", overlap) == ([1] * n, [1] * n)
+    assert ask("in the table") == ([1] + [8] * 8 + [3] * 3, [0] * n)
+    one = lib.coopt_workspace_bytes(batch, hq, hkv, d, width, 0, batch)
+    assert ask("apart", room=one)[0] == [8] * 8 + [4] * 4
+    assert lib.coopt_selftest_layers_launch(None, n, 0, table, width, lens, batch, hq, one, 0, None, None) == -1
