@@ -144,7 +144,10 @@ __device__ __forceinline__ void arrive_one(uint64_t* bar) {
   asm volatile("{\n .reg .pred q;\n elect.sync _|q, 0xffffffff;\n @q mbarrier.arrive.shared::cta.b64 _, [%0];\n}" ::"r"(smem_u32(bar)) : "memory");
 }
 
-template <int D, bool kE5m2>
+// kTurns: the two tiles of a CTA take turns at the exponentials.  A launch with one tile a CTA has a kernel without that code, which
+// nothing waits in there but which costs all the same (256 new tokens behind 2 x 8192, G = 8, 115.4 / 113.2 us; 24 sequences of
+// 335..671 tokens, one head, 23.8 / 23.4).
+template <int D, bool kE5m2, bool kTurns>
 __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const PrefillParams p, const __grid_constant__ CUtensorMap map_part,
                                                                     const __grid_constant__ CUtensorMap map_hdr) {
   using C = Cfg<D>;
@@ -438,7 +441,7 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
       // behind tile 0's h, as long as the other tile has such a half.  Side by side they would each take twice as long, and then
       // leave the units idle while both load logits and look for the maximum.
       const int turn = x == 0 ? h - 1 : h;
-      if (turn >= 0 && turn < other_halves) ok = wait_warp(&bar_turn[4 * (1 - x) + (warp & 3)], turn & 1u, abort_flag);
+      if (kTurns && turn >= 0 && turn < other_halves) ok = wait_warp(&bar_turn[4 * (1 - x) + (warp & 3)], turn & 1u, abort_flag);
       if (!ok) break;
       // p * pv = 2^(s * cf - m + log2 pv): the V scale rides in the exponent, and a block's sum of p is recovered from the sum
       // of p * pv (pv: the block's V scale over the reference, at most 2^4, a zero one replaced by 2^-24)
@@ -464,7 +467,7 @@ __global__ void __launch_bounds__(kThreads, 1) paged_prefill_kernel(const Prefil
           const float2 u = f32_both(add2(add2(add2(y[0], y[1]), add2(y[2], y[3])), add2(add2(y[4], y[5]), add2(y[6], y[7]))));
           l_row += (u.x + u.y) * (c == 0 ? inv.x : c == 1 ? inv.y : c == 2 ? inv.z : inv.w);
         }
-        if (i == 1) arrive_one(&bar_turn[4 * x + (warp & 3)]);       // (ahead of the store: behind it 394 us, here 385)
+        if (kTurns && i == 1) arrive_one(&bar_turn[4 * x + (warp & 3)]);       // (ahead of the store: behind it 394 us, here 385)
         tmem_st16(s_cols + kHalf * buf + 16 * i, pw);
       }
       tmem_st_wait();
@@ -776,8 +779,11 @@ int launch_one(const coopt_cache* c, const PrefillParams& p, dim3 grid, cudaStre
   const long long granules = static_cast<long long>(c->num_blocks) * c->num_kv_heads;
   if (!encode_cache_map(&map_part, c->data, granules, C::kGran, C::kPart / 8) || !encode_cache_map(&map_hdr, c->data, granules, C::kGran, kFp8Header / 8))
     return COOPT_ERR_CUDA;
-  if (!configure_kernel_smem(reinterpret_cast<const void*>(&paged_prefill_kernel<D, kE5m2>), C::kSmemBytes)) return COOPT_ERR_CUDA;
-  return launch_dependent(paged_prefill_kernel<D, kE5m2>, grid, kThreads, C::kSmemBytes, stream, p, map_part, map_hdr) ? COOPT_OK : COOPT_ERR_CUDA;
+  auto launch = [&](auto* kernel) {
+    if (!configure_kernel_smem(reinterpret_cast<const void*>(kernel), C::kSmemBytes)) return COOPT_ERR_CUDA;
+    return launch_dependent(kernel, grid, kThreads, C::kSmemBytes, stream, p, map_part, map_hdr) ? COOPT_OK : COOPT_ERR_CUDA;
+  };
+  return p.tiles == 2 ? launch(&paged_prefill_kernel<D, kE5m2, true>) : launch(&paged_prefill_kernel<D, kE5m2, false>);
 }
 
 }  // namespace

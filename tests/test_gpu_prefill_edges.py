@@ -106,3 +106,16 @@ def test_on_both_sides_of_as_many_tiles_as_multiprocessors(d, more):
     """16 queries a tile; the launch reckons with one tile more than the sequence fills."""
     n = 16 * (torch.cuda.get_device_properties(0).multi_processor_count - 1 + more)
     _check([n + 5], [n], 8, 1, d, seed=more)
+
+
+@pytest.mark.parametrize("causal", [True, False])
+@pytest.mark.parametrize("hkv,d", [(20, 64), (20, 128), (2, 64), (2, 128)])
+def test_runs_of_one_to_five_tiles_with_and_without_turns(hkv, d, causal):
+    """From the start of their context and behind others: with twenty kv heads a CTA has two tiles, which take turns at the
+    exponentials, as long and unequally long as they come; with two it has one, by another kernel.  (Without loud channels: at
+    head_dim 128 a logit's error is up to sm_scale 2^-17 max|q| sum|k|, with them 2^-17 * 80 * 160 / 11.3 = 0.009 of a
+    probability, and of values of 80 among 4.8 million one is off by 0.05; without 2^-17 * 5.5 * 130 / 11.3 = 0.0005.)"""
+    def mutate(w):
+        for x in (w.q, w.k, w.v):
+            x.clamp_(-5.5, 5.5)
+    _check([64, 65, 128, 300, 300, 500], [64, 65, 128, 129, 300, 257], 2 * hkv, hkv, d, causal=causal, seed=d + hkv, mutate=mutate)
