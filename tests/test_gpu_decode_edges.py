@@ -302,3 +302,95 @@ def test_an_infinite_value_is_an_infinite_result(d):
     plan = torch.empty(binding.plan_bytes(w.batch, 2, table.shape[1]), dtype=torch.uint8, device="cuda")
     binding.decode_layers(layers, table, lens_t, 6, w.sm_scale, plan, ws)
     assert torch.equal(outs[0], want) and torch.equal(outs[1], want)
+
+
+@pytest.mark.parametrize("hq,hkv,d,fmt", [(64, 8, 128, "e4m3"), (16, 8, 128, "e5m2"), (64, 8, 64, "e4m3")])
+def test_long_layers_in_one_launch_equal_layers_one_by_one(hq, hkv, d, fmt):
+    """Three layers of 64 sequences in block tables of 128 columns, 440 blocks a multiprocessor: units cut between warps and CTAs
+    in every layer, with appended tokens.  All sequences have their first 95 blocks in common, and what follows to themselves."""
+    B, shared, width, n = 64, 95, 128, 3
+    gen = torch.Generator("cuda").manual_seed(hq + d)
+    draw = lambda *shape: torch.randn(*shape, generator=gen, device="cuda").to(torch.bfloat16)
+    lens = [shared * 16 + 1 + (37 * b) % (16 * (width - shared)) for b in range(B)]
+    own = width - shared
+    table = torch.full((B, width), -1, dtype=torch.int32)
+    for b, L in enumerate(lens):
+        table[b, :shared] = torch.arange(shared)
+        k = -(-L // 16) - shared
+        table[b, shared:shared + k] = shared + own * b + torch.arange(k)
+    blocks = shared + own * B
+    table, lens_t = table.cuda(), torch.tensor(lens, dtype=torch.int32).cuda()
+    last = lens_t.long() - 1
+    slots = table.gather(1, (last // 16)[:, None])[:, 0].long() * 16 + last % 16
+    kind = {"e4m3": binding.KV_FP8_E4M3, "e5m2": binding.KV_FP8_E5M2}[fmt]
+    ws = binding.new_workspace(B, hq, hkv, d, width)
+    ios, want, want_bytes = [], [], []
+    for y in range(n):
+        cache = binding.Cache(blocks, hkv, d, kind)
+        binding.kv_write(cache, draw(blocks * 16, hkv, d), draw(blocks * 16, hkv, d), torch.arange(blocks * 16, device="cuda"))
+        io = {"cache": cache, "q": draw(B, hq, d), "out": torch.full((B, hq, d), float("nan"), dtype=torch.bfloat16, device="cuda"),
+              "k_new": draw(B, hkv, d), "v_new": draw(B, hkv, d), "slot_mapping": slots}
+        twin = binding.Cache(blocks, hkv, d, kind)
+        twin.data.copy_(cache.data)
+        binding.kv_write(twin, io["k_new"], io["v_new"], slots)
+        want.append(binding.paged_decode(twin, io["q"], table, lens_t, d ** -0.5, ws))
+        want_bytes.append(twin.data)
+        ios.append(io)
+    plan = torch.empty(binding.plan_bytes(B, hkv, width), dtype=torch.uint8, device="cuda")
+    for keys in (set(ios[0]), {"cache", "q", "out"}):                       # with the new tokens, and over what they have left
+        layer_set = binding.LayerSet([{k: v for k, v in io.items() if k in keys} for io in ios])
+        for io in ios:
+            io["out"].fill_(float("nan"))
+        binding.decode_layers(layer_set, table, lens_t, hq, d ** -0.5, plan, ws)
+        torch.cuda.synchronize()
+        assert binding.workspace_status(ws) == 0
+        for y, io in enumerate(ios):
+            assert torch.equal(io["out"], want[y]), f"layer {y}: outputs"
+            assert torch.equal(io["cache"].data, want_bytes[y]), f"layer {y}: cache bytes"
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_bf16_values_past_the_context_do_not_count(d):
+    lens = [1, 5, 16, 17, 31, 33, 47, 700, 2049]
+    w = workloads.make_workload("past the end", lens, 6, 2, d, seed=d)
+    cache = helpers.gpu_fill(w, dtype=binding.KV_BF16)
+    out, ws = helpers.gpu_decode(w, cache)
+    raw = cache.data.view(torch.int16)
+    at = [binding.cache_offset(cache, int(w.block_table[b, (L - 1) // 16]), g, which, t, e) // 2
+          for b, L in enumerate(lens) for g in range(2) for which in (0, 1) for t in range((L - 1) % 16 + 1, 16) for e in range(d)]
+    raw[torch.tensor(at, device="cuda")] = 0x7FC0                           # no number
+    assert torch.equal(binding.paged_decode(cache, w.q.cuda(), w.block_table.cuda(), w.context_lens_tensor.cuda(), w.sm_scale, ws), out)
+    assert torch.equal(helpers.gpu_decode(w, cache, chunk_size=512)[0][:7], out[:7])      # contexts of a single chunk
+
+
+@pytest.mark.parametrize("fmt", ["e4m3", "e5m2"])
+@pytest.mark.parametrize("d", [64, 128])
+def test_a_token_appended_in_front_of_codes_that_are_no_numbers(d, fmt):
+    """The one-launch step adds a token to a block whose later slots hold codes that are no numbers: output and cache bytes
+    are those of the write followed by the decode, the later slots' codes among them."""
+    lens = [2, 5, 16, 18, 31, 33, 47, 50, 63, 700, 2049]                   # (2049: the token begins its block, which is cleared)
+    kind = {"e4m3": binding.KV_FP8_E4M3, "e5m2": binding.KV_FP8_E5M2}[fmt]
+    w = workloads.make_workload("append in front", lens, 6, 2, d, seed=d)
+    hist = np.concatenate([np.arange(w.kv_offsets[b], w.kv_offsets[b] + L - 1) for b, L in enumerate(lens)])
+    new = torch.tensor([w.kv_offsets[b] + L - 1 for b, L in enumerate(lens)])
+    # K and V that are small next to the block's scale, so that the write leaves the scale and the other codes as they are
+    k_new, v_new, slots = (w.k[new] * 0.01).cuda(), (w.v[new] * 0.01).cuda(), w.slot_mapping[new].cuda()
+    table, lens_t = w.block_table.cuda(), w.context_lens_tensor.cuda()
+    caches = [helpers.gpu_fill(w, dtype=kind, calls=[hist]) for _ in range(3)]
+    at = [binding.cache_offset(caches[0], int(w.block_table[b, (L - 1) // 16]), g, which, t, e)
+          for b, L in enumerate(lens) for g in range(2) for which in (0, 1) for t in range((L - 1) % 16 + 1, 16) for e in range(d)]
+    for c in caches:
+        c.data[torch.tensor(at, device="cuda")] = 0x7F
+    ws = binding.new_workspace(w.batch, 6, 2, d, table.shape[1])
+    binding.kv_write(caches[0], k_new, v_new, slots)
+    want = binding.paged_decode(caches[0], w.q.cuda(), table, lens_t, w.sm_scale, ws)
+    assert torch.isfinite(want.float()).all()
+    plan = binding.decode_plan(table, lens_t, 2, w.num_blocks)
+    got = binding.decode_step_planned(caches[1], plan, w.q.cuda(), table.shape[1], w.sm_scale, ws, k_new, v_new, slots)
+    assert torch.equal(got, want) and torch.equal(caches[1].data, caches[0].data)
+    outs = [torch.full_like(want, float("nan")) for _ in range(2)]         # two layers in one launch, one of which appends
+    layers = binding.LayerSet([{"cache": caches[0], "q": w.q.cuda(), "out": outs[0]},
+                               {"cache": caches[2], "q": w.q.cuda(), "out": outs[1], "k_new": k_new, "v_new": v_new, "slot_mapping": slots}])
+    layers.kv_stride = 2 * d
+    binding.decode_layers(layers, table, lens_t, 6, w.sm_scale, plan, ws)
+    assert torch.equal(outs[0], want) and torch.equal(outs[1], want) and torch.equal(caches[2].data, caches[0].data)
