@@ -253,13 +253,16 @@ int coopt_decode_step_planned(const coopt_cache* cache, const void* plan, size_t
 
 /*
  * coopt_decode_layers -- the decode loop of Section 2 over the layers of a model for one step: one plan,
- * then the layers' fused steps, enqueued back to back on `stream`: a launch per layer, or one for up to eight
- * layers whose buffers are apart where a layer is small.  Results are those of one call per layer.
+ * then the layers' fused steps, enqueued back to back on `stream`.  Up to eight layers that follow one another,
+ * of any size, share a launch and may run at the same time if their buffers are apart (nothing that one of them
+ * writes is read or written by another, or part of the block table or the context lengths) and the workspace has
+ * room for their pieces (coopt_workspace_bytes says how much eight need), whatever the flags; other layers run one
+ * after the other.  Results are those of one call per layer.
  *   layers        HOST array of num_layers entries; every pointer inside is DEVICE memory: the layer's cache
  *                 (all of one shape), its new token's k/v and slots (all NULL = no append), its q and out
  *   block_table, context_lens, plan, workspace   shared by all layers
- *   flags         COOPT_FLAG_OVERLAP_PREVIOUS lets layer l + 1 start while layer l drains (it reads only the
- *                 plan and its own cache until layer l has finished)
+ *   flags         COOPT_FLAG_OVERLAP_PREVIOUS lets a launch start while the launch of the layers before it drains (it
+ *                 reads only the plan and its own caches until that one has finished)
  * Errors: as the calls it makes; every argument of every layer is checked before anything is launched.
  */
 typedef struct coopt_layer_io {

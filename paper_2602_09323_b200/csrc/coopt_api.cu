@@ -213,8 +213,10 @@ static LayersLaunch next_layers(const coopt_layer_io* layers, int left, bool fir
                                 int max_blocks_per_seq, const int32_t* context_lens, int batch, int num_q_heads, size_t workspace_bytes, bool overlap) {
   const coopt_cache& c = *layers[0].cache;
   // Layers whose buffers are apart go into one launch, up to eight: what a launch costs once is then shared, and the pieces of a
-  // layer are merged while the blocks of the next are under way.  (Apart / together: eight layers of 8 sequences of 1..28
-  // tokens 53 / 11.4 us; three of 54 of 4072..8144, G = 2, 185 / 171; four of 24 of 300..4000, G = 8, 96.8 / 93.2.)
+  // layer are merged while the blocks of the next are under way.  (Apart / together, us: eight layers of 8 sequences of 1..28
+  // tokens 71 / 10.1; three of 54 of 4072..8144, G = 2, 185 / 174; four of 24 of 300..4000, G = 8, 101.5 / 89.4; four of 32 x
+  // 8192, G = 6, 7 and 8, 374 / 358, 376 / 359 and 377 / 360; head_dim 64, 64 of 100..5000, G = 4, four layers of eight kv heads
+  // 153.5 / 141.9, eight layers of four 203 / 181.)
   int n = std::min(left, kManyLayers);
   while (n > 1 && workspace_bytes < workspace_need(batch, num_q_heads, c.num_kv_heads, c.head_dim, max_blocks_per_seq, 0, n)) --n;
   auto apart = [&](int n) { return layers_are_apart(layers, n, kv_token_stride, block_table, max_blocks_per_seq, context_lens, batch, num_q_heads); };

@@ -79,8 +79,8 @@ struct LayerPtrs {
   const __nv_bfloat16* v_new;
   const long long* slot_mapping;
 };
-// A launch serves one layer, or up to kManyLayers whose buffers do not touch each other (every one has room of its own for
-// its pieces in the workspace; what a launch costs once is small against eight layers).
+// A launch serves one layer, or up to kManyLayers of any size whose buffers do not touch each other (every one has room of its
+// own for its pieces in the workspace; what a launch costs once is small against eight layers).
 constexpr int kManyLayers = 8;
 template <int L>
 struct LayerTable {
