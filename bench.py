@@ -723,7 +723,7 @@ def run_layers(args):
 
 # dram__bytes_read.sum + dram__bytes_write.sum of one decode launch on this workload, from the
 # ncu capture summarised under profiles/ (None while the kernel is newer than the capture).
-DRAM_TRAFFIC_PER_LAUNCH = 139022592 + 5901312   # dram__bytes_read.sum + dram__bytes_write.sum of one launch (profiles/)
+DRAM_TRAFFIC_PER_LAUNCH = 139028736 + 4793088   # dram__bytes_read.sum + dram__bytes_write.sum of one launch (profiles/)
 
 if __name__ == "__main__":
     main()
